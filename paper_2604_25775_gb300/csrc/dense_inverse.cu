@@ -22,6 +22,7 @@
 
 #include <algorithm>
 
+#include "fp64_mma.cuh"
 #include "scale_internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -554,38 +555,596 @@ cudaError_t run_gj(cudaStream_t st, TW* mats, int n, int B, const int32_t* list,
   return cudaGetLastError();
 }
 
+// ---- FP64 elimination with the rank-16 updates on the tensor cores -------------------------
+// Gauss-Jordan in blocks of 16 pivots, the products of a block taken as split FP16 products
+// (fp64_mma.cuh): of the 16 DFMA per element and block one rounded FP64 addition is left. Pivot
+// choices, the panel's elimination and every stored value are FP64.
+//
+//  (1) Panel: LU with partial pivoting of the block's 16 columns, one thread per row, the row in
+//      registers; the inverse's earlier pivot rows take the same steps. Pivot: the largest
+//      |value| among the rows without a pivot, ties to the lowest row, by warp reductions on
+//      integer keys.
+//  (2) X = L11^-1 and (inverse) U11^-1 by warp 0, the column slices of the old pivot rows P by
+//      the other warps.
+//  (3) The left factor U = -L21 X of the rows without a pivot, U11^-1 X of the block's pivot rows,
+//      as split products (its fragment order is that of (4)'s operand, so it stays in registers);
+//      U is also the block's columns of the matrix after the sweep.
+//  (4) A[i][c] += sum_k U[i][k] P[k][c] outside the block, a pivot row starting from zero.
+//
+// Scales: rows of U by their largest exponent, columns of P per column; between the two, pivot
+// k's column of U is multiplied by the power of two that divides its row of P, the largest
+// exponent of that row of the input matrix, so that rows of very different size do not cost the
+// products of the small ones their low digits. A block whose factors hold an infinity, a NaN
+// or a scale far from 1 (2^+-100 for input rows, 2^+-200 inside the panel, 2^+-300 for the
+// columns: the products' exponents then stay in range) takes (3) and (4) in plain FP64.
+constexpr int kSW = 16;        // pivots per block = k of one mma
+constexpr int kSLd = kSW + 2;  // panel row stride in doubles: 16-byte rows without bank conflicts
+constexpr int kSTd = kSW + 1;  // row stride of the 16 x 16 blocks
+constexpr int kSCols = 224;    // columns whose slices are staged at a time
+constexpr int kSplitMaxN = 448;
+constexpr int kSMs = 152;
+
+struct SplitSmem {
+  size_t panel, tri, xs, xf, xe, prow, inv, bf, fexp, rexp, rho, piv, qinv, act, used, total;
+};
+__host__ __device__ inline SplitSmem split_smem(int n, int ch) {
+  SplitSmem s{};
+  size_t off = sizeof(double) * (size_t)((n + 1) & ~1);  // pabs
+  auto take = [&](size_t bytes) {
+    const size_t at = off;
+    off = (off + bytes + 15) & ~size_t(15);
+    return at;
+  };
+  s.panel = take(sizeof(double) * (size_t)n * kSLd);
+  s.tri = take(sizeof(double) * kSW * kSTd);
+  s.xs = take(sizeof(double) * kSW * kSTd);
+  s.xf = take((size_t)2 * kSplit * 32 * sizeof(uint2));
+  s.xe = take(sizeof(int) * kSW);
+  s.prow = take(sizeof(double) * kSW);
+  s.inv = take(sizeof(double) * kSW);
+  s.bf = take((size_t)(ch / 8) * kSplit * 32 * sizeof(uint2));
+  s.fexp = take(sizeof(int) * ch);
+  s.rexp = take(sizeof(int) * n);
+  s.rho = take(sizeof(int) * kSW);
+  s.piv = take(sizeof(int) * n);
+  s.qinv = take(sizeof(int) * n);
+  s.act = take(sizeof(int) * n);
+  s.used = take(n);
+  s.total = off;
+  return s;
+}
+
+__device__ __forceinline__ uint64_t dbits(double x) { return (uint64_t)__double_as_longlong(x); }
+
+// Exponent field within 2^+-lim of 1, or the value zero (also rejects infinities and NaN).
+__device__ __forceinline__ bool exp_near(int e, bool nonzero, int lim) {
+  return !nonzero || (e >= 1023 - lim && e <= 1023 + lim);
+}
+
+// Slices of the B fragment of one 8-column tile from the lane's values x[q] (row k = 2t + (q & 1)
+// + 8 (q >> 1) of the lane's column g) multiplied by 2^-rho_k; the column's scale to *fe (t == 0).
+// Returns whether the scale is usable.
+__device__ __forceinline__ bool split_column_tile(const uint64_t (&x)[4], const int* rho, uint2* bf, int* fe) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int2 r0 = *reinterpret_cast<const int2*>(rho + 2 * t), r1 = *reinterpret_cast<const int2*>(rho + 2 * t + 8);
+  int e = max(max(exp_scaled(x[0], -r0.x), exp_scaled(x[1], -r0.y)), max(exp_scaled(x[2], -r1.x), exp_scaled(x[3], -r1.y)));
+  int nz = ((x[0] | x[1] | x[2] | x[3]) << 1) != 0;
+#pragma unroll
+  for (int off = 1; off < 4; off <<= 1) {
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
+    nz |= __shfl_xor_sync(0xffffffffu, nz, off);
+  }
+  if (t == 0) fe[g] = e;
+  uint32_t s0[kSplit], s1[kSplit];
+  split_pair(split_fixed(x[0], e + r0.x), split_fixed(x[1], e + r0.y), s0);
+  split_pair(split_fixed(x[2], e + r1.x), split_fixed(x[3], e + r1.y), s1);
+#pragma unroll
+  for (int l = 0; l < kSplit; ++l) bf[l * 32 + lane] = make_uint2(s0[l], s1[l]);
+  return exp_near(e, nz != 0, 300);
+}
+
+// Slices of the A fragment of 16 rows from the lane's values v[q][0..1] (row g + 8 (q & 1), columns
+// 2t, 2t + 1 at q < 2 and 2t + 8, 2t + 9 at q >= 2) times 2^rho of their column; the scales of
+// the lane's two rows come back in ex.
+__device__ __forceinline__ void split_row_tile(const double (&v)[4][2], const int* rho, uint32_t (&a)[kSplit][4],
+                                               int (&ex)[2]) {
+  const int t = threadIdx.x & 3;
+  const int2 r0 = *reinterpret_cast<const int2*>(rho + 2 * t), r1 = *reinterpret_cast<const int2*>(rho + 2 * t + 8);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int e = max(max(exp_scaled(dbits(v[h][0]), r0.x), exp_scaled(dbits(v[h][1]), r0.y)),
+                max(exp_scaled(dbits(v[2 + h][0]), r1.x), exp_scaled(dbits(v[2 + h][1]), r1.y)));
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+    ex[h] = e;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int2 rk = q < 2 ? r0 : r1;
+    uint32_t s[kSplit];
+    split_pair(split_fixed(dbits(v[q][0]), ex[q & 1] - rk.x), split_fixed(dbits(v[q][1]), ex[q & 1] - rk.y), s);
+#pragma unroll
+    for (int l = 0; l < kSplit; ++l) a[l][q] = s[l];
+  }
+}
+
+// One matrix by one CTA of TH >= n threads.
+template <typename TOUT, bool kInverse, int TH>
+__device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats, int n, int ch, int b,
+                             TOUT* __restrict__ binv, double* __restrict__ logabs_out, int32_t* __restrict__ sign_out,
+                             int32_t* __restrict__ status) {
+  constexpr int NW = TH / 32;
+  const SplitSmem S = split_smem(n, ch);
+  double* pabs = reinterpret_cast<double*>(smem_raw);            // [n] |pivot| of column k
+  double* panel = reinterpret_cast<double*>(smem_raw + S.panel);  // [n][kSLd], row r = matrix row act[r]
+  double* tri = reinterpret_cast<double*>(smem_raw + S.tri);      // [16][kSTd] L11 below, U11 on and above the diagonal
+  double* xs = reinterpret_cast<double*>(smem_raw + S.xs);        // [16][kSTd] X = L11^-1
+  uint2* xf = reinterpret_cast<uint2*>(smem_raw + S.xf);          // its slices, two tiles
+  int* xe = reinterpret_cast<int*>(smem_raw + S.xe);              // [16] its column scales
+  double* prow = reinterpret_cast<double*>(smem_raw + S.prow);    // [16] the pivot row right of the pivot
+  double* inv = reinterpret_cast<double*>(smem_raw + S.inv);      // [16] reciprocal pivots
+  uint2* bf = reinterpret_cast<uint2*>(smem_raw + S.bf);          // [ch / 8][kSplit][32] slices of P
+  int* fexp = reinterpret_cast<int*>(smem_raw + S.fexp);          // [ch] column scales of P
+  int* rexp = reinterpret_cast<int*>(smem_raw + S.rexp);          // [n] exponent of the largest value of an input row
+  int* rho = reinterpret_cast<int*>(smem_raw + S.rho);            // [16] those of the block's pivot rows
+  int* piv = reinterpret_cast<int*>(smem_raw + S.piv);            // [n] pivot row of column k
+  int* qinv = reinterpret_cast<int*>(smem_raw + S.qinv);          // [n]
+  int* act = reinterpret_cast<int*>(smem_raw + S.act);            // [n] rows in work: all, or those without a pivot
+  unsigned char* used = smem_raw + S.used;                        // [n] 0, or 1 + block that pivoted the row
+  __shared__ uint4 cand[NW];
+  __shared__ int prr[kSW];  // panel rows of the block's pivots
+  __shared__ int s_wild, s_nact, s_sgn;
+
+  double* A = mats + (size_t)b * n * n;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+  const bool vec = (n & 1) == 0;  // rows of A start on 16 bytes
+
+  for (int i = tid; i < n; i += TH) {
+    used[i] = 0;
+    act[i] = i;
+  }
+  if (tid == 0) {
+    s_nact = n;
+    s_sgn = 1;
+  }
+  for (int i = warp; i < n; i += NW) {
+    int e = 0;
+    for (int c = lane; c < n; c += 32) e = max(e, exp_field(dbits(A[(size_t)i * n + c])));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) rexp[i] = (e == 0 || e == 2047) ? 0 : e - 1023;
+  }
+  __syncthreads();
+
+  bool singular = false;
+  for (int K0 = 0; K0 < n; K0 += kSW) {
+    const int w = min(kSW, n - K0), nact = s_nact;
+    const unsigned char blk = (unsigned char)(1 + K0 / kSW);
+    // (1) panel: thread r holds row act[r]
+    const int row = tid < nact ? act[tid] : -1;
+    const bool open = row >= 0 && !used[row];  // may become a pivot row
+    int own = -1;                              // the pivot this row became
+    double a[kSW];
+    {
+      const double* src = A + (size_t)max(row, 0) * n + K0;
+      if (vec && w == kSW) {
+#pragma unroll
+        for (int k = 0; k < kSW; k += 2) {
+          const double2 v = row >= 0 ? *reinterpret_cast<const double2*>(src + k) : make_double2(0.0, 0.0);
+          a[k] = v.x;
+          a[k + 1] = v.y;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < kSW; ++k) a[k] = (row >= 0 && k < w) ? src[k] : 0.0;
+      }
+    }
+    if (tid == 0) s_wild = 0;
+    if (tid < kSW * kSW) tri[(tid / kSW) * kSTd + tid % kSW] = tid / kSW == tid % kSW ? 1.0 : 0.0;
+    for (int q = TH + tid; q < kSW * kSW; q += TH) tri[(q / kSW) * kSTd + q % kSW] = q / kSW == q % kSW ? 1.0 : 0.0;
+    if (tid < kSW) {
+      inv[tid] = 1.0;
+      rho[tid] = 0;
+      prr[tid] = -1;
+    }
+#pragma unroll
+    for (int jj = 0; jj < kSW; ++jj) {
+      if (jj >= w || singular) continue;  // uniform
+      // the candidate of each warp: largest key (0: none; the key's upper word + 1, lower word)
+      const bool valid = open && own < 0;
+      const uint64_t key = dbits(a[jj]) & 0x7fffffffffffffffull;
+      const unsigned hi = valid ? (unsigned)(key >> 32) + 1u : 0u, lo = valid ? (unsigned)key : 0u;
+      const unsigned m1 = __reduce_max_sync(0xffffffffu, hi);
+      const unsigned m2 = __reduce_max_sync(0xffffffffu, hi == m1 ? lo : 0u);
+      const unsigned bal = __ballot_sync(0xffffffffu, hi == m1 && lo == m2);
+      if (lane == 0) cand[warp] = make_uint4(m1, m2, (unsigned)(warp * 32 + __ffs(bal) - 1), 0u);
+      __syncthreads();
+      const uint4 c = lane < NW ? cand[lane] : make_uint4(0u, 0u, 0u, 0u);
+      const unsigned g1 = __reduce_max_sync(0xffffffffu, c.x);
+      const unsigned g2 = __reduce_max_sync(0xffffffffu, c.x == g1 ? c.y : 0u);
+      const unsigned bal2 = __ballot_sync(0xffffffffu, lane < NW && c.x == g1 && c.y == g2);
+      const int rp = (int)__shfl_sync(0xffffffffu, c.z, __ffs(bal2) - 1);
+      // no row left, a zero column, or a NaN in it
+      if (g1 == 0u || (g1 == 1u && g2 == 0u) || g1 > 0x7ff00001u || (g1 == 0x7ff00001u && g2 != 0u)) {
+        singular = true;
+        continue;
+      }
+      if (warp == (rp >> 5)) {
+        const double pv = __shfl_sync(0xffffffffu, a[jj], rp & 31);
+        const double ip = __drcp_rn(pv);
+        if (lane == (rp & 31)) {
+          own = jj;
+#pragma unroll
+          for (int k = jj + 1; k < kSW; ++k) prow[k] = a[k];
+          inv[jj] = ip;
+          prr[jj] = rp;
+          piv[K0 + jj] = row;
+          used[row] = blk;
+          rho[jj] = rexp[row];
+          pabs[K0 + jj] = __longlong_as_double((long long)key);
+          if (dbits(pv) >> 63) s_sgn = -s_sgn;
+        }
+      }
+      __syncthreads();
+      if (row >= 0 && own < 0) {  // the inverse's earlier pivot rows too
+        const double l = a[jj] * inv[jj];
+        a[jj] = l;
+#pragma unroll
+        for (int k = jj + 1; k < kSW; ++k) a[k] = fma(-l, prow[k], a[k]);
+      }
+    }
+    if (singular) break;
+    const int c_lo = kInverse ? 0 : K0 + w;
+    if (c_lo >= n) break;  // determinant: the last block is done
+    if (own >= 0) {
+#pragma unroll
+      for (int k = 0; k < kSW; ++k) tri[own * kSTd + k] = a[k];
+    }
+    __syncthreads();
+    if (row >= 0 && own < 0) {
+      int e = 0;
+      uint64_t nz = 0;
+#pragma unroll
+      for (int k = 0; k < kSW; ++k) {
+        e = max(e, exp_scaled(dbits(a[k]), 0));
+        nz |= dbits(a[k]) << 1;
+      }
+      if (!exp_near(e, nz != 0, 200)) atomicOr(&s_wild, 1);
+#pragma unroll
+      for (int k = 0; k < kSW; k += 2) *reinterpret_cast<double2*>(panel + tid * kSLd + k) = make_double2(a[k], a[k + 1]);
+    }
+    if (tid < kSW && (rho[tid] > 100 || rho[tid] < -100)) atomicOr(&s_wild, 1);
+    // (2)
+    if (warp == 0) {
+      // lanes 0..15: column `lane` of L11^-1 by forward substitution; lanes 16..31 (inverse): column
+      // lane - 16 of U11^-1 by backward substitution, with every index reversed (i -> 15 - i)
+      const bool up = lane >= kSW;
+      const int col = up ? 2 * kSW - 1 - lane : lane;
+      const double* tp = up ? tri + (kSW - 1) * (kSTd + 1) : tri;
+      const int dir = up ? -1 : 1;
+      double x[kSW];
+#pragma unroll
+      for (int i = 0; i < kSW; ++i) x[i] = i == col ? 1.0 : 0.0;
+#pragma unroll
+      for (int s = 0; s < kSW; ++s) {
+        double l[kSW];
+#pragma unroll
+        for (int i = s + 1; i < kSW; ++i) l[i] = tp[dir * (i * kSTd + s)];
+        if (kInverse) x[s] *= up ? inv[kSW - 1 - s] : 1.0;
+#pragma unroll
+        for (int i = s + 1; i < kSW; ++i) x[i] = fma(-l[i], x[s], x[i]);
+      }
+      int e = 0;
+      uint64_t nz = 0;
+#pragma unroll
+      for (int i = 0; i < kSW; ++i) {
+        e = max(e, exp_scaled(dbits(x[i]), 0));
+        nz |= dbits(x[i]) << 1;
+      }
+      if ((kInverse || !up) && !exp_near(e, nz != 0, 200)) atomicOr(&s_wild, 1);
+      if (!up) {
+#pragma unroll
+        for (int i = 0; i < kSW; ++i) xs[i * kSTd + col] = x[i];
+      } else if (kInverse) {  // the pivot rows of (3): -U11^-1
+#pragma unroll
+        for (int i = 0; i < kSW; ++i)
+          if (prr[kSW - 1 - i] >= 0) panel[prr[kSW - 1 - i] * kSLd + kSW - 1 - col] = -x[i];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt) {
+        uint64_t v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = dbits(xs[(2 * t + (q & 1) + 8 * (q >> 1)) * kSTd + 8 * nt + g]);
+        split_column_tile(v, rho, xf + nt * kSplit * 32, xe + 8 * nt);
+      }
+    }
+    for (int cb = c_lo; cb < n; cb += ch) {
+      const int ncol = min(ch, n - cb), ntile = (ncol + 7) >> 3;
+      // column slices of the block's old pivot rows: a warp per 8-column tile (warp 0 joins late)
+      const int w0 = cb == c_lo ? (warp + NW - 1) % NW : warp;
+      for (int nt = w0; nt < ntile; nt += NW) {
+        const int c = cb + 8 * nt + g;
+        if (kInverse && (unsigned)(cb + 8 * nt - K0) < (unsigned)kSW) continue;
+        uint64_t x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int k = 2 * t + (q & 1) + 8 * (q >> 1);
+          x[q] = (k < w && c < n) ? dbits(A[(size_t)piv[K0 + k] * n + c]) : 0ull;
+        }
+        if (!split_column_tile(x, rho, bf + (size_t)nt * kSplit * 32, fexp + 8 * nt)) atomicOr(&s_wild, 1);
+      }
+      __syncthreads();
+      if (!s_wild) {
+        // strips of 16 rows in runs of column tiles; as many runs per strip as even out the warps
+        // best (a run's row slices cost about five tiles)
+        const int nstrip = (nact + 15) >> 4;
+        int cs = 1, best = 1 << 30;
+        for (int q = 1; q <= min(ntile, 8); ++q) {
+          const int cost = ((nstrip * q + NW - 1) / NW) * ((ntile + q - 1) / q + 5);
+          if (cost < best) {
+            best = cost;
+            cs = q;
+          }
+        }
+        const int per = (ntile + cs - 1) / cs;
+        for (int task = warp; task < nstrip * cs; task += NW) {
+          const int strip = task % nstrip, run = task / nstrip;
+          const int r0 = strip * 16 + g, r1 = r0 + 8;
+          const int i0 = r0 < nact ? act[r0] : 0, i1 = r1 < nact ? act[r1] : 0;
+          // rows to write; a pivot row of this block starts from zero (inverse) or is done with
+          const bool on0 = r0 < nact && (kInverse || !used[i0]), on1 = r1 < nact && (kInverse || !used[i1]);
+          const bool add0 = on0 && !(kInverse && used[i0] == blk), add1 = on1 && !(kInverse && used[i1] == blk);
+          double* A0 = A + (size_t)i0 * n;
+          double* A1 = A + (size_t)i1 * n;
+          uint32_t as[kSplit][4];
+          int ex[2];
+          float acc[kSplit][4];
+          // (3)
+          double u[4][2];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            double2 v = make_double2(0.0, 0.0);
+            if ((q & 1) ? on1 : on0)
+              v = *reinterpret_cast<const double2*>(panel + ((q & 1) ? r1 : r0) * kSLd + 2 * t + 8 * (q >> 1));
+            u[q][0] = v.x;
+            u[q][1] = v.y;
+          }
+          split_row_tile(u, rho, as, ex);
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) {
+            split_mma(acc, as, xf + nt * kSplit * 32);
+            const int2 f = *reinterpret_cast<const int2*>(xe + 8 * nt + 2 * t);
+            u[2 * nt][0] = -split_value(acc, 0, ex[0], f.x);
+            u[2 * nt][1] = -split_value(acc, 1, ex[0], f.y);
+            u[2 * nt + 1][0] = -split_value(acc, 2, ex[1], f.x);
+            u[2 * nt + 1][1] = -split_value(acc, 3, ex[1], f.y);
+          }
+          if (kInverse && run == 0 && cb == c_lo) {  // the block's columns after the sweep
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              double* dst = ((q & 1) ? A1 : A0) + K0;
+              const int c = 2 * t + 8 * (q >> 1);
+              if (!((q & 1) ? on1 : on0)) continue;
+              if (c < w) dst[c] = u[q][0];
+              if (c + 1 < w) dst[c + 1] = u[q][1];
+            }
+          }
+          split_row_tile(u, rho, as, ex);
+          // (4)
+          for (int nt = run * per; nt < min(ntile, (run + 1) * per); ++nt) {
+            if (kInverse && (unsigned)(cb + 8 * nt - K0) < (unsigned)kSW) continue;
+            const int cc = 8 * nt + 2 * t, c = cb + cc;
+            const bool in0 = c < n, in1 = c + 1 < n;
+            double v[4] = {0.0, 0.0, 0.0, 0.0};
+            if (vec) {
+              if (in0 && add0) {
+                const double2 q = *reinterpret_cast<const double2*>(A0 + c);
+                v[0] = q.x;
+                v[1] = q.y;
+              }
+              if (in0 && add1) {
+                const double2 q = *reinterpret_cast<const double2*>(A1 + c);
+                v[2] = q.x;
+                v[3] = q.y;
+              }
+            } else {
+              if (in0 && add0) v[0] = A0[c];
+              if (in1 && add0) v[1] = A0[c + 1];
+              if (in0 && add1) v[2] = A1[c];
+              if (in1 && add1) v[3] = A1[c + 1];
+            }
+            split_mma(acc, as, bf + (size_t)nt * kSplit * 32);
+            const int2 f = *reinterpret_cast<const int2*>(fexp + cc);
+            v[0] += split_value(acc, 0, ex[0], f.x);
+            v[1] += split_value(acc, 1, ex[0], f.y);
+            v[2] += split_value(acc, 2, ex[1], f.x);
+            v[3] += split_value(acc, 3, ex[1], f.y);
+            if (vec) {
+              if (on0 && in0) *reinterpret_cast<double2*>(A0 + c) = make_double2(v[0], v[1]);
+              if (on1 && in0) *reinterpret_cast<double2*>(A1 + c) = make_double2(v[2], v[3]);
+            } else {
+              if (on0 && in0) A0[c] = v[0];
+              if (on0 && in1) A0[c + 1] = v[1];
+              if (on1 && in0) A1[c] = v[2];
+              if (on1 && in1) A1[c + 1] = v[3];
+            }
+          }
+        }
+      } else {
+        // (3) and (4) in plain FP64: U takes the place of the panel rows (once per block: bit 1 of
+        // s_wild, which keeps the block's later chunks here), the old pivot rows are staged where
+        // the slices were
+        double* pr = reinterpret_cast<double*>(bf);  // [kSW][ch]
+        __syncthreads();
+        if (!(s_wild & 2)) {
+          for (int r = warp; r < nact; r += NW) {
+            double s = 0.0;
+            if (lane < kSW)
+              for (int k = 0; k < kSW; ++k) s -= panel[r * kSLd + k] * xs[k * kSTd + lane];
+            __syncwarp();
+            if (lane < kSW) {
+              panel[r * kSLd + lane] = s;
+              if (kInverse && lane < w) A[(size_t)act[r] * n + K0 + lane] = s;
+            }
+            __syncwarp();
+          }
+        }
+        for (int q = tid; q < w * ncol; q += TH) {
+          const int k = q / ncol, cc = q - k * ncol;
+          pr[k * ch + cc] = A[(size_t)piv[K0 + k] * n + cb + cc];
+        }
+        __syncthreads();
+        if (tid == 0) atomicOr(&s_wild, 2);
+        for (int r = warp; r < nact; r += NW) {
+          const int i = act[r];
+          if (!kInverse && used[i]) continue;
+          const bool add = !(kInverse && used[i] == blk);
+          for (int cc = lane; cc < ncol; cc += 32) {
+            const int c = cb + cc;
+            if (kInverse && (unsigned)(c - K0) < (unsigned)kSW) continue;
+            double v = add ? A[(size_t)i * n + c] : 0.0;
+            for (int k = 0; k < w; ++k) v += panel[r * kSLd + k] * pr[k * ch + cc];
+            A[(size_t)i * n + c] = v;
+          }
+        }
+      }
+      __syncthreads();
+    }
+    if (!kInverse && warp == 0) {  // the rows not yet pivoted, compacted in place
+      int m = 0;
+      for (int r0 = 0; r0 < nact; r0 += 32) {
+        const int i = r0 + lane < nact ? act[r0 + lane] : 0;
+        const bool on = r0 + lane < nact && !used[i];
+        const unsigned bal = __ballot_sync(0xffffffffu, on);
+        if (on) act[m + __popc(bal & ((1u << lane) - 1u))] = i;
+        m += __popc(bal);
+        __syncwarp();
+      }
+      if (lane == 0) s_nact = m;
+    }
+    __syncthreads();
+  }
+  __syncthreads();
+
+  const double logdet = warp == 0 ? sum_log_pivots(pabs, n, singular) : 0.0;  // on thread 0
+  if (tid == 0) {
+    int st = 0;
+    double la = logdet;
+    int sg = s_sgn;
+    if (singular) {
+      st = SCALE_SAMPLE_SINGULAR;
+      la = -INFINITY;
+      sg = 0;
+    } else {
+      // sign of the permutation k -> piv[k]
+      for (int k = 0; k < n; ++k) qinv[k] = 0;
+      int parity = 0;
+      for (int k = 0; k < n; ++k) {
+        if (qinv[k]) continue;
+        int j = k, len = 0;
+        while (!qinv[j]) {
+          qinv[j] = 1;
+          j = piv[j];
+          ++len;
+        }
+        parity += len - 1;
+      }
+      if (parity & 1) sg = -sg;
+    }
+    if (logabs_out) logabs_out[b] = la;
+    if (sign_out) sign_out[b] = sg;
+    if (status && st) status[b] |= st;
+  }
+  if (!kInverse) return;
+  __syncthreads();
+  if (singular) {
+    if (binv)
+      for (int q = tid; q < n * n; q += TH) binv[(size_t)b * n * n + q] = TOUT(0);
+    return;
+  }
+  for (int k = tid; k < n; k += TH) qinv[piv[k]] = k;
+  __syncthreads();
+  // Binv[s][cf] = A^-1[cf][s] = A_final[piv[cf]][qinv[s]]
+  for (int q = tid; q < n * n; q += TH) {
+    const int s = q / n, cf = q - s * n;
+    binv[(size_t)b * n * n + q] = (TOUT)A[(size_t)piv[cf] * n + qinv[s]];
+  }
+}
+
+// All B matrices, the listed ones (entries below 0 are skipped), or the first *count entries of a
+// compacted list, from a grid of at most the resident CTAs in that case.
+template <typename TOUT, bool kInverse, int TH, int MINB>
+__global__ void __launch_bounds__(TH, MINB) k_gj_split(double* __restrict__ mats, int n, int ch, int B,
+                                                       const int32_t* __restrict__ list, const int32_t* __restrict__ count,
+                                                       TOUT* __restrict__ binv, double* __restrict__ logabs_out,
+                                                       int32_t* __restrict__ sign_out, int32_t* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int total = count ? min(*count, B) : B;
+  for (int e = blockIdx.x; e < total; e += gridDim.x) {
+    const int b = list ? list[e] : e;
+    if (b >= 0) gj_split_one<TOUT, kInverse, TH>(smem_raw, mats, n, ch, b, binv, logabs_out, sign_out, status);
+    __syncthreads();  // the next matrix takes the same shared memory
+  }
+}
+
+template <typename TOUT, bool kInverse, int TH, int MINB>
+cudaError_t run_gj_split(cudaStream_t st, double* mats, int n, int B, const int32_t* list, const int32_t* count,
+                         TOUT* binv, double* la, int32_t* sg, int32_t* status) {
+  const int ch = std::min((n + 7) & ~7, kSCols);
+  const size_t smem = split_smem(n, ch).total;
+  auto kern = k_gj_split<TOUT, kInverse, TH, MINB>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int grid = count ? std::min(B, kSMs * MINB) : B;
+  kern<<<grid, TH, smem, st>>>(mats, n, ch, B, list, count, binv, la, sg, status);
+  return cudaGetLastError();
+}
+
+// Launch shapes of k_gj_split, n <= kSplitMaxN (ms per call, 1500 matrices, kernel before -> now):
+//   n <= 128: 128 threads, four CTAs per SM   (n = 56: inverse 2.12 -> 0.59, determinant 0.50 -> 0.43)
+//   n <= 256: 256 threads, two CTAs per SM    (n = 224: inverse 38.3 -> 8.72, determinant 13.3 -> 4.75),
+//             or, for no more matrices than SMs, 512 threads and one CTA: the warps share one
+//             matrix's updates (one inverse 3.83 -> 1.05 ms against 1.29 with 256 threads)
+//   above:    512 threads, one row per thread
+template <typename TOUT, bool kInverse>
+cudaError_t gj_split(cudaStream_t st, double* mats, int n, int B, const int32_t* list, const int32_t* count, bool few,
+                     TOUT* binv, double* la, int32_t* sg, int32_t* status) {
+  if (n <= 128) return run_gj_split<TOUT, kInverse, 128, 4>(st, mats, n, B, list, count, binv, la, sg, status);
+  if (n <= 256 && !few) return run_gj_split<TOUT, kInverse, 256, 2>(st, mats, n, B, list, count, binv, la, sg, status);
+  return run_gj_split<TOUT, kInverse, 512, 1>(st, mats, n, B, list, count, binv, la, sg, status);
+}
+
 }  // namespace
 
 // FP64 inverse (out_fp64: Binv in double, else float) or determinant only, for B matrices
-// [B][n][n] stored in Phi (overwritten).
+// [B][n][n] stored in Phi (overwritten). count (optional, device): the list is compacted, its
+// first *count entries are taken. few: the caller expects no more matrices than SMs.
 cudaError_t launch_gj(scale_ctx* c, const double* Phi, int n, int B, const int32_t* list, bool inverse,
-                      bool out_fp64, void* Binv, double* logabs, int32_t* sign, int32_t* status) {
+                      bool out_fp64, void* Binv, double* logabs, int32_t* sign, int32_t* status, const int32_t* count,
+                      bool few) {
   double* A = const_cast<double*>(Phi);
   if (B <= 0) return cudaSuccess;
+  if (n <= kSplitMaxN) {
+    few = few || B <= kSMs;
+    if (!inverse)
+      return gj_split<double, false>(c->stream, A, n, B, list, count, few, nullptr, logabs, sign, status);
+    return out_fp64 ? gj_split<double, true>(c->stream, A, n, B, list, count, few, (double*)Binv, logabs, sign, status)
+                    : gj_split<float, true>(c->stream, A, n, B, list, count, few, (float*)Binv, logabs, sign, status);
+  }
   if (inverse) {
-    // A listed refresh (a few samples whose counter came due) of matrices above 448 rows is
-    // latency-bound: one such FP64 inverse takes a single SM about 0.2 s, so it is split
-    // over an 8-CTA cluster. Loads and smaller matrices keep one CTA per matrix, which has
-    // the higher throughput (measured at 224 rows: a 4-CTA cluster inverts one matrix only
-    // 1.5x faster, the serial panel steps and per-block barriers dominate).
-    if (n > 448 && list) {
+    // A listed refresh (a few samples whose counter came due) is latency-bound: one such FP64
+    // inverse takes a single SM about 0.2 s, so it is split over an 8-CTA cluster. Loads keep
+    // one CTA per matrix, which has the higher throughput.
+    if (list) {
       const cudaError_t e =
           out_fp64 ? run_gj_cluster<double, 8, 8>(c->stream, A, n, B, list, (double*)Binv, logabs, sign, status)
                    : run_gj_cluster<float, 8, 8>(c->stream, A, n, B, list, (float*)Binv, logabs, sign, status);
       if (e != cudaErrorNotSupported) return e;
     }
-    if (out_fp64) {
-      if (n > 448) return run_gj<double, double, true, 8>(c->stream, A, n, B, list, (double*)Binv, logabs, sign, status);
-      return run_gj<double, double, true, 16>(c->stream, A, n, B, list, (double*)Binv, logabs, sign, status);
-    }
-    if (n > 448) return run_gj<double, float, true, 8>(c->stream, A, n, B, list, (float*)Binv, logabs, sign, status);
-    return run_gj<double, float, true, 16>(c->stream, A, n, B, list, (float*)Binv, logabs, sign, status);
+    return out_fp64 ? run_gj<double, double, true, 8>(c->stream, A, n, B, list, (double*)Binv, logabs, sign, status)
+                    : run_gj<double, float, true, 8>(c->stream, A, n, B, list, (float*)Binv, logabs, sign, status);
   }
-  if (n > 448) return run_gj<double, double, false, 8, 512>(c->stream, A, n, B, list, (double*)nullptr, logabs, sign, status);
-  // several matrices per SM: small CTAs overlap one's pivot steps with the others' updates;
-  // fewer matrices than a few per SM: one wide CTA per matrix
-  if (B < 4 * 152) return run_gj<double, double, false, 16>(c->stream, A, n, B, list, (double*)nullptr, logabs, sign, status);
-  return run_gj<double, double, false, 8, 256>(c->stream, A, n, B, list, (double*)nullptr, logabs, sign, status);
+  return run_gj<double, double, false, 8, 512>(c->stream, A, n, B, list, (double*)nullptr, logabs, sign, status);
 }
 
 }  // namespace scale

@@ -233,8 +233,8 @@ cudaError_t launch_eloc_full(scale_ctx* c, double* eloc) {
                                             c->full_owner, c->full_list, c->full_vcount);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = launch_forward_phi(c, c->full_occ, G, c->full_list, c->full_vcount, c->Phi64)) != cudaSuccess) return e;
-    if ((e = launch_gj(c, c->Phi64, Ne, G, c->full_list, false, true, nullptr, c->full_la, c->full_sg, nullptr)) !=
-        cudaSuccess)
+    if ((e = launch_gj(c, c->Phi64, Ne, G, c->full_list, false, true, nullptr, c->full_la, c->full_sg, nullptr,
+                       c->full_vcount)) != cudaSuccess)
       return e;
     k_scatter_dets<<<(G + 255) / 256, 256, 0, c->stream>>>(G, c->full_owner, c->full_la, c->full_sg, c->full_la_all,
                                                            c->full_sg_all);

@@ -295,7 +295,7 @@ cudaError_t launch_forward(scale_ctx* c, const int8_t* occ, int B, const int32_t
 cudaError_t launch_slots(scale_ctx* c, const int8_t* occ, int B);
 cudaError_t launch_gj(scale_ctx* c, const double* Phi, int n, int B, const int32_t* list,
                       bool inverse, bool out_fp64, void* Binv, double* logabs, int32_t* sign,
-                      int32_t* status);
+                      int32_t* status, const int32_t* count = nullptr, bool few = false);
 cudaError_t launch_projector(scale_ctx* c, int B, const int32_t* list, const int32_t* count = nullptr);
 // G0t = (M0 + proj_b) Binv^T of the listed samples (all B when list is null).
 cudaError_t launch_build_g0(scale_ctx* c, int B, const int32_t* list, const int32_t* count = nullptr);
