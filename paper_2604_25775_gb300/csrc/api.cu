@@ -243,14 +243,14 @@ scale_status require_lowrank(scale_ctx* c) {
 namespace scale {
 
 // FP64 re-factorisation of the samples selected by the commit counter / drift flag (or
-// all of them): network forward, ascending slot maps, Phi, Gauss-Jordan inverse, projector.
-cudaError_t refresh_samples(scale_ctx* c, bool force_all, bool counters_due) {
+// all of them; expect: about how many, 0 = all): network forward, ascending slot maps, Phi, Gauss-Jordan inverse, projector.
+cudaError_t refresh_samples(scale_ctx* c, bool force_all, bool counters_due, int expect) {
   cudaError_t e;
   if ((e = launch_mark_refresh(c, force_all, counters_due)) != cudaSuccess) return e;
   if ((e = launch_forward(c, c->occ, c->B, c->list, true, c->Phi64, c->list_count)) != cudaSuccess) return e;
   if ((e = launch_slots_list(c, c->list, c->B)) != cudaSuccess) return e;
   if ((e = launch_gj(c, c->Phi64, c->Ne, c->B, c->list, true, c->fp64, c->Binv, c->logabs, c->sign_slot, c->status,
-                     c->list_count, !force_all)) != cudaSuccess)
+                     c->list_count, expect)) != cudaSuccess)
     return e;
   return launch_projector(c, c->B, c->list, c->list_count);
 }
@@ -524,7 +524,8 @@ scale_status scale_commit(scale_ctx* c, const int32_t* moves) {
   if (!moves) return SCALE_EINVAL;
   if ((s = require_lowrank(c)) != SCALE_OK) return s;
   SCALE_TRY(c, launch_commit(c, moves));
-  SCALE_TRY(c, refresh_samples(c, false));
+  // the counters are staggered: about 1 / refresh_every of the samples come due
+  SCALE_TRY(c, refresh_samples(c, false, true, std::max(1, c->B / c->arch.refresh_every)));
   return SCALE_OK;
 }
 
@@ -545,7 +546,10 @@ scale_status scale_sweep(scale_ctx* c, int32_t n_steps, const int32_t* pick, con
     const size_t off = (size_t)k * c->B;
     SCALE_TRY(c, launch_metropolis(c, pick + off, dir + off, u + off, accepted));
     const bool due = (k % kSweepRefreshStride) == kSweepRefreshStride - 1 || k == n_steps - 1;
-    SCALE_TRY(c, refresh_samples(c, false, due));
+    // few samples drift in a step; at an acceptance of about 1/3 the counters of 8 steps bring
+    // some 3 / refresh_every of them
+    const int expect = due ? std::max(1, (int)(3ll * c->B / c->arch.refresh_every)) : 1;
+    SCALE_TRY(c, refresh_samples(c, false, due, expect));
   }
   // The Metropolis commits leave the cached G0t rows behind the inverse (keeping them current
   // per accepted move costs more than the sweep's ratios save); one GEMM per sample restores them.

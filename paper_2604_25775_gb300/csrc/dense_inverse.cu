@@ -1,19 +1,20 @@
 // dense_inverse.cu -- batched Gauss-Jordan elimination with partial pivoting.
 //
-// One CTA per matrix. It returns log|det|, the sign and (inverse mode) the inverse in the
-// library's dual-row layout Binv[c][k] = (A^-1)[k][c]; "det-only" mode restricts the
-// elimination to the rows not yet pivoted and the columns to the right, which is LU with
-// partial pivoting (n^3/3 multiply-adds) -- both are the "single LU decomposition" of
-// Sec. II.C giving the determinant and the inverse together.
+// It returns log|det|, the sign and (inverse mode) the inverse in the library's dual-row layout
+// Binv[c][k] = (A^-1)[k][c]; "det-only" mode restricts the elimination to the rows not yet
+// pivoted and the columns to the right, which is LU with partial pivoting (n^3/3 multiply-adds)
+// -- both are the "single LU decomposition" of Sec. II.C giving the determinant and the inverse
+// together.
 //
-// Blocking. Pivots are taken W columns at a time. The W-column panel is swept in shared
-// memory; the W elementary row operations of the block combine into T = I + U P^T, where
-// the columns of U are the swept panel columns minus the unit vectors of the pivot rows
-// and P selects the pivot rows. Every other column then takes one rank-W update
+// Blocking. Pivots are taken a panel of columns at a time; the elementary row operations of the
+// block combine into T = I + U P^T, where the columns of U are the swept panel columns minus
+// the unit vectors of the pivot rows and P selects the pivot rows. Every other column then takes
+// one update
 //     A[i][c] += sum_j U[i][j] A_old[p_j][c]
-// so each matrix element is read and written once per W pivots. The matrix stays in
-// global memory (L2-resident while the CTAs in flight fit), the work is the FMA pipe of
-// the working type; on sm_103a FP64 this kernel is DFMA-bound.
+// so each matrix element is read and written once per block. The matrix stays in global memory
+// (L2-resident while the CTAs in flight fit). Up to 1024 rows (k_gj_split) the update runs on the
+// 16-bit tensor cores as split products; above, where its panel exceeds shared memory, k_gj takes
+// it on the FP64 pipe (8 columns a block, one CTA per matrix).
 //
 // Pivot choice: largest |value| among unpivoted rows, ties to the lowest row index.
 // Pivoting is implicit (no row swaps); the pivot row of column k is p[k] and the final
@@ -31,14 +32,7 @@ namespace scale {
 
 namespace {
 
-constexpr int kThreads = 1024;  // 32 warps: DFMA latency hidden within one CTA (refresh batches
-                                 // are often one CTA per SM)
-
-template <typename TW>
-struct ArgMax {
-  TW v;
-  int i;
-};
+constexpr int kThreads = 1024;  // 32 warps: DFMA latency hidden within one CTA
 
 // Pivot search on integer keys: the bit pattern of |x| orders like |x| (and puts NaN above
 // every number), so the search runs on the integer pipe instead of FP64 compares.
@@ -113,11 +107,8 @@ __device__ __forceinline__ double sum_log_pivots(const double* pabs, int n, bool
   return part;
 }
 
-// TW: working precision; TOUT: inverse output precision.
-// TH threads per CTA (one matrix): 1024 hides the DFMA latency inside one CTA; the
-// determinant-only path runs 256-thread CTAs with 8-column panels, several per SM, so that
-// one matrix's serial pivot steps overlap the trailing updates of the others (measured on
-// 1024 matrices of 224: W 8 / 256 threads 1.8x faster than W 16 / 1024 threads).
+// Matrices above 1024 rows. TW: working precision; TOUT: inverse output precision; TH threads per
+// CTA (one matrix).
 //
 // The FP64 pipe of sm_103a issues one warp-wide DFMA per SM sub-partition about every 64
 // cycles, so the serial part of a pivot step (search, reciprocal, log) is kept off it: the
@@ -308,242 +299,6 @@ __global__ void __launch_bounds__(TH) k_gj(TW* __restrict__ mats, int n, const i
   }
 }
 
-// Inverse mode split over a thread-block cluster of C CTAs per matrix (FP64 working
-// precision). The columns are cut into C contiguous ranges of whole W-column blocks; CTA q
-// owns its range, and only it reads or writes those columns of A. For each block the owner
-// sweeps the W-column panel in its shared memory exactly as k_gj does; after one cluster
-// barrier every CTA copies the swept panel and the block's pivot rows from the owner's
-// shared memory (distributed shared memory) and applies the rank-W update to its own
-// columns. The panel alternates between two buffers, so the owner of the next block can
-// sweep while the others still copy: one cluster barrier per block. Every element sees the
-// same operations in the same order as in k_gj, so the two kernels give the same bits; the
-// cluster version spreads the O(n^3) FP64 update of one matrix over C SMs, which shortens
-// the refresh of a large matrix (the serial panel steps stay on one SM).
-template <typename TOUT, int W, int C>
-__global__ void __launch_bounds__(kThreads) k_gj_cluster(double* __restrict__ mats, int n,
-                                                         const int32_t* __restrict__ list, TOUT* __restrict__ binv,
-                                                         double* __restrict__ logabs_out, int32_t* __restrict__ sign_out,
-                                                         int32_t* __restrict__ status) {
-  extern __shared__ unsigned char smem_raw[];
-  cg::cluster_group cluster = cg::this_cluster();
-  const int q = (int)cluster.block_rank();
-  const int mat = blockIdx.x / C;
-  const int b = list ? list[mat] : mat;
-  if (b < 0) return;  // the whole cluster shares mat, so it leaves together
-  double* A = mats + (size_t)b * n * n;
-  const int nblocks = (n + W - 1) / W;
-  const int bpc = (nblocks + C - 1) / C;  // blocks per CTA
-  const int c_lo = min(n, q * bpc * W), c_hi = min(n, (q + 1) * bpc * W);
-  const int ncol = c_hi - c_lo, ldp = bpc * W;
-  double* pabs = reinterpret_cast<double*>(smem_raw);    // [n] |pivot| of the columns this CTA owns
-  double* panels = pabs + n;                             // [2][n][W]
-  double* prow = panels + (size_t)2 * n * W;             // [W][ldp]
-  double* colk = prow + (size_t)W * ldp;                 // [n]
-  double* rowp = colk + n;                               // [W]
-  int* piv = reinterpret_cast<int*>(rowp + W);           // [n]
-  int* qinv = piv + n;                                   // [n]
-  unsigned char* used = reinterpret_cast<unsigned char*>(qinv + n);  // [n]
-  __shared__ unsigned long long red_k[kThreads / 32];
-  __shared__ int red_i[kThreads / 32];
-  __shared__ double s_inv;
-  __shared__ int s_p;
-  __shared__ int s_singular;
-  __shared__ int s_sgn;
-
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < n; i += kThreads) used[i] = 0;
-  if (tid == 0) {
-    s_singular = 0;
-    s_sgn = 1;
-  }
-  __syncthreads();
-  cluster.sync();  // every CTA of the cluster runs before any reads another's shared memory
-
-  bool singular = false;
-  for (int blk = 0; blk < nblocks; ++blk) {
-    const int K0 = blk * W, w = min(W, n - K0);
-    const int owner = blk / bpc;
-    double* panel = panels + (size_t)(blk & 1) * n * W;
-    if (q == owner) {
-      for (int e = tid; e < n * W; e += kThreads) {
-        const int i = e / W, j = e % W;
-        if (j < w) panel[e] = A[(size_t)i * n + K0 + j];
-      }
-      __syncthreads();
-      for (int jj = 0; jj < w; ++jj) {
-        const int k = K0 + jj;
-        const int bi = pivot_search<double, kThreads>(panel, W, jj, n, used, red_k, red_i);
-        if (tid == 0) {
-          if (bi >= n || !(fabs(panel[bi * W + jj]) > 0.0)) {
-            s_singular = 1;
-          } else {
-            const double pv = panel[bi * W + jj];
-            s_inv = 1.0 / pv;
-            s_p = bi;
-            piv[k] = bi;
-            used[bi] = 1;
-            pabs[k] = fabs(pv);
-            if (pv < 0.0) s_sgn = -s_sgn;
-          }
-        }
-        __syncthreads();
-        if (s_singular) break;
-        const int p = s_p;
-        const double inv = s_inv;
-        for (int j = tid; j < w; j += kThreads) rowp[j] = (j == jj) ? inv : panel[p * W + j] * inv;
-        for (int i = tid; i < n; i += kThreads) colk[i] = panel[i * W + jj];
-        __syncthreads();
-        for (int e = tid; e < n * W; e += kThreads) {
-          const int i = e / W, j = e % W;
-          if (j >= w) continue;
-          if (i == p) {
-            panel[e] = rowp[j];
-          } else {
-            const double f = colk[i];
-            const double base = (j == jj) ? 0.0 : panel[e];
-            panel[e] = base - f * rowp[j];
-          }
-        }
-        __syncthreads();
-      }
-    }
-    cluster.sync();  // the owner's swept panel, pivots and singular flag are visible
-    const int* o_sing = cluster.map_shared_rank(&s_singular, owner);
-    if (*o_sing) {
-      singular = true;
-      break;
-    }
-    if (q != owner) {
-      const double* o_panel = cluster.map_shared_rank(panel, owner);
-      const int* o_piv = cluster.map_shared_rank(piv, owner);
-      for (int e = tid; e < n * W; e += kThreads)
-        if (e % W < w) panel[e] = o_panel[e];
-      for (int j = tid; j < w; j += kThreads) piv[K0 + j] = o_piv[K0 + j];
-      __syncthreads();
-      for (int j = tid; j < w; j += kThreads) used[piv[K0 + j]] = 1;
-    }
-    // old pivot rows of the block on this CTA's columns (outside the panel)
-    for (int e = tid; e < w * ncol; e += kThreads) {
-      const int j = e / ncol, cc = e - j * ncol;
-      prow[j * ldp + cc] = A[(size_t)piv[K0 + j] * n + c_lo + cc];
-    }
-    __syncthreads();
-    // rank-w update of this CTA's columns outside the panel (the order of k_gj)
-    for (int i = warp; i < n; i += kThreads / 32) {
-      double u[W];
-#pragma unroll
-      for (int j = 0; j < W; ++j) u[j] = (j < w) ? panel[i * W + j] - ((piv[K0 + j] == i) ? 1.0 : 0.0) : 0.0;
-      double* Ai = A + (size_t)i * n;
-      int c = c_lo + lane;
-      for (; c + 32 < c_hi; c += 64) {
-        const int c2 = c + 32;
-        const bool in1 = !(c >= K0 && c < K0 + w);
-        const bool in2 = !(c2 >= K0 && c2 < K0 + w);
-        double a1 = in1 ? Ai[c] : 0.0;
-        double a2 = in2 ? Ai[c2] : 0.0;
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-          if (j < w) {
-            a1 += u[j] * prow[j * ldp + (c - c_lo)];
-            a2 += u[j] * prow[j * ldp + (c2 - c_lo)];
-          }
-        }
-        if (in1) Ai[c] = a1;
-        if (in2) Ai[c2] = a2;
-      }
-      if (c < c_hi && !(c >= K0 && c < K0 + w)) {
-        double a1 = Ai[c];
-#pragma unroll
-        for (int j = 0; j < W; ++j)
-          if (j < w) a1 += u[j] * prow[j * ldp + (c - c_lo)];
-        Ai[c] = a1;
-      }
-    }
-    if (q == owner) {
-      for (int e = tid; e < n * W; e += kThreads) {
-        const int i = e / W, j = e % W;
-        if (j < w) A[(size_t)i * n + K0 + j] = panel[e];
-      }
-    }
-    __syncthreads();
-  }
-  cluster.sync();  // all pivots and flags final: rank 0 gathers the pivots of every block
-  if (q == 0) {
-    // each column's pivot from the CTA that owns its block, summed as in k_gj
-    if (!singular)
-      for (int k = tid; k < n; k += kThreads) pabs[k] = cluster.map_shared_rank(pabs, (k / W) / bpc)[k];
-    __syncthreads();
-    const double logdet = warp == 0 ? sum_log_pivots(pabs, n, singular) : 0.0;
-    if (tid == 0) {
-      double la = logdet;
-      int sg = 1;
-      for (int r = 0; r < C; ++r) sg *= *cluster.map_shared_rank(&s_sgn, r);
-      if (singular) {
-        la = -INFINITY;
-        sg = 0;
-        if (status) status[b] |= SCALE_SAMPLE_SINGULAR;
-      } else {
-        for (int k = 0; k < n; ++k) qinv[k] = 0;
-        int parity = 0;
-        for (int k = 0; k < n; ++k) {
-          if (qinv[k]) continue;
-          int j = k, len = 0;
-          while (!qinv[j]) {
-            qinv[j] = 1;
-            j = piv[j];
-            ++len;
-          }
-          parity += len - 1;
-        }
-        if (parity & 1) sg = -sg;
-      }
-      if (logabs_out) logabs_out[b] = la;
-      if (sign_out) sign_out[b] = sg;
-    }
-  }
-  if (singular) {
-    // zero this CTA's share of the rows of Binv
-    const int r0 = (int)((long long)n * q / C), r1 = (int)((long long)n * (q + 1) / C);
-    for (int e = tid; e < (r1 - r0) * n; e += kThreads) binv[(size_t)b * n * n + (size_t)r0 * n + e] = TOUT(0);
-  } else {
-    // Binv[s][cf] = A^-1[cf][s] = A_final[piv[cf]][col] with s = piv[col], col in this CTA's range
-    for (int e = tid; e < ncol * n; e += kThreads) {
-      const int cc = e / n, cf = e - cc * n, col = c_lo + cc;
-      binv[(size_t)b * n * n + (size_t)piv[col] * n + cf] = (TOUT)A[(size_t)piv[cf] * n + col];
-    }
-  }
-  cluster.sync();  // rank 0 read the others' pivots and signs
-}
-
-template <typename TOUT, int W, int C>
-cudaError_t run_gj_cluster(cudaStream_t st, double* mats, int n, int B, const int32_t* list, TOUT* binv, double* la,
-                           int32_t* sg, int32_t* status) {
-  const int nblocks = (n + W - 1) / W, bpc = (nblocks + C - 1) / C;
-  const size_t smem =
-      sizeof(double) * ((size_t)n + 2 * n * W + (size_t)W * bpc * W + n + W) + sizeof(int) * 2 * n + n + 16;
-  auto kern = k_gj_cluster<TOUT, W, C>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)B * C);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
-    cudaGetLastError();  // clear; the caller falls back to one CTA per matrix
-    return cudaErrorNotSupported;
-  }
-  return cudaLaunchKernelEx(&cfg, kern, mats, n, list, binv, la, sg, status);
-}
-
 template <typename TW, typename TOUT, bool kInverse, int W, int TH = kThreads>
 cudaError_t run_gj(cudaStream_t st, TW* mats, int n, int B, const int32_t* list, TOUT* binv, double* la,
                    int32_t* sg, int32_t* status) {
@@ -581,7 +336,8 @@ constexpr int kSW = 16;        // pivots per block = k of one mma
 constexpr int kSLd = kSW + 2;  // panel row stride in doubles: 16-byte rows without bank conflicts
 constexpr int kSTd = kSW + 1;  // row stride of the 16 x 16 blocks
 constexpr int kSCols = 224;    // columns whose slices are staged at a time
-constexpr int kSplitMaxN = 448;
+constexpr int kSColsTall = 128;  // beside a panel of more than 512 rows
+constexpr int kSplitMaxN = 1024;
 constexpr int kSMs = 152;
 
 struct SplitSmem {
@@ -668,8 +424,11 @@ __device__ __forceinline__ void split_row_tile(const double (&v)[4][2], const in
   }
 }
 
-// One matrix by one CTA of TH >= n threads.
-template <typename TOUT, bool kInverse, int TH>
+// One matrix by a cluster of C CTAs of TH threads, R TH >= n, R rows of the panel per thread. The
+// column blocks are dealt out to the CTAs in turn; every CTA takes the panel, (2) and (3) itself,
+// with the same bits, and updates its own columns, so a block costs one cluster barrier and no
+// exchange but through the matrix.
+template <typename TOUT, bool kInverse, int TH, int R, int C>
 __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats, int n, int ch, int b,
                              TOUT* __restrict__ binv, double* __restrict__ logabs_out, int32_t* __restrict__ sign_out,
                              int32_t* __restrict__ status) {
@@ -691,6 +450,11 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
   int* qinv = reinterpret_cast<int*>(smem_raw + S.qinv);          // [n]
   int* act = reinterpret_cast<int*>(smem_raw + S.act);            // [n] rows in work: all, or those without a pivot
   unsigned char* used = smem_raw + S.used;                        // [n] 0, or 1 + block that pivoted the row
+  const int cta = C == 1 ? 0 : (int)cg::this_cluster().block_rank();
+  auto sync_all = [] {
+    if constexpr (C == 1) __syncthreads();
+    else cg::this_cluster().sync();
+  };
   __shared__ uint4 cand[NW];
   __shared__ int prr[kSW];  // panel rows of the block's pivots
   __shared__ int s_wild, s_nact, s_sgn;
@@ -719,23 +483,26 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
   for (int K0 = 0; K0 < n; K0 += kSW) {
     const int w = min(kSW, n - K0), nact = s_nact;
     const unsigned char blk = (unsigned char)(1 + K0 / kSW);
-    // (1) panel: thread r holds row act[r]
-    const int row = tid < nact ? act[tid] : -1;
-    const bool open = row >= 0 && !used[row];  // may become a pivot row
-    int own = -1;                              // the pivot this row became
-    double a[kSW];
-    {
-      const double* src = A + (size_t)max(row, 0) * n + K0;
+    // (1) panel: the thread's rows act[tid + TH m] (past L1: another CTA may have written them)
+    int row[R], own[R];  // own: the pivot the row became
+    bool open[R];        // may become a pivot row
+    double a[R][kSW];
+#pragma unroll
+    for (int m = 0; m < R; ++m) {
+      row[m] = tid + TH * m < nact ? act[tid + TH * m] : -1;
+      open[m] = row[m] >= 0 && !used[row[m]];
+      own[m] = -1;
+      const double* src = A + (size_t)max(row[m], 0) * n + K0;
       if (vec && w == kSW) {
 #pragma unroll
         for (int k = 0; k < kSW; k += 2) {
-          const double2 v = row >= 0 ? *reinterpret_cast<const double2*>(src + k) : make_double2(0.0, 0.0);
-          a[k] = v.x;
-          a[k + 1] = v.y;
+          const double2 v = row[m] >= 0 ? __ldcg(reinterpret_cast<const double2*>(src + k)) : make_double2(0.0, 0.0);
+          a[m][k] = v.x;
+          a[m][k + 1] = v.y;
         }
       } else {
 #pragma unroll
-        for (int k = 0; k < kSW; ++k) a[k] = (row >= 0 && k < w) ? src[k] : 0.0;
+        for (int k = 0; k < kSW; ++k) a[m][k] = (row[m] >= 0 && k < w) ? __ldcg(src + k) : 0.0;
       }
     }
     if (tid == 0) s_wild = 0;
@@ -749,68 +516,93 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
 #pragma unroll
     for (int jj = 0; jj < kSW; ++jj) {
       if (jj >= w || singular) continue;  // uniform
-      // the candidate of each warp: largest key (0: none; the key's upper word + 1, lower word)
-      const bool valid = open && own < 0;
-      const uint64_t key = dbits(a[jj]) & 0x7fffffffffffffffull;
-      const unsigned hi = valid ? (unsigned)(key >> 32) + 1u : 0u, lo = valid ? (unsigned)key : 0u;
-      const unsigned m1 = __reduce_max_sync(0xffffffffu, hi);
-      const unsigned m2 = __reduce_max_sync(0xffffffffu, hi == m1 ? lo : 0u);
-      const unsigned bal = __ballot_sync(0xffffffffu, hi == m1 && lo == m2);
-      if (lane == 0) cand[warp] = make_uint4(m1, m2, (unsigned)(warp * 32 + __ffs(bal) - 1), 0u);
+      // the candidate of each warp: largest key (0: none; the key's upper word + 1, lower word),
+      // ties to the lowest row
+      unsigned hi[R], lo[R], h = 0u, l = 0u;
+#pragma unroll
+      for (int m = 0; m < R; ++m) {
+        const uint64_t key = dbits(a[m][jj]) & 0x7fffffffffffffffull;
+        const bool valid = open[m] && own[m] < 0;
+        hi[m] = valid ? (unsigned)(key >> 32) + 1u : 0u;
+        lo[m] = valid ? (unsigned)key : 0u;
+        h = max(h, hi[m]);
+      }
+      const unsigned m1 = __reduce_max_sync(0xffffffffu, h);
+#pragma unroll
+      for (int m = 0; m < R; ++m) l = max(l, hi[m] == m1 ? lo[m] : 0u);
+      const unsigned m2 = __reduce_max_sync(0xffffffffu, l);
+      unsigned r = 0x7fffffffu;
+#pragma unroll
+      for (int m = R - 1; m >= 0; --m)
+        if (hi[m] == m1 && lo[m] == m2) r = (unsigned)(tid + TH * m);
+      r = __reduce_min_sync(0xffffffffu, r);
+      if (lane == 0) cand[warp] = make_uint4(m1, m2, r, 0u);
       __syncthreads();
-      const uint4 c = lane < NW ? cand[lane] : make_uint4(0u, 0u, 0u, 0u);
+      const uint4 c = lane < NW ? cand[lane] : make_uint4(0u, 0u, 0x7fffffffu, 0u);
       const unsigned g1 = __reduce_max_sync(0xffffffffu, c.x);
       const unsigned g2 = __reduce_max_sync(0xffffffffu, c.x == g1 ? c.y : 0u);
-      const unsigned bal2 = __ballot_sync(0xffffffffu, lane < NW && c.x == g1 && c.y == g2);
-      const int rp = (int)__shfl_sync(0xffffffffu, c.z, __ffs(bal2) - 1);
+      const int rp = (int)__reduce_min_sync(0xffffffffu, c.x == g1 && c.y == g2 ? c.z : 0x7fffffffu);
       // no row left, a zero column, or a NaN in it
       if (g1 == 0u || (g1 == 1u && g2 == 0u) || g1 > 0x7ff00001u || (g1 == 0x7ff00001u && g2 != 0u)) {
         singular = true;
         continue;
       }
-      if (warp == (rp >> 5)) {
-        const double pv = __shfl_sync(0xffffffffu, a[jj], rp & 31);
-        const double ip = __drcp_rn(pv);
-        if (lane == (rp & 31)) {
-          own = jj;
+      const int rt = rp % TH, rm = rp / TH;
+      if (warp == (rt >> 5)) {
+        double pv = a[0][jj];
 #pragma unroll
-          for (int k = jj + 1; k < kSW; ++k) prow[k] = a[k];
+        for (int m = 1; m < R; ++m) pv = rm == m ? a[m][jj] : pv;
+        pv = __shfl_sync(0xffffffffu, pv, rt & 31);
+        const double ip = __drcp_rn(pv);
+#pragma unroll
+        for (int m = 0; m < R; ++m) {
+          if (lane != (rt & 31) || rm != m) continue;
+          own[m] = jj;
+#pragma unroll
+          for (int k = jj + 1; k < kSW; ++k) prow[k] = a[m][k];
           inv[jj] = ip;
           prr[jj] = rp;
-          piv[K0 + jj] = row;
-          used[row] = blk;
-          rho[jj] = rexp[row];
-          pabs[K0 + jj] = __longlong_as_double((long long)key);
+          piv[K0 + jj] = row[m];
+          used[row[m]] = blk;
+          rho[jj] = rexp[row[m]];
+          pabs[K0 + jj] = fabs(pv);
           if (dbits(pv) >> 63) s_sgn = -s_sgn;
         }
       }
       __syncthreads();
-      if (row >= 0 && own < 0) {  // the inverse's earlier pivot rows too
-        const double l = a[jj] * inv[jj];
-        a[jj] = l;
 #pragma unroll
-        for (int k = jj + 1; k < kSW; ++k) a[k] = fma(-l, prow[k], a[k]);
+      for (int m = 0; m < R; ++m) {
+        if (row[m] < 0 || own[m] >= 0) continue;  // the inverse's earlier pivot rows take part
+        const double f = a[m][jj] * inv[jj];
+        a[m][jj] = f;
+#pragma unroll
+        for (int k = jj + 1; k < kSW; ++k) a[m][k] = fma(-f, prow[k], a[m][k]);
       }
     }
     if (singular) break;
     const int c_lo = kInverse ? 0 : K0 + w;
     if (c_lo >= n) break;  // determinant: the last block is done
-    if (own >= 0) {
 #pragma unroll
-      for (int k = 0; k < kSW; ++k) tri[own * kSTd + k] = a[k];
+    for (int m = 0; m < R; ++m) {
+      if (own[m] < 0) continue;
+#pragma unroll
+      for (int k = 0; k < kSW; ++k) tri[own[m] * kSTd + k] = a[m][k];
     }
     __syncthreads();
-    if (row >= 0 && own < 0) {
+#pragma unroll
+    for (int m = 0; m < R; ++m) {
+      if (row[m] < 0 || own[m] >= 0) continue;
       int e = 0;
       uint64_t nz = 0;
 #pragma unroll
       for (int k = 0; k < kSW; ++k) {
-        e = max(e, exp_scaled(dbits(a[k]), 0));
-        nz |= dbits(a[k]) << 1;
+        e = max(e, exp_scaled(dbits(a[m][k]), 0));
+        nz |= dbits(a[m][k]) << 1;
       }
       if (!exp_near(e, nz != 0, 200)) atomicOr(&s_wild, 1);
 #pragma unroll
-      for (int k = 0; k < kSW; k += 2) *reinterpret_cast<double2*>(panel + tid * kSLd + k) = make_double2(a[k], a[k + 1]);
+      for (int k = 0; k < kSW; k += 2)
+        *reinterpret_cast<double2*>(panel + (tid + TH * m) * kSLd + k) = make_double2(a[m][k], a[m][k + 1]);
     }
     if (tid < kSW && (rho[tid] > 100 || rho[tid] < -100)) atomicOr(&s_wild, 1);
     // (2)
@@ -858,13 +650,18 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
         split_column_tile(v, rho, xf + nt * kSplit * 32, xe + 8 * nt);
       }
     }
-    for (int cb = c_lo; cb < n; cb += ch) {
-      const int ncol = min(ch, n - cb), ntile = (ncol + 7) >> 3;
+    // this CTA's column blocks from c_lo on: tile nt is half of block jb0 + (nt >> 1) C
+    const int nb = (n + kSW - 1) / kSW, lo_b = c_lo / kSW;
+    const int jb0 = lo_b + ((cta - lo_b) % C + C) % C;
+    const int ntiles = jb0 < nb ? 2 * ((nb - 1 - jb0) / C + 1) : 0;
+    for (int t0 = 0; t0 < ntiles; t0 += ch / 8) {
+      const int ntile = min(ch / 8, ntiles - t0);
+      auto tile_col = [&](int nt) { return (jb0 + ((t0 + nt) >> 1) * C) * kSW + 8 * ((t0 + nt) & 1); };
       // column slices of the block's old pivot rows: a warp per 8-column tile (warp 0 joins late)
-      const int w0 = cb == c_lo ? (warp + NW - 1) % NW : warp;
+      const int w0 = t0 == 0 ? (warp + NW - 1) % NW : warp;
       for (int nt = w0; nt < ntile; nt += NW) {
-        const int c = cb + 8 * nt + g;
-        if (kInverse && (unsigned)(cb + 8 * nt - K0) < (unsigned)kSW) continue;
+        const int c0 = tile_col(nt), c = c0 + g;
+        if (kInverse && (unsigned)(c0 - K0) < (unsigned)kSW) continue;
         uint64_t x[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -919,7 +716,7 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
             u[2 * nt + 1][0] = -split_value(acc, 2, ex[1], f.x);
             u[2 * nt + 1][1] = -split_value(acc, 3, ex[1], f.y);
           }
-          if (kInverse && run == 0 && cb == c_lo) {  // the block's columns after the sweep
+          if (kInverse && run == 0 && t0 == 0 && (K0 / kSW) % C == cta) {  // the block's columns after the sweep
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               double* dst = ((q & 1) ? A1 : A0) + K0;
@@ -932,8 +729,8 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
           split_row_tile(u, rho, as, ex);
           // (4)
           for (int nt = run * per; nt < min(ntile, (run + 1) * per); ++nt) {
-            if (kInverse && (unsigned)(cb + 8 * nt - K0) < (unsigned)kSW) continue;
-            const int cc = 8 * nt + 2 * t, c = cb + cc;
+            const int c0 = tile_col(nt), c = c0 + 2 * t;
+            if (kInverse && (unsigned)(c0 - K0) < (unsigned)kSW) continue;
             const bool in0 = c < n, in1 = c + 1 < n;
             double v[4] = {0.0, 0.0, 0.0, 0.0};
             if (vec) {
@@ -954,7 +751,7 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
               if (in1 && add1) v[3] = A1[c + 1];
             }
             split_mma(acc, as, bf + (size_t)nt * kSplit * 32);
-            const int2 f = *reinterpret_cast<const int2*>(fexp + cc);
+            const int2 f = *reinterpret_cast<const int2*>(fexp + 8 * nt + 2 * t);
             v[0] += split_value(acc, 0, ex[0], f.x);
             v[1] += split_value(acc, 1, ex[0], f.y);
             v[2] += split_value(acc, 2, ex[1], f.x);
@@ -984,14 +781,15 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
             __syncwarp();
             if (lane < kSW) {
               panel[r * kSLd + lane] = s;
-              if (kInverse && lane < w) A[(size_t)act[r] * n + K0 + lane] = s;
+              if (kInverse && lane < w && (K0 / kSW) % C == cta) A[(size_t)act[r] * n + K0 + lane] = s;
             }
             __syncwarp();
           }
         }
+        const int ncol = 8 * ntile;
         for (int q = tid; q < w * ncol; q += TH) {
-          const int k = q / ncol, cc = q - k * ncol;
-          pr[k * ch + cc] = A[(size_t)piv[K0 + k] * n + cb + cc];
+          const int k = q / ncol, cc = q - k * ncol, c = tile_col(cc >> 3) + (cc & 7);
+          pr[k * ch + cc] = c < n ? A[(size_t)piv[K0 + k] * n + c] : 0.0;
         }
         __syncthreads();
         if (tid == 0) atomicOr(&s_wild, 2);
@@ -1000,8 +798,8 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
           if (!kInverse && used[i]) continue;
           const bool add = !(kInverse && used[i] == blk);
           for (int cc = lane; cc < ncol; cc += 32) {
-            const int c = cb + cc;
-            if (kInverse && (unsigned)(c - K0) < (unsigned)kSW) continue;
+            const int c = tile_col(cc >> 3) + (cc & 7);
+            if (c >= n || (kInverse && (unsigned)(c - K0) < (unsigned)kSW)) continue;
             double v = add ? A[(size_t)i * n + c] : 0.0;
             for (int k = 0; k < w; ++k) v += panel[r * kSLd + k] * pr[k * ch + cc];
             A[(size_t)i * n + c] = v;
@@ -1022,12 +820,12 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
       }
       if (lane == 0) s_nact = m;
     }
-    __syncthreads();
+    sync_all();
   }
   __syncthreads();
 
   const double logdet = warp == 0 ? sum_log_pivots(pabs, n, singular) : 0.0;  // on thread 0
-  if (tid == 0) {
+  if (tid == 0 && cta == 0) {
     int st = 0;
     double la = logdet;
     int sg = s_sgn;
@@ -1059,91 +857,120 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
   __syncthreads();
   if (singular) {
     if (binv)
-      for (int q = tid; q < n * n; q += TH) binv[(size_t)b * n * n + q] = TOUT(0);
+      for (int q = cta * TH + tid; q < n * n; q += C * TH) binv[(size_t)b * n * n + q] = TOUT(0);
     return;
   }
   for (int k = tid; k < n; k += TH) qinv[piv[k]] = k;
   __syncthreads();
   // Binv[s][cf] = A^-1[cf][s] = A_final[piv[cf]][qinv[s]]
-  for (int q = tid; q < n * n; q += TH) {
+  for (int q = cta * TH + tid; q < n * n; q += C * TH) {
     const int s = q / n, cf = q - s * n;
-    binv[(size_t)b * n * n + q] = (TOUT)A[(size_t)piv[cf] * n + qinv[s]];
+    binv[(size_t)b * n * n + q] = (TOUT)__ldcg(A + (size_t)piv[cf] * n + qinv[s]);
   }
+  if constexpr (C > 1) cg::this_cluster().sync();  // the matrix is read before another takes its place
 }
 
 // All B matrices, the listed ones (entries below 0 are skipped), or the first *count entries of a
 // compacted list, from a grid of at most the resident CTAs in that case.
-template <typename TOUT, bool kInverse, int TH, int MINB>
+template <typename TOUT, bool kInverse, int TH, int MINB, int R, int C>
 __global__ void __launch_bounds__(TH, MINB) k_gj_split(double* __restrict__ mats, int n, int ch, int B,
                                                        const int32_t* __restrict__ list, const int32_t* __restrict__ count,
                                                        TOUT* __restrict__ binv, double* __restrict__ logabs_out,
                                                        int32_t* __restrict__ sign_out, int32_t* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int total = count ? min(*count, B) : B;
-  for (int e = blockIdx.x; e < total; e += gridDim.x) {
+  for (int e = blockIdx.x / C; e < total; e += gridDim.x / C) {
     const int b = list ? list[e] : e;
-    if (b >= 0) gj_split_one<TOUT, kInverse, TH>(smem_raw, mats, n, ch, b, binv, logabs_out, sign_out, status);
+    if (b >= 0) gj_split_one<TOUT, kInverse, TH, R, C>(smem_raw, mats, n, ch, b, binv, logabs_out, sign_out, status);
     __syncthreads();  // the next matrix takes the same shared memory
   }
 }
 
-template <typename TOUT, bool kInverse, int TH, int MINB>
-cudaError_t run_gj_split(cudaStream_t st, double* mats, int n, int B, const int32_t* list, const int32_t* count,
-                         TOUT* binv, double* la, int32_t* sg, int32_t* status) {
-  const int ch = std::min((n + 7) & ~7, kSCols);
-  const size_t smem = split_smem(n, ch).total;
-  auto kern = k_gj_split<TOUT, kInverse, TH, MINB>;
+struct GjArgs {
+  cudaStream_t st;
+  double* mats;
+  int n, B;
+  const int32_t* list;
+  const int32_t* count;
+  int expect;  // matrices the caller expects in this call (<= B)
+  double* la;
+  int32_t* sg;
+  int32_t* status;
+};
+
+template <typename TOUT, bool kInverse, int TH, int MINB, int R, int C>
+cudaError_t run_gj_split(const GjArgs& a, TOUT* binv) {
+  const int ch = std::min((a.n + 15) & ~15, R == 1 ? kSCols : kSColsTall);
+  auto kern = k_gj_split<TOUT, kInverse, TH, MINB, R, C>;
+  const size_t smem = split_smem(a.n, ch).total;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int grid = count ? std::min(B, kSMs * MINB) : B;
-  kern<<<grid, TH, smem, st>>>(mats, n, ch, B, list, count, binv, la, sg, status);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(a.count ? std::min(a.B, kSMs * MINB / C) : a.B) * C);
+  cfg.blockDim = dim3(TH);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = a.st;
+  cudaLaunchAttribute attr[1];
+  if (C > 1) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+  e = cudaLaunchKernelEx(&cfg, kern, a.mats, a.n, ch, a.B, a.list, a.count, binv, a.la, a.sg, a.status);
+  if constexpr (C > 1) {  // a partition without room for a cluster: one CTA per matrix, the same bits
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return run_gj_split<TOUT, kInverse, TH, MINB, R, 1>(a, binv);
+    }
+  }
+  return e;
 }
 
-// Launch shapes of k_gj_split, n <= kSplitMaxN (ms per call, 1500 matrices, kernel before -> now):
-//   n <= 128: 128 threads, four CTAs per SM   (n = 56: inverse 2.12 -> 0.59, determinant 0.50 -> 0.43)
-//   n <= 256: 256 threads, two CTAs per SM    (n = 224: inverse 38.3 -> 8.72, determinant 13.3 -> 4.75),
-//             or, for no more matrices than SMs, 512 threads and one CTA: the warps share one
-//             matrix's updates (one inverse 3.83 -> 1.05 ms against 1.29 with 256 threads)
-//   above:    512 threads, one row per thread
+// Launch shapes (inverses of n x n, ms per call on a GB300; "old": every product on the FP64 pipe):
+//   n <= 128: 128 threads, four CTAs per SM. n = 56: 1500 matrices 0.59 (old 2.12).
+//   n <= 256: many matrices 256 threads, two CTAs per SM, one matrix's panel beside the other's
+//     updates: n = 224, 1500 matrices 8.7 (old 38.3). Up to one per SM 512 threads, whose warps
+//     share the updates: 1.02 alone (1.20 with 256 threads, old 3.83). Up to 32 matrices clusters
+//     of 4 CTAs: 0.69. (Clusters of 4 fill the GPCs' SMs at about 36: 38 matrices 1.37.)
+//   n <= 512: 512 threads; clusters of 4 also pay in two waves: n = 448 alone 2.37 against 5.36,
+//     38 matrices 4.75 against 5.37.
+//   n <= 1024: two panel rows per thread; n = 896: 152 matrices 43.5 (old 189); alone 39.3, in a
+//     cluster of 8 CTAs 8.1 (old cluster of 8 about 30); clusters of 8 run one wave up to 14.
 template <typename TOUT, bool kInverse>
-cudaError_t gj_split(cudaStream_t st, double* mats, int n, int B, const int32_t* list, const int32_t* count, bool few,
-                     TOUT* binv, double* la, int32_t* sg, int32_t* status) {
-  if (n <= 128) return run_gj_split<TOUT, kInverse, 128, 4>(st, mats, n, B, list, count, binv, la, sg, status);
-  if (n <= 256 && !few) return run_gj_split<TOUT, kInverse, 256, 2>(st, mats, n, B, list, count, binv, la, sg, status);
-  return run_gj_split<TOUT, kInverse, 512, 1>(st, mats, n, B, list, count, binv, la, sg, status);
+cudaError_t gj_split(const GjArgs& a, TOUT* binv) {
+  if (a.n <= 128) return run_gj_split<TOUT, kInverse, 128, 4, 1, 1>(a, binv);
+  if (a.n <= 512) {
+    if (a.expect <= (a.n <= 256 ? 32 : 64)) return run_gj_split<TOUT, kInverse, 512, 1, 1, 4>(a, binv);
+    if (a.n <= 256 && a.expect > kSMs) return run_gj_split<TOUT, kInverse, 256, 2, 1, 1>(a, binv);
+    return run_gj_split<TOUT, kInverse, 512, 1, 1, 1>(a, binv);
+  }
+  if (a.expect <= 14) return run_gj_split<TOUT, kInverse, 512, 1, 2, 8>(a, binv);
+  if (a.expect <= 64) return run_gj_split<TOUT, kInverse, 512, 1, 2, 4>(a, binv);
+  return run_gj_split<TOUT, kInverse, 512, 1, 2, 1>(a, binv);
 }
 
 }  // namespace
 
 // FP64 inverse (out_fp64: Binv in double, else float) or determinant only, for B matrices
 // [B][n][n] stored in Phi (overwritten). count (optional, device): the list is compacted, its
-// first *count entries are taken. few: the caller expects no more matrices than SMs.
+// first *count entries are taken. expect: how many matrices the caller expects (0: B); it
+// chooses the launch shape and no result depends on it.
 cudaError_t launch_gj(scale_ctx* c, const double* Phi, int n, int B, const int32_t* list, bool inverse,
                       bool out_fp64, void* Binv, double* logabs, int32_t* sign, int32_t* status, const int32_t* count,
-                      bool few) {
+                      int expect) {
   double* A = const_cast<double*>(Phi);
   if (B <= 0) return cudaSuccess;
   if (n <= kSplitMaxN) {
-    few = few || B <= kSMs;
-    if (!inverse)
-      return gj_split<double, false>(c->stream, A, n, B, list, count, few, nullptr, logabs, sign, status);
-    return out_fp64 ? gj_split<double, true>(c->stream, A, n, B, list, count, few, (double*)Binv, logabs, sign, status)
-                    : gj_split<float, true>(c->stream, A, n, B, list, count, few, (float*)Binv, logabs, sign, status);
+    const GjArgs a{c->stream, A, n, B, list, count, expect > 0 ? std::min(expect, B) : B, logabs, sign, status};
+    if (!inverse) return gj_split<double, false>(a, nullptr);
+    return out_fp64 ? gj_split<double, true>(a, (double*)Binv) : gj_split<float, true>(a, (float*)Binv);
   }
-  if (inverse) {
-    // A listed refresh (a few samples whose counter came due) is latency-bound: one such FP64
-    // inverse takes a single SM about 0.2 s, so it is split over an 8-CTA cluster. Loads keep
-    // one CTA per matrix, which has the higher throughput.
-    if (list) {
-      const cudaError_t e =
-          out_fp64 ? run_gj_cluster<double, 8, 8>(c->stream, A, n, B, list, (double*)Binv, logabs, sign, status)
-                   : run_gj_cluster<float, 8, 8>(c->stream, A, n, B, list, (float*)Binv, logabs, sign, status);
-      if (e != cudaErrorNotSupported) return e;
-    }
+  if (inverse)
     return out_fp64 ? run_gj<double, double, true, 8>(c->stream, A, n, B, list, (double*)Binv, logabs, sign, status)
                     : run_gj<double, float, true, 8>(c->stream, A, n, B, list, (float*)Binv, logabs, sign, status);
-  }
   return run_gj<double, double, false, 8, 512>(c->stream, A, n, B, list, (double*)nullptr, logabs, sign, status);
 }
 

@@ -295,7 +295,7 @@ cudaError_t launch_forward(scale_ctx* c, const int8_t* occ, int B, const int32_t
 cudaError_t launch_slots(scale_ctx* c, const int8_t* occ, int B);
 cudaError_t launch_gj(scale_ctx* c, const double* Phi, int n, int B, const int32_t* list,
                       bool inverse, bool out_fp64, void* Binv, double* logabs, int32_t* sign,
-                      int32_t* status, const int32_t* count = nullptr, bool few = false);
+                      int32_t* status, const int32_t* count = nullptr, int expect = 0);
 cudaError_t launch_projector(scale_ctx* c, int B, const int32_t* list, const int32_t* count = nullptr);
 // G0t = (M0 + proj_b) Binv^T of the listed samples (all B when list is null).
 cudaError_t launch_build_g0(scale_ctx* c, int B, const int32_t* list, const int32_t* count = nullptr);
@@ -314,7 +314,7 @@ cudaError_t launch_log_psi_sym(scale_ctx* c, int G, const int32_t* perms, const 
                                int32_t* sign);
 cudaError_t launch_eloc_full(scale_ctx* c, double* eloc);
 cudaError_t launch_grad(scale_ctx* c, double* grad, int recompute);
-cudaError_t refresh_samples(scale_ctx* c, bool force_all, bool counters_due = true);
+cudaError_t refresh_samples(scale_ctx* c, bool force_all, bool counters_due = true, int expect = 0);
 cudaError_t launch_mark_refresh(scale_ctx* c, bool force_all, bool counters_due);
 cudaError_t launch_slots_list(scale_ctx* c, const int32_t* list, int B);
 cudaError_t launch_forward_phi(scale_ctx* c, const int8_t* occ, int B, const int32_t* list, const int32_t* vcount,

@@ -1,6 +1,7 @@
 """FP64 elimination with its block products as split FP16 tensor-core products (dense_inverse.cu,
 fp64_mma.cuh): log|det|, sign and inverse at the edges of its blocks (16 pivots), tiles (8
-columns, 16 rows), launch shapes (128 / 256 / 448 rows) and scale rules, against numpy in FP64.
+columns, 16 rows), launch shapes (128 / 256 / 512 / 1024 rows, clusters of 4 and 8 CTAs) and
+scale rules, against numpy in FP64.
 
 The network's weights are zero, so Phi is the chosen reference orbitals' rows; the tolerance is
 the one of the other FP64 tests, cond(Phi) x 1e3 x 2^-53."""
@@ -13,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 
 def _problem(ne, prec=I.PREC_FP64):
-    L = 4 if ne <= 32 else 8 if ne <= 128 else 16
+    L = 4 if ne <= 32 else 8 if ne <= 128 else 16 if ne <= 512 else 24
     up = (ne + 1) // 2
     return I.Problem(L, L, 1, 1, up, ne - up, I.MODEL_HUBBARD, 1.0, 0.0, 4.0, 0.0, 1, 1, [1], [0], I.ACT_TANH, 1, prec,
                      64, 1e-10)
@@ -46,7 +47,7 @@ def _check_inverse(ctx, pb, M0, occ, Phi, tol):
 
 
 @pytest.mark.parametrize("ne", [1, 2, 7, 8, 9, 15, 16, 17, 24, 31, 32, 33, 47, 49, 63, 64, 65, 127, 128, 129, 160, 223, 225,
-                                255, 256, 257, 447, 448])
+                                255, 256, 257, 447, 449, 512, 513, 800, 1024, 1025])
 def test_block_edges(ne):
     pb = _problem(ne)
     rng = np.random.default_rng(ne)
@@ -62,6 +63,8 @@ def test_block_edges(ne):
     assert (np.abs(la - ref[1]) <= tol).all()
     if ne < 2 * pb.N:
         _check_inverse(ctx, pb, M0, occ, Phi, tol)
+    if ne > 512:
+        return
     # determinants alone (the full-recompute entry), many and few matrices a call
     e_low = ctx.local_energy(0).cpu().numpy()
     e_full = ctx.local_energy(1).cpu().numpy()
@@ -114,3 +117,19 @@ def test_zero_row_nan_and_infinity():
                 assert st[b] == 4 and sg[b] == 0 and np.isneginf(la[b])
             else:
                 assert not np.isfinite(la[b])
+
+
+@pytest.mark.parametrize("ne,many", [(140, 160), (140, 60), (300, 70), (460, 70), (530, 20), (530, 70)])
+def test_launch_shapes_agree_bit_for_bit(ne, many):
+    """A matrix gives the same bits alone (a cluster of CTAs) and among many (one CTA each)."""
+    import torch
+    pb = _problem(ne, I.PREC_MIXED)
+    rng = np.random.default_rng(ne)
+    M0 = rng.normal(size=(2 * pb.N, ne)) / np.sqrt(ne)
+    occ = I.random_configs(pb, many, 4)
+    mv = torch.from_numpy(I.random_hop_moves(pb, occ, 8)[:, None, :].copy()).cuda()
+    ctx, la, sg, _ = _run(pb, M0, occ)
+    r = ctx.ratios(mv).cpu().numpy()
+    few, la2, sg2, _ = _run(pb, M0, occ[:3])
+    r2 = few.ratios(mv[:3].contiguous()).cpu().numpy()
+    assert np.array_equal(la[:3], la2) and np.array_equal(sg[:3], sg2) and np.array_equal(r[:3], r2)
