@@ -1,5 +1,5 @@
 // lowrank.cu -- local energies and amplitude ratios by the cached-network + rank-r
-// determinant update of Sec. II.C, and the projector P_s = W_s Phi^-1 it relies on.
+// determinant update of Sec. II.C.
 //
 // One CTA per sample. Connected configurations are enumerated on the device in the fixed
 // order of eloc_common.cuh, compacted chunk by chunk, and handed to the warps (one move per
@@ -175,64 +175,6 @@ __global__ void __launch_bounds__(kWarps * 32) k_ratios(LowrankArgs a, Net<T> ne
   }
 }
 
-// Pt[s][c][:] = W_s Binv[c], i.e. the GEMM Pt[s] = Binv (Ne x Ne) * W_s^T (Ne x h),
-// W_s^T[k][cc] = proj_w[cc][s*Ne + k]. 32 rows per CTA, K tiles of 32.
-template <typename T>
-__global__ void __launch_bounds__(256) k_project(int Ne, int h, const T* __restrict__ proj_w,
-                                                 const T* __restrict__ Binv, T* __restrict__ Pt,
-                                                 const int32_t* __restrict__ list, int B,
-                                                 const int32_t* __restrict__ count) {
-  __shared__ T Bs[32][33];
-  __shared__ T Ws[32][2 * kMaxH + 1];
-  const int nrows = count ? min(*count, B) : B;  // a compacted list: its first *count entries
-  for (int lrow = blockIdx.y; lrow < nrows; lrow += gridDim.y) {
-  __syncthreads();  // the previous sample's tiles are consumed
-  const int b = list ? list[lrow] : lrow;
-  if (b < 0) continue;
-  const int c0 = blockIdx.x * 32;
-  const int tid = threadIdx.x;
-  const int row = tid >> 3, grp = tid & 7;
-  const int ncol = 2 * h;
-  T acc[16];
-#pragma unroll
-  for (int u = 0; u < 16; ++u) acc[u] = T(0);
-  const T* Bb = Binv + (size_t)b * Ne * Ne;
-  for (int k0 = 0; k0 < Ne; k0 += 32) {
-    for (int q = tid; q < 32 * 32; q += 256) {
-      const int rr = q >> 5, kk = q & 31;
-      const int c = c0 + rr, k = k0 + kk;
-      Bs[rr][kk] = (c < Ne && k < Ne) ? Bb[(size_t)c * Ne + k] : T(0);
-    }
-    for (int q = tid; q < 32 * ncol; q += 256) {
-      const int kk = q / ncol, col = q - kk * ncol;
-      const int s = col / h, cc = col - s * h, k = k0 + kk;
-      Ws[kk][col] = (k < Ne) ? proj_w[(size_t)cc * 2 * Ne + s * Ne + k] : T(0);
-    }
-    __syncthreads();
-    for (int kk = 0; kk < 32; ++kk) {
-      const T bv = Bs[row][kk];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const int col = grp + 8 * u;
-        if (col < ncol) acc[u] += bv * Ws[kk][col];
-      }
-    }
-    __syncthreads();
-  }
-  const int c = c0 + row;
-  if (c < Ne) {
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int col = grp + 8 * u;
-      if (col < ncol) {
-        const int s = col / h, cc = col - s * h;
-        Pt[(((size_t)b * 2 + s) * Ne + c) * h + cc] = acc[u];
-      }
-    }
-  }
-  }
-}
-
 template <typename T, int H, int WARPS>
 size_t eloc_smem(int N) {
   return sizeof(MoveScratch<T, H>) * WARPS + (sizeof(uint32_t) + sizeof(double)) * kMoveChunk +
@@ -287,81 +229,6 @@ cudaError_t ratios_t(scale_ctx* c, const int32_t* moves, int M, double* ratio) {
   return cudaGetLastError();
 }
 
-// G0t[b][j][o] = (M0[o] + proj_b[s(o)]) . Binv[b][j]: the part of every Slater row's
-// product with the inverse that does not depend on the network features (the moved rows of
-// R need it for the target orbital). A GEMM per sample: CTA tiles of 64 slots x 64 orbitals,
-// 4 x 4 per thread, K staged 32 at a time through shared memory; the listed samples only
-// (their first *count entries when count is given).
-template <typename T>
-__global__ void __launch_bounds__(256) k_build_g0(int Ne, int No, const T* __restrict__ Binv,
-                                                  const T* __restrict__ M0b, T* __restrict__ G0t,
-                                                  const int32_t* __restrict__ list, int B,
-                                                  const int32_t* __restrict__ count) {
-  __shared__ T As[32][65];  // As[k][j] = Binv[j][k]
-  __shared__ T Ms[32][65];  // Ms[k][o] = M0b[o][k]
-  const int nrows = count ? min(*count, B) : B;
-  const int j0 = blockIdx.x * 64, o0 = blockIdx.y * 64;
-  const int tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
-  for (int lrow = blockIdx.z; lrow < nrows; lrow += gridDim.z) {
-    const int b = list ? list[lrow] : lrow;
-    if (b < 0) continue;
-    const T* Bb = Binv + (size_t)b * Ne * Ne;
-    T acc[4][4] = {};
-    for (int k0 = 0; k0 < Ne; k0 += 32) {
-      __syncthreads();  // the previous tiles are consumed
-      for (int q = tid; q < 64 * 32; q += 256) {
-        const int rr = q >> 5, kk = q & 31, k = k0 + kk;
-        As[kk][rr] = (j0 + rr < Ne && k < Ne) ? Bb[(size_t)(j0 + rr) * Ne + k] : T(0);
-        Ms[kk][rr] = (o0 + rr < No && k < Ne) ? M0b[(size_t)(o0 + rr) * Ne + k] : T(0);
-      }
-      __syncthreads();
-#pragma unroll 4
-      for (int kk = 0; kk < 32; ++kk) {
-        T x[4], y[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          x[u] = As[kk][tr + 16 * u];
-          y[u] = Ms[kk][tc + 16 * u];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) acc[u][v] += x[u] * y[v];
-      }
-    }
-    T* out = G0t + (size_t)b * Ne * No;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int j = j0 + tr + 16 * u;
-      if (j >= Ne) continue;
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const int o = o0 + tc + 16 * v;
-        if (o < No) out[(size_t)j * No + o] = acc[u][v];
-      }
-    }
-  }
-}
-
-template <typename T>
-cudaError_t build_g0_t(scale_ctx* c, int B, const int32_t* list, const int32_t* count) {
-  const int No = 2 * c->N;
-  const dim3 g0grid((c->Ne + 63) / 64, (No + 63) / 64, count ? std::min(B, 256) : std::min(B, 65535));
-  k_build_g0<T><<<g0grid, 256, 0, c->stream>>>(c->Ne, No, (const T*)c->Binv, (const T*)c->M0b, (T*)c->G0t, list, B,
-                                               count);
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t project_t(scale_ctx* c, int B, const int32_t* list, const int32_t* count) {
-  dim3 grid((c->Ne + 31) / 32, count ? std::min(B, 1024) : B);
-  k_project<T><<<grid, 256, 0, c->stream>>>(c->Ne, c->h, make_net<T>(c).proj_w, (const T*)c->Binv, (T*)c->Pt, list,
-                                            B, count);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return build_g0_t<T>(c, B, list, count);
-}
-
 }  // namespace
 
 #define SCALE_DISPATCH_H(c, FN, ...)                                                          \
@@ -384,14 +251,6 @@ cudaError_t launch_eloc_lowrank_list(scale_ctx* c, const int32_t* list, int n, d
 
 cudaError_t launch_ratios(scale_ctx* c, const int32_t* moves, int M, double* ratio) {
   return SCALE_DISPATCH_H(c, ratios_t, c, moves, M, ratio);
-}
-
-cudaError_t launch_projector(scale_ctx* c, int B, const int32_t* list, const int32_t* count) {
-  return c->fp64 ? project_t<double>(c, B, list, count) : project_t<float>(c, B, list, count);
-}
-
-cudaError_t launch_build_g0(scale_ctx* c, int B, const int32_t* list, const int32_t* count) {
-  return c->fp64 ? build_g0_t<double>(c, B, list, count) : build_g0_t<float>(c, B, list, count);
 }
 
 }  // namespace scale
