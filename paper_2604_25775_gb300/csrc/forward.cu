@@ -1,4 +1,4 @@
-// forward.cu -- network forward (Sec. II.B), slot bookkeeping, Slater-matrix build,
+// forward.cu -- network forward (Sec. II.B), slot bookkeeping,
 // layer-0 conv-of-embedding table and the log|psi| output convention.
 #include <algorithm>
 
@@ -8,6 +8,12 @@
 namespace scale {
 
 namespace {
+
+// Four consecutive values, 16-byte aligned (rows of h % 4 == 0 values of an aligned array).
+__device__ __forceinline__ void load4g(const float* p, float (&v)[4]) {
+  const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+  v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+}
 
 // One network layer for every (sample, site, channel):
 //   out_i[c] = res * in_i[c] + act(b[c] + sum_{offsets d} sum_c' in_{i+d}[c'] K[d][c'][c])
@@ -52,6 +58,104 @@ __global__ void k_layer(Lattice lat, Net<T> net, int l, const int8_t* __restrict
   }
   out[(size_t)b * N * h + idx] = self + act_fn<T>(net.act, z);
   if (zout) zout[(size_t)b * N * h + idx] = z;
+  }
+}
+
+// Layer 0 in FP64 from the conv-of-embedding table, z_i[c] = b[c] + sum_d KE[i + d][n_{i+d}][d][c]: one
+// addition per tap instead of h multiply-adds on the FP64 pipe.
+__global__ void k_layer0_table(Lattice lat, Net<double> net, const int8_t* __restrict__ occ,
+                               const int32_t* __restrict__ list, double* __restrict__ out, double* __restrict__ zout,
+                               int B, const int32_t* __restrict__ count) {
+  const int h = net.h, N = lat.N, taps = net.taps0, k = net.ksize[0], r = (k - 1) / 2;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= N * h) return;
+  const int i = idx / h, c = idx - i * h;
+  const double bias = net.bias[0][c];
+  const int nrows = count ? min(*count, B) : B;
+  for (int row = blockIdx.y; row < nrows; row += gridDim.y) {
+    const int b = list ? list[row] : row;
+    if (b < 0) continue;
+    const int8_t* ob = occ + (size_t)b * N;
+    double z = bias;
+    int tap = 0;
+    for (int ky = 0; ky < k; ++ky)
+      for (int kx = 0; kx < k; ++kx) {
+        if (!stencil_in(net.stencil, k, kx - r, ky - r)) continue;
+        const int d = tap++;
+        const int j = site_off(lat, i, kx - r, ky - r);
+        if (j >= 0) z += net.KE[(((size_t)(net.per_site ? j : 0) * 4 + (ob[j] & 3)) * taps + d) * h + c];
+      }
+    const double self = net.resid[0] ? net.embed[((size_t)(net.per_site ? i * 4 : 0) + (ob[i] & 3)) * h + c] : 0.0;
+    out[(size_t)b * N * h + idx] = self + act_fn<double>(net.act, z);
+    if (zout) zout[(size_t)b * N * h + idx] = z;
+  }
+}
+
+// The FP32 layer, 4 sites x 4 channels per thread (h % 4 == 0; HC the width as a constant, or 0),
+// in the same order (bias, taps row-major, input channels ascending), so with the same bits.
+// One output per thread issues two loads per multiply-add; the tile eight 16-byte loads per 64.
+// (FP32, 1500 samples of 16x16, h = 32, 3x3: 1148 us by k_layer, 264 us here.)
+template <int HC>
+__global__ void __launch_bounds__(128) k_layer_tile(Lattice lat, Net<float> net, int l, const int8_t* __restrict__ occ,
+                                                    const int32_t* __restrict__ list, const float* __restrict__ in,
+                                                    float* __restrict__ out, float* __restrict__ zout, int B,
+                                                    const int32_t* __restrict__ count) {
+  const int h = HC ? HC : net.h, N = lat.N, hq = h >> 2, k = net.ksize[l], r = (k - 1) / 2;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= ((N + 3) >> 2) * hq) return;
+  const int i0 = (q / hq) * 4, c0 = (q % hq) * 4;
+  const int nrows = count ? min(*count, B) : B;
+  for (int row = blockIdx.y; row < nrows; row += gridDim.y) {
+    const int b = list ? list[row] : row;
+    if (b < 0) continue;
+    const int8_t* ob = occ + (size_t)b * N;
+    auto input = [&](int j) {  // layer 0 reads the embedding tables
+      return l == 0 ? net.embed + ((size_t)(net.per_site ? j * 4 : 0) + (ob[j] & 3)) * h : in + ((size_t)b * N + j) * h;
+    };
+    float acc[4][4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) acc[s][m] = net.bias[l][c0 + m];
+    int tap = 0;
+    for (int ky = 0; ky < k; ++ky)
+      for (int kx = 0; kx < k; ++kx) {
+        if (!stencil_in(net.stencil, k, kx - r, ky - r)) continue;
+        const float* w = net.kernel[l] + (size_t)tap++ * h * h + c0;
+        const float* x[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const int j = i0 + s < N ? site_off(lat, i0 + s, kx - r, ky - r) : -1;
+          x[s] = j < 0 ? nullptr : input(j);
+        }
+#pragma unroll 4
+        for (int ci = 0; ci < h; ci += 4) {
+          float wv[4][4];
+#pragma unroll
+          for (int a = 0; a < 4; ++a) load4g(w + (size_t)(ci + a) * h, wv[a]);
+#pragma unroll
+          for (int s = 0; s < 4; ++s) {
+            if (!x[s]) continue;
+            float xv[4];
+            load4g(x[s] + ci, xv);
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+              for (int m = 0; m < 4; ++m) acc[s][m] = fma(xv[a], wv[a][m], acc[s][m]);
+          }
+        }
+      }
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      if (i0 + s >= N) break;
+      const size_t o = ((size_t)b * N + i0 + s) * h + c0;
+      const float* self = net.resid[l] ? input(i0 + s) + c0 : nullptr;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        out[o + m] = (self ? self[m] : 0.f) + act_fn<float>(net.act, acc[s][m]);
+        if (zout) zout[o + m] = acc[s][m];
+      }
+    }
   }
 }
 
@@ -132,52 +236,6 @@ __global__ void k_slots(Lattice lat, const int8_t* __restrict__ occ, const int32
   if (threadIdx.x == 0) {
     status[b] = st;
     if (commits) commits[b] = stagger > 0 ? b % stagger : 0;
-  }
-}
-
-// The orbital projection's parameters in precision TP.
-template <typename TP>
-struct Proj {
-  int h;
-  const TP* proj_w;  // [h][2Ne]
-  const TP* proj_b;  // [2Ne]
-  const TP* M0;      // [2N][Ne]
-};
-
-// Slater matrix in ascending orbital order (Sec. II.B "Orbital Projection"):
-//   Phi[a][k] = M0[o_a][k] + proj_b[s*Ne+k] + sum_c H(L)_i[c] proj_w[c][s*Ne+k],
-// o_a = s*N + i the a-th occupied orbital, from features H(L) of type TH, computed in TP and
-// stored as FP64. The load and the refresh project in the mode's precision; the
-// full-recompute path projects in FP64 (it divides two determinants, where an FP32 rounding
-// of the entries would not cancel as the low-rank update's differences do).
-template <typename TH, typename TP>
-__global__ void k_phi(Lattice lat, Proj<TP> net, const int8_t* __restrict__ occ, const int32_t* __restrict__ list,
-                      const TH* __restrict__ HL, double* __restrict__ phi, int B, const int32_t* __restrict__ count) {
-  extern __shared__ int sm[];
-  const int nrows = count ? min(*count, B) : B;
-  for (int row = blockIdx.x; row < nrows; row += gridDim.x) {
-  __syncthreads();  // the previous sample's use of shared memory is over
-  const int b = list ? list[row] : row;
-  if (b < 0) continue;
-  const int N = lat.N, Ne = lat.Ne, h = net.h;
-  int* olist = sm;
-  int* tmp = sm + 2 * N;
-  const int n = occupied_list(occ + (size_t)b * N, N, olist, tmp);
-  double* P = phi + (size_t)b * Ne * Ne;
-  if (n != Ne) {  // invalid sample: leave a zero matrix (singular)
-    for (int q = threadIdx.x; q < Ne * Ne; q += blockDim.x) P[q] = 0.0;
-    continue;
-  }
-  const TH* Hb = HL + (size_t)b * N * h;
-  for (int q = threadIdx.x; q < Ne * Ne; q += blockDim.x) {
-    const int a = q / Ne, k = q - a * Ne;
-    const int o = olist[a], s = o / N, i = o - s * N;
-    TP v = net.M0[(size_t)o * Ne + k] + net.proj_b[s * Ne + k];
-    const TP* w = net.proj_w + s * Ne + k;
-    const TH* x = Hb + (size_t)i * h;
-    for (int c = 0; c < h; ++c) v += (TP)x[c] * w[(size_t)c * 2 * Ne];
-    P[q] = (double)v;
-  }
   }
 }
 
@@ -441,7 +499,20 @@ cudaError_t forward_t(scale_ctx* c, const int8_t* occ, int B, const int32_t* lis
   for (int l = 0; l < (mma ? 1 : c->L); ++l) {
     T* out = (l == c->L - 1 && keep_cache) ? (T*)c->HL : bufs[l & 1];
     T* zo = (l == 0 && keep_cache) ? (T*)c->z0 : nullptr;
-    k_layer<T><<<grid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);
+    bool done = false;
+    if constexpr (sizeof(T) == 8) {
+      if (l == 0 && net.KE) {  // (the allocation-free entry has no table)
+        k_layer0_table<<<grid, 128, 0, c->stream>>>(c->lat, net, occ, list, out, zo, B, count);
+        done = true;
+      }
+    } else if (h % 4 == 0) {  // every embedding, kernel and activation row starts on 16 bytes
+      const dim3 tgrid((((N + 3) / 4) * (h / 4) + 127) / 128, Bgrid);
+      if (h == 16) k_layer_tile<16><<<tgrid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);
+      else if (h == 32) k_layer_tile<32><<<tgrid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);
+      else k_layer_tile<0><<<tgrid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);
+      done = true;
+    }
+    if (!done) k_layer<T><<<grid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);
     in = out;
   }
   if constexpr (sizeof(T) == 4) {
@@ -461,20 +532,9 @@ cudaError_t forward_t(scale_ctx* c, const int8_t* occ, int B, const int32_t* lis
       in = (const T*)out;
     }
   }
-  const size_t smem = sizeof(int) * (2 * N + 257);
-  const int Bphi = count ? std::min(B, 1024) : B;
-  if (phi_out) {
-    if (proj64 && !c->fp64) {
-      // FP64 projection parameters: the flat FP64 vector at the offsets of make_net
-      const int64_t off_w = (const T*)net.proj_w - (const T*)c->params32;
-      const Proj<double> p64{c->h, c->params64 + off_w, c->params64 + off_w + (int64_t)c->h * 2 * c->Ne, c->M0_64};
-      k_phi<T, double><<<Bphi, 256, smem, c->stream>>>(c->lat, p64, occ, list, in, phi_out, B, count);
-    } else {
-      const Proj<T> pt{c->h, net.proj_w, net.proj_b, net.M0};
-      k_phi<T, T><<<Bphi, 256, smem, c->stream>>>(c->lat, pt, occ, list, in, phi_out, B, count);
-    }
-  }
-  return cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || !phi_out) return e;
+  return launch_phi(c, occ, B, list, count, in, phi_out, proj64);
 }
 }  // namespace
 

@@ -292,6 +292,9 @@ cudaError_t launch_offsets(scale_ctx* c, int B, const int32_t* count, int extra,
 // count (optional, device): sample_list is compacted, its first *count entries are used
 cudaError_t launch_forward(scale_ctx* c, const int8_t* occ, int B, const int32_t* sample_list,
                            bool keep_cache, double* phi_out, const int32_t* count = nullptr);
+// FP64 Slater matrices from features HL (mode's precision); proj64: projected in FP64 in every mode
+cudaError_t launch_phi(scale_ctx* c, const int8_t* occ, int B, const int32_t* list, const int32_t* count, const void* HL,
+                       double* phi, bool proj64);
 cudaError_t launch_slots(scale_ctx* c, const int8_t* occ, int B);
 cudaError_t launch_gj(scale_ctx* c, const double* Phi, int n, int B, const int32_t* list,
                       bool inverse, bool out_fp64, void* Binv, double* logabs, int32_t* sign,
