@@ -66,7 +66,7 @@ def parse():
 # DRAM traffic of the local-energy kernel per walker, from the ncu capture summarised in
 # this file; used only while the kernel sources still hash to the value recorded there.
 ELOC_PROFILE = os.path.join(ROOT, "profiles", "k_eloc_hubbard16x16.md")
-ELOC_SOURCES = ["lowrank.cu", "eloc_common.cuh", "move.cuh", "mlp_mma.cuh", "scale_internal.cuh"]
+ELOC_SOURCES = ["eloc.cuh", "eloc_common.cuh", "move.cuh", "mlp_mma.cuh", "scale_internal.cuh"]
 
 
 # The shared header contributes only its device part (geometry, parameter view, activation

@@ -17,7 +17,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libscale.so")
-UNITS = ["api.cu", "forward.cu", "slater.cu", "dense_inverse.cu", "lowrank.cu", "project.cu", "eloc_tc.cu", "commit.cu", "full.cu", "grad.cu", "serve.cu", "noalloc.cu", "symmetry.cu", "ace.cu", "wide_lowrank.cu"]
+# the longest compilations first
+UNITS = ["dense_inverse.cu", "eloc_f32.cu", "commit.cu", "ace.cu", "eloc_f64.cu", "lowrank.cu", "grad.cu", "wide_lowrank.cu",
+         "eloc_tc.cu", "forward.cu", "slater.cu", "project.cu", "api.cu", "full.cu", "serve.cu", "noalloc.cu", "symmetry.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

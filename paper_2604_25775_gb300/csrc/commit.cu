@@ -62,7 +62,7 @@ __device__ T warp_inverse(T (*R)[kRMax + 1], T (*Ri)[kRMax + 1], int r) {
   __syncwarp();
   T det = T(1);
   for (int k = 0; k < r; ++k) {
-    const int p = warp_pivot<T>(R, k, r);
+    const int p = warp_pivot<T, kRMax + 1>(R, k, r);
     if (p != k) {
       if (lane < r) {
         T t = R[k][lane]; R[k][lane] = R[p][lane]; R[p][lane] = t;
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kCommitThreads, 2) k_commit(CommitArgs a, Net<
       ms.spin = spin;
     }
     __syncwarp();
-    move_features<T, H>(a.lat, net, a.k0, sv, a.mf, ms, z0n);
+    move_features<T, H>(a.lat, net, lane_tap(a.lat, net, a.k0), sv, a.mf, ms, z0n);
     const int r = move_matrix<T, H, true>(a.lat, net, sv, ms);
     T det = T(0);
     if (r > 0 && !singular) det = warp_inverse<T>(ms.R, Ri, r);

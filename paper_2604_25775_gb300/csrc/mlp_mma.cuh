@@ -137,6 +137,36 @@ struct MmaShape {
   static constexpr int KT = KIND == kTF32 ? H / 8 : H / 16;
 };
 
+// act_fast of G tiles' values by the whole warp, the same values: where every |z| of the warp is
+// below 1/2, which one vote tells, the tanh of each is its polynomial alone (half of its
+// instructions; the site-wise layers' activations are small while the features are).
+template <int G>
+__device__ __forceinline__ void act_tiles(int act, float (&c)[G][4]) {
+  if (act == SCALE_ACT_TANH) {
+    float m = 0.f;
+#pragma unroll
+    for (int u = 0; u < G; ++u)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) m = fmaxf(m, fabsf(c[u][q]));
+    if (__any_sync(0xffffffffu, !(m < 0.5f))) {
+#pragma unroll
+      for (int u = 0; u < G; ++u)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[u][q] = tanh_f32(c[u][q]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < G; ++u)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[u][q] = tanh_f32_small(c[u][q]);
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < G; ++u)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) c[u][q] = act_fast(act, c[u][q]);
+  }
+}
+
 // Layers 1..L-1 (all site-wise) on the 16-row tile held in x (C-fragment layout, FP32):
 //   x <- res_l * x + act(bias_l + x W_l).
 // wf: fragments [L][KT][NT][32], bias: per layer (FP32 copies); oscale (kFP16 only): per layer
@@ -173,42 +203,48 @@ __device__ __forceinline__ void mlp_tile(float (&x)[H / 8][4], const WFrag* __re
     const float* bl = bias[l];
     const int res = resid[l];
     const float om = KIND == kFP16 ? oscale[l] : 1.f;
+    // G column tiles at a time, so that one vote covers their activations
+    constexpr int G = NT <= 4 ? NT : 2;
 #pragma unroll
-    for (int j = 0; j < NT; ++j) {
-      const float b0 = bl[8 * j + 2 * t], b1 = bl[8 * j + 2 * t + 1];
-      // the accumulators start at the bias (kFP16: at zero, the bias added after unscaling)
-      float c[4] = {b0, b1, b0, b1};
-      if constexpr (KIND == kFP16) c[0] = c[1] = c[2] = c[3] = 0.f;
+    for (int j0 = 0; j0 < NT; j0 += G) {
+      float c[G][4];
 #pragma unroll
-      for (int kk = 0; kk < KT; ++kk) {
-        const WFrag w = wl[(kk * NT + j) * 32 + lane];
-        if constexpr (KIND == kTF32) {
-          mma_tf32(c, ah[kk], w.v[0], w.v[1]);
-          mma_tf32(c, al[kk], w.v[0], w.v[1]);
-          mma_tf32(c, ah[kk], w.v[2], w.v[3]);
-        } else if constexpr (KIND == kFP16) {
-          mma_f16(c, ah[kk], w.v[0], w.v[1]);
-          mma_f16(c, al[kk], w.v[0], w.v[1]);
-          mma_f16(c, ah[kk], w.v[2], w.v[3]);
-        } else {
-          mma_bf16(c, ah[kk], w.v[0], w.v[1]);
-          mma_bf16(c, al[kk], w.v[0], w.v[1]);
-          mma_bf16(c, ah[kk], w.v[2], w.v[3]);
+      for (int u = 0; u < G; ++u) {
+        const int j = j0 + u;
+        const float b0 = bl[8 * j + 2 * t], b1 = bl[8 * j + 2 * t + 1];
+        // the accumulators start at the bias (kFP16: at zero, the bias added after unscaling)
+        c[u][0] = c[u][2] = b0;
+        c[u][1] = c[u][3] = b1;
+        if constexpr (KIND == kFP16) c[u][0] = c[u][1] = c[u][2] = c[u][3] = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < KT; ++kk) {
+          const WFrag w = wl[(kk * NT + j) * 32 + lane];
+          if constexpr (KIND == kTF32) {
+            mma_tf32(c[u], ah[kk], w.v[0], w.v[1]);
+            mma_tf32(c[u], al[kk], w.v[0], w.v[1]);
+            mma_tf32(c[u], ah[kk], w.v[2], w.v[3]);
+          } else if constexpr (KIND == kFP16) {
+            mma_f16(c[u], ah[kk], w.v[0], w.v[1]);
+            mma_f16(c[u], al[kk], w.v[0], w.v[1]);
+            mma_f16(c[u], ah[kk], w.v[2], w.v[3]);
+          } else {
+            mma_bf16(c[u], ah[kk], w.v[0], w.v[1]);
+            mma_bf16(c[u], al[kk], w.v[0], w.v[1]);
+            mma_bf16(c[u], ah[kk], w.v[2], w.v[3]);
+          }
+        }
+        if constexpr (KIND == kFP16) {
+          c[u][0] = fmaf(c[u][0], om, b0);
+          c[u][1] = fmaf(c[u][1], om, b1);
+          c[u][2] = fmaf(c[u][2], om, b0);
+          c[u][3] = fmaf(c[u][3], om, b1);
         }
       }
-      if constexpr (KIND == kFP16) {
-        c[0] = fmaf(c[0], om, b0);
-        c[1] = fmaf(c[1], om, b1);
-        c[2] = fmaf(c[2], om, b0);
-        c[3] = fmaf(c[3], om, b1);
-      }
-      if (res) {  // uniform
+      act_tiles<G>(act, c);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) x[j][q] += act_fast(act, c[q]);
-      } else {
+      for (int u = 0; u < G; ++u)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) x[j][q] = act_fast(act, c[q]);
-      }
+        for (int q = 0; q < 4; ++q) x[j0 + u][q] = res ? x[j0 + u][q] + c[u][q] : c[u][q];  // res: uniform
     }
   }
 }

@@ -26,16 +26,31 @@ namespace scale {
 constexpr int kSMax = 18;  // affected sites for two touched sites and a 3x3 box or the 13-site plus
 constexpr int kRMax = 32;  // electrons on the affected sites (lane per column)
 
-template <typename T, int H>
+// Scratch of one move. SM sites, RM electrons. Compact (the local-energy kernel, whose moves are
+// neighbour hops): Delta H takes the place of H' in feat, and only the touched sites' H' are kept
+// beside it (hl[0] of src, hl[1] of dst); the commit needs both on all of S.
+// EXACT: the network's width is H, so that rows have a constant length.
+template <typename T, int H, int SM = kSMax, int RM = kRMax, bool COMPACT = false, bool EXACT = false>
 struct MoveScratch {
+  static constexpr bool kCompact = COMPACT, kExact = EXACT;
+  static constexpr int kSites = SM, kRows = RM;
   int nS, r, kind, src, dst, spin;
-  int site[kSMax];
-  int nold[kSMax], nnew[kSMax];
+  int site[SM];
+  int nold[SM], nnew[SM];
   int pair_s[2 * 13];  // S index of each (touched site, tap) pair, -1 if none (up to 13 taps)
-  int slot[kRMax], orb[kRMax], sidx[kRMax], moved[kRMax];
-  alignas(16) T feat[kSMax][H];   // new features H'(L) on S (tile loads/stores stop at nS)
-  alignas(16) T hl[kSMax][H];     // cached features H(L) on S
-  alignas(16) T R[kRMax][kRMax + 1];  // also the embedding rows of S while the features are built
+  int slot[RM], orb[RM], sidx[RM];
+  int moved[RM];                           // 0, or 1 + (the electron now sits on dst)
+  int mpos[2];                             // list position of the electron that moved to src, dst (-1: none)
+  uint16_t tap[SM];                        // compact: taps of src (low byte) and dst that reach the site, 0xff none
+  alignas(16) T feat[SM][H];               // new features H'(L) on S (tile loads/stores stop at nS)
+  alignas(16) T hl[COMPACT ? 2 : SM][H];   // cached features H(L) on S, then Delta H (compact: see above)
+  alignas(16) T R[RM][RM + 1];             // also the embedding rows of S while the features are built
+  // the row of electron a in R = delta + row . Pt: H' if it moved, Delta H if it kept its orbital
+  // (compact: sidx counts on into hl, which follows feat)
+  __device__ __forceinline__ const T* row(int a) const {
+    if constexpr (COMPACT) return &feat[0][0] + sidx[a] * H;
+    return moved[a] ? feat[sidx[a]] : hl[sidx[a]];
+  }
 };
 
 // 16-byte asynchronous global -> shared copies (the warp waits for its own copies and then
@@ -90,9 +105,9 @@ __device__ __forceinline__ bool move_allowed(const Lattice& lat, int kind, int s
 // Site-wise layers 1..L-1 on the rows of ms.feat (FP FMA path): lane = channel, four sites
 // per pass, weights read through L1. Summation order: bias first, then c' ascending, the
 // same as the forward layer kernel.
-template <typename T, int H>
-__device__ void mlp_simt(const Net<T>& net, MoveScratch<T, H>& ms, int nS) {
-  const int lane = threadIdx.x & 31, h = net.h;
+template <typename T, int H, typename MS>
+__device__ void mlp_simt(const Net<T>& net, MS& ms, int nS) {
+  const int lane = threadIdx.x & 31, h = MS::kExact ? H : net.h;
   for (int l = 1; l < net.L; ++l) {
     const T* W = net.kernel[l];
     const T* bl = net.bias[l];
@@ -139,23 +154,50 @@ __device__ void mlp_simt(const Net<T>& net, MoveScratch<T, H>& ms, int nS) {
   }
 }
 
+// What a lane keeps for all moves of a kernel: the layer-0 offset of its (touched site, tap) pair --
+// lane p < taps is tap p of src, lane taps + p of dst -- and a reciprocal of the lattice width.
+struct LaneTap {
+  int dx, dy;
+  uint32_t inv_lx;  // ceil(2^20 / Lx): (i inv_lx) >> 20 = i / Lx for i < 4096, Lx <= 128
+  bool unique;      // no site lies under two taps of one site (periodic extents cover the stencil)
+};
+template <typename T>
+__device__ __forceinline__ LaneTap lane_tap(const Lattice& lat, const Net<T>& net, int k0) {
+  const int lane = threadIdx.x & 31, kk = net.taps0;
+  LaneTap t{};
+  if (lane < 2 * kk) stencil_tap(net.stencil, k0, lane < kk ? lane : lane - kk, t.dx, t.dy);
+  t.inv_lx = ((1u << 20) + lat.Lx - 1) / lat.Lx;
+  t.unique = (!lat.pbc_x || lat.Lx >= k0) && (!lat.pbc_y || lat.Ly >= k0);
+  return t;
+}
+// site_off for offsets smaller than the periodic extents (|dx|, |dy| <= 2, extents >= 3).
+__device__ __forceinline__ int site_near(const Lattice& lat, const LaneTap& lt, int i, int dx, int dy) {
+  const int y0 = (int)(((uint32_t)i * lt.inv_lx) >> 20);
+  int x = i - y0 * lat.Lx + dx, y = y0 + dy;
+  if (x < 0 || x >= lat.Lx) {
+    if (!lat.pbc_x) return -1;
+    x += x < 0 ? lat.Lx : -lat.Lx;
+  }
+  if (y < 0 || y >= lat.Ly) {
+    if (!lat.pbc_y) return -1;
+    y += y < 0 ? lat.Ly : -lat.Ly;
+  }
+  return y * lat.Lx + x;
+}
+
 // Steps 1-3: S and the new last-layer features H'(L) on S in ms.feat, the cached H(L) in
-// ms.hl. All lanes of the warp participate. z0_new (optional) receives z0' on S.
-template <typename T, int H>
-__device__ void move_features(const Lattice& lat, const Net<T>& net, int k0, const SampleView<T>& sv,
-                              const MlpFrags& mf, MoveScratch<T, H>& ms, T (*z0_new)[H] = nullptr) {
+// ms.hl (not in a compact scratch). All lanes of the warp participate. z0_new (optional)
+// receives z0' on S.
+template <typename T, int H, typename MS>
+__device__ void move_features(const Lattice& lat, const Net<T>& net, const LaneTap& lt, const SampleView<T>& sv,
+                              const MlpFrags& mf, MS& ms, T (*z0_new)[H] = nullptr) {
   const int lane = threadIdx.x & 31;
-  const int h = net.h, kk = net.taps0;  // taps of layer 0 (9 for the 3x3 box, 13 for the plus)
-  const int npairs = 2 * kk;            // <= 32: one lane per pair
+  const int h = MS::kExact ? H : net.h, kk = net.taps0;  // taps of layer 0 (9 for the 3x3 box, 13 for the plus)
+  const int npairs = 2 * kk;                             // <= 32: one lane per pair
+  const bool by_rows = MS::kCompact && H <= 32 && lt.unique;  // how the layer-0 rows are built below
   // pairs (t, d): t = src (pair < kk) or dst; the site reached is t - offset(d)
   int s_site = -1;
-  if (lane < npairs) {
-    const int t = (lane < kk) ? ms.src : ms.dst;
-    const int d = lane % kk;
-    int dx, dy;
-    stencil_tap(net.stencil, k0, d, dx, dy);
-    s_site = site_off(lat, t, -dx, -dy);
-  }
+  if (lane < npairs) s_site = site_near(lat, lt, (lane < kk) ? ms.src : ms.dst, -lt.dx, -lt.dy);
   const unsigned act_mask = __ballot_sync(0xffffffffu, s_site >= 0);
   const unsigned same = __match_any_sync(0xffffffffu, s_site);
   const int first = __ffs(same & act_mask) - 1;
@@ -166,12 +208,16 @@ __device__ void move_features(const Lattice& lat, const Net<T>& net, int k0, con
   const int n_dst_new = move_new_state(ms.kind, ms.spin, false, n_src_old, n_dst_old);
   if (s_site >= 0) {
     const int pos = __popc(firsts & ((1u << first) - 1u));
-    ms.pair_s[lane] = pos;
+    if (!by_rows) ms.pair_s[lane] = pos;
     if (is_first) {
       ms.site[pos] = s_site;
       const int n_old = sv.occ[s_site] & 3;
       ms.nold[pos] = n_old;
       ms.nnew[pos] = (s_site == ms.src) ? n_src_new : (s_site == ms.dst) ? n_dst_new : n_old;
+      if constexpr (MS::kCompact) {  // the taps of src and of dst that reach the site
+        const unsigned ts = same & ((1u << kk) - 1u), td = same >> kk;
+        ms.tap[pos] = (uint16_t)((ts ? __ffs(ts) - 1 : 0xff) | ((td ? __ffs(td) - 1 : 0xff) << 8));
+      }
     }
   } else if (lane < npairs) {
     ms.pair_s[lane] = -1;
@@ -180,8 +226,46 @@ __device__ void move_features(const Lattice& lat, const Net<T>& net, int k0, con
   if (lane == 0) ms.nS = nS;
   __syncwarp();
   const int ts_src = net.per_site ? ms.src : 0, ts_dst = net.per_site ? ms.dst : 0;
+  if (by_rows) {
+    // a site's z0 row takes the table deltas of at most one tap of src and one of dst: row by row
+    // (two at a time with 16 channels), lane = channel, every load of kG rows in flight before the
+    // first use, straight from the cache and the tables into the activation
+    constexpr int kG = 4, RP = H == 16 ? 2 : 1;
+    const T* ks = net.KE + (size_t)ts_src * 4 * kk * h;
+    const T* kd = net.KE + (size_t)ts_dst * 4 * kk * h;
+    const int c = lane & (32 / RP - 1), sub = RP == 2 ? lane >> 4 : 0;
+    if (MS::kExact || c < h) {
+#pragma unroll 1
+      for (int s0 = sub; s0 < nS; s0 += kG * RP) {
+        T z[kG], sn[kG], so[kG], dn[kG], dold[kG], ev[kG];
+#pragma unroll
+        for (int g = 0; g < kG; ++g) {
+          z[g] = sn[g] = so[g] = dn[g] = dold[g] = ev[g] = T(0);
+          const int s = s0 + g * RP;
+          if (s < nS) {
+            const int site = ms.site[s], tap = ms.tap[s], a = tap & 0xff, b = tap >> 8;
+            z[g] = sv.z0[(size_t)site * h + c];
+            if (a != 0xff) {
+              sn[g] = ks[(n_src_new * kk + a) * h + c];
+              so[g] = ks[(n_src_old * kk + a) * h + c];
+            }
+            if (b != 0xff) {
+              dn[g] = kd[(n_dst_new * kk + b) * h + c];
+              dold[g] = kd[(n_dst_old * kk + b) * h + c];
+            }
+            if (net.resid[0]) ev[g] = net.embed[((size_t)(net.per_site ? site * 4 : 0) + ms.nnew[s]) * h + c];
+          }
+        }
+#pragma unroll
+        for (int g = 0; g < kG; ++g)
+          if (s0 + g * RP < nS)
+            ms.feat[s0 + g * RP][c] = ev[g] + act_fn<T>(net.act, (z[g] + (sn[g] - so[g])) + (dn[g] - dold[g]));
+      }
+    }
+  } else {
   // stage z0 and H(L) rows of S, add the layer-0 table deltas, activation + residual.
-  constexpr bool kCopyRows = H <= 32 && kSMax * H <= kRMax * (kRMax + 1);
+  constexpr bool kCopyRows = H <= 32 && MS::kSites * H <= MS::kRows * (MS::kRows + 1);
+  constexpr int kParts = MS::kCompact ? 1 : 2;  // z0 rows, and H(L) rows where they are kept
   if (kCopyRows && (h * (int)sizeof(T)) % 16 == 0) {
     // z0 -> feat, H(L) -> hl and the residual embedding rows -> the R area by asynchronous
     // 16-byte copies; the table-delta loads go out while they travel (two rounds of nine
@@ -189,17 +273,17 @@ __device__ void move_features(const Lattice& lat, const Net<T>& net, int k0, con
     constexpr int E = 16 / (int)sizeof(T);
     const int cpr = h / E;  // chunks per row
     T* emb = &ms.R[0][0];   // [nS][h]
-    const int nrows = nS * (net.resid[0] ? 3 : 2);
+    const int nrows = nS * (net.resid[0] ? kParts + 1 : kParts);
     for (int q = lane; q < nrows * cpr; q += 32) {
       const int row = q / cpr, v = q - row * cpr;
-      const int part = row / nS, s = row - part * nS;
+      const int part = (row >= nS) + (kParts == 2 && row >= 2 * nS), s = row - part * nS;
       const int site = ms.site[s];
       const T* src;
       T* dst;
       if (part == 0) {
         src = sv.z0 + (size_t)site * h;
         dst = ms.feat[s];
-      } else if (part == 1) {
+      } else if (part < kParts) {
         src = sv.HL + (size_t)site * h;
         dst = ms.hl[s];
       } else {
@@ -220,8 +304,8 @@ __device__ void move_features(const Lattice& lat, const Net<T>& net, int k0, con
         const int p = p0 + g;
         kn[g] = ko[g] = T(0);
         if (on_c && p < npairs && ms.pair_s[p] >= 0) {
-          const int d = p % kk;
           const bool from_src = p < kk;
+          const int d = from_src ? p : p - kk;
           const int ts = from_src ? ts_src : ts_dst;
           const int nn = from_src ? n_src_new : n_dst_new;
           const int no = from_src ? n_src_old : n_dst_old;
@@ -259,13 +343,13 @@ __device__ void move_features(const Lattice& lat, const Net<T>& net, int k0, con
         const bool on = s0 + g < nS;
         const int site = on ? ms.site[s0 + g] : 0;
         z[g] = on ? sv.z0[(size_t)site * h + c] : T(0);
-        hv[g] = on ? sv.HL[(size_t)site * h + c] : T(0);
+        hv[g] = on && !MS::kCompact ? sv.HL[(size_t)site * h + c] : T(0);
       }
 #pragma unroll
       for (int g = 0; g < kG; ++g)
         if (s0 + g < nS) {
           ms.feat[s0 + g][c] = z[g];
-          ms.hl[s0 + g][c] = hv[g];
+          if constexpr (!MS::kCompact) ms.hl[s0 + g][c] = hv[g];
         }
     }
     // (b) layer-0 table deltas of the touched (site, offset) pairs
@@ -277,8 +361,8 @@ __device__ void move_features(const Lattice& lat, const Net<T>& net, int k0, con
         const int p = p0 + g;
         kn[g] = ko[g] = T(0);
         if (p < npairs && ms.pair_s[p] >= 0) {
-          const int d = p % kk;
           const bool from_src = p < kk;
+          const int d = from_src ? p : p - kk;
           const int ts = from_src ? ts_src : ts_dst;
           const int nn = from_src ? n_src_new : n_dst_new;
           const int no = from_src ? n_src_old : n_dst_old;
@@ -312,6 +396,7 @@ __device__ void move_features(const Lattice& lat, const Net<T>& net, int k0, con
     }
   }
   }
+  }
   __syncwarp();
   if (net.L > 1) {
     if constexpr (sizeof(T) == 4 && H % 16 == 0) {
@@ -340,16 +425,19 @@ __device__ void move_features(const Lattice& lat, const Net<T>& net, int k0, con
 // all lanes), or -1 when r exceeds kRMax or a slot map is inconsistent.
 // kDotFallback: sv.G0t may be null (a Metropolis commit), so the dot-product path is compiled
 // in; the local-energy and ratio kernels always have the cache and leave it out.
-template <typename T, int H, bool kDotFallback = false>
-__device__ int move_matrix(const Lattice& lat, const Net<T>& net, const SampleView<T>& sv, MoveScratch<T, H>& ms) {
+template <typename T, int H, bool kDotFallback = false, typename MS>
+__device__ int move_matrix(const Lattice& lat, const Net<T>& net, const SampleView<T>& sv, MS& ms) {
+  constexpr int RM = MS::kRows;
   const int lane = threadIdx.x & 31;
-  const int N = lat.N, Ne = lat.Ne, h = net.h;
+  const int N = lat.N, Ne = lat.Ne, h = MS::kExact ? H : net.h;
   const int nS = ms.nS;
   // electrons on S after the move: spin-up ones first, then spin-down, each group in S
   // order, compacted with ballots (the determinant does not depend on the row order
   // because rows and columns of R follow the same list)
   int r = 0, r_up = 0;
   bool bad = false;
+  if (lane < 2) ms.mpos[lane] = -1;
+  __syncwarp();
   for (int sp = 0; sp < 2; ++sp) {
     if (sp == 1) r_up = r;
     for (int base = 0; base < nS; base += 32) {
@@ -364,10 +452,10 @@ __device__ int move_matrix(const Lattice& lat, const Net<T>& net, const SampleVi
             slot = sv.slot_of_orb[sp * N + site];  // same electron, same orbital
           } else if (ms.kind == 0) {
             slot = sv.slot_of_orb[sp * N + ms.src];  // the hopping electron
-            mv = 1;
+            mv = 2;
           } else {
             slot = sv.slot_of_orb[sp * N + (site == ms.src ? ms.dst : ms.src)];  // exchanged spin
-            mv = 1;
+            mv = site == ms.src ? 1 : 2;
           }
         }
       }
@@ -375,11 +463,12 @@ __device__ int move_matrix(const Lattice& lat, const Net<T>& net, const SampleVi
       if (occ) {
         const int pos = r + __popc(bal & ((1u << lane) - 1u));
         if (slot < 0) bad = true;
-        if (pos < kRMax) {
+        if (pos < RM) {
           ms.slot[pos] = slot;
           ms.orb[pos] = sp * N + ms.site[s];
-          ms.sidx[pos] = s;
+          ms.sidx[pos] = MS::kCompact && mv ? MS::kSites + mv - 1 : s;
           ms.moved[pos] = mv;
+          if (mv) ms.mpos[mv - 1] = pos;
         }
       }
       r += __popc(bal);
@@ -388,10 +477,33 @@ __device__ int move_matrix(const Lattice& lat, const Net<T>& net, const SampleVi
   bad = __any_sync(0xffffffffu, bad);
   if (lane == 0) ms.r = r;
   __syncwarp();
-  if (r > kRMax || bad) return -1;
-  // Delta H in place of the cached rows: ms.hl[s] <- H'_s - H_s
-  for (int c = lane; c < h; c += 32)
-    for (int s = 0; s < nS; ++s) ms.hl[s][c] = ms.feat[s][c] - ms.hl[s][c];
+  if (r > RM || bad) return -1;
+  if constexpr (MS::kCompact) {
+    // Delta H in place of the new rows, the touched sites' H' beside them; the cached rows go out
+    // as many loads at a time as registers hold
+    constexpr int kG = 7, RP = H == 16 ? 2 : 1;
+    for (int c = lane & (32 / RP - 1); c < h; c += 32)
+#pragma unroll 1
+      for (int s0 = RP == 2 ? lane >> 4 : 0; s0 < nS; s0 += kG * RP) {
+        T hv[kG];
+#pragma unroll
+        for (int g = 0; g < kG; ++g) hv[g] = s0 + g * RP < nS ? sv.HL[(size_t)ms.site[s0 + g * RP] * h + c] : T(0);
+#pragma unroll
+        for (int g = 0; g < kG; ++g) {
+          const int s = s0 + g * RP;
+          if (s >= nS) continue;
+          const T v = ms.feat[s][c];
+          const int site = ms.site[s];
+          if (site == ms.src) ms.hl[0][c] = v;
+          if (site == ms.dst) ms.hl[1][c] = v;
+          ms.feat[s][c] = v - hv[g];
+        }
+      }
+  } else {
+    // Delta H in place of the cached rows: ms.hl[s] <- H'_s - H_s
+    for (int c = lane; c < h; c += 32)
+      for (int s = 0; s < nS; ++s) ms.hl[s][c] = ms.feat[s][c] - ms.hl[s][c];
+  }
   __syncwarp();
   const int cb = ms.slot[lane < r ? lane : 0];
   // Pt terms, column b = lane: the Pt[spin][c_b] row in registers (16 channels at a time),
@@ -412,17 +524,17 @@ __device__ int move_matrix(const Lattice& lat, const Net<T>& net, const SampleVi
 #pragma unroll
         for (int u = 0; u < HH; ++u) pv[u] = (hc * HH + u < h) ? pt[u] : T(0);
         for (int a = a0; a < a1; ++a) {
-          const T* row = (ms.moved[a] ? ms.feat[ms.sidx[a]] : ms.hl[ms.sidx[a]]) + hc * HH;
+          const T* row = ms.row(a) + hc * HH;
           T v[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
           for (int u = 0; u < HH; ++u)
             if (hc * HH + u < h) v[u & 3] += row[u] * pv[u];
           const T part = (v[0] + v[1]) + (v[2] + v[3]);
           const T tot = part + __shfl_xor_sync(0xffffffffu, part, 16);
-          const T init = (!ms.moved[a] && a == bb) ? T(1) : T(0);
-          if (hc == 0 && bb < r) ms.R[a][bb] = init + tot;
+          if (hc == 0 && bb < r) ms.R[a][bb] = tot;
         }
       }
+      if (hc == 0 && bb < r && !ms.moved[bb]) ms.R[bb][bb] += T(1);  // the lane's own column
       __syncwarp();
     } else {
     // the whole Pt row of the lane's column in registers; every row of R written once
@@ -434,15 +546,15 @@ __device__ int move_matrix(const Lattice& lat, const Net<T>& net, const SampleVi
 #pragma unroll
       for (int u = 0; u < H; ++u) pv[u] = (u < h) ? pt[u] : T(0);
       for (int a = a0; a < a1; ++a) {
-        const T* row = ms.moved[a] ? ms.feat[ms.sidx[a]] : ms.hl[ms.sidx[a]];
+        const T* row = ms.row(a);
         T v[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
         for (int u = 0; u < H; ++u)
           if (u < h) v[u & 3] += row[u] * pv[u];
-        const T init = (!ms.moved[a] && a == lane) ? T(1) : T(0);
-        if (lane < r) ms.R[a][lane] = init + ((v[0] + v[1]) + (v[2] + v[3]));
+        if (lane < r) ms.R[a][lane] = (v[0] + v[1]) + (v[2] + v[3]);
       }
     }
+    if (lane < r && !ms.moved[lane]) ms.R[lane][lane] += T(1);
     __syncwarp();
     }
   } else {
@@ -458,7 +570,7 @@ __device__ int move_matrix(const Lattice& lat, const Net<T>& net, const SampleVi
 #pragma unroll
       for (int u = 0; u < 16; ++u) pv[u] = (c0 + u < h) ? pt[c0 + u] : T(0);
       for (int a = a0; a < a1; ++a) {
-        const T* row = (ms.moved[a] ? ms.feat[ms.sidx[a]] : ms.hl[ms.sidx[a]]) + c0;
+        const T* row = ms.row(a) + c0;
         T v0 = T(0), v1 = T(0);
 #pragma unroll
         for (int u = 0; u < 16; u += 2) {
@@ -475,9 +587,10 @@ __device__ int move_matrix(const Lattice& lat, const Net<T>& net, const SampleVi
   // without the cache (a Metropolis sweep, which does not keep it current) the dot products
   // against the inverse, lanes split k, one warp reduction per b
   if (!kDotFallback || sv.G0t) {
-    for (int a = 0; a < r; ++a) {
-      if (!ms.moved[a]) continue;
-      if (lane < r) ms.R[a][lane] += sv.G0t[(size_t)ms.slot[lane] * 2 * N + ms.orb[a]];
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      const int a = ms.mpos[m];
+      if (a >= 0 && lane < r) ms.R[a][lane] += sv.G0t[(size_t)ms.slot[lane] * 2 * N + ms.orb[a]];
     }
   } else if constexpr (kDotFallback) {
     for (int a = 0; a < r; ++a) {
@@ -523,8 +636,8 @@ __device__ __forceinline__ double recip(double x) { return __drcp_rn(x); }
 
 // Pivot row of column k among rows [k, r) of R (lane i holds row i): the largest |R[i][k]|,
 // ties to the lowest row. Same value in every lane.
-template <typename T>
-__device__ __forceinline__ int warp_pivot(const T (*R)[kRMax + 1], int k, int r) {
+template <typename T, int LD>
+__device__ __forceinline__ int warp_pivot(const T (*R)[LD], int k, int r) {
   const int lane = threadIdx.x & 31;
   const bool mine = lane >= k && lane < r;
   if constexpr (sizeof(T) == 4) {
@@ -551,12 +664,12 @@ __device__ __forceinline__ int warp_pivot(const T (*R)[kRMax + 1], int k, int r)
 // Step 5: det of R (r x r, r <= kRMax) by LU with partial pivoting, lane j owning column j;
 // the pivot search is a warp argmax over the rows, one reciprocal per column. R is destroyed.
 // Returns the determinant (same value in all lanes).
-template <typename T>
-__device__ T warp_det_R(T (*R)[kRMax + 1], int r) {
+template <typename T, int LD>
+__device__ T warp_det_R(T (*R)[LD], int r) {
   const int lane = threadIdx.x & 31;
   T det = T(1);
   for (int k = 0; k < r; ++k) {
-    const int p = warp_pivot<T>(R, k, r);
+    const int p = warp_pivot<T, LD>(R, k, r);
     if (p != k) {
       if (lane < r) {
         const T t = R[k][lane];
@@ -582,8 +695,8 @@ __device__ T warp_det_R(T (*R)[kRMax + 1], int r) {
   return det;
 }
 
-template <typename T, int H>
-__device__ T warp_det(MoveScratch<T, H>& ms, int r) {
+template <typename T, typename MS>
+__device__ T warp_det(MS& ms, int r) {
   return warp_det_R<T>(ms.R, r);
 }
 

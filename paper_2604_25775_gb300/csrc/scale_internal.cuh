@@ -309,6 +309,8 @@ cudaError_t launch_logpsi_list(scale_ctx* c, const int32_t* list, int n, double*
 cudaError_t launch_load_list(scale_ctx* c, const int8_t* occ, const int32_t* list, int n);
 cudaError_t launch_logpsi_out(scale_ctx* c, double* logabs, int32_t* sign);
 cudaError_t launch_eloc_lowrank(scale_ctx* c, double* eloc);
+cudaError_t launch_eloc_f32(scale_ctx* c, double* eloc, const int32_t* list, int n);
+cudaError_t launch_eloc_f64(scale_ctx* c, double* eloc, const int32_t* list, int n);
 cudaError_t launch_ratios(scale_ctx* c, const int32_t* moves, int M, double* ratio);
 cudaError_t launch_commit(scale_ctx* c, const int32_t* moves);
 cudaError_t launch_metropolis(scale_ctx* c, const int32_t* pick, const int32_t* dir, const double* u,
