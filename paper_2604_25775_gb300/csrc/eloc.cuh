@@ -14,13 +14,19 @@
 // particle-hole transformed Hubbard model U sum_i n_up (1 - n_dn).
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "eloc_common.cuh"
 
+namespace cg = cooperative_groups;
+
 namespace scale {
 
 namespace {
+
+constexpr int kElocList = 2048;  // moves of one list
 
 // WARPS warps per sample; the sample's cached rows (Pt, z0, H(L), G0t) are read through L1/L2,
 // shared memory holds the per-warp move scratch and the move list. Bound by the instructions and
@@ -37,28 +43,36 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_eloc(LowrankArgs a, Net<T> ne
   extern __shared__ __align__(16) unsigned char smem[];
   const int N = a.lat.N, Ne = a.lat.Ne, h = MS::kExact ? H : net.h;
   MS* ms_all = reinterpret_cast<MS*>(smem);
-  uint32_t* mlist = reinterpret_cast<uint32_t*>(ms_all + WARPS);     // [kMoveChunk]
-  double* contrib = reinterpret_cast<double*>(mlist + kMoveChunk);   // [kMoveChunk]
-  int32_t* slot_s = reinterpret_cast<int32_t*>(contrib + kMoveChunk);
+  uint32_t* mlist = reinterpret_cast<uint32_t*>(ms_all + WARPS);    // [kElocList]
+  double* contrib = reinterpret_cast<double*>(mlist + kElocList);   // [kElocList]
+  int32_t* slot_s = reinterpret_cast<int32_t*>(contrib + kElocList);
   int8_t* occ_s = reinterpret_cast<int8_t*>(slot_s + 2 * N);
   __shared__ int warp_cnt[WARPS];
-  __shared__ double s_diag;
-  __shared__ int s_next;
+  __shared__ int s_diag, s_next;
 
-  const int b = a.list ? a.list[blockIdx.x] : blockIdx.x;
+  // the CTAs of a cluster share one sample's moves: CTA `rank` takes moves rank, rank + cs, ... of
+  // the list they all enumerate, and the first one collects and sums the contributions
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int cs = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int w = blockIdx.x / cs;
+  const int b = a.list ? a.list[w] : w;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int st = a.status[b];
   if (st & (SCALE_SAMPLE_BAD_COUNT | SCALE_SAMPLE_DOUBLE_OCC | SCALE_SAMPLE_SINGULAR)) {
-    if (tid == 0) {
+    if (tid == 0 && rank == 0) {
       a.out[b] = CUDART_NAN;
       if (a.move_count) a.move_count[b] = 0;
     }
     return;
   }
+  if (tid == 0) s_diag = 0;
   for (int i = tid; i < N; i += blockDim.x) occ_s[i] = a.occ[(size_t)b * N + i];
   for (int o = tid; o < 2 * N; o += blockDim.x) slot_s[o] = a.slot_of_orb[(size_t)b * 2 * N + o];
   __syncthreads();
-  if (tid == 0) s_diag = diag_energy(a, occ_s);
+  if (rank == 0) {
+    const int d = __reduce_add_sync(0xffffffffu, diag_count(a, occ_s, tid, WARPS * 32));
+    if (lane == 0) atomicAdd(&s_diag, d);
+  }
   SampleView<T> sv;
   sv.occ = occ_s;
   sv.slot_of_orb = slot_s;
@@ -71,19 +85,22 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_eloc(LowrankArgs a, Net<T> ne
 
   const LaneTap lt = lane_tap(a.lat, net, a.k0);
   const int ncand = candidate_count(a);
+  double* sums = cs == 1 ? contrib : cluster.map_shared_rank(contrib, 0);
   double total = 0.0;  // thread 0
   int nmoves = 0;
-  for (int cs = 0; cs < ncand; cs += kMoveChunk) {
-    const int ce = min(ncand, cs + kMoveChunk);
-    // enumerate and compact the allowed moves of this chunk (enumeration order)
-    const int nm = enumerate_chunk<WARPS>(a, occ_s, cs, ce, mlist, warp_cnt);
+  for (int id = 0; id < ncand;) {
+    // the allowed moves of as many candidates as surely fit the list (enumeration order)
+    int nm = 0;
+    for (; id < ncand && nm + WARPS * 32 <= kElocList; id += WARPS * 32)
+      nm = enumerate_window<WARPS>(a, occ_s, id, ncand, nm, mlist, warp_cnt);
     if (tid == 0) s_next = 0;
-    __syncthreads();
+    if (cs == 1) __syncthreads();
+    else cluster.sync();  // the first CTA has summed the previous list
     // warps take the next move as they finish the previous one
     for (;;) {
       int mi = 0;
       if (lane == 0) mi = atomicAdd(&s_next, 1);
-      mi = __shfl_sync(0xffffffffu, mi, 0);
+      mi = __shfl_sync(0xffffffffu, mi, 0) * cs + rank;
       if (mi >= nm) break;
       const uint32_t pm = mlist[mi];
       if (lane == 0) {
@@ -97,13 +114,14 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_eloc(LowrankArgs a, Net<T> ne
       move_features<T, H>(a.lat, net, lt, sv, a.mf, ms);
       const int r = move_matrix<T, H>(a.lat, net, sv, ms);
       const T det = (r < 0) ? T(CUDART_NAN) : warp_det<T>(ms, r);
-      if (lane == 0) contrib[mi] = move_coeff(a.lat, pm) * (double)det;
+      if (lane == 0) sums[mi] = move_coeff(a.lat, pm) * (double)det;
       __syncwarp();
     }
-    __syncthreads();
-    // fixed-order sum of the chunk: lane l adds contributions l, l+32, ..., then an xor tree
+    if (cs == 1) __syncthreads();
+    else cluster.sync();
+    // fixed-order sum of the list: lane l adds contributions l, l+32, ..., then an xor tree
     // (both orders independent of which warp evaluated which move)
-    if (warp == 0) {
+    if (warp == 0 && rank == 0) {
       double s = 0.0;
       for (int q = lane; q < nm; q += 32) s += contrib[q];
 #pragma unroll
@@ -113,10 +131,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_eloc(LowrankArgs a, Net<T> ne
         nmoves += nm;
       }
     }
-    __syncthreads();
+    if (cs == 1) __syncthreads();
   }
-  if (tid == 0) {
-    a.out[b] = s_diag + total;
+  if (tid == 0 && rank == 0) {
+    a.out[b] = (a.lat.model == SCALE_MODEL_TJ ? (0.25 * a.lat.J) * s_diag : a.lat.U * s_diag) + total;
     if (a.move_count) a.move_count[b] = nmoves;
   }
 }
@@ -130,17 +148,57 @@ using ElocDisk = MoveScratch<T, H, kSMax, kRMax, true, EXACT>;
 
 template <int WARPS, typename MS>
 size_t eloc_smem(int N) {
-  return sizeof(MS) * WARPS + (sizeof(uint32_t) + sizeof(double)) * kMoveChunk + sizeof(int32_t) * 2 * N + N + 16;
+  return sizeof(MS) * WARPS + (sizeof(uint32_t) + sizeof(double)) * kElocList + sizeof(int32_t) * 2 * N + N + 16;
 }
 
 template <int H>
 constexpr int kElocWarps = H == 64 ? 16 : 28;  // 64 channels keep 32 activations a lane: registers
+// CTAs per sample for n samples: the number that takes the fewest rounds of moves, ceil(n / slots) / C,
+// with 3% per further CTA for the repeated set-up and enumeration. slots: samples in flight -- one CTA
+// per SM, and clusters of 4 and 8 leave SMs of a GPC over (measured: 38 clusters of 4 and 16 of 8 run
+// as two waves). Local energies do not depend on it. (us, one CTA each / split: 16x16 Hubbard 1
+// walker 665 / 102, 38 walkers 669 / 350, 100 walkers 694 / 542, 333 walkers 1948 / 1760; 64 walkers of
+// 8x8 106 / 61.)
+inline int eloc_split(int n) {
+  constexpr int kSlots[4] = {152, 76, 36, 14};
+  int best = 1;
+  double cost = 1e30;
+  for (int k = 0; k < 4; ++k) {
+    const int C = 1 << k;
+    const double v = (double)((n + kSlots[k] - 1) / kSlots[k]) / C * (1.0 + 0.03 * (C - 1));
+    if (v < cost) {
+      cost = v;
+      best = C;
+    }
+  }
+  return best;
+}
+
 template <typename T, int H, int WARPS, typename MS>
 cudaError_t eloc_launch(scale_ctx* c, const LowrankArgs& a, int n) {
   const size_t smem = eloc_smem<WARPS, MS>(c->N);
-  cudaError_t e = cudaFuncSetAttribute(k_eloc<T, H, WARPS, MS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kern = k_eloc<T, H, WARPS, MS>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_eloc<T, H, WARPS, MS><<<n, WARPS * 32, smem, c->stream>>>(a, make_net<T>(c));
+  const int C = eloc_split(n);
+  if (C > 1) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)n * C);
+    cfg.blockDim = dim3(WARPS * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kern, a, make_net<T>(c));
+    if (e == cudaSuccess) return e;
+    cudaGetLastError();  // a partition without room for a cluster: one CTA per sample
+  }
+  kern<<<n, WARPS * 32, smem, c->stream>>>(a, make_net<T>(c));
   return cudaGetLastError();
 }
 

@@ -151,6 +151,41 @@ __device__ int enumerate_chunk(const LowrankArgs& a, const int8_t* occ_s, int cs
   return nm;
 }
 
+// The same, one candidate id per thread: the allowed moves among ids [id0, id0 + 32 NWARPS), appended
+// to the nm moves of the list; returns their new number. Two barriers.
+template <int NWARPS>
+__device__ int enumerate_window(const LowrankArgs& a, const int8_t* occ_s, int id0, int ncand, int nm, uint32_t* mlist,
+                                int* warp_cnt) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, id = id0 + tid;
+  int cls = 0;
+  MoveDesc m{-1, 0, 0, 0};
+  if (id < ncand) m = candidate(a, occ_s, id, &cls);
+  const unsigned bal = __ballot_sync(0xffffffffu, m.kind >= 0);
+  if (lane == 0) warp_cnt[warp] = __popc(bal);
+  __syncthreads();
+  const int mine = lane < NWARPS ? warp_cnt[lane] : 0;
+  const int before = __reduce_add_sync(0xffffffffu, lane < warp ? mine : 0);
+  if (m.kind >= 0) mlist[nm + before + __popc(bal & ((1u << lane) - 1u))] = pack_move(m, cls);
+  const int all = nm + __reduce_add_sync(0xffffffffu, mine);
+  __syncthreads();
+  return all;
+}
+
+// diag_energy's integer count over one thread's share of the sites or bonds.
+__device__ __forceinline__ int diag_count(const LowrankArgs& a, const int8_t* occ_s, int t, int threads) {
+  int cnt = 0;
+  if (a.lat.model == SCALE_MODEL_TJ) {
+    for (int q = t; q < a.nb_nn; q += threads) {
+      const int oi = occ_s[a.bonds[2 * q]], oj = occ_s[a.bonds[2 * q + 1]];
+      cnt += ((oi & 1) - ((oi >> 1) & 1)) * ((oj & 1) - ((oj >> 1) & 1));
+    }
+  } else {
+    const int want = a.lat.model == SCALE_MODEL_HUBBARD ? 3 : 1;
+    for (int i = t; i < a.lat.N; i += threads) cnt += occ_s[i] == want;
+  }
+  return cnt;
+}
+
 inline LowrankArgs make_args(scale_ctx* c) {
   LowrankArgs a{};
   a.lat = c->lat;
