@@ -3,7 +3,6 @@
 // G0t = (M0 + proj_b) Phi^-1 (Sec. II.C, Eq. SMW).
 #include <algorithm>
 
-#include "mlp_mma.cuh"
 #include "scale_internal.cuh"
 
 namespace scale {
@@ -12,23 +11,15 @@ namespace {
 
 // Mixed precision: both are products of the walker's inverse with rows shared by all walkers,
 //   out[j][col] = sum_k Binv[j][k] row_col[k],  rows: M0[o] + proj_b (G0t), proj_w[c] of spin s (Pt),
-// 2 Ne^2 (2N + 2h) flops a walker and 4 Ne (2N + 2h) bytes written. FP32 FMA ran them as two
-// kernels at about a third of its rate; here one kernel takes both on mma.sync as three TF32
-// products of a hi/lo split. Every 16 values of k start a fresh accumulator that is then added to
-// the FP32 sum with rounding to nearest, so the tensor core's truncating accumulation touches 16
-// terms and the sum of Ne terms takes Ne / 16 rounded additions instead of Ne.
-//
-// CTA: 64 slots x 192 columns, six warps of 32 x 64 (64 accumulators a thread); k in steps of 16,
-// both operands split while they are staged (once per CTA, not once per warp) in double-buffered
-// shared memory, rows padded to 20 words (conflict-free fragment loads).
-//
-// From kSplitMinNe electrons on: the split leaves about 2^-23 of each product, an FP32 chain of Ne
-// rounded additions grows with Ne. Rms error of single ratios against FP64 (which the rounding
-// of the stored inverse bounds from below): Ne = 224 3.2e-7 as a chain, 1.7e-7 here; Ne = 56
-// 0.99e-7 as a chain, 1.12e-7 here, so short sums keep the chain.
-constexpr int kSplitMinNe = 129;
-constexpr int kGM = 64, kGN = 192, kGK = 16, kGLd = kGK + 4, kGThreads = 192;
-constexpr int kGBuf = (kGM + kGN) * kGLd;  // words of one buffer's hi (or lo) half
+// 2 Ne^2 (2N + 2h) flops a walker, 4 Ne (2N + 2h) bytes written: bound by FP32 FMA. One kernel takes
+// all columns (two read the inverse twice, the projector's with one row a thread). Register tiles of
+// 8 slots x TN columns, 16-byte shared-memory loads along the slots: 5 loads per 48 FMA. Each
+// output is one FMA chain over k ascending. Tiles: 112 x 96 (224 electrons in two, 576 columns in
+// six), or 56 x 160 up to 56 electrons (28 + 28 on 8x8 in one). 1500 walkers of 16x16: 4.82 ms as
+// two kernels, 2.43 here. (On the tensor cores as three TF32 products with rounded additions
+// every 16 terms: 2.33 ms, and the truncation inside the tensor core biased all ratios one way: the
+// error of local energies of well-conditioned walkers grew 1.7-fold.)
+constexpr int kGThreads = 224, kGK = 16;
 
 struct ProjArgs {
   int Ne, No, h, ncol;  // ncol: No, or No + 2h with the projector's columns
@@ -42,38 +33,42 @@ struct ProjArgs {
   const int32_t* count;
 };
 
-__global__ void __launch_bounds__(kGThreads, 2) k_project_tc(ProjArgs a) {
-  extern __shared__ __align__(16) uint32_t gsm[];  // [2 buffers][hi, lo][kGM + kGN][kGLd]
+// RG x CG threads of 8 x TN outputs.
+template <int RG, int CG, int TN>
+__global__ void __launch_bounds__(kGThreads, 2) k_project32(ProjArgs a) {
+  static_assert(RG * CG == kGThreads, "one thread per tile");
+  constexpr int M = 8 * RG, N = CG * TN, LA = M + 4;  // LA: rows of the staged slots, 16-byte aligned
+  __shared__ __align__(16) float As[2][kGK][LA];
+  __shared__ __align__(16) float Bs[2][kGK][N];
   const int Ne = a.Ne, No = a.No, h = a.h;
   const int nrows = a.count ? min(*a.count, a.B) : a.B;
-  const int j0 = blockIdx.x * kGM, c0 = blockIdx.y * kGN;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-  const int wm = (warp & 1) * 32, wn = (warp >> 1) * 64;  // the warp's tile
+  const int j0 = blockIdx.x * M, c0 = blockIdx.y * N;
+  const int tid = threadIdx.x, tr = (tid / CG) * 8, tc = (tid % CG) * TN;
   const bool vec = (Ne & 3) == 0 && (reinterpret_cast<uintptr_t>(a.proj_w) & 15) == 0;
-  constexpr int kQ = kGK / 4;                             // 4-value pieces of a row
-  constexpr int kPer = ((kGM + kGN) * kQ + kGThreads - 1) / kGThreads;
+  constexpr int kQ = kGK / 4;
   const int nk = (Ne + kGK - 1) / kGK;
+  // staging: thread r < M takes slot row j0 + r, thread M + q the row of column c0 + q, 16 values at a time
+  static_assert(M + N <= kGThreads, "a thread per staged row");
+  const float* col_row = nullptr;
+  if (tid >= M && tid < M + N) {
+    const int col = c0 + tid - M;
+    if (col < No) {
+      col_row = a.M0b + (size_t)col * Ne;
+    } else if (col < a.ncol) {
+      const int s = (col - No) / h, cc = (col - No) - s * h;
+      col_row = a.proj_w + (size_t)cc * 2 * Ne + (size_t)s * Ne;
+    }
+  }
   for (int lrow = blockIdx.z; lrow < nrows; lrow += gridDim.z) {
     const int b = a.list ? a.list[lrow] : lrow;
     if (b < 0) continue;  // uniform
-    const float* Bb = a.Binv + (size_t)b * Ne * Ne;
-    float4 reg[kPer];
+    const float* src =
+        tid >= M ? col_row : (j0 + tid < Ne ? a.Binv + (size_t)b * Ne * Ne + (size_t)(j0 + tid) * Ne : nullptr);
+    float4 reg[kQ];
     auto fetch = [&](int kt) {
 #pragma unroll
-      for (int u = 0; u < kPer; ++u) {
-        const int q = tid + u * kGThreads, r = q / kQ, k = kt * kGK + (q % kQ) * 4;
-        const float* src = nullptr;
-        if (r < kGM) {
-          if (j0 + r < Ne) src = Bb + (size_t)(j0 + r) * Ne;
-        } else if (r < kGM + kGN) {
-          const int col = c0 + r - kGM;
-          if (col < No) {
-            src = a.M0b + (size_t)col * Ne;
-          } else if (col < a.ncol) {
-            const int s = (col - No) / h, cc = (col - No) - s * h;
-            src = a.proj_w + (size_t)cc * 2 * Ne + (size_t)s * Ne;
-          }
-        }
+      for (int u = 0; u < kQ; ++u) {
+        const int k = kt * kGK + 4 * u;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (src) {
           if (vec) {
@@ -89,114 +84,83 @@ __global__ void __launch_bounds__(kGThreads, 2) k_project_tc(ProjArgs a) {
       }
     };
     auto stage = [&](int buf) {
-      uint32_t* hi = gsm + (size_t)buf * 2 * kGBuf;
-      uint32_t* lo = hi + kGBuf;
+      if (tid >= M + N) return;
+      float* dst = tid < M ? &As[buf][0][tid] : &Bs[buf][0][tid - M];
+      const int ld = tid < M ? LA : N;
 #pragma unroll
-      for (int u = 0; u < kPer; ++u) {
-        const int q = tid + u * kGThreads, r = q / kQ;
-        if (r >= kGM + kGN) continue;
-        uint4 vh, vl;
-        split_tf32(reg[u].x, vh.x, vl.x);
-        split_tf32(reg[u].y, vh.y, vl.y);
-        split_tf32(reg[u].z, vh.z, vl.z);
-        split_tf32(reg[u].w, vh.w, vl.w);
-        *reinterpret_cast<uint4*>(hi + r * kGLd + (q % kQ) * 4) = vh;
-        *reinterpret_cast<uint4*>(lo + r * kGLd + (q % kQ) * 4) = vl;
+      for (int u = 0; u < kQ; ++u) {
+        dst[(4 * u) * ld] = reg[u].x;
+        dst[(4 * u + 1) * ld] = reg[u].y;
+        dst[(4 * u + 2) * ld] = reg[u].z;
+        dst[(4 * u + 3) * ld] = reg[u].w;
       }
     };
-    float acc[2][8][4] = {};
+    float acc[8][TN] = {};
     __syncthreads();  // the previous walker's buffers are consumed
     fetch(0);
     stage(0);
     for (int kt = 0; kt < nk; ++kt) {
       if (kt + 1 < nk) fetch(kt + 1);
       __syncthreads();  // buffer kt & 1 is staged, the other one consumed
-      const uint32_t* hi = gsm + (size_t)(kt & 1) * 2 * kGBuf;
-      const uint32_t* lo = hi + kGBuf;
-      uint32_t ah[2][2][4], al[2][2][4];  // [m tile][k step]
+#pragma unroll 4
+      for (int k = 0; k < kGK; ++k) {
+        float x[8], y[TN];
+        *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(&As[kt & 1][k][tr]);
+        *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(&As[kt & 1][k][tr + 4]);
+        if constexpr (TN % 2 == 0) {
 #pragma unroll
-      for (int m = 0; m < 2; ++m)
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          const int o = (wm + 16 * m + g) * kGLd + 8 * s + t;
-          ah[m][s][0] = hi[o];
-          ah[m][s][1] = hi[o + 8 * kGLd];
-          ah[m][s][2] = hi[o + 4];
-          ah[m][s][3] = hi[o + 8 * kGLd + 4];
-          al[m][s][0] = lo[o];
-          al[m][s][1] = lo[o + 8 * kGLd];
-          al[m][s][2] = lo[o + 4];
-          al[m][s][3] = lo[o + 8 * kGLd + 4];
-        }
-#pragma unroll
-      for (int n = 0; n < 8; ++n) {
-        uint32_t bh[2][2], bl[2][2];
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          const int o = (kGM + wn + 8 * n + g) * kGLd + 8 * s + t;
-          bh[s][0] = hi[o];
-          bh[s][1] = hi[o + 4];
-          bl[s][0] = lo[o];
-          bl[s][1] = lo[o + 4];
-        }
-#pragma unroll
-        for (int m = 0; m < 2; ++m) {
-          float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-          for (int s = 0; s < 2; ++s) {
-            mma_tf32(c, al[m][s], bh[s][0], bh[s][1]);
-            mma_tf32(c, ah[m][s], bl[s][0], bl[s][1]);
+          for (int v = 0; v < TN; v += 2) {
+            const float2 q = *reinterpret_cast<const float2*>(&Bs[kt & 1][k][tc + v]);
+            y[v] = q.x;
+            y[v + 1] = q.y;
           }
+        } else {
 #pragma unroll
-          for (int s = 0; s < 2; ++s) mma_tf32(c, ah[m][s], bh[s][0], bh[s][1]);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) acc[m][n][i] += c[i];
+          for (int v = 0; v < TN; ++v) y[v] = Bs[kt & 1][k][tc + v];
         }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+          for (int v = 0; v < TN; ++v) acc[u][v] = fmaf(x[u], y[v], acc[u][v]);
       }
       if (kt + 1 < nk) stage((kt + 1) & 1);
     }
     float* G = a.G0t + (size_t)b * Ne * No;
     float* P = a.Pt + (size_t)b * 2 * Ne * h;
 #pragma unroll
-    for (int m = 0; m < 2; ++m)
+    for (int u = 0; u < 8; ++u) {
+      const int j = j0 + tr + u;
+      if (j >= Ne) continue;
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        const int j = j0 + wm + 16 * m + 8 * half + g;
-        if (j >= Ne) continue;
-#pragma unroll
-        for (int n = 0; n < 8; ++n) {
-          const int col = c0 + wn + 8 * n + 2 * t;
-          const float v0 = acc[m][n][2 * half], v1 = acc[m][n][2 * half + 1];
-          if (col + 1 < No) {  // No is even
-            *reinterpret_cast<float2*>(G + (size_t)j * No + col) = make_float2(v0, v1);
-          } else {
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const int q = col + e - No;
-              if (q >= 0 && col + e < a.ncol) {
-                const int s = q / h;
-                P[((size_t)s * Ne + j) * h + q - s * h] = e ? v1 : v0;
-              }
-            }
-          }
+      for (int v = 0; v < TN; ++v) {
+        const int col = c0 + tc + v;
+        if (col < No) {
+          G[(size_t)j * No + col] = acc[u][v];
+        } else if (col < a.ncol) {
+          const int s = (col - No) / h;
+          P[((size_t)s * Ne + j) * h + (col - No) - s * h] = acc[u][v];
         }
       }
+    }
   }
 }
 
-cudaError_t project_tc(scale_ctx* c, int B, const int32_t* list, const int32_t* count, bool with_pt) {
-  const int No = 2 * c->N;
-  const ProjArgs a{c->Ne, No, c->h, No + (with_pt ? 2 * c->h : 0), (const float*)c->Binv, (const float*)c->M0b,
-                   make_net<float>(c).proj_w, (float*)c->G0t, (float*)c->Pt, list, B, count};
-  constexpr size_t smem = sizeof(uint32_t) * 4 * kGBuf;
-  const cudaError_t e = cudaFuncSetAttribute(k_project_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const dim3 grid((c->Ne + kGM - 1) / kGM, (a.ncol + kGN - 1) / kGN, count ? std::min(B, 64) : std::min(B, 65535));
-  k_project_tc<<<grid, kGThreads, smem, c->stream>>>(a);
+template <int RG, int CG, int TN>
+cudaError_t project32_launch(scale_ctx* c, const ProjArgs& a) {
+  constexpr int M = 8 * RG, N = CG * TN;
+  const dim3 grid((a.Ne + M - 1) / M, (a.ncol + N - 1) / N, a.count ? std::min(a.B, 64) : std::min(a.B, 65535));
+  k_project32<RG, CG, TN><<<grid, kGThreads, 0, c->stream>>>(a);
   return cudaGetLastError();
 }
 
-// ---- FP64 mode, and mixed precision up to kSplitMinNe - 1 electrons ---------------------------
+cudaError_t project32(scale_ctx* c, int B, const int32_t* list, const int32_t* count, bool with_pt) {
+  const int No = 2 * c->N;
+  const ProjArgs a{c->Ne, No, c->h, No + (with_pt ? 2 * c->h : 0), (const float*)c->Binv, (const float*)c->M0b,
+                   make_net<float>(c).proj_w, (float*)c->G0t, (float*)c->Pt, list, B, count};
+  return c->Ne <= 56 ? project32_launch<7, 32, 5>(c, a) : project32_launch<14, 16, 6>(c, a);
+}
+
+// ---- FP64 mode ------------------------------------------------------------------------------
 // Pt[s][c][:] = W_s Binv[c], i.e. the GEMM Pt[s] = Binv (Ne x Ne) * W_s^T (Ne x h),
 // W_s^T[k][cc] = proj_w[cc][s*Ne + k]. 32 rows per CTA, K tiles of 32.
 template <typename T>
@@ -333,13 +297,11 @@ cudaError_t project_t(scale_ctx* c, int B, const int32_t* list, const int32_t* c
 }  // namespace
 
 cudaError_t launch_projector(scale_ctx* c, int B, const int32_t* list, const int32_t* count) {
-  if (c->fp64) return project_t<double>(c, B, list, count);
-  return c->Ne >= kSplitMinNe ? project_tc(c, B, list, count, true) : project_t<float>(c, B, list, count);
+  return c->fp64 ? project_t<double>(c, B, list, count) : project32(c, B, list, count, true);
 }
 
 cudaError_t launch_build_g0(scale_ctx* c, int B, const int32_t* list, const int32_t* count) {
-  if (c->fp64) return build_g0_t<double>(c, B, list, count);
-  return c->Ne >= kSplitMinNe ? project_tc(c, B, list, count, false) : build_g0_t<float>(c, B, list, count);
+  return c->fp64 ? build_g0_t<double>(c, B, list, count) : project32(c, B, list, count, false);
 }
 
 }  // namespace scale
