@@ -243,11 +243,17 @@ __global__ void k_din_tile(Lattice lat, Net<T> net, int l, const T* __restrict__
   }
 }
 
-// ---- the forward and dK with one sample's slabs staged in shared memory --------------------
-// CTA per sample: the layer input rows (the embedding rows for layer 0) and, for dK, dz copied
-// to shared memory once with coalesced loads, and the site table nbr[i][t] (the site reached
-// from i by tap t; -1 past an open edge). The register tiles and the summation order are those
-// of the kernels above, so the results are the same.
+// ---- one sample's slabs staged in shared memory (up to kStagedSites sites) ------------------
+// CTA per sample: the rows a layer reads (its input, the embedding rows for layer 0, or dz) copied
+// to shared memory once with coalesced loads, and the site table nbr[t][i] (the site reached
+// from i by tap t; -1 past an open edge). The summation order is that of the kernels above, so the
+// results are the same. Row stride h plus one 16-byte vector: rows read by the lanes of one warp
+// then lie in different banks (with stride h four site groups hit the same ones).
+constexpr int kStagedSites = 128;
+constexpr int kSM = 2;  // sites per thread of the convolutions
+constexpr int kConvThreads = 512;
+template <typename T>
+constexpr int kDkThreads = sizeof(T) == 4 ? 512 : 288;  // at 4 x 8 sums per thread, registers for one full block
 __device__ __forceinline__ void lds4(const float* p, float (&v)[4]) {
   const float4 q = *reinterpret_cast<const float4*>(p);
   v[0] = q.x;
@@ -263,119 +269,170 @@ __device__ __forceinline__ void lds4(const double* p, double (&v)[4]) {
   v[3] = c.y;
 }
 
-__device__ __forceinline__ void stage_nbr(const Lattice& lat, int stencil, int k, int taps, int sgn, int* nbr) {
+__device__ __forceinline__ void stage_nbr(const Lattice& lat, int stencil, int k, int taps, int sgn, int16_t* nbr) {
   for (int q = threadIdx.x; q < lat.N * taps; q += blockDim.x) {
-    const int i = q / taps, t = q - i * taps;
+    const int t = q / lat.N, i = q - t * lat.N;
     int dx, dy;
     stencil_tap(stencil, k, t, dx, dy);
-    nbr[q] = site_off(lat, i, sgn * dx, sgn * dy);
+    nbr[q] = (int16_t)site_off(lat, i, sgn * dx, sgn * dy);
   }
 }
 
-// Bytes of shared memory of the staged kernels: [slabs][N][h] rows and the [N][taps] table.
-inline size_t grad_smem_bytes(int N, int h, int taps, int slabs, size_t tsize) {
-  return (size_t)slabs * N * h * tsize + (size_t)N * taps * sizeof(int);
+template <typename T>
+__host__ __device__ constexpr int staged_ld(int h) {
+  return h + (int)(16 / sizeof(T));
+}
+// Bytes of shared memory of the staged kernels: [slabs][N][staged_ld] rows and the [taps][N] table.
+template <typename T>
+inline size_t staged_bytes(int N, int h, int taps, int slabs) {
+  return (size_t)slabs * N * staged_ld<T>(h) * sizeof(T) + (size_t)N * taps * sizeof(int16_t);
 }
 
-template <typename T, int HC>
-__global__ void k_fwd_smem(Lattice lat, Net<T> net, int l, int taps, const int8_t* __restrict__ occ,
-                           const T* __restrict__ in, T* __restrict__ out, T* __restrict__ zout) {
+// SM sites x 4 channels per thread of
+//   BACK = 0: out = res in + act(z), zout = z = b + sum_d W[d]^T in_{i+d}     (W = kernel)
+//   BACK = 1: out = res dout + sum_d W[d]^T dz_{i-d}, dz = dout act'(z)       (W = kernel transposed)
+// a: in, or dout; z: zout (written), or z (read).
+template <typename T, int HC, int SM, int BACK>
+__global__ void __launch_bounds__(kConvThreads) k_conv_staged(Lattice lat, Net<T> net, int l, int taps, const T* __restrict__ W,
+                              const int8_t* __restrict__ occ, const T* __restrict__ a, T* __restrict__ z,
+                              T* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char gsm[];
-  const int h = HC ? HC : net.h, N = lat.N, hq = h >> 2;
+  const int h = HC ? HC : net.h, N = lat.N, hq = h >> 2, ld = staged_ld<T>(h);
   const int b = blockIdx.x;
   T* xs = reinterpret_cast<T*>(gsm);
-  int* nbr = reinterpret_cast<int*>(xs + (size_t)N * h);
+  int16_t* nbr = reinterpret_cast<int16_t*>(xs + (size_t)N * ld);
   const int8_t* ob = occ + (size_t)b * N;
-  const T* in_b = in + (size_t)b * N * h;
+  const size_t base = (size_t)b * N * h;
   for (int q = threadIdx.x; q < N * h; q += blockDim.x) {
     const int i = q / h, c = q - i * h;
-    xs[q] = layer_in_row(net, l, ob, in_b, i, h)[c];
+    if constexpr (BACK)
+      xs[i * ld + c] = a[base + q] * act_grad<T>(net.act, z[base + q]);
+    else
+      xs[i * ld + c] = layer_in_row(net, l, ob, a + base, i, h)[c];
   }
-  stage_nbr(lat, net.stencil, net.ksize[l], taps, 1, nbr);
+  stage_nbr(lat, net.stencil, net.ksize[l], taps, BACK ? -1 : 1, nbr);
   __syncthreads();
-  const int tiles = ((N + 3) >> 2) * hq;
+  const int tiles = ((N + SM - 1) / SM) * hq;
   for (int q = threadIdx.x; q < tiles; q += blockDim.x) {
-    const int sq = q / hq, c0 = (q - sq * hq) * 4;
-    T acc[4][4];
+    const int i0 = (q / hq) * SM, c0 = (q % hq) * 4;
+    T acc[SM][4];
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+    for (int s = 0; s < SM; ++s)
 #pragma unroll
-      for (int m = 0; m < 4; ++m) acc[s][m] = net.bias[l][c0 + m];
-    for (int t = 0; t < taps; ++t) {
-      int row[4];
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int i = sq * 4 + s;
-        row[s] = i < N ? nbr[i * taps + t] : -1;
+      for (int m = 0; m < 4; ++m) {
+        if constexpr (BACK)
+          acc[s][m] = (net.resid[l] && i0 + s < N) ? a[base + (size_t)(i0 + s) * h + c0 + m] : T(0);
+        else
+          acc[s][m] = net.bias[l][c0 + m];
       }
-      const T* w = net.kernel[l] + (size_t)t * h * h + c0;
+    for (int t = 0; t < taps; ++t) {
+      int row[SM];
+#pragma unroll
+      for (int s = 0; s < SM; ++s) row[s] = i0 + s < N ? nbr[t * N + i0 + s] : -1;
+      const T* w = W + (size_t)t * h * h + c0;
 #pragma unroll
       for (int ci = 0; ci < h; ci += 4) {
         T wv[4][4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) ld4(w + (size_t)(ci + a) * h, wv[a]);
+        for (int k = 0; k < 4; ++k) ld4(w + (size_t)(ci + k) * h, wv[k]);
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
+        for (int s = 0; s < SM; ++s) {
           if (row[s] < 0) continue;
           T xv[4];
-          lds4(xs + (size_t)row[s] * h + ci, xv);
+          lds4(xs + row[s] * ld + ci, xv);
 #pragma unroll
-          for (int a = 0; a < 4; ++a)
+          for (int k = 0; k < 4; ++k)
 #pragma unroll
-            for (int m = 0; m < 4; ++m) acc[s][m] = fma(xv[a], wv[a][m], acc[s][m]);
+            for (int m = 0; m < 4; ++m) acc[s][m] = fma(xv[k], wv[k][m], acc[s][m]);
         }
       }
     }
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const int i = sq * 4 + s;
+    for (int s = 0; s < SM; ++s) {
+      const int i = i0 + s;
       if (i >= N) break;
-      const size_t o = ((size_t)b * N + i) * h + c0;
+      const size_t o = base + (size_t)i * h + c0;
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        out[o + m] = (net.resid[l] ? xs[(size_t)i * h + c0 + m] : T(0)) + act_fn<T>(net.act, acc[s][m]);
-        zout[o + m] = acc[s][m];
+        if constexpr (BACK) {
+          out[o + m] = acc[s][m];
+        } else {
+          out[o + m] = (net.resid[l] ? xs[i * ld + c0 + m] : T(0)) + act_fn<T>(net.act, acc[s][m]);
+          z[o + m] = acc[s][m];
+        }
       }
     }
   }
 }
 
+// dK, and the bias gradient by the block's last warps. dz = dout act'(z) is formed while it is staged.
+// Four sites of a tap at a time, their loads in flight before the first use.
 template <typename T, int HC>
-__global__ void k_dk_smem(Lattice lat, Net<T> net, int l, int taps, const int8_t* __restrict__ occ,
-                          const T* __restrict__ in, const T* __restrict__ dz, int64_t off_k, int64_t P,
-                          double* __restrict__ grad) {
+__global__ void __launch_bounds__(kDkThreads<T> + 64) k_dk_staged(Lattice lat, Net<T> net, int l, int taps, int dk_threads, const int8_t* __restrict__ occ,
+                            const T* __restrict__ in, const T* __restrict__ dout, const T* __restrict__ z, int64_t off_k,
+                            int64_t off_b, int64_t P, double* __restrict__ grad) {
   extern __shared__ __align__(16) unsigned char gsm[];
-  const int N = lat.N, h = HC ? HC : net.h, hq = h >> 2, ho = h >> 3;
+  const int N = lat.N, h = HC ? HC : net.h, hq = h >> 2, ho = h >> 3, ld = staged_ld<T>(h);
   const int b = blockIdx.x;
   T* xs = reinterpret_cast<T*>(gsm);
-  T* gs = xs + (size_t)N * h;
-  int* nbr = reinterpret_cast<int*>(gs + (size_t)N * h);
+  T* gs = xs + (size_t)N * ld;
+  int16_t* nbr = reinterpret_cast<int16_t*>(gs + (size_t)N * ld);
   const int8_t* ob = occ + (size_t)b * N;
-  const T* in_b = in + (size_t)b * N * h;
-  const T* dz_b = dz + (size_t)b * N * h;
+  const size_t base = (size_t)b * N * h;
   for (int q = threadIdx.x; q < N * h; q += blockDim.x) {
     const int i = q / h, c = q - i * h;
-    xs[q] = layer_in_row(net, l, ob, in_b, i, h)[c];
-    gs[q] = dz_b[q];
+    xs[i * ld + c] = layer_in_row(net, l, ob, in + base, i, h)[c];
+    gs[i * ld + c] = dout[base + q] * act_grad<T>(net.act, z[base + q]);
   }
   stage_nbr(lat, net.stencil, net.ksize[l], taps, 1, nbr);
   __syncthreads();
-  for (int q = threadIdx.x; q < taps * hq * ho; q += blockDim.x) {
+  double* g0 = grad + (size_t)b * P;
+  if ((int)threadIdx.x >= dk_threads) {  // db = sum_i dz_i
+    for (int c = threadIdx.x - dk_threads; c < h; c += blockDim.x - dk_threads) {
+      double acc = 0.0;
+      for (int i = 0; i < N; ++i) acc += (double)gs[i * ld + c];
+      g0[off_b + c] = acc;
+    }
+    return;
+  }
+  for (int q = threadIdx.x; q < taps * hq * ho; q += dk_threads) {
     const int t = q / (hq * ho), rem = q - t * hq * ho, ci0 = (rem / ho) * 4, co0 = (rem % ho) * 8;
     T acc[4][8] = {};
-    for (int i = 0; i < N; ++i) {
-      const int j = nbr[i * taps + t];
+    const int16_t* nt = nbr + t * N;
+    constexpr int U = 4;
+    int i = 0;
+    for (; i + U <= N; i += U) {
+      T xv[U][4], gv[U][2][4];
+      int j[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        j[u] = nt[i + u];
+        lds4(xs + (j[u] < 0 ? 0 : j[u]) * ld + ci0, xv[u]);
+        lds4(gs + (i + u) * ld + co0, gv[u][0]);
+        lds4(gs + (i + u) * ld + co0 + 4, gv[u][1]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (j[u] < 0) continue;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int m = 0; m < 8; ++m) acc[a][m] = fma(xv[u][a], gv[u][m >> 2][m & 3], acc[a][m]);
+      }
+    }
+    for (; i < N; ++i) {
+      const int j = nt[i];
       if (j < 0) continue;
       T xv[4], gv[2][4];
-      lds4(xs + (size_t)j * h + ci0, xv);
-      lds4(gs + (size_t)i * h + co0, gv[0]);
-      lds4(gs + (size_t)i * h + co0 + 4, gv[1]);
+      lds4(xs + j * ld + ci0, xv);
+      lds4(gs + i * ld + co0, gv[0]);
+      lds4(gs + i * ld + co0 + 4, gv[1]);
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int m = 0; m < 8; ++m) acc[a][m] = fma(xv[a], gv[m >> 2][m & 3], acc[a][m]);
     }
-    double* g = grad + (size_t)b * P + off_k + (size_t)t * h * h + co0;
+    double* g = g0 + off_k + (size_t)t * h * h + co0;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -532,18 +589,18 @@ __global__ void k_nan_bad(int B, int64_t P, const int32_t* __restrict__ status, 
   for (int64_t q = threadIdx.x; q < P; q += blockDim.x) grad[(size_t)b * P + q] = CUDART_NAN;
 }
 
-// One CTA per sample with `smem` bytes of staged slabs; the block covers the sample's work
-// (one tile per thread up to 1024 tiles, beyond that each thread loops over its share).
+// One CTA per sample of `block` threads with `smem` bytes of staged slabs.
 template <typename... KA, typename... A>
-cudaError_t staged_launch(void (*kern)(KA...), int B, int work, size_t smem, cudaStream_t st, A... args) {
+cudaError_t staged_launch(void (*kern)(KA...), int B, int block, size_t smem, cudaStream_t st, A... args) {
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  const int block = std::min(1024, std::max(32, (work + 31) / 32 * 32));  // one tile per thread
   kern<<<B, block, smem, st>>>(args...);
   return cudaGetLastError();
 }
+// Threads for `work` items: one each up to `most`, beyond that each thread loops over its share.
+inline int staged_block(int work, int most) { return std::min(most, std::max(32, (work + 31) / 32 * 32)); }
 
 constexpr size_t kGradSmemMax = 96 * 1024;  // staged slabs up to this size (a few CTAs per SM)
 
@@ -558,7 +615,7 @@ cudaError_t grad_t(scale_ctx* c, double* grad, int recompute) {
   // the tiled kernels with one sample's slabs staged in shared memory: small lattices (the
   // 16x4 cylinder: forward 109 -> 96 us, dK 216 -> 140 us per 2048 walkers); at 256 sites the
   // 73 KB of staged slabs per sample cost more than the L1-served kernels (measured)
-  const bool staged = tiled && N <= 128 && grad_smem_bytes(N, h, max_taps, 2, sizeof(T)) <= kGradSmemMax;
+  const bool staged = tiled && N <= kStagedSites && staged_bytes<T>(N, h, max_taps, 2) <= kGradSmemMax;
   // stored: every layer's input and pre-activation kept from the one forward pass; recompute:
   // only every stride-th layer input, each segment's forward recomputed during the backward
   const int stride = recompute ? std::max(1, (int)std::ceil(std::sqrt((double)L))) : 1;
@@ -619,21 +676,24 @@ cudaError_t grad_t(scale_ctx* c, double* grad, int recompute) {
     case 64: KERNEL<T, 64><<<GRID, 128, 0, c->stream>>>(__VA_ARGS__); break;               \
     default: KERNEL<T, 0><<<GRID, 128, 0, c->stream>>>(__VA_ARGS__);                       \
   }
-#define SCALE_GRAD_STAGED(KERNEL, WORK, SMEM, ...)                                                            \
-  switch (h) {                                                                                               \
-    case 8: e = staged_launch(KERNEL<T, 8>, B, WORK, SMEM, c->stream, __VA_ARGS__); break;                   \
-    case 16: e = staged_launch(KERNEL<T, 16>, B, WORK, SMEM, c->stream, __VA_ARGS__); break;                 \
-    case 32: e = staged_launch(KERNEL<T, 32>, B, WORK, SMEM, c->stream, __VA_ARGS__); break;                 \
-    case 64: e = staged_launch(KERNEL<T, 64>, B, WORK, SMEM, c->stream, __VA_ARGS__); break;                 \
-    default: e = staged_launch(KERNEL<T, 0>, B, WORK, SMEM, c->stream, __VA_ARGS__);                         \
+#define SCALE_GRAD_STAGED(CALL)     \
+  switch (h) {                      \
+    case 8: CALL(8); break;         \
+    case 16: CALL(16); break;       \
+    case 32: CALL(32); break;       \
+    case 64: CALL(64); break;       \
+    default: CALL(0);               \
   }
-  const int site_tiles = ((N + 3) / 4) * (h / 4);
+  const int conv_block = staged_block(((N + kSM - 1) / kSM) * (h / 4), kConvThreads);
   cudaError_t e = cudaSuccess;
   auto fwd = [&](int l, const T* in, T* out, T* z) {
     if (staged) {
       const int tl = stencil_taps(net.stencil, net.ksize[l]);
-      SCALE_GRAD_STAGED(k_fwd_smem, site_tiles, grad_smem_bytes(N, h, tl, 1, sizeof(T)), c->lat, net, l, tl, c->occ,
-                        in, out, z);
+#define SCALE_CALL(HC)                                                                                            \
+  e = staged_launch(k_conv_staged<T, HC, kSM, 0>, B, conv_block, staged_bytes<T>(N, h, tl, 1), c->stream, c->lat, net, l, \
+                    tl, net.kernel[l], c->occ, in, z, out)
+      SCALE_GRAD_STAGED(SCALE_CALL)
+#undef SCALE_CALL
     } else if (tiled) {
       SCALE_GRAD_TILED(k_fwd_tile, gridT, c->lat, net, l, c->occ, in, out, z);
     } else {
@@ -671,15 +731,23 @@ cudaError_t grad_t(scale_ctx* c, double* grad, int recompute) {
     }
     for (int l = l1 - 1; l >= l0; --l) {
       const T* lin = (l == 0) ? nullptr : (l == l0 ? ck + (size_t)sg * slab : segH + (size_t)(l - l0) * slab);
-      const T* zl = recompute ? segZ + (size_t)(l - l0) * slab : segZ + (size_t)l * slab;
-      k_grad_dz<T><<<B, 256, 0, c->stream>>>(c->lat, net, l, dcur, zl, dZ, offB[l], c->P, grad);
+      T* zl = recompute ? segZ + (size_t)(l - l0) * slab : segZ + (size_t)l * slab;
       const int kq = tiled ? taps[l] * (h / 4) * (h / 8) : taps[l] * h * h;
+      if (!staged) k_grad_dz<T><<<B, 256, 0, c->stream>>>(c->lat, net, l, dcur, zl, dZ, offB[l], c->P, grad);
       if (staged) {
-        SCALE_GRAD_STAGED(k_dk_smem, kq, grad_smem_bytes(N, h, taps[l], 2, sizeof(T)), c->lat, net, l, taps[l], c->occ,
-                          lin, dZ, offK[l], c->P, grad);
+        const int dkb = staged_block(kq, kDkThreads<T>);
+#define SCALE_CALL(HC)                                                                                              \
+  e = staged_launch(k_dk_staged<T, HC>, B, dkb + std::min(64, (h + 31) / 32 * 32), staged_bytes<T>(N, h, taps[l], 2),   \
+                    c->stream, c->lat, net, l, taps[l], dkb, c->occ, lin, dcur, zl, offK[l], offB[l], c->P, grad)
+        SCALE_GRAD_STAGED(SCALE_CALL)
+#undef SCALE_CALL
         if (e != cudaSuccess) return e;
-        // the input gradient reads dz through L1 as fast as from a staged copy (measured)
-        SCALE_GRAD_TILED(k_din_tile, gridT, c->lat, net, l, KTl[l], dcur, dZ, dnext);
+#define SCALE_CALL(HC)                                                                                             \
+  e = staged_launch(k_conv_staged<T, HC, kSM, 1>, B, conv_block, staged_bytes<T>(N, h, taps[l], 1), c->stream, c->lat, net, \
+                    l, taps[l], KTl[l], c->occ, dcur, zl, dnext)
+        SCALE_GRAD_STAGED(SCALE_CALL)
+#undef SCALE_CALL
+        if (e != cudaSuccess) return e;
       } else if (tiled) {
         const dim3 gridK((kq + 127) / 128, B);
         SCALE_GRAD_TILED(k_dk_tile, gridK, c->lat, net, l, taps[l], c->occ, lin, dZ, offK[l], c->P, grad);
