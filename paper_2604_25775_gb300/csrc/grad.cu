@@ -15,6 +15,7 @@
 #include <cmath>
 
 #include "scale_internal.cuh"
+#include "tcgen05.cuh"
 
 namespace scale {
 
@@ -245,15 +246,38 @@ __global__ void k_din_tile(Lattice lat, Net<T> net, int l, const T* __restrict__
 
 // ---- one sample's slabs staged in shared memory (up to kStagedSites sites) ------------------
 // CTA per sample: the rows a layer reads (its input, the embedding rows for layer 0, or dz) copied
-// to shared memory once with coalesced loads, and the site table nbr[t][i] (the site reached
+// to shared memory once with 16-byte loads, and the site table nbr[t][i] (the site reached
 // from i by tap t; -1 past an open edge). The summation order is that of the kernels above, so the
 // results are the same. Row stride h plus one 16-byte vector: rows read by the lanes of one warp
-// then lie in different banks (with stride h four site groups hit the same ones).
+// then lie in different banks (with stride h four site groups hit the same ones). The weights come
+// through shared memory in chunks ahead of their use: all walkers' CTAs run in one wave and step through
+// the taps together, so each read of a weight row through L1 waited for L2.
+// What bounds them: 512 walkers are 3.4 CTAs per SM, so staging, sums and output of a layer follow one
+// another with little to overlap (sums about half of it). Per layer of the 16x4 cylinder, 512 walkers:
+// forward 45 -> 25 us, input gradient with dz 53 -> 25, dK 50 -> 29 (of which the FP64 output of
+// 38 MB takes 7).
 constexpr int kStagedSites = 128;
-constexpr int kSM = 2;  // sites per thread of the convolutions
-constexpr int kConvThreads = 512;
+constexpr int kConvThreads = 256;
+// Sites per thread of the convolutions and input rows per thread of dK, by 8 channels. In FP32 a
+// 16-byte load from shared memory occupies the SM for four cycles and a warp's FMA for a quarter:
+// 2 x 4 sums per thread ran at the loads' rate (33 us a layer of the 16x4 cylinder, 512 walkers; the
+// FMAs alone take 8), 2 x 8 take 25 and 4 x 8 29 (two warps per walker hide too little). In FP64 the
+// FP64 pipe is the limit and one site per thread keeps more warps (an update of 8x8, 200 walkers:
+// 1.42 ms, with two sites 1.55, with four 1.73). dK by 8 x 8: 31 us a layer against 29 by 4 x 8.
 template <typename T>
-constexpr int kDkThreads = sizeof(T) == 4 ? 512 : 288;  // at 4 x 8 sums per thread, registers for one full block
+constexpr int kConvSites = sizeof(T) == 4 ? 2 : 1;
+constexpr int kDkRows = 4;
+template <typename T>
+constexpr int kDkThreads = sizeof(T) == 4 ? 640 : 288;  // registers for a full block
+__host__ __device__ constexpr int bias_threads(int h) { return (h + 31) / 32 * 32; }
+// The conversion to FP64 in integers (the FP64 pipe is 64 times narrower): exponent and mantissa of
+// a normal number; the rest by the instruction.
+__device__ __forceinline__ double to_double(float x) {
+  const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u;
+  if (e == 0 || e == 0x7f800000u) return (double)x;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double to_double(double x) { return x; }
 __device__ __forceinline__ void lds4(const float* p, float (&v)[4]) {
   const float4 q = *reinterpret_cast<const float4*>(p);
   v[0] = q.x;
@@ -269,13 +293,18 @@ __device__ __forceinline__ void lds4(const double* p, double (&v)[4]) {
   v[3] = c.y;
 }
 
-__device__ __forceinline__ void stage_nbr(const Lattice& lat, int stencil, int k, int taps, int sgn, int16_t* nbr) {
-  for (int q = threadIdx.x; q < lat.N * taps; q += blockDim.x) {
-    const int t = q / lat.N, i = q - t * lat.N;
-    int dx, dy;
-    stencil_tap(stencil, k, t, dx, dy);
-    nbr[q] = (int16_t)site_off(lat, i, sgn * dx, sgn * dy);
-  }
+// The table of a layer lies in device memory (k_grad_prep; with the divisions per CTA the staging
+// took longer than the sums), padded to whole 16-byte pieces.
+__host__ __device__ constexpr int nbr_size(int N, int taps) { return (N * taps + 7) & ~7; }
+__device__ __forceinline__ void stage_nbr(const int16_t* __restrict__ table, int n, int16_t* nbr) {
+  for (int q = threadIdx.x * 8; q < n; q += blockDim.x * 8) tc::cp_async16(nbr + q, table + q);
+}
+__device__ __forceinline__ void sts4(float* p, const float (&v)[4]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void sts4(double* p, const double (&v)[4]) {
+  *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+  *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
 }
 
 template <typename T>
@@ -285,66 +314,125 @@ __host__ __device__ constexpr int staged_ld(int h) {
 // Bytes of shared memory of the staged kernels: [slabs][N][staged_ld] rows and the [taps][N] table.
 template <typename T>
 inline size_t staged_bytes(int N, int h, int taps, int slabs) {
-  return (size_t)slabs * N * staged_ld<T>(h) * sizeof(T) + (size_t)N * taps * sizeof(int16_t);
+  return (size_t)slabs * N * staged_ld<T>(h) * sizeof(T) + (size_t)nbr_size(N, taps) * sizeof(int16_t);
 }
 
-// SM sites x 4 channels per thread of
+// Weight rows of one tap that are in shared memory at a time: at most 8 KB, a divisor of h.
+constexpr int kWStages = 3;
+template <typename T>
+__host__ __device__ constexpr int conv_rows(int h) {
+  int r = h;
+  while (r > 4 && ((size_t)r * h * sizeof(T) > 8192 || h % r || r % 4)) r -= 4;
+  return r;
+}
+template <typename T>
+inline size_t conv_bytes(int N, int h, int taps) {
+  return staged_bytes<T>(N, h, taps, 1) + (size_t)kWStages * conv_rows<T>(h) * h * sizeof(T);
+}
+
+// SM sites x CM channels per thread of
 //   BACK = 0: out = res in + act(z), zout = z = b + sum_d W[d]^T in_{i+d}     (W = kernel)
-//   BACK = 1: out = res dout + sum_d W[d]^T dz_{i-d}, dz = dout act'(z)       (W = kernel transposed)
+//   BACK = 1: out = res dout + sum_d W[d]^T dz_{i-d}, dz = dout act'(z)       (W = kernel transposed),
+//             kept for dK, and the bias gradient sum_i dz_i by the block's last threads
 // a: in, or dout; z: zout (written), or z (read).
-template <typename T, int HC, int SM, int BACK>
-__global__ void __launch_bounds__(kConvThreads) k_conv_staged(Lattice lat, Net<T> net, int l, int taps, const T* __restrict__ W,
-                              const int8_t* __restrict__ occ, const T* __restrict__ a, T* __restrict__ z,
-                              T* __restrict__ out) {
+template <typename T, int HC, int BACK>
+__global__ void __launch_bounds__(kConvThreads + 64, 2)
+    k_conv_staged(Lattice lat, Net<T> net, int l, int taps, const int16_t* __restrict__ table,
+                  const T* __restrict__ W, const int8_t* __restrict__ occ, const T* __restrict__ a, T* __restrict__ z, T* __restrict__ out, T* __restrict__ dz, int64_t off_b, int64_t P,
+                  double* __restrict__ grad) {
+  constexpr int SM = kConvSites<T>, CM = 8;
   extern __shared__ __align__(16) unsigned char gsm[];
-  const int h = HC ? HC : net.h, N = lat.N, hq = h >> 2, ld = staged_ld<T>(h);
+  const int h = HC ? HC : net.h, N = lat.N, hq = h / CM, ld = staged_ld<T>(h);
+  const int R = conv_rows<T>(h), per = h / R, chunks = taps * per;
   const int b = blockIdx.x;
-  T* xs = reinterpret_cast<T*>(gsm);
+  T* ws = reinterpret_cast<T*>(gsm);  // [kWStages][R][h] weight rows
+  T* xs = ws + (size_t)kWStages * R * h;
   int16_t* nbr = reinterpret_cast<int16_t*>(xs + (size_t)N * ld);
   const int8_t* ob = occ + (size_t)b * N;
   const size_t base = (size_t)b * N * h;
-  for (int q = threadIdx.x; q < N * h; q += blockDim.x) {
-    const int i = q / h, c = q - i * h;
-    if constexpr (BACK)
-      xs[i * ld + c] = a[base + q] * act_grad<T>(net.act, z[base + q]);
-    else
-      xs[i * ld + c] = layer_in_row(net, l, ob, a + base, i, h)[c];
-  }
-  stage_nbr(lat, net.stencil, net.ksize[l], taps, BACK ? -1 : 1, nbr);
-  __syncthreads();
-  const int tiles = ((N + SM - 1) / SM) * hq;
-  for (int q = threadIdx.x; q < tiles; q += blockDim.x) {
-    const int i0 = (q / hq) * SM, c0 = (q % hq) * 4;
-    T acc[SM][4];
+  constexpr int V = 16 / sizeof(T);
+  auto load = [&](int k) {  // one commit group per call, empty past the last chunk
+    if (k < chunks)
+      for (int q = threadIdx.x * V; q < R * h; q += blockDim.x * V)
+        tc::cp_async16(ws + (size_t)(k % kWStages) * R * h + q, W + (size_t)k * R * h + q);
+    tc::cp_async_commit();
+  };
+  const int tiles = ((N + SM - 1) / SM) * hq, workers = BACK ? blockDim.x - bias_threads(h) : blockDim.x;
+  const int cb = BACK ? (int)threadIdx.x - workers : -1, bsites = (N + chunks - 1) / chunks;
+  double db = 0.0;
+  for (int q0 = 0; q0 < tiles; q0 += workers) {
+    if (q0 == 0) stage_nbr(table, nbr_size(N, taps), nbr);  // in the group of the first chunk
+    for (int k = 0; k < kWStages - 1; ++k) load(k);
+    if (q0 == 0) {
+#pragma unroll 4
+      for (int q = threadIdx.x * 4; q < N * h; q += blockDim.x * 4) {
+        const int i = q / h, c = q - i * h;
+        T v[4];
+        if constexpr (BACK) {
+          T zv[4];
+          ld4(a + base + q, v);
+          ld4(z + base + q, zv);
+#pragma unroll
+          for (int m = 0; m < 4; ++m) v[m] *= act_grad<T>(net.act, zv[m]);
+          sts4(dz + base + q, v);
+        } else {
+          ld4(layer_in_row(net, l, ob, a + base, i, h) + c, v);
+        }
+        sts4(xs + i * ld + c, v);
+      }
+    }
+    const int q = q0 + threadIdx.x;
+    // i0 = N: no sites (a thread past the tiles, or of the bias sums)
+    const int i0 = q < tiles && (int)threadIdx.x < workers ? (q / hq) * SM : N, c0 = (q % hq) * CM;
+    T acc[SM][CM];
 #pragma unroll
     for (int s = 0; s < SM; ++s)
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
+      for (int m = 0; m < CM; ++m) {
         if constexpr (BACK)
           acc[s][m] = (net.resid[l] && i0 + s < N) ? a[base + (size_t)(i0 + s) * h + c0 + m] : T(0);
         else
           acc[s][m] = net.bias[l][c0 + m];
       }
-    for (int t = 0; t < taps; ++t) {
-      int row[SM];
+    for (int k = 0; k < chunks; ++k) {
+      tc::cp_async_wait<kWStages - 2>();
+      __syncthreads();  // chunk k has landed for every thread; chunk k - 1 is no longer read
+      load(k + kWStages - 1);
+      if (BACK && q0 == 0 && cb >= 0 && cb < h)  // a few sites per chunk, in order
+        for (int i = k * bsites; i < min(N, (k + 1) * bsites); ++i) db += to_double(xs[i * ld + cb]);
+      const int t = k / per, ci0 = (k - t * per) * R;
+      int row[SM], n_in = 0;
 #pragma unroll
-      for (int s = 0; s < SM; ++s) row[s] = i0 + s < N ? nbr[t * N + i0 + s] : -1;
-      const T* w = W + (size_t)t * h * h + c0;
+      for (int s = 0; s < SM; ++s) {
+        row[s] = i0 + s < N ? nbr[t * N + i0 + s] : -1;
+        n_in += row[s] >= 0;
+      }
+      const T* w = ws + (size_t)(k % kWStages) * R * h + c0;
+      const T* x = xs + ci0;
+      auto step = [&](int ci, bool all) {
+        T xv[SM][4];
 #pragma unroll
-      for (int ci = 0; ci < h; ci += 4) {
-        T wv[4][4];
+        for (int s = 0; s < SM; ++s)
+          if (all || row[s] >= 0) lds4(x + row[s] * ld + ci, xv[s]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) ld4(w + (size_t)(ci + k) * h, wv[k]);
+        for (int r = 0; r < 4; ++r) {
+          T wv[CM];
 #pragma unroll
-        for (int s = 0; s < SM; ++s) {
-          if (row[s] < 0) continue;
-          T xv[4];
-          lds4(xs + row[s] * ld + ci, xv);
+          for (int m = 0; m < CM; m += 4) lds4(w + (ci + r) * h + m, reinterpret_cast<T(&)[4]>(wv[m]));
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
+          for (int s = 0; s < SM; ++s) {
+            if (!all && row[s] < 0) continue;
 #pragma unroll
-            for (int m = 0; m < 4; ++m) acc[s][m] = fma(xv[k], wv[k][m], acc[s][m]);
+            for (int m = 0; m < CM; ++m) acc[s][m] = fma(xv[s][r], wv[m], acc[s][m]);
+          }
         }
+      };
+      if (n_in == SM) {
+#pragma unroll 2
+        for (int ci = 0; ci < R; ci += 4) step(ci, true);
+      } else if (n_in) {
+#pragma unroll 1
+        for (int ci = 0; ci < R; ci += 4) step(ci, false);
       }
     }
 #pragma unroll
@@ -353,90 +441,98 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_staged(Lattice lat, Net<T
       if (i >= N) break;
       const size_t o = base + (size_t)i * h + c0;
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        if constexpr (BACK) {
-          out[o + m] = acc[s][m];
+      for (int m = 0; m < CM; m += 4) {
+        T(&v)[4] = reinterpret_cast<T(&)[4]>(acc[s][m]);
+        if constexpr (!BACK) {
+          T r[4] = {};
+          if (net.resid[l]) lds4(xs + i * ld + c0 + m, r);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) r[e] += act_fn<T>(net.act, v[e]);
+          sts4(z + o + m, v);
+          sts4(out + o + m, r);
         } else {
-          out[o + m] = (net.resid[l] ? xs[i * ld + c0 + m] : T(0)) + act_fn<T>(net.act, acc[s][m]);
-          z[o + m] = acc[s][m];
+          sts4(out + o + m, v);
         }
       }
     }
+    __syncthreads();  // the weight rows of this pass are no longer read
   }
+  if (BACK && cb >= 0 && cb < h) grad[(size_t)b * P + off_b + cb] = db;
 }
 
-// dK, and the bias gradient by the block's last warps. dz = dout act'(z) is formed while it is staged.
-// Four sites of a tap at a time, their loads in flight before the first use.
+// dK: RI input x 8 output channels of a tap per thread.
+// U sites of a tap at a time, their loads in flight before the first use. A thread's eight columns
+// are co = m h/8 + its group, so that the lanes of a store write neighbouring words; the columns of dz
+// lie in that order in shared memory.
 template <typename T, int HC>
-__global__ void __launch_bounds__(kDkThreads<T> + 64) k_dk_staged(Lattice lat, Net<T> net, int l, int taps, int dk_threads, const int8_t* __restrict__ occ,
-                            const T* __restrict__ in, const T* __restrict__ dout, const T* __restrict__ z, int64_t off_k,
-                            int64_t off_b, int64_t P, double* __restrict__ grad) {
+__global__ void __launch_bounds__(kDkThreads<T>)
+    k_dk_staged(Lattice lat, Net<T> net, int l, int taps, const int16_t* __restrict__ table,
+                const int8_t* __restrict__ occ, const T* __restrict__ in, const T* __restrict__ dz, int64_t off_k, int64_t P,
+                double* __restrict__ grad) {
+  constexpr int RI = kDkRows, U = 4;
   extern __shared__ __align__(16) unsigned char gsm[];
-  const int N = lat.N, h = HC ? HC : net.h, hq = h >> 2, ho = h >> 3, ld = staged_ld<T>(h);
+  const int N = lat.N, h = HC ? HC : net.h, hq = h / RI, ho = h >> 3, ld = staged_ld<T>(h);
   const int b = blockIdx.x;
   T* xs = reinterpret_cast<T*>(gsm);
   T* gs = xs + (size_t)N * ld;
   int16_t* nbr = reinterpret_cast<int16_t*>(gs + (size_t)N * ld);
   const int8_t* ob = occ + (size_t)b * N;
   const size_t base = (size_t)b * N * h;
-  for (int q = threadIdx.x; q < N * h; q += blockDim.x) {
+  stage_nbr(table, nbr_size(N, taps), nbr);
+  tc::cp_async_commit();
+#pragma unroll 4
+  for (int q = threadIdx.x * 4; q < N * h; q += blockDim.x * 4) {
     const int i = q / h, c = q - i * h;
-    xs[i * ld + c] = layer_in_row(net, l, ob, in + base, i, h)[c];
-    gs[i * ld + c] = dout[base + q] * act_grad<T>(net.act, z[base + q]);
+    T v[4], gv[4];
+    ld4(layer_in_row(net, l, ob, in + base, i, h) + c, v);
+    ld4(dz + base + q, gv);
+    sts4(xs + i * ld + c, v);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) gs[i * ld + ((c + m) % ho) * 8 + (c + m) / ho] = gv[m];
   }
-  stage_nbr(lat, net.stencil, net.ksize[l], taps, 1, nbr);
+  tc::cp_async_wait<0>();
   __syncthreads();
-  double* g0 = grad + (size_t)b * P;
-  if ((int)threadIdx.x >= dk_threads) {  // db = sum_i dz_i
-    for (int c = threadIdx.x - dk_threads; c < h; c += blockDim.x - dk_threads) {
-      double acc = 0.0;
-      for (int i = 0; i < N; ++i) acc += (double)gs[i * ld + c];
-      g0[off_b + c] = acc;
-    }
-    return;
-  }
-  for (int q = threadIdx.x; q < taps * hq * ho; q += dk_threads) {
-    const int t = q / (hq * ho), rem = q - t * hq * ho, ci0 = (rem / ho) * 4, co0 = (rem % ho) * 8;
-    T acc[4][8] = {};
+  for (int q = threadIdx.x; q < taps * hq * ho; q += blockDim.x) {
+    const int t = q / (hq * ho), rem = q - t * hq * ho, ci0 = (rem / ho) * RI, cg = rem % ho;
+    T acc[RI][8] = {};
     const int16_t* nt = nbr + t * N;
-    constexpr int U = 4;
+    const T* x = xs + ci0;
+    const T* gp = gs + cg * 8;
     int i = 0;
     for (; i + U <= N; i += U) {
-      T xv[U][4], gv[U][2][4];
+      T xv[U][RI], gv[U][8];
       int j[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         j[u] = nt[i + u];
-        lds4(xs + (j[u] < 0 ? 0 : j[u]) * ld + ci0, xv[u]);
-        lds4(gs + (i + u) * ld + co0, gv[u][0]);
-        lds4(gs + (i + u) * ld + co0 + 4, gv[u][1]);
+#pragma unroll
+        for (int a = 0; a < RI; a += 4)
+          lds4(x + (j[u] < 0 ? 0 : j[u]) * ld + a, reinterpret_cast<T(&)[4]>(xv[u][a]));
+        lds4(gp + (i + u) * ld, reinterpret_cast<T(&)[4]>(gv[u][0]));
+        lds4(gp + (i + u) * ld + 4, reinterpret_cast<T(&)[4]>(gv[u][4]));
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (j[u] < 0) continue;
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < RI; ++a)
 #pragma unroll
-          for (int m = 0; m < 8; ++m) acc[a][m] = fma(xv[u][a], gv[u][m >> 2][m & 3], acc[a][m]);
+          for (int m = 0; m < 8; ++m) acc[a][m] = fma(xv[u][a], gv[u][m], acc[a][m]);
       }
     }
     for (; i < N; ++i) {
       const int j = nt[i];
       if (j < 0) continue;
-      T xv[4], gv[2][4];
-      lds4(xs + j * ld + ci0, xv);
-      lds4(gs + i * ld + co0, gv[0]);
-      lds4(gs + i * ld + co0 + 4, gv[1]);
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int a = 0; a < RI; ++a)
 #pragma unroll
-        for (int m = 0; m < 8; ++m) acc[a][m] = fma(xv[a], gv[m >> 2][m & 3], acc[a][m]);
+        for (int m = 0; m < 8; ++m) acc[a][m] = fma(x[j * ld + a], gp[i * ld + m], acc[a][m]);
     }
-    double* g = g0 + off_k + (size_t)t * h * h + co0;
+    double* g = grad + (size_t)b * P + off_k + (size_t)t * h * h + cg;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < RI; ++a)
 #pragma unroll
-      for (int m = 0; m < 8; ++m) g[(size_t)(ci0 + a) * h + m] = (double)acc[a][m];
+      for (int m = 0; m < 8; ++m) g[(size_t)(ci0 + a) * h + m * ho] = to_double(acc[a][m]);
   }
 }
 
@@ -452,21 +548,46 @@ __global__ void k_grad_proj(Lattice lat, Net<T> net, const int32_t* __restrict__
   const T* Hb = HLr + (size_t)b * N * h;
   double* g = grad + (size_t)b * P;
   const int32_t* os = orb_of_slot + (size_t)b * Ne;
-  for (int q = threadIdx.x; q < 2 * Ne * (h + 1); q += blockDim.x) {
-    const int s = q / (Ne * (h + 1));
-    const int rem = q - s * Ne * (h + 1);
-    const int c = rem / Ne, k = rem - c * Ne;  // c == h: bias
-    T acc = T(0);  // the mode's precision, as the layer gradients
+  const int groups = (h + 7) / 8 + 1;  // eight channels each; the last is the bias
+  for (int q = threadIdx.x; q < 2 * Ne * groups; q += blockDim.x) {
+    const int s = q / (Ne * groups);
+    const int rem = q - s * Ne * groups;
+    const int cg = rem / Ne, k = rem - cg * Ne;
+    if (cg == groups - 1) {
+      T acc = T(0);  // the mode's precision, as the layer gradients
+      for (int a = 0; a < Ne; ++a) {
+        const int i = os[a] - s * N;
+        if (i >= 0 && i < N) acc += Bb[(size_t)a * Ne + k];  // else a slot of the other spin
+      }
+      g[off_pb + s * Ne + k] = to_double(acc);
+      continue;
+    }
+    const int c0 = cg * 8, nc = min(8, h - c0);
+    T acc[8] = {};
     for (int a = 0; a < Ne; ++a) {
       const int i = os[a] - s * N;
-      if (i < 0 || i >= N) continue;  // a slot of the other spin
+      if (i < 0 || i >= N) continue;
       const T bv = Bb[(size_t)a * Ne + k];
-      acc += (c == h) ? bv : Hb[(size_t)i * h + c] * bv;
+      const T* hr = Hb + (size_t)i * h + c0;
+      if (h % 4 == 0) {
+        T v[4];
+        ld4(hr, v);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) acc[m] += v[m] * bv;
+        if (nc > 4) {
+          ld4(hr + 4, v);
+#pragma unroll
+          for (int m = 0; m < 4; ++m) acc[4 + m] += v[m] * bv;
+        }
+      } else {
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+          if (m < nc) acc[m] += hr[m] * bv;
+      }
     }
-    if (c == h)
-      g[off_pb + s * Ne + k] = (double)acc;
-    else
-      g[off_pw + (size_t)c * 2 * Ne + s * Ne + k] = (double)acc;
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+      if (m < nc) g[off_pw + (size_t)(c0 + m) * 2 * Ne + s * Ne + k] = to_double(acc[m]);
   }
   const int32_t* so = slot_of_orb + (size_t)b * 2 * N;
   const T* Pb = Pt + (size_t)b * 2 * Ne * h;
@@ -523,14 +644,26 @@ __global__ void k_grad_kernel(Lattice lat, Net<T> net, int l, int taps, const in
   grad[(size_t)b * P + off_k + q] = (double)acc;
 }
 
-// KT[d][co][ci] = K[d][ci][co] of one layer (the loads of k_grad_din are then consecutive
-// across the lanes of a warp).
+// KT[d][co][ci] = K[d][ci][co] of every layer (blockIdx.y), one after another (the loads of
+// k_grad_din are then consecutive across the lanes of a warp), and, with `table`, each layer's site
+// tables: [2][taps][N], by i + d and by i - d.
 template <typename T>
-__global__ void k_transpose_taps(const T* __restrict__ K, int taps, int h, T* __restrict__ KT) {
-  const int total = taps * h * h;
+__global__ void k_grad_prep(Lattice lat, Net<T> net, T* __restrict__ KT, int16_t* __restrict__ table) {
+  const int h = net.h, l = blockIdx.y, total = stencil_taps(net.stencil, net.ksize[l]) * h * h;
+  const T* K = net.kernel[l];
+  for (int m = 0; m < l; ++m) KT += (size_t)stencil_taps(net.stencil, net.ksize[m]) * h * h;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
     const int d = q / (h * h), rem = q - d * h * h, ci = rem / h, co = rem - ci * h;
     KT[(size_t)d * h * h + (size_t)co * h + ci] = K[q];
+  }
+  if (!table) return;
+  const int N = lat.N, taps = total / (h * h), k = net.ksize[l];
+  for (int m = 0; m < l; ++m) table += 2 * nbr_size(N, stencil_taps(net.stencil, net.ksize[m]));
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < 2 * N * taps; q += gridDim.x * blockDim.x) {
+    const int neg = q >= N * taps, e = q - neg * N * taps, t = e / N, i = e - t * N;
+    int dx, dy;
+    stencil_tap(net.stencil, k, t, dx, dy);
+    table[neg * nbr_size(N, taps) + e] = (int16_t)site_off(lat, i, neg ? -dx : dx, neg ? -dy : dy);
   }
 }
 
@@ -612,10 +745,10 @@ cudaError_t grad_t(scale_ctx* c, double* grad, int recompute) {
   const bool tiled = h % 8 == 0;          // the register-tiled kernels (vector loads of 4)
   int max_taps = 1;
   for (int l = 0; l < L; ++l) max_taps = std::max(max_taps, stencil_taps(net.stencil, net.ksize[l]));
-  // the tiled kernels with one sample's slabs staged in shared memory: small lattices (the
-  // 16x4 cylinder: forward 109 -> 96 us, dK 216 -> 140 us per 2048 walkers); at 256 sites the
-  // 73 KB of staged slabs per sample cost more than the L1-served kernels (measured)
-  const bool staged = tiled && N <= kStagedSites && staged_bytes<T>(N, h, max_taps, 2) <= kGradSmemMax;
+  // one sample's slabs staged in shared memory on small lattices; at 256 sites the 73 KB of slabs
+  // per sample cost more than the L1-served kernels (measured)
+  const bool staged = tiled && N <= kStagedSites && staged_bytes<T>(N, h, max_taps, 2) <= kGradSmemMax &&
+                      conv_bytes<T>(N, h, max_taps) <= kGradSmemMax + 32 * 1024;
   // stored: every layer's input and pre-activation kept from the one forward pass; recompute:
   // only every stride-th layer input, each segment's forward recomputed during the backward
   const int stride = recompute ? std::max(1, (int)std::ceil(std::sqrt((double)L))) : 1;
@@ -625,7 +758,9 @@ cudaError_t grad_t(scale_ctx* c, double* grad, int recompute) {
   const size_t n_seg = recompute ? (size_t)(stride + 1) + stride : (size_t)L;
   size_t ktaps = 0;  // transposed kernels of every layer
   for (int l = 0; l < L; ++l) ktaps += (size_t)stencil_taps(net.stencil, net.ksize[l]) * h * h;
-  const size_t need = sizeof(T) * (slab * (n_ck + n_seg + 4) + ktaps);
+  size_t ntab = 0;  // site tables of the staged kernels
+  for (int l = 0; staged && l < L; ++l) ntab += 2 * (size_t)nbr_size(N, stencil_taps(net.stencil, net.ksize[l]));
+  const size_t need = sizeof(T) * (slab * (n_ck + n_seg + 4) + ktaps) + sizeof(int16_t) * ntab;
   if (need > c->grad_scratch_bytes) {
     if (c->grad_scratch) cudaFree(c->grad_scratch);
     c->grad_scratch = nullptr;
@@ -645,14 +780,19 @@ cudaError_t grad_t(scale_ctx* c, double* grad, int recompute) {
   T* dZ = dB + slab;
   T* KT = dZ + slab;  // [sum over layers of taps * h * h]
   T* KTl[kMaxLayers];
+  int16_t* table = reinterpret_cast<int16_t*>(KT + ktaps);
+  const int16_t* tabl[kMaxLayers];
   {
-    size_t o = 0;
+    size_t o = 0, ot = 0;
     for (int l = 0; l < L; ++l) {
       const int tl = stencil_taps(net.stencil, net.ksize[l]);
       KTl[l] = KT + o;
-      k_transpose_taps<T><<<(tl * h * h + 255) / 256, 256, 0, c->stream>>>(net.kernel[l], tl, h, KTl[l]);
+      tabl[l] = table + ot;
+      ot += 2 * nbr_size(N, tl);
       o += (size_t)tl * h * h;
     }
+    k_grad_prep<T><<<dim3((max_taps * h * h + 255) / 256, L), 256, 0, c->stream>>>(c->lat, net, KT,
+                                                                                  staged ? table : nullptr);
   }
   // offsets (every parameter is written below: no clearing pass over the B x P gradients)
   int64_t off = (int64_t)(c->arch.per_site_embed ? N : 1) * 4 * h;
@@ -684,14 +824,14 @@ cudaError_t grad_t(scale_ctx* c, double* grad, int recompute) {
     case 64: CALL(64); break;       \
     default: CALL(0);               \
   }
-  const int conv_block = staged_block(((N + kSM - 1) / kSM) * (h / 4), kConvThreads);
+  const int conv_block = staged_block(((N + kConvSites<T> - 1) / kConvSites<T>) * (h / 8), kConvThreads);
   cudaError_t e = cudaSuccess;
   auto fwd = [&](int l, const T* in, T* out, T* z) {
     if (staged) {
       const int tl = stencil_taps(net.stencil, net.ksize[l]);
-#define SCALE_CALL(HC)                                                                                            \
-  e = staged_launch(k_conv_staged<T, HC, kSM, 0>, B, conv_block, staged_bytes<T>(N, h, tl, 1), c->stream, c->lat, net, l, \
-                    tl, net.kernel[l], c->occ, in, z, out)
+#define SCALE_CALL(HC)                                                                                                \
+  e = staged_launch(k_conv_staged<T, HC, 0>, B, conv_block, conv_bytes<T>(N, h, tl), c->stream, c->lat, net, l, tl,   \
+                    tabl[l], net.kernel[l], c->occ, in, z, out, (T*)nullptr, (int64_t)0, c->P, grad)
       SCALE_GRAD_STAGED(SCALE_CALL)
 #undef SCALE_CALL
     } else if (tiled) {
@@ -735,16 +875,17 @@ cudaError_t grad_t(scale_ctx* c, double* grad, int recompute) {
       const int kq = tiled ? taps[l] * (h / 4) * (h / 8) : taps[l] * h * h;
       if (!staged) k_grad_dz<T><<<B, 256, 0, c->stream>>>(c->lat, net, l, dcur, zl, dZ, offB[l], c->P, grad);
       if (staged) {
-        const int dkb = staged_block(kq, kDkThreads<T>);
-#define SCALE_CALL(HC)                                                                                              \
-  e = staged_launch(k_dk_staged<T, HC>, B, dkb + std::min(64, (h + 31) / 32 * 32), staged_bytes<T>(N, h, taps[l], 2),   \
-                    c->stream, c->lat, net, l, taps[l], dkb, c->occ, lin, dcur, zl, offK[l], offB[l], c->P, grad)
+#define SCALE_CALL(HC)                                                                                               \
+  e = staged_launch(k_conv_staged<T, HC, 1>, B, conv_block + bias_threads(h), conv_bytes<T>(N, h, taps[l]), c->stream, \
+                    c->lat, net, l, taps[l], tabl[l] + nbr_size(N, taps[l]), KTl[l], c->occ, dcur, zl, dnext, dZ,     \
+                    offB[l], c->P, grad)
         SCALE_GRAD_STAGED(SCALE_CALL)
 #undef SCALE_CALL
         if (e != cudaSuccess) return e;
-#define SCALE_CALL(HC)                                                                                             \
-  e = staged_launch(k_conv_staged<T, HC, kSM, 1>, B, conv_block, staged_bytes<T>(N, h, taps[l], 1), c->stream, c->lat, net, \
-                    l, taps[l], KTl[l], c->occ, dcur, zl, dnext)
+#define SCALE_CALL(HC)                                                                                               \
+  e = staged_launch(k_dk_staged<T, HC>, B, staged_block(taps[l] * (h / kDkRows) * (h / 8), kDkThreads<T>),          \
+                    staged_bytes<T>(N, h, taps[l], 2), c->stream, c->lat, net, l, taps[l], tabl[l], c->occ, lin, dZ,  \
+                    offK[l], c->P, grad)
         SCALE_GRAD_STAGED(SCALE_CALL)
 #undef SCALE_CALL
         if (e != cudaSuccess) return e;

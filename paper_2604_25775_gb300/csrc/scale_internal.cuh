@@ -260,7 +260,7 @@ __host__ __device__ inline bool stencil_has(int stencil, int k, int dx, int dy) 
   const int r = (k - 1) / 2;
   return stencil == SCALE_STENCIL_BOX || dx * dx + dy * dy <= r * r;
 }
-inline int stencil_taps(int stencil, int k) {
+__host__ __device__ inline int stencil_taps(int stencil, int k) {
   int n = 0;
   for (int dy = -(k - 1) / 2; dy <= (k - 1) / 2; ++dy)
     for (int dx = -(k - 1) / 2; dx <= (k - 1) / 2; ++dx) n += stencil_has(stencil, k, dx, dy);
