@@ -348,10 +348,9 @@ __global__ void __launch_bounds__(256, (NTW > 18 || NTW == 16 ? 1 : 2)) k_ace_mm
 
 // ---- conv blocks on tcgen05 ---------------------------------------------------------------
 constexpr int kTcRows = 128;  // M of a tile = TMEM lanes
-constexpr int kTcThreads = 256;  // two threads per row
+constexpr int kTcCopy = 256;               // copying threads, two per row
+constexpr int kTcThreads = kTcCopy + 32;  // and a warp that issues the MMAs
 constexpr int kTcKC = 8;      // input channels per pipeline stage (one K = 8 MMA step)
-constexpr int kTcStages = 6;  // shared-memory ring
-constexpr int kTcAhead = 4;   // stages whose copies are in flight ahead of the MMA
 constexpr uint32_t kTcWaitPolls = 1u << 24;  // bound of every mbarrier wait
 
 // Byte offset of element (r, k) of an [R x 8] tf32 tile in the K-major core-matrix layout:
@@ -374,7 +373,9 @@ struct TcShape {
   static constexpr uint32_t A_BYTES = kTcRows * kTcKC * 4;  // one half (hi or lo) of the A tile
   static constexpr uint32_t B_BYTES = N * kTcKC * 4;        // one half of the weight tile
   static constexpr uint32_t STAGE = 2 * A_BYTES + 2 * B_BYTES;
-  static constexpr uint32_t SMEM = kTcStages * STAGE + 2 * kTcStages * 8 + 16 + 1024;  // + barriers, slot, alignment
+  // Ring slots: what fits one CTA per SM (wide tiles) or two, AHEAD of them with copies in flight.
+  static constexpr int STAGES = N > 192 ? 9 : (N > 144 ? 10 : 6), AHEAD = STAGES - 2;
+  static constexpr uint32_t SMEM = STAGES * STAGE + 2 * STAGES * 8 + 16 + 1024;  // + barriers, slot, alignment
   static constexpr uint32_t TCOLS = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
 };
 
@@ -437,6 +438,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
   // input row (C == CO). A normalised block is one tile wide: C == CO == N.
   if constexpr (LN) C = CO = N;
   using S = TcShape<N>;
+  constexpr int kStages = S::STAGES, kAhead = S::AHEAD;
   const int KC = C / kTcKC;
   const int STEPS = taps * KC;
   // Grid (column tile, row tile): the CO / N column tiles of the same 128 rows are adjacent
@@ -447,25 +449,26 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte aligned ring (descriptors address 16-byte units; core matrices 128 bytes)
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kTcStages * S::STAGE);
-  uint64_t* done = full + kTcStages;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + kTcStages);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * S::STAGE);
+  uint64_t* done = full + kStages;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + kStages);
   __shared__ int s_abort;
   __shared__ float s_sum[2][kTcRows], s_sq[2][kTcRows];  // per-half row sums for the normalisation
-  const int tid = threadIdx.x, warp = tid >> 5, row = tid & (kTcRows - 1), part = tid >> 7;
+  const int tid = threadIdx.x, warp = tid >> 5, row = tid & (kTcRows - 1), part = (tid >> 7) & 1;
+  const bool copier = tid < kTcCopy;
   const int Ns = lat.N;
   // rows past the valid configurations of a chunk (vcfg: their count on the device): a tile
   // that holds none of them leaves before any barrier, mbarrier or TMEM allocation
   if (vcfg) rows = min(rows, (long long)*vcfg * Ns);
   if (row0 + (long long)blockIdx.y * kTcRows >= rows) return;
   const long long R = row0 + (long long)blockIdx.y * kTcRows + row;
-  const bool valid = R < rows;
+  const bool valid = copier && R < rows;
   const long long cfg = valid ? R / Ns : 0;
   const int site = valid ? (int)(R - cfg * Ns) : 0;
 
   if (tid == 0) {
-    for (int s = 0; s < kTcStages; ++s) {
-      tc::mbar_init(&full[s], 1);
+    for (int s = 0; s < kStages; ++s) {
+      tc::mbar_init(&full[s], 1 + kTcCopy / 32);  // the weights' copy and the copying warps
       tc::mbar_init(&done[s], 1);
     }
     tc::mbar_fence_init();
@@ -495,7 +498,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
   const uint32_t a_off0 = part * S::A_BYTES + tc_off(row, 0), a_off1 = part * S::A_BYTES + tc_off(row, 4);
   auto issue_next = [&]() {
     if (is < STEPS) {
-      const int b = is % kTcStages;
+      const int b = is % kStages;
       unsigned char* st = smem + b * S::STAGE;
       const size_t src = isrc + (size_t)ikc * kTcKC;
       tc::cp_async16_zfill(st + a_off0, in_part + src, inb);
@@ -515,43 +518,48 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
     tc::cp_async_commit();
   };
 
+  // Copying warps: stage s into its slot once the MMAs of stage s - kStages are done; stage
+  // s - kAhead, whose copies have landed then, is handed to the MMA warp. No barrier of the block in the loop.
+  if (copier) {
 #pragma unroll 1
-  for (int p = 0; p < kTcAhead; ++p) issue_next();
-#pragma unroll 1
-  for (int s = 0; s < STEPS; ++s) {
-    const int b = s % kTcStages;
-    const int s1 = s + kTcAhead;
-    // the ring slot of stage s1 last held stage s1 - kTcStages (two MMA stages back)
-    bool ok = true;
-    if (s1 < STEPS && s1 >= kTcStages)
-      ok = tc::mbar_wait(&done[s1 % kTcStages], (uint32_t)((s1 / kTcStages) - 1) & 1u, kTcWaitPolls);
-    if (ok) {
-      issue_next();  // stage s1
-    } else {
-      s_abort = 1;
-      tc::cp_async_commit();
-    }
-    tc::cp_async_wait<kTcAhead>();  // this thread's copies of stage s have landed
-    tc::fence_proxy_async();        // ... and are visible to the tensor core
-    __syncthreads();
-    if (s_abort) break;
-    if (tid == 0) {
-      if (!tc::mbar_wait(&full[b], (uint32_t)(s / kTcStages) & 1u, kTcWaitPolls)) {
-        s_abort = 1;
-      } else {
-        tc::fence_after_sync();
-        const uint32_t a0 = tc::smem_u32(smem + b * S::STAGE);
-        const uint64_t ah = tc::smem_desc_kmajor(a0, kTcLBO, kTcSBO);
-        const uint64_t al = tc::smem_desc_kmajor(a0 + S::A_BYTES, kTcLBO, kTcSBO);
-        const uint64_t bh = tc::smem_desc_kmajor(a0 + 2 * S::A_BYTES, kTcLBO, kTcSBO);
-        const uint64_t bl = tc::smem_desc_kmajor(a0 + 2 * S::A_BYTES + S::B_BYTES, kTcLBO, kTcSBO);
-        tc::mma_tf32(tmem, ah, bh, IDESC, s > 0 ? 1u : 0u);
-        tc::mma_tf32(tmem, al, bh, IDESC, 1u);
-        tc::mma_tf32(tmem, ah, bl, IDESC, 1u);
-        tc::mma_commit(&done[b]);
+    for (int s = 0; s < STEPS + kAhead; ++s) {
+      if (s >= kStages && s < STEPS &&
+          !__all_sync(~0u, tc::mbar_wait(&done[s % kStages], (uint32_t)((s / kStages) - 1) & 1u, kTcWaitPolls))) {
+        s_abort = 1;  // the whole warp leaves
+        break;
       }
+      issue_next();
+      if (s < kAhead) continue;
+      tc::cp_async_wait<kAhead>();  // this thread's copies of stage s - kAhead have landed
+      tc::fence_proxy_async();      // ... and are visible to the tensor core
+      __syncwarp();
+      if ((tid & 31) == 0) tc::mbar_arrive(&full[(s - kAhead) % kStages]);
     }
+  } else if (tid == kTcCopy) {
+#pragma unroll 1
+    for (int s = 0; s < STEPS; ++s) {
+      const int b = s % kStages;
+      if (!tc::mbar_wait(&full[b], (uint32_t)(s / kStages) & 1u, kTcWaitPolls)) {
+        s_abort = 1;
+        break;
+      }
+      tc::fence_after_sync();
+      tc::fence_proxy_async();
+      const uint32_t a0 = tc::smem_u32(smem + b * S::STAGE);
+      const uint64_t ah = tc::smem_desc_kmajor(a0, kTcLBO, kTcSBO);
+      const uint64_t al = tc::smem_desc_kmajor(a0 + S::A_BYTES, kTcLBO, kTcSBO);
+      const uint64_t bh = tc::smem_desc_kmajor(a0 + 2 * S::A_BYTES, kTcLBO, kTcSBO);
+      const uint64_t bl = tc::smem_desc_kmajor(a0 + 2 * S::A_BYTES + S::B_BYTES, kTcLBO, kTcSBO);
+      tc::mma_tf32(tmem, ah, bh, IDESC, s > 0 ? 1u : 0u);
+      tc::mma_tf32(tmem, al, bh, IDESC, 1u);
+      tc::mma_tf32(tmem, ah, bl, IDESC, 1u);
+      tc::mma_commit(&done[b]);
+    }
+    // every MMA of this thread, before the accumulator is read and the ring's copies are all drained
+    const int sl = STEPS - 1;
+    if (!s_abort && !tc::mbar_wait(&done[sl % kStages], (uint32_t)(sl / kStages) & 1u, kTcWaitPolls)) s_abort = 1;
   }
+  __syncwarp();
   // this thread's half of the tile's residual row (independent of the MMAs: loaded under them);
   // the 256-column tiles (site-wise layers, no residual) stream their epilogue instead
   constexpr bool kStream = N == 256;
@@ -576,14 +584,10 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
     for (int c = 0; c < H2; ++c) u[c] = 0.f;
   }
   (void)u;
-  if (!s_abort && tid == 0) {
-    const int sl = STEPS - 1;
-    if (!tc::mbar_wait(&done[sl % kTcStages], (uint32_t)(sl / kTcStages) & 1u, kTcWaitPolls)) s_abort = 1;
-  }
   tc::cp_async_wait<0>();
   __syncthreads();
   tc::fence_after_sync();
-  const bool run = !s_abort;
+  const bool aborted = s_abort, run = !aborted && copier;
   if constexpr (kStream) {  // 8 columns at a time: TMEM -> bias, activation -> (split) store
     if (run) {
       const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0;
@@ -613,7 +617,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
           }
         }
       }
-    } else if (tid == 0) {
+    } else if (aborted && tid == 0) {
       atomicExch(err, 1);
     }
     tc::fence_before_sync();
@@ -674,7 +678,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
         }
       }
     }
-  } else if (tid == 0) {
+  } else if (aborted && tid == 0) {
     atomicExch(err, 1);
   }
   tc::fence_before_sync();
