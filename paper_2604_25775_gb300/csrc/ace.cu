@@ -373,8 +373,8 @@ struct TcShape {
   static constexpr uint32_t A_BYTES = kTcRows * kTcKC * 4;  // one half (hi or lo) of the A tile
   static constexpr uint32_t B_BYTES = N * kTcKC * 4;        // one half of the weight tile
   static constexpr uint32_t STAGE = 2 * A_BYTES + 2 * B_BYTES;
-  // Ring slots: what fits one CTA per SM (wide tiles) or two, AHEAD of them with copies in flight.
-  static constexpr int STAGES = N > 192 ? 9 : (N > 144 ? 10 : 6), AHEAD = STAGES - 2;
+  // Ring slots: what fits one CTA per SM (160 and 192 columns) or two, AHEAD of them with copies in flight.
+  static constexpr int STAGES = N > 192 ? 4 : (N > 144 ? 10 : 6), AHEAD = STAGES - 2;
   static constexpr uint32_t SMEM = STAGES * STAGE + 2 * STAGES * 8 + 16 + 1024;  // + barriers, slot, alignment
   static constexpr uint32_t TCOLS = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
 };
@@ -427,12 +427,12 @@ __global__ void k_ace_embed_split(int N, int h, int per_site, const float* __res
 // a wait ran out. 256 threads: thread t serves row t % 128 -- copies of its hi (t < 128) or
 // lo half, and in the epilogue the tile's columns [0, N/2) (warps 0-3) or [N/2, N) (warps
 // 4-7); a warp reads the TMEM lanes of its quarter (warp % 4).
-template <int N, bool LN>
-__global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
+template <int N, bool LN, bool BIN>
+__global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ace_conv_tc(
     Lattice lat, const float* __restrict__ bimg, const float* __restrict__ bias, const float* __restrict__ gam,
     const float* __restrict__ bet, int act, float eps, int C, int CO, int res, int ks, int stencil, int taps,
     const float* __restrict__ in_hi, const float* __restrict__ in_lo, float* __restrict__ out_hi,
-    float* __restrict__ out_lo, long long row0, long long rows, int* __restrict__ err,
+    float* __restrict__ out_lo, int bout, long long row0, long long rows, int* __restrict__ err,
     const int* __restrict__ vcfg) {
   // C input channels (K = taps x C), CO output channels (this CTA: [cb, cb + N)); res: add the
   // input row (C == CO). A normalised block is one tile wide: C == CO == N.
@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
 
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
-      tc::mbar_init(&full[s], 1 + kTcCopy / 32);  // the weights' copy and the copying warps
+      tc::mbar_init(&full[s], BIN ? 1 : 1 + kTcCopy / 32);  // the bulk copies, and the copying warps
       tc::mbar_init(&done[s], 1);
     }
     tc::mbar_fence_init();
@@ -520,7 +520,23 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
 
   // Copying warps: stage s into its slot once the MMAs of stage s - kStages are done; stage
   // s - kAhead, whose copies have landed then, is handed to the MMA warp. No barrier of the block in the loop.
-  if (copier) {
+  if (BIN && tid == 0) {  // blocked input: the whole stage by bulk copies
+    const float* src = in_hi + (size_t)(R / kTcRows) * kTcRows * 2 * C;
+#pragma unroll 1
+    for (int s = 0; s < STEPS; ++s) {
+      const int b = s % kStages;
+      if (s >= kStages && !tc::mbar_wait(&done[b], (uint32_t)((s / kStages) - 1) & 1u, kTcWaitPolls)) {
+        s_abort = 1;
+        break;
+      }
+      unsigned char* st = smem + b * S::STAGE;
+      const float* w = bimg + (size_t)s * 2 * CO * kTcKC + (size_t)cb * kTcKC;
+      tc::mbar_arrive_expect_tx(&full[b], S::STAGE);
+      tc::bulk_g2s(st, src + (size_t)s * 2 * kTcRows * kTcKC, 2 * S::A_BYTES, &full[b]);
+      tc::bulk_g2s(st + 2 * S::A_BYTES, w, S::B_BYTES, &full[b]);
+      tc::bulk_g2s(st + 2 * S::A_BYTES + S::B_BYTES, w + CO * kTcKC, S::B_BYTES, &full[b]);
+    }
+  } else if (!BIN && copier) {
 #pragma unroll 1
     for (int s = 0; s < STEPS + kAhead; ++s) {
       if (s >= kStages && s < STEPS &&
@@ -588,6 +604,14 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
   __syncthreads();
   tc::fence_after_sync();
   const bool aborted = s_abort, run = !aborted && copier;
+  // where columns [c, c + 4) of this thread's half go; blocked: the stages of the layer that reads them
+  // (its lo half one A tile behind), a warp's stores then cover whole 128-byte pieces
+  auto out_at = [&](int c) {
+    const int col = cb + c0 + c;
+    return bout ? (size_t)(R / kTcRows) * kTcRows * 2 * CO + (size_t)(col / kTcKC) * 2 * kTcRows * kTcKC +
+                      tc_off(row, col % kTcKC) / 4
+                : (size_t)R * CO + col;
+  };
   if constexpr (kStream) {  // 8 columns at a time: TMEM -> bias, activation -> (split) store
     if (run) {
       const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0;
@@ -598,16 +622,17 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
 #pragma unroll
         for (int q = 0; q < 8; ++q) z[q] = act_tc(act, z[q] + __ldg(bias + cb + c0 + cc * 8 + q));
         if (valid) {
-          const size_t o = (size_t)R * CO + cb + c0 + cc * 8;
+          const size_t o = out_at(cc * 8);
           if (out_lo) {
+            const int e4 = bout ? 32 : 4;  // the next four columns
             uint32_t hi[8], lo[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) split_tf32(z[e], hi[e], lo[e]);
 #pragma unroll
             for (int e = 0; e < 8; e += 4) {
-              *reinterpret_cast<float4*>(out_hi + o + e) = make_float4(
+              *reinterpret_cast<float4*>(out_hi + o + (e ? e4 : 0)) = make_float4(
                   __uint_as_float(hi[e]), __uint_as_float(hi[e + 1]), __uint_as_float(hi[e + 2]), __uint_as_float(hi[e + 3]));
-              *reinterpret_cast<float4*>(out_lo + o + e) = make_float4(
+              *reinterpret_cast<float4*>(out_lo + o + (e ? e4 : 0)) = make_float4(
                   __uint_as_float(lo[e]), __uint_as_float(lo[e + 1]), __uint_as_float(lo[e + 2]), __uint_as_float(lo[e + 3]));
             }
           } else {
@@ -664,7 +689,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
         else y[e] = u[c + e];
       }
       if (valid) {
-        const size_t o = (size_t)R * CO + cb + c0 + c;
+        const size_t o = out_at(c);
         if (out_lo) {
           uint32_t hi[4], lo[4];
 #pragma unroll
@@ -686,22 +711,22 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 ? 1 : 2)) k_ace_conv_tc(
   if (warp == 0) tc::tmem_dealloc(tmem, S::TCOLS);
 }
 
-template <int N, bool LN>
+template <int N, bool LN, bool BIN = false>
 cudaError_t run_conv_tc(cudaStream_t st, const Lattice& lat, const float* bimg, const float* bias, const float* g,
                         const float* be, int act, float eps, int C, int CO, int res, int ks, int stencil,
-                        const float* in_hi, const float* in_lo, float* out_hi, float* out_lo, long long rows,
-                        int* err, const int* vcfg) {
+                        const float* in_hi, const float* in_lo, float* out_hi, float* out_lo, int bout,
+                        long long rows, int* err, const int* vcfg) {
   using S = TcShape<N>;
   cudaError_t e =
-      cudaFuncSetAttribute(k_ace_conv_tc<N, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+      cudaFuncSetAttribute(k_ace_conv_tc<N, LN, BIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
   if (e != cudaSuccess) return e;
   // rows [row0, rows) per launch, at most 65535 row tiles (the grid's y limit) each
   const long long tiles = (rows + kTcRows - 1) / kTcRows;
   for (long long t0 = 0; t0 < tiles; t0 += 65535) {
     const dim3 grid((unsigned)(CO / N), (unsigned)std::min<long long>(65535, tiles - t0));
-    k_ace_conv_tc<N, LN><<<grid, kTcThreads, S::SMEM, st>>>(lat, bimg, bias, g, be, act, eps, C, CO, res, ks,
-                                                            stencil, stencil_taps(stencil, ks), in_hi, in_lo,
-                                                            out_hi, out_lo, t0 * kTcRows, rows, err, vcfg);
+    k_ace_conv_tc<N, LN, BIN><<<grid, kTcThreads, S::SMEM, st>>>(
+        lat, bimg, bias, g, be, act, eps, C, CO, res, ks, stencil, stencil_taps(stencil, ks), in_hi, in_lo, out_hi,
+        out_lo, bout, t0 * kTcRows, rows, err, vcfg);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -719,12 +744,15 @@ bool tc_sitewise(int cin, int cout) { return cin % kTcKC == 0 && cout % 128 == 0
 
 cudaError_t launch_conv_tc(const scale_ctx* c, const Lattice& lat, bool ln, int cin, int cout, int res, int ks,
                            const float* bimg, const float* bias, const float* g, const float* be, int act, float eps,
-                           const float* in_hi, const float* in_lo, float* out_hi, float* out_lo, long long rows,
-                           const int* vcfg) {
+                           const float* in_hi, const float* in_lo, float* out_hi, float* out_lo, int bin, int bout,
+                           long long rows, const int* vcfg) {
   const int st = c->arch.stencil;
 #define SCALE_TC(NT, LNV) \
   run_conv_tc<NT, LNV>(c->stream, lat, bimg, bias, g, be, act, eps, cin, cout, res, ks, st, in_hi, in_lo, \
-                       out_hi, out_lo, rows, c->ace_err, vcfg)
+                       out_hi, out_lo, bout, rows, c->ace_err, vcfg)
+  if (bin)
+    return run_conv_tc<256, false, true>(c->stream, lat, bimg, bias, g, be, act, eps, cin, cout, res, ks, st, in_hi,
+                                         in_lo, out_hi, out_lo, bout, rows, c->ace_err, vcfg);
   if (ln) {
     if (cout == 48) return SCALE_TC(48, true);
     if (cout == 144) return SCALE_TC(144, true);
@@ -908,13 +936,23 @@ bool tc_layer(const scale_ctx* c, int l) {
   return true;
 }
 
-// Layers [l0, l1) on `rows` rows: a holds the input of layer l0 (as (hi, lo) halves of the
-// buffer when split), b is the other buffer; on return *out points at the buffer holding the
+// Layers that read blocked rows: [row tile of 128][8 channels][hi, lo] A tiles, each in the order of the
+// operand's core matrices, so that a stage arrives by one bulk copy (gathered 16 bytes at a time, the
+// loads of 32 different rows per instruction bounded the layers: the four 512-wide layers of SCALE-L on the
+// 400,000 rows of 24 walkers of 16x16 6.4 ms, blocked 2.5). The site-wise layers in tiles of 256 columns, when the padded last tile fits the buffers.
+bool tc_blocked(const scale_ctx* c, int l, long long rows) {
+  const long long fc = std::max(c->B_max, c->full_chunk);
+  return tc_layer(c, l) && c->arch.ksize[l] == 1 && !c->arch.residual[l] && ace_width_out(c->arch, l) % 256 == 0 &&
+         (rows + kTcRows - 1) / kTcRows * kTcRows * ace_width_in(c->arch, l) <= fc * c->N * c->hmax;
+}
+
+// Layers [l0, l1) on `rows` rows: a holds the input of layer l0 (split = 1: as (hi, lo) halves of the
+// buffer, 2: blocked), b is the other buffer; on return *out points at the buffer holding the
 // output of layer l1 - 1 and *out_split tells whether it is split. Rows are the sites of
 // configurations of lat (rows = configurations x lat.N); the site-wise (1 x 1) layers read
 // row r alone, so they also run on a buffer of gathered rows whose lattice is a stand-in.
 template <typename T>
-cudaError_t ace_layers_t(scale_ctx* c, const Lattice& lat, int l0, int l1, T* a, T* b, long long rows, bool split,
+cudaError_t ace_layers_t(scale_ctx* c, const Lattice& lat, int l0, int l1, T* a, T* b, long long rows, int split,
                          const int* vcfg, T** out, bool* out_split) {
   const AceNet<T> net = make_ace_net<T>(c);
   size_t frag_off = 0;
@@ -925,13 +963,14 @@ cudaError_t ace_layers_t(scale_ctx* c, const Lattice& lat, int l0, int l1, T* a,
       if (split && tc_layer(c, l)) {  // on tcgen05; split output when the next layer is too
         const float* bimg = (const float*)((const char*)c->ace_frag + frag_off);
         const long long tin = rows * net.cin[l], tout = rows * net.cout[l];
-        float* olo = (l + 1 < l1 && tc_layer(c, l + 1)) ? b + tout : nullptr;
+        const bool next = l + 1 < l1 && tc_layer(c, l + 1), bout = next && tc_blocked(c, l + 1, rows);
+        float* olo = next ? b + (bout ? kTcRows * kTcKC : tout) : nullptr;
         const cudaError_t e =
             launch_conv_tc(c, lat, net.ln_g[l] != nullptr, net.cin[l], net.cout[l], c->arch.residual[l], net.ks[l],
                            bimg, net.bias[l], net.ln_g[l], net.ln_b[l], net.act, (float)net.eps, a, a + tin, b, olo,
-                           rows, vcfg);
+                           split == 2, bout, rows, vcfg);
         if (e != cudaSuccess) return e;
-        split = olo != nullptr;
+        split = !next ? 0 : (bout ? 2 : 1);
         done = true;
       } else if (c->ace_mma) {
         const MmaPlan p = plan_of(c->arch, l);
@@ -953,7 +992,7 @@ cudaError_t ace_layers_t(scale_ctx* c, const Lattice& lat, int l0, int l1, T* a,
     std::swap(a, b);
   }
   *out = a;
-  *out_split = split;
+  *out_split = split != 0;
   return cudaSuccess;
 }
 
@@ -977,7 +1016,7 @@ cudaError_t ace_forward_t(scale_ctx* c, const int8_t* occ, int C, double* phi64,
   if (!split) k_ace_embed<T><<<eblocks, 256, 0, c->stream>>>(N, c->h, net.per_site, net.embed, occ, total, a, vcfg);
   T* hL = nullptr;
   bool hsplit = false;
-  cudaError_t e = ace_layers_t<T>(c, c->lat, 0, c->L, a, b, rows, split, vcfg, &hL, &hsplit);
+  cudaError_t e = ace_layers_t<T>(c, c->lat, 0, c->L, a, b, rows, split ? 1 : 0, vcfg, &hL, &hsplit);
   if (e != cudaSuccess) return e;
   const int hl = net.cout[c->L - 1];
   if (hl_out) {  // the last layer's features (plain rows: the last layer never writes a split)
@@ -1059,12 +1098,13 @@ cudaError_t launch_ace_forward(scale_ctx* c, const int8_t* occ, int C, double* p
 // Layers [l0, l1) on a buffer of rows (see ace_layers_t); *out receives the buffer of the
 // last output.
 cudaError_t launch_ace_layers(scale_ctx* c, const Lattice& lat, int l0, int l1, void* a, void* b, long long rows,
-                              bool split, const int* vcfg, void** out) {
+                              int split, const int* vcfg, void** out) {
   bool os = false;
-  if (c->fp64) return ace_layers_t<double>(c, lat, l0, l1, (double*)a, (double*)b, rows, false, vcfg, (double**)out, &os);
+  if (c->fp64) return ace_layers_t<double>(c, lat, l0, l1, (double*)a, (double*)b, rows, 0, vcfg, (double**)out, &os);
   return ace_layers_t<float>(c, lat, l0, l1, (float*)a, (float*)b, rows, split, vcfg, (float**)out, &os);
 }
 
 bool ace_tc_layer(const scale_ctx* c, int l) { return tc_layer(c, l); }
+bool ace_tc_blocked(const scale_ctx* c, int l, long long rows) { return tc_blocked(c, l, rows); }
 
 }  // namespace scale

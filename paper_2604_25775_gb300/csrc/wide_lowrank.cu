@@ -178,10 +178,12 @@ __global__ void __launch_bounds__(32 * NW) k_wl_enum(LowrankArgs a, const int64_
   }
 }
 
+constexpr int kWlCols = 4;   // R's columns per pass of the finishing kernel
 constexpr int kWlWarps = 4;  // warps (moves) per CTA of the staging and finishing kernels
 
-// Staging: warp j of the chunk takes move g0 + j. SPLIT: rows as TF32 (hi, lo) halves.
-template <typename T, bool SPLIT>
+// Staging: warp j of the chunk takes move g0 + j. SPLIT = 1: rows as TF32 (hi, lo) halves, 2: in the
+// blocked order of the layer that reads them (rows_lo unused).
+template <typename T, int SPLIT>
 __global__ void __launch_bounds__(32 * kWlWarps) k_wl_stage(WideView<T> v, int64_t g0, int MC, T* __restrict__ rows,
                                                             T* __restrict__ rows_lo, int32_t* __restrict__ nvalid) {
   __shared__ T buf[kWlWarps][kSMax][33];
@@ -253,7 +255,25 @@ __global__ void __launch_bounds__(32 * kWlWarps) k_wl_stage(WideView<T> v, int64
       }
     }
     __syncwarp();
-    if (on) {
+    if constexpr (SPLIT == 2) {  // lane = row slot: four channels at a time, 16 bytes next to the next row's
+      for (int s = 0; s < nS; ++s) {
+        T x = act_wide<T>(v.act, buf[warp][s][lane]);
+        if (v.res0 && on) x += v.embed[((size_t)(v.per_site ? m.site[s] : 0) * 4 + m.nnew[s]) * h + c];
+        buf[warp][s][lane] = x;
+      }
+      __syncwarp();
+      if (lane < v.rpm) {
+        for (int q = 0; q < 32 && c0 + q < h; q += 4) {
+          uint32_t hi[4] = {}, lo[4] = {};  // padding slots past S hold zeros
+          if (lane < nS)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) split_tf32((float)buf[warp][lane][q + e], hi[e], lo[e]);
+          T* o = rows + ace_blk_off((long long)row0 + lane, h, c0 + q);
+          *reinterpret_cast<uint4*>(o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+          *reinterpret_cast<uint4*>(o + kAceBlkLo) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        }
+      }
+    } else if (on) {
       for (int s = 0; s < v.rpm; ++s) {
         T x = T(0);  // padding slots past S hold zeros
         if (s < nS) {
@@ -262,7 +282,7 @@ __global__ void __launch_bounds__(32 * kWlWarps) k_wl_stage(WideView<T> v, int64
           if (v.res0) x += v.embed[((size_t)(v.per_site ? site : 0) * 4 + m.nnew[s]) * h + c];
         }
         const size_t q = (row0 + s) * h + c;
-        if constexpr (SPLIT) {
+        if constexpr (SPLIT == 1) {
           uint32_t hi, lo;
           split_tf32((float)x, hi, lo);
           rows[q] = __uint_as_float(hi);
@@ -277,10 +297,10 @@ __global__ void __launch_bounds__(32 * kWlWarps) k_wl_stage(WideView<T> v, int64
 }
 
 // Finishing: R of Eq. SMW from the new features on S, det R, the move's term.
-template <typename T>
+template <typename T, int kWlRows>
 __global__ void __launch_bounds__(32 * kWlWarps) k_wl_finish(WideView<T> v, int64_t g0, int MC,
                                                              const T* __restrict__ feat, double* __restrict__ terms) {
-  extern __shared__ __align__(16) unsigned char wsm[];  // [kWlWarps][hl]: the row a's vector
+  extern __shared__ __align__(16) unsigned char wsm[];  // [kWlWarps][kWlRows][hl]: the rows' vectors
   __shared__ T Rs[kWlWarps][kRMax][kRMax + 1];
   __shared__ int sl_slot[kWlWarps][kRMax], sl_sidx[kWlWarps][kRMax], sl_moved[kWlWarps][kRMax], sl_orb[kWlWarps][kRMax];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -340,49 +360,69 @@ __global__ void __launch_bounds__(32 * kWlWarps) k_wl_finish(WideView<T> v, int6
     if (lane == 0) terms[g] = CUDART_NAN;
     return;
   }
-  // R, one row a at a time: its feature row (H'(L) - H(L) if the orbital is kept) staged in
-  // shared memory once, then dotted against the Pt rows of its spin four columns per pass
-  // (lanes over channels, one reduction round per pass)
+  // R, kWlRows rows of one spin at a time: their feature rows (H'(L) - H(L) if the orbital is kept)
+  // staged in shared memory, then dotted against the Pt rows of the spin, kWlCols columns per pass
+  // (lanes over channels, one reduction round per pass). The Pt rows come from L2 (16 rows of 2 KB
+  // per spin and move): one row at a time read them r times a move and that was the kernel's time.
   const T* Ptb = v.Pt + (size_t)b * 2 * Ne * hl;
   const T* HLb = v.HL + (size_t)b * N * hl;
   const T* Bb = v.Binv + (size_t)b * Ne * Ne;
-  T* dh = reinterpret_cast<T*>(wsm) + (size_t)warp * hl;
-  for (int a = 0; a < r; ++a) {
-    const int sp = a >= r_up;
-    const int s = sidx[a];
-    const bool kept = !moved[a];
-    const T* x = feat + ((size_t)j * v.rpm + s) * hl;
-    const T* hrow = HLb + (size_t)m.site[s] * hl;
-    for (int c = lane; c < hl; c += 32) dh[c] = kept ? x[c] - hrow[c] : x[c];
-    __syncwarp();
-    for (int b0 = 0; b0 < r; b0 += 4) {
-      const T* p[4];
+  T* dh = reinterpret_cast<T*>(wsm) + (size_t)warp * kWlRows * hl;
+  for (int sp = 0; sp < 2; ++sp) {
+    const int a1 = sp ? r : r_up;
+    for (int a0 = sp ? r_up : 0; a0 < a1; a0 += kWlRows) {
+      const int na = min(kWlRows, a1 - a0);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) p[u] = Ptb + ((size_t)sp * Ne + slot[min(b0 + u, r - 1)]) * hl;
-      T acc[4] = {T(0), T(0), T(0), T(0)};
-      for (int c = lane; c < hl; c += 32) {
-        const T d = dh[c];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] += d * p[u][c];
+      for (int w = 0; w < kWlRows; ++w) {
+        const int a = a0 + min(w, na - 1), s = sidx[a];  // past the last row: that row again
+        const T* x = feat + ((size_t)j * v.rpm + s) * hl;
+        const T* hrow = HLb + (size_t)m.site[s] * hl;
+        const bool kept = !moved[a];
+        for (int c = lane; c < hl; c += 32) dh[(size_t)w * hl + c] = kept ? x[c] - hrow[c] : x[c];
       }
-      if (!kept) {  // + (M0 + proj_b)[o'_a] . Binv[c_b]
-        const T* mb = v.M0b + (size_t)orb[a] * Ne;
-        for (int k = lane; k < Ne; k += 32) {
-          const T mk = mb[k];
+      __syncwarp();
+      for (int b0 = 0; b0 < r; b0 += kWlCols) {
+        const T* p[kWlCols];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) acc[u] += mk * Bb[(size_t)slot[min(b0 + u, r - 1)] * Ne + k];
+        for (int u = 0; u < kWlCols; ++u) p[u] = Ptb + ((size_t)sp * Ne + slot[min(b0 + u, r - 1)]) * hl;
+        T acc[kWlRows][kWlCols] = {};
+#pragma unroll 2
+        for (int c = lane; c < hl; c += 32) {
+          T pv[kWlCols];
+#pragma unroll
+          for (int u = 0; u < kWlCols; ++u) pv[u] = p[u][c];
+#pragma unroll
+          for (int w = 0; w < kWlRows; ++w) {
+            const T d = dh[(size_t)w * hl + c];
+#pragma unroll
+            for (int u = 0; u < kWlCols; ++u) acc[w][u] += d * pv[u];
+          }
+        }
+#pragma unroll
+        for (int w = 0; w < kWlRows; ++w) {
+          const int a = a0 + w;
+          if (w >= na) break;
+          const bool kept = !moved[a];
+          if (!kept) {  // + (M0 + proj_b)[o'_a] . Binv[c_b]
+            const T* mb = v.M0b + (size_t)orb[a] * Ne;
+            for (int k = lane; k < Ne; k += 32) {
+              const T mk = mb[k];
+#pragma unroll
+              for (int u = 0; u < kWlCols; ++u) acc[w][u] += mk * Bb[(size_t)slot[min(b0 + u, r - 1)] * Ne + k];
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < kWlCols; ++u)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc[w][u] += __shfl_xor_sync(0xffffffffu, acc[w][u], o);
+          if (lane == 0)
+#pragma unroll
+            for (int u = 0; u < kWlCols; ++u)
+              if (b0 + u < r) R[a][b0 + u] = (kept && a == b0 + u ? T(1) : T(0)) + acc[w][u];
         }
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
-      if (lane == 0)
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (b0 + u < r) R[a][b0 + u] = (kept && a == b0 + u ? T(1) : T(0)) + acc[u];
+      __syncwarp();
     }
-    __syncwarp();
   }
   __syncwarp();
   const T det = warp_det_R<T>(R, r);
@@ -493,24 +533,29 @@ cudaError_t wide_eloc_t(scale_ctx* c, double* eloc) {
   const int MC = c->wl_chunk;
   const int h = c->h;
   const long long rows = (long long)MC * c->wl_rows;
-  const bool split = !c->fp64 && ace_tc_layer(c, 1);
+  const int split = c->fp64 || !ace_tc_layer(c, 1) ? 0 : (ace_tc_blocked(c, 1, rows) ? 2 : 1);
   const int64_t bound = (int64_t)B * (int64_t)cap;  // the device-side total is at most this
   T* ra = (T*)c->act_a;
-  const size_t fsm = (size_t)kWlWarps * v.hl * sizeof(T);  // the finishing warps' row vectors
-  if (fsm > 48 * 1024 &&
-      (e = cudaFuncSetAttribute(k_wl_finish<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm)) != cudaSuccess)
-    return e;
+  // the finishing warps' row vectors: as many rows at a time as 48 KB hold, else one
+  const size_t row_bytes = (size_t)kWlWarps * v.hl * sizeof(T);
+  const int wr = 4 * row_bytes <= 48 * 1024 ? 4 : (2 * row_bytes <= 48 * 1024 ? 2 : 1);
+  const size_t fsm = wr * row_bytes;
+  auto* finish = wr == 4 ? k_wl_finish<T, 4> : (wr == 2 ? k_wl_finish<T, 2> : k_wl_finish<T, 1>);
+  if ((e = cudaFuncSetAttribute(finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm)) != cudaSuccess)
+    return e;  // with the static arrays above 48 KB
   for (int64_t g0 = 0; g0 < bound; g0 += MC) {
     const unsigned grid = (unsigned)((MC + kWlWarps - 1) / kWlWarps);
-    if (split)
-      k_wl_stage<T, true><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, ra + rows * h, c->full_vcount);
+    if (split == 2)
+      k_wl_stage<T, sizeof(T) == 4 ? 2 : 0><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, nullptr, c->full_vcount);
+    else if (split)
+      k_wl_stage<T, 1><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, ra + rows * h, c->full_vcount);
     else
-      k_wl_stage<T, false><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, nullptr, c->full_vcount);
+      k_wl_stage<T, 0><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, nullptr, c->full_vcount);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     void* out = nullptr;
     if ((e = launch_ace_layers(c, rl, 1, c->L, c->act_a, c->act_b, rows, split, c->full_vcount, &out)) != cudaSuccess)
       return e;
-    k_wl_finish<T><<<grid, 32 * kWlWarps, fsm, c->stream>>>(v, g0, MC, (const T*)out, c->full_coeff);
+    finish<<<grid, 32 * kWlWarps, fsm, c->stream>>>(v, g0, MC, (const T*)out, c->full_coeff);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   k_wl_reduce<<<(B + 127) / 128, 128, 0, c->stream>>>(B, c->full_offsets, c->full_diag, c->full_coeff, c->status,
