@@ -18,15 +18,15 @@
 //   k_ace_conv_tc (mixed mode: the ACE conv blocks of width 48, 144 or 192, the wide SCALE
 //               conv of width 384 or 640, and the site-wise layers that follow them while
 //               their output widths are multiples of 128): the 5th-generation tensor cores.
-//               One CTA of 256 threads (two per row) owns 128 rows (TMEM lanes) and a tile
+//               One CTA (256 copying threads and a warp that issues the MMAs) owns 128 rows (TMEM lanes) and a tile
 //               of N output channels (TMEM columns; the whole width for a normalised block,
 //               else 128 to 192); the column tiles of the same rows are adjacent in the
 //               grid, so they share the gathered rows through L2. The K loop runs over (offset d, 8-channel chunk) stages
-//               in a 6-slot shared-memory ring with 4 stages of copies in flight: each
-//               thread gathers its row's 8 input channels, hi or lo part, from the
-//               neighbour site with 16-byte cp.async (zero fill past an open edge),
+//               in a shared-memory ring of 4 to 10 slots: eight
+//               warps gather the rows' 8 input channels, hi and lo parts, from the
+//               neighbour sites with 16-byte cp.async (zero fill past an open edge),
 //               the pre-split weight tile arrives by one bulk copy per half (hi, lo) on an
-//               mbarrier, and one thread issues the three TF32 products
+//               mbarrier, and the MMA warp issues the three TF32 products
 //               x_hi W_hi + x_lo W_hi + x_hi W_lo per K=8 step (tcgen05.mma, FP32
 //               accumulation in TMEM) and commits them to the stage's mbarrier. Between two
 //               tensor-core layers the activations are stored already split (hi, lo).
@@ -353,6 +353,12 @@ constexpr int kTcThreads = kTcCopy + 32;  // and a warp that issues the MMAs
 constexpr int kTcKC = 8;      // input channels per pipeline stage (one K = 8 MMA step)
 constexpr uint32_t kTcWaitPolls = 1u << 24;  // bound of every mbarrier wait
 
+// Split rows: eight channels' hi parts, then their lo parts.
+__host__ __device__ __forceinline__ size_t split_off(long long row, int C, int c) {
+  return (size_t)row * 2 * C + (c >> 3) * 16 + (c & 7);
+}
+constexpr int kSplitLo = 8;
+
 // Byte offset of element (r, k) of an [R x 8] tf32 tile in the K-major core-matrix layout:
 // core matrix (r / 8, k / 4) at ((r / 8) * 2 + k / 4) * 128, its row r % 8 at 16 bytes.
 // Neighbours along K are 128 bytes apart (descriptor LBO), along rows 256 (SBO).
@@ -402,10 +408,10 @@ __global__ void k_ace_build_bimg(const float* __restrict__ K, int CI, int N, int
   }
 }
 
-// H0 rows split for the tensor cores: out_hi = tf32(E), out_lo = tf32(E - out_hi).
+// H0 rows split for the tensor cores: hi = tf32(E), lo = tf32(E - hi).
 __global__ void k_ace_embed_split(int N, int h, int per_site, const float* __restrict__ embed,
-                                  const int8_t* __restrict__ occ, long long total, float* __restrict__ out_hi,
-                                  float* __restrict__ out_lo, const int* __restrict__ vcfg) {
+                                  const int8_t* __restrict__ occ, long long total, float* __restrict__ out,
+                                  const int* __restrict__ vcfg) {
   if (vcfg) total = min(total, (long long)*vcfg * N * h);
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
        q += (long long)gridDim.x * blockDim.x) {
@@ -415,24 +421,25 @@ __global__ void k_ace_embed_split(int N, int h, int per_site, const float* __res
     const float e = embed[((size_t)(per_site ? i : 0) * 4 + (occ[row] & 3)) * h + c];
     uint32_t hi, lo;
     split_tf32(e, hi, lo);
-    out_hi[q] = __uint_as_float(hi);
-    out_lo[q] = __uint_as_float(lo);
+    const size_t o = split_off(row, h, c);
+    out[o] = __uint_as_float(hi);
+    out[o + kSplitLo] = __uint_as_float(lo);
   }
 }
 
 // One conv layer (ks x ks stencil, C -> C channels) on tcgen05: ACE blocks with the layer
 // normalisation in the epilogue (LN, one column tile of N = C), or the wide SCALE conv (no
-// normalisation, column tiles of N: blockIdx.y selects columns [N y, N y + N)). out_lo ==
-// nullptr writes plain FP32 rows to out_hi (the input of the site-wise layers). err: set when
-// a wait ran out. 256 threads: thread t serves row t % 128 -- copies of its hi (t < 128) or
-// lo half, and in the epilogue the tile's columns [0, N/2) (warps 0-3) or [N/2, N) (warps
+// normalisation, column tiles of N: blockIdx.x selects columns [N x, N x + N)). in: split rows
+// (split_off; BIN: blocked), out: plain FP32 rows (omode 0), split (1) or blocked (2). err: set when
+// a wait ran out. Copying thread t takes the 16-byte piece t % 4 of rows t / 4 and t / 4 + 64 (four lanes a
+// row: 64 contiguous bytes; one lane a row, with hi and lo in separate slabs, asked for 32 lines per load: the
+// blocks of ACE 16x16, 96 walkers, 2.54 ms, now HERE). In the epilogue thread t serves row t % 128, the tile's columns [0, N/2) (warps 0-3) or [N/2, N) (warps
 // 4-7); a warp reads the TMEM lanes of its quarter (warp % 4).
 template <int N, bool LN, bool BIN>
 __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ace_conv_tc(
     Lattice lat, const float* __restrict__ bimg, const float* __restrict__ bias, const float* __restrict__ gam,
     const float* __restrict__ bet, int act, float eps, int C, int CO, int res, int ks, int stencil, int taps,
-    const float* __restrict__ in_hi, const float* __restrict__ in_lo, float* __restrict__ out_hi,
-    float* __restrict__ out_lo, int bout, long long row0, long long rows, int* __restrict__ err,
+    const float* __restrict__ in, float* __restrict__ out, int omode, long long row0, long long rows, int* __restrict__ err,
     const int* __restrict__ vcfg) {
   // C input channels (K = taps x C), CO output channels (this CTA: [cb, cb + N)); res: add the
   // input row (C == CO). A normalised block is one tile wide: C == CO == N.
@@ -463,8 +470,6 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   if (row0 + (long long)blockIdx.y * kTcRows >= rows) return;
   const long long R = row0 + (long long)blockIdx.y * kTcRows + row;
   const bool valid = copier && R < rows;
-  const long long cfg = valid ? R / Ns : 0;
-  const int site = valid ? (int)(R - cfg * Ns) : 0;
 
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -483,26 +488,39 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   // Copies of the stages in order, one per call; each call closes one cp.async group
   // (empty past the last stage). The neighbour row of the current tap is recomputed only
   // when the tap changes (every KC stages).
-  const float* in_part = part ? in_lo : in_hi;
   int is = 0, id = 0, ikc = 0;
-  size_t isrc = 0;
-  uint32_t inb = 0;
+  const int piece = tid & 3, arow = (tid & (kTcCopy - 1)) >> 2;
+  long long acfg[2] = {0, 0};
+  int asite[2] = {-1, -1};
+  const float* isrc[2] = {in, in};
+  uint32_t inb[2] = {0, 0};
+  if (!BIN) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const long long q = row0 + (long long)blockIdx.y * kTcRows + arow + 64 * u;
+      if (q >= rows) continue;
+      acfg[u] = q / Ns;
+      asite[u] = (int)(q - acfg[u] * Ns);
+    }
+  }
   auto tap_row = [&](int d) {
     int dx, dy;
     stencil_tap(stencil, ks, d, dx, dy);
-    const int j = valid ? site_off(lat, site, dx, dy) : -1;
-    isrc = j >= 0 ? ((size_t)cfg * Ns + j) * C : 0;
-    inb = j >= 0 ? 16u : 0u;  // zero fill past an open edge or the last row
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int j = asite[u] >= 0 ? site_off(lat, asite[u], dx, dy) : -1;
+      isrc[u] = in + (j >= 0 ? split_off(acfg[u] * Ns + j, C, 0) + piece * 4 : 0);
+      inb[u] = j >= 0 ? 16u : 0u;  // zero fill past an open edge or the last row
+    }
   };
-  tap_row(0);
-  const uint32_t a_off0 = part * S::A_BYTES + tc_off(row, 0), a_off1 = part * S::A_BYTES + tc_off(row, 4);
+  if (!BIN) tap_row(0);
+  const uint32_t a_off = (piece >> 1) * S::A_BYTES + tc_off(arow, (piece & 1) * 4);
   auto issue_next = [&]() {
     if (is < STEPS) {
       const int b = is % kStages;
       unsigned char* st = smem + b * S::STAGE;
-      const size_t src = isrc + (size_t)ikc * kTcKC;
-      tc::cp_async16_zfill(st + a_off0, in_part + src, inb);
-      tc::cp_async16_zfill(st + a_off1, in_part + src + 4, inb);
+      tc::cp_async16_zfill(st + a_off, isrc[0] + ikc * 2 * kTcKC, inb[0]);
+      tc::cp_async16_zfill(st + a_off + tc_off(64, 0), isrc[1] + ikc * 2 * kTcKC, inb[1]);
       if (tid == 0) {
         const float* w = bimg + ((size_t)id * KC + ikc) * 2 * CO * kTcKC + (size_t)cb * kTcKC;
         tc::mbar_arrive_expect_tx(&full[b], 2 * S::B_BYTES);
@@ -521,7 +539,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   // Copying warps: stage s into its slot once the MMAs of stage s - kStages are done; stage
   // s - kAhead, whose copies have landed then, is handed to the MMA warp. No barrier of the block in the loop.
   if (BIN && tid == 0) {  // blocked input: the whole stage by bulk copies
-    const float* src = in_hi + (size_t)(R / kTcRows) * kTcRows * 2 * C;
+    const float* src = in + (size_t)(R / kTcRows) * kTcRows * 2 * C;
 #pragma unroll 1
     for (int s = 0; s < STEPS; ++s) {
       const int b = s % kStages;
@@ -584,12 +602,12 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   if constexpr (kStream) {
     u[0] = 0.f;
   } else if (LN || res) {  // the normalised conv blocks are residual
-    const float* xh = in_hi + (size_t)(valid ? R : 0) * C + cb + c0;
-    const float* xl = in_lo + (size_t)(valid ? R : 0) * C + cb + c0;
+    const float* xr = in + split_off(valid ? R : 0, C, cb + c0);
 #pragma unroll
     for (int c = 0; c < H2; c += 4) {
-      const float4 h4 = __ldg(reinterpret_cast<const float4*>(xh + c));
-      const float4 l4 = __ldg(reinterpret_cast<const float4*>(xl + c));
+      const float* x = xr + split_off(0, C, c);
+      const float4 h4 = __ldg(reinterpret_cast<const float4*>(x));
+      const float4 l4 = __ldg(reinterpret_cast<const float4*>(x + kSplitLo));
       u[c] = h4.x + l4.x;
       u[c + 1] = h4.y + l4.y;
       u[c + 2] = h4.z + l4.z;
@@ -604,13 +622,19 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   __syncthreads();
   tc::fence_after_sync();
   const bool aborted = s_abort, run = !aborted && copier;
-  // where columns [c, c + 4) of this thread's half go; blocked: the stages of the layer that reads them
-  // (its lo half one A tile behind), a warp's stores then cover whole 128-byte pieces
-  auto out_at = [&](int c) {
+  // columns [c, c + 4) of this thread's half of the row
+  auto put = [&](int c, const float(&y)[4]) {
     const int col = cb + c0 + c;
-    return bout ? (size_t)(R / kTcRows) * kTcRows * 2 * CO + (size_t)(col / kTcKC) * 2 * kTcRows * kTcKC +
-                      tc_off(row, col % kTcKC) / 4
-                : (size_t)R * CO + col;
+    if (omode == 0) {
+      *reinterpret_cast<float4*>(out + (size_t)R * CO + col) = make_float4(y[0], y[1], y[2], y[3]);
+      return;
+    }
+    float* o = out + (omode == 2 ? ace_blk_off(R, CO, col) : split_off(R, CO, col));
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) split_tf32(y[e], hi[e], lo[e]);
+    *reinterpret_cast<uint4*>(o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(o + (omode == 2 ? kAceBlkLo : kSplitLo)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
   };
   if constexpr (kStream) {  // 8 columns at a time: TMEM -> bias, activation -> (split) store
     if (run) {
@@ -622,24 +646,8 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
 #pragma unroll
         for (int q = 0; q < 8; ++q) z[q] = act_tc(act, z[q] + __ldg(bias + cb + c0 + cc * 8 + q));
         if (valid) {
-          const size_t o = out_at(cc * 8);
-          if (out_lo) {
-            const int e4 = bout ? 32 : 4;  // the next four columns
-            uint32_t hi[8], lo[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) split_tf32(z[e], hi[e], lo[e]);
-#pragma unroll
-            for (int e = 0; e < 8; e += 4) {
-              *reinterpret_cast<float4*>(out_hi + o + (e ? e4 : 0)) = make_float4(
-                  __uint_as_float(hi[e]), __uint_as_float(hi[e + 1]), __uint_as_float(hi[e + 2]), __uint_as_float(hi[e + 3]));
-              *reinterpret_cast<float4*>(out_lo + o + (e ? e4 : 0)) = make_float4(
-                  __uint_as_float(lo[e]), __uint_as_float(lo[e + 1]), __uint_as_float(lo[e + 2]), __uint_as_float(lo[e + 3]));
-            }
-          } else {
-#pragma unroll
-            for (int e = 0; e < 8; e += 4)
-              *reinterpret_cast<float4*>(out_hi + o + e) = make_float4(z[e], z[e + 1], z[e + 2], z[e + 3]);
-          }
+          put(cc * 8, reinterpret_cast<const float(&)[4]>(z[0]));
+          put(cc * 8 + 4, reinterpret_cast<const float(&)[4]>(z[4]));
         }
       }
     } else if (aborted && tid == 0) {
@@ -688,20 +696,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
         if constexpr (LN) y[e] = (u[c + e] - mean) * inv * __ldg(gam + c0 + c + e) + __ldg(bet + c0 + c + e);
         else y[e] = u[c + e];
       }
-      if (valid) {
-        const size_t o = out_at(c);
-        if (out_lo) {
-          uint32_t hi[4], lo[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) split_tf32(y[e], hi[e], lo[e]);
-          *reinterpret_cast<float4*>(out_hi + o) = make_float4(__uint_as_float(hi[0]), __uint_as_float(hi[1]),
-                                                               __uint_as_float(hi[2]), __uint_as_float(hi[3]));
-          *reinterpret_cast<float4*>(out_lo + o) = make_float4(__uint_as_float(lo[0]), __uint_as_float(lo[1]),
-                                                               __uint_as_float(lo[2]), __uint_as_float(lo[3]));
-        } else {
-          *reinterpret_cast<float4*>(out_hi + o) = make_float4(y[0], y[1], y[2], y[3]);
-        }
-      }
+      if (valid) put(c, y);
     }
   } else if (aborted && tid == 0) {
     atomicExch(err, 1);
@@ -714,8 +709,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
 template <int N, bool LN, bool BIN = false>
 cudaError_t run_conv_tc(cudaStream_t st, const Lattice& lat, const float* bimg, const float* bias, const float* g,
                         const float* be, int act, float eps, int C, int CO, int res, int ks, int stencil,
-                        const float* in_hi, const float* in_lo, float* out_hi, float* out_lo, int bout,
-                        long long rows, int* err, const int* vcfg) {
+                        const float* in, float* out, int omode, long long rows, int* err, const int* vcfg) {
   using S = TcShape<N>;
   cudaError_t e =
       cudaFuncSetAttribute(k_ace_conv_tc<N, LN, BIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
@@ -725,8 +719,8 @@ cudaError_t run_conv_tc(cudaStream_t st, const Lattice& lat, const float* bimg, 
   for (long long t0 = 0; t0 < tiles; t0 += 65535) {
     const dim3 grid((unsigned)(CO / N), (unsigned)std::min<long long>(65535, tiles - t0));
     k_ace_conv_tc<N, LN, BIN><<<grid, kTcThreads, S::SMEM, st>>>(
-        lat, bimg, bias, g, be, act, eps, C, CO, res, ks, stencil, stencil_taps(stencil, ks), in_hi, in_lo, out_hi,
-        out_lo, bout, t0 * kTcRows, rows, err, vcfg);
+        lat, bimg, bias, g, be, act, eps, C, CO, res, ks, stencil, stencil_taps(stencil, ks), in, out, omode,
+        t0 * kTcRows, rows, err, vcfg);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -744,15 +738,14 @@ bool tc_sitewise(int cin, int cout) { return cin % kTcKC == 0 && cout % 128 == 0
 
 cudaError_t launch_conv_tc(const scale_ctx* c, const Lattice& lat, bool ln, int cin, int cout, int res, int ks,
                            const float* bimg, const float* bias, const float* g, const float* be, int act, float eps,
-                           const float* in_hi, const float* in_lo, float* out_hi, float* out_lo, int bin, int bout,
-                           long long rows, const int* vcfg) {
+                           const float* in, float* out, int bin, int omode, long long rows, const int* vcfg) {
   const int st = c->arch.stencil;
 #define SCALE_TC(NT, LNV) \
-  run_conv_tc<NT, LNV>(c->stream, lat, bimg, bias, g, be, act, eps, cin, cout, res, ks, st, in_hi, in_lo, \
-                       out_hi, out_lo, bout, rows, c->ace_err, vcfg)
+  run_conv_tc<NT, LNV>(c->stream, lat, bimg, bias, g, be, act, eps, cin, cout, res, ks, st, in, out, omode, rows, \
+                       c->ace_err, vcfg)
   if (bin)
-    return run_conv_tc<256, false, true>(c->stream, lat, bimg, bias, g, be, act, eps, cin, cout, res, ks, st, in_hi,
-                                         in_lo, out_hi, out_lo, bout, rows, c->ace_err, vcfg);
+    return run_conv_tc<256, false, true>(c->stream, lat, bimg, bias, g, be, act, eps, cin, cout, res, ks, st, in,
+                                         out, omode, rows, c->ace_err, vcfg);
   if (ln) {
     if (cout == 48) return SCALE_TC(48, true);
     if (cout == 144) return SCALE_TC(144, true);
@@ -946,8 +939,8 @@ bool tc_blocked(const scale_ctx* c, int l, long long rows) {
          (rows + kTcRows - 1) / kTcRows * kTcRows * ace_width_in(c->arch, l) <= fc * c->N * c->hmax;
 }
 
-// Layers [l0, l1) on `rows` rows: a holds the input of layer l0 (split = 1: as (hi, lo) halves of the
-// buffer, 2: blocked), b is the other buffer; on return *out points at the buffer holding the
+// Layers [l0, l1) on `rows` rows: a holds the input of layer l0 (split = 1: split rows, 2: blocked),
+// b is the other buffer; on return *out points at the buffer holding the
 // output of layer l1 - 1 and *out_split tells whether it is split. Rows are the sites of
 // configurations of lat (rows = configurations x lat.N); the site-wise (1 x 1) layers read
 // row r alone, so they also run on a buffer of gathered rows whose lattice is a stand-in.
@@ -962,15 +955,13 @@ cudaError_t ace_layers_t(scale_ctx* c, const Lattice& lat, int l0, int l1, T* a,
     if constexpr (sizeof(T) == 4) {
       if (split && tc_layer(c, l)) {  // on tcgen05; split output when the next layer is too
         const float* bimg = (const float*)((const char*)c->ace_frag + frag_off);
-        const long long tin = rows * net.cin[l], tout = rows * net.cout[l];
-        const bool next = l + 1 < l1 && tc_layer(c, l + 1), bout = next && tc_blocked(c, l + 1, rows);
-        float* olo = next ? b + (bout ? kTcRows * kTcKC : tout) : nullptr;
+        const int omode = l + 1 < l1 && tc_layer(c, l + 1) ? (tc_blocked(c, l + 1, rows) ? 2 : 1) : 0;
         const cudaError_t e =
             launch_conv_tc(c, lat, net.ln_g[l] != nullptr, net.cin[l], net.cout[l], c->arch.residual[l], net.ks[l],
-                           bimg, net.bias[l], net.ln_g[l], net.ln_b[l], net.act, (float)net.eps, a, a + tin, b, olo,
-                           split == 2, bout, rows, vcfg);
+                           bimg, net.bias[l], net.ln_g[l], net.ln_b[l], net.act, (float)net.eps, a, b, split == 2,
+                           omode, rows, vcfg);
         if (e != cudaSuccess) return e;
-        split = !next ? 0 : (bout ? 2 : 1);
+        split = omode;
         done = true;
       } else if (c->ace_mma) {
         const MmaPlan p = plan_of(c->arch, l);
@@ -1009,7 +1000,7 @@ cudaError_t ace_forward_t(scale_ctx* c, const int8_t* occ, int C, double* phi64,
   if constexpr (sizeof(T) == 4) {
     if (c->ace_tc) {
       k_ace_embed_split<<<eblocks, 256, 0, c->stream>>>(N, c->h, net.per_site, net.embed, occ, total, a,
-                                                        a + total, vcfg);
+                                                        vcfg);
       split = true;
     }
   }

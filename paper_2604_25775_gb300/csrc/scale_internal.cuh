@@ -277,7 +277,7 @@ cudaError_t launch_ace_forward(scale_ctx* c, const int8_t* occ, int C, double* p
 cudaError_t launch_ace_layers(scale_ctx* c, const Lattice& lat, int l0, int l1, void* a, void* b, long long rows,
                               int split, const int* vcfg, void** out);
 bool ace_tc_layer(const scale_ctx* c, int l);
-// Layer l reads blocked rows (offset of element (row, c) in ace_blk_off); false: (hi, lo) halves.
+// Layer l reads blocked rows (offset of element (row, c) in ace_blk_off); false: split rows.
 bool ace_tc_blocked(const scale_ctx* c, int l, long long rows);
 __device__ __forceinline__ size_t ace_blk_off(long long row, int C, int c) {
   return (size_t)(row >> 7) * 256 * C + (size_t)(c >> 3) * 2048 + ((row & 127) >> 3) * 64 + ((c >> 2) & 1) * 32 +

@@ -181,11 +181,11 @@ __global__ void __launch_bounds__(32 * NW) k_wl_enum(LowrankArgs a, const int64_
 constexpr int kWlCols = 4;   // R's columns per pass of the finishing kernel
 constexpr int kWlWarps = 4;  // warps (moves) per CTA of the staging and finishing kernels
 
-// Staging: warp j of the chunk takes move g0 + j. SPLIT = 1: rows as TF32 (hi, lo) halves, 2: in the
-// blocked order of the layer that reads them (rows_lo unused).
+// Staging: warp j of the chunk takes move g0 + j. SPLIT = 1: rows as TF32 (hi, lo) parts, eight
+// channels of each in turn, 2: in the blocked order of the layer that reads them.
 template <typename T, int SPLIT>
 __global__ void __launch_bounds__(32 * kWlWarps) k_wl_stage(WideView<T> v, int64_t g0, int MC, T* __restrict__ rows,
-                                                            T* __restrict__ rows_lo, int32_t* __restrict__ nvalid) {
+                                                            int32_t* __restrict__ nvalid) {
   __shared__ T buf[kWlWarps][kSMax][33];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int j = blockIdx.x * kWlWarps + warp;
@@ -239,19 +239,27 @@ __global__ void __launch_bounds__(32 * kWlWarps) k_wl_stage(WideView<T> v, int64
   const int ts_src = v.per_site ? mv.src : 0, ts_dst = v.per_site ? mv.dst : 0;
   const T* z0b = v.z0 + (size_t)b * N * h;
   const size_t row0 = (size_t)j * v.rpm;
+  const int my_site = lane < nS ? m.site[lane] : 0;
+  // the changes of z0 at the pairs of the source, then of the destination: rows (n', d) - (n, d) of KE
+  const T* ke_new[2] = {v.KE + ((size_t)ts_src * 4 + n_src_new) * kk * h, v.KE + ((size_t)ts_dst * 4 + n_dst_new) * kk * h};
+  const T* ke_old[2] = {v.KE + ((size_t)ts_src * 4 + n_src_old) * kk * h, v.KE + ((size_t)ts_dst * 4 + n_dst_old) * kk * h};
   for (int c0 = 0; c0 < h; c0 += 32) {
     const int c = c0 + lane;
     const bool on = c < h;
-    for (int s = 0; s < nS; ++s) buf[warp][s][lane] = on ? z0b[(size_t)m.site[s] * h + c] : T(0);
+#pragma unroll 6
+    for (int s = 0; s < nS; ++s) {
+      const int site = __shfl_sync(0xffffffffu, my_site, s);
+      buf[warp][s][lane] = on ? __ldg(z0b + (size_t)site * h + c) : T(0);
+    }
     __syncwarp();
-    for (int p = 0; p < npairs; ++p) {
-      const int ps = __shfl_sync(0xffffffffu, pair_s, p);
-      if (ps >= 0 && on) {
-        const bool fs = p < kk;
-        const int d = fs ? p : p - kk;
-        const int ts = fs ? ts_src : ts_dst, nn = fs ? n_src_new : n_dst_new, no = fs ? n_src_old : n_dst_old;
-        buf[warp][ps][lane] +=
-            v.KE[(((size_t)ts * 4 + nn) * kk + d) * h + c] - v.KE[(((size_t)ts * 4 + no) * kk + d) * h + c];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const T *kn = ke_new[e] + (on ? c : 0), *ko = ke_old[e] + (on ? c : 0);
+#pragma unroll 5
+      for (int d = 0; d < kk; ++d) {
+        const int ps = __shfl_sync(0xffffffffu, pair_s, e * kk + d);
+        const T x = __ldg(kn + (size_t)d * h) - __ldg(ko + (size_t)d * h);
+        if (ps >= 0 && on) buf[warp][ps][lane] += x;
       }
     }
     __syncwarp();
@@ -281,14 +289,14 @@ __global__ void __launch_bounds__(32 * kWlWarps) k_wl_stage(WideView<T> v, int64
           x = act_wide<T>(v.act, buf[warp][s][lane]);
           if (v.res0) x += v.embed[((size_t)(v.per_site ? site : 0) * 4 + m.nnew[s]) * h + c];
         }
-        const size_t q = (row0 + s) * h + c;
         if constexpr (SPLIT == 1) {
           uint32_t hi, lo;
           split_tf32((float)x, hi, lo);
-          rows[q] = __uint_as_float(hi);
-          rows_lo[q] = __uint_as_float(lo);
+          T* o = rows + (row0 + s) * 2 * h + (c >> 3) * 16 + (c & 7);
+          o[0] = __uint_as_float(hi);
+          o[8] = __uint_as_float(lo);
         } else {
-          rows[q] = x;
+          rows[(row0 + s) * h + c] = x;
         }
       }
     }
@@ -531,7 +539,6 @@ cudaError_t wide_eloc_t(scale_ctx* c, double* eloc) {
   rl.pbc_x = rl.pbc_y = 1;
   rl.N = c->wl_rows;
   const int MC = c->wl_chunk;
-  const int h = c->h;
   const long long rows = (long long)MC * c->wl_rows;
   const int split = c->fp64 || !ace_tc_layer(c, 1) ? 0 : (ace_tc_blocked(c, 1, rows) ? 2 : 1);
   const int64_t bound = (int64_t)B * (int64_t)cap;  // the device-side total is at most this
@@ -546,11 +553,11 @@ cudaError_t wide_eloc_t(scale_ctx* c, double* eloc) {
   for (int64_t g0 = 0; g0 < bound; g0 += MC) {
     const unsigned grid = (unsigned)((MC + kWlWarps - 1) / kWlWarps);
     if (split == 2)
-      k_wl_stage<T, sizeof(T) == 4 ? 2 : 0><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, nullptr, c->full_vcount);
+      k_wl_stage<T, sizeof(T) == 4 ? 2 : 0><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, c->full_vcount);
     else if (split)
-      k_wl_stage<T, 1><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, ra + rows * h, c->full_vcount);
+      k_wl_stage<T, 1><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, c->full_vcount);
     else
-      k_wl_stage<T, 0><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, nullptr, c->full_vcount);
+      k_wl_stage<T, 0><<<grid, 32 * kWlWarps, 0, c->stream>>>(v, g0, MC, ra, c->full_vcount);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     void* out = nullptr;
     if ((e = launch_ace_layers(c, rl, 1, c->L, c->act_a, c->act_b, rows, split, c->full_vcount, &out)) != cudaSuccess)
