@@ -379,8 +379,8 @@ struct TcShape {
   static constexpr uint32_t A_BYTES = kTcRows * kTcKC * 4;  // one half (hi or lo) of the A tile
   static constexpr uint32_t B_BYTES = N * kTcKC * 4;        // one half of the weight tile
   static constexpr uint32_t STAGE = 2 * A_BYTES + 2 * B_BYTES;
-  // Ring slots: what fits one CTA per SM (160 and 192 columns) or two, AHEAD of them with copies in flight.
-  static constexpr int STAGES = N > 192 ? 4 : (N > 144 ? 10 : 6), AHEAD = STAGES - 2;
+  // Ring slots: what fits one CTA per SM (160 and 192 columns) or two.
+  static constexpr int STAGES = N > 192 ? 4 : (N > 144 ? 10 : 6);
   static constexpr uint32_t SMEM = STAGES * STAGE + 2 * STAGES * 8 + 16 + 1024;  // + barriers, slot, alignment
   static constexpr uint32_t TCOLS = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
 };
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   // input row (C == CO). A normalised block is one tile wide: C == CO == N.
   if constexpr (LN) C = CO = N;
   using S = TcShape<N>;
-  constexpr int kStages = S::STAGES, kAhead = S::AHEAD;
+  constexpr int kStages = S::STAGES;
   const int KC = C / kTcKC;
   const int STEPS = taps * KC;
   // Grid (column tile, row tile): the CO / N column tiles of the same 128 rows are adjacent
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
 
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
-      tc::mbar_init(&full[s], BIN ? 1 : 1 + kTcCopy / 32);  // the bulk copies, and the copying warps
+      tc::mbar_init(&full[s], BIN ? 1 : 1 + kTcCopy);  // the bulk copies, and the copying threads
       tc::mbar_init(&done[s], 1);
     }
     tc::mbar_fence_init();
@@ -485,10 +485,9 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   tc::fence_after_sync();
   const uint32_t tmem = *tslot;
 
-  // Copies of the stages in order, one per call; each call closes one cp.async group
-  // (empty past the last stage). The neighbour row of the current tap is recomputed only
+  // Copies of the stages in order, one per call. The neighbour row of the current tap is recomputed only
   // when the tap changes (every KC stages).
-  int is = 0, id = 0, ikc = 0;
+  int id = 0, ikc = 0;
   const int piece = tid & 3, arow = (tid & (kTcCopy - 1)) >> 2;
   long long acfg[2] = {0, 0};
   int asite[2] = {-1, -1};
@@ -515,29 +514,25 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   };
   if (!BIN) tap_row(0);
   const uint32_t a_off = (piece >> 1) * S::A_BYTES + tc_off(arow, (piece & 1) * 4);
-  auto issue_next = [&]() {
-    if (is < STEPS) {
-      const int b = is % kStages;
-      unsigned char* st = smem + b * S::STAGE;
-      tc::cp_async16_zfill(st + a_off, isrc[0] + ikc * 2 * kTcKC, inb[0]);
-      tc::cp_async16_zfill(st + a_off + tc_off(64, 0), isrc[1] + ikc * 2 * kTcKC, inb[1]);
-      if (tid == 0) {
-        const float* w = bimg + ((size_t)id * KC + ikc) * 2 * CO * kTcKC + (size_t)cb * kTcKC;
-        tc::mbar_arrive_expect_tx(&full[b], 2 * S::B_BYTES);
-        tc::bulk_g2s(st + 2 * S::A_BYTES, w, S::B_BYTES, &full[b]);
-        tc::bulk_g2s(st + 2 * S::A_BYTES + S::B_BYTES, w + CO * kTcKC, S::B_BYTES, &full[b]);
-      }
-      ++is;
-      if (++ikc == KC) {
-        ikc = 0;
-        if (++id < taps) tap_row(id);
-      }
+  auto issue_next = [&](int b) {
+    unsigned char* st = smem + b * S::STAGE;
+    tc::cp_async16_zfill(st + a_off, isrc[0] + ikc * 2 * kTcKC, inb[0]);
+    tc::cp_async16_zfill(st + a_off + tc_off(64, 0), isrc[1] + ikc * 2 * kTcKC, inb[1]);
+    if (tid == 0) {
+      const float* w = bimg + ((size_t)id * KC + ikc) * 2 * CO * kTcKC + (size_t)cb * kTcKC;
+      tc::mbar_arrive_expect_tx(&full[b], 2 * S::B_BYTES);
+      tc::bulk_g2s(st + 2 * S::A_BYTES, w, S::B_BYTES, &full[b]);
+      tc::bulk_g2s(st + 2 * S::A_BYTES + S::B_BYTES, w + CO * kTcKC, S::B_BYTES, &full[b]);
     }
-    tc::cp_async_commit();
+    if (++ikc == KC) {
+      ikc = 0;
+      if (++id < taps) tap_row(id);
+    }
   };
 
-  // Copying warps: stage s into its slot once the MMAs of stage s - kStages are done; stage
-  // s - kAhead, whose copies have landed then, is handed to the MMA warp. No barrier of the block in the loop.
+  // Copying warps: stage s into its slot once the MMAs of stage s - kStages are done; the copies
+  // themselves arrive on the stage's barrier, so the warps never wait for them. No barrier of the block in the
+  // loop; the MMA warp fences the copies (generic proxy) against its reads.
   if (BIN && tid == 0) {  // blocked input: the whole stage by bulk copies
     const float* src = in + (size_t)(R / kTcRows) * kTcRows * 2 * C;
 #pragma unroll 1
@@ -555,19 +550,20 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
       tc::bulk_g2s(st + 2 * S::A_BYTES + S::B_BYTES, w + CO * kTcKC, S::B_BYTES, &full[b]);
     }
   } else if (!BIN && copier) {
+    int b = 0;
+    uint32_t ph = 1;  // parity of the slot's last MMAs, from the second round on
 #pragma unroll 1
-    for (int s = 0; s < STEPS + kAhead; ++s) {
-      if (s >= kStages && s < STEPS &&
-          !__all_sync(~0u, tc::mbar_wait(&done[s % kStages], (uint32_t)((s / kStages) - 1) & 1u, kTcWaitPolls))) {
+    for (int s = 0; s < STEPS; ++s) {
+      if (s >= kStages && !__all_sync(~0u, tc::mbar_wait(&done[b], ph, kTcWaitPolls))) {
         s_abort = 1;  // the whole warp leaves
         break;
       }
-      issue_next();
-      if (s < kAhead) continue;
-      tc::cp_async_wait<kAhead>();  // this thread's copies of stage s - kAhead have landed
-      tc::fence_proxy_async();      // ... and are visible to the tensor core
-      __syncwarp();
-      if ((tid & 31) == 0) tc::mbar_arrive(&full[(s - kAhead) % kStages]);
+      issue_next(b);
+      tc::cp_async_arrive(&full[b]);  // once this thread's copies have landed
+      if (++b == kStages) {
+        b = 0;
+        ph ^= 1;
+      }
     }
   } else if (tid == kTcCopy) {
 #pragma unroll 1
@@ -618,7 +614,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
     for (int c = 0; c < H2; ++c) u[c] = 0.f;
   }
   (void)u;
-  tc::cp_async_wait<0>();
+  tc::cp_async_wait_all();
   __syncthreads();
   tc::fence_after_sync();
   const bool aborted = s_abort, run = !aborted && copier;
