@@ -374,13 +374,14 @@ __device__ __forceinline__ float act_tc(int act, float z) {
   return tanh_f32(z);
 }
 
-template <int N>
+template <int N, bool BIN>
 struct TcShape {
   static constexpr uint32_t A_BYTES = kTcRows * kTcKC * 4;  // one half (hi or lo) of the A tile
   static constexpr uint32_t B_BYTES = N * kTcKC * 4;        // one half of the weight tile
-  static constexpr uint32_t STAGE = 2 * A_BYTES + 2 * B_BYTES;
-  // Ring slots: what fits one CTA per SM (160 and 192 columns) or two.
-  static constexpr int STAGES = N > 192 ? 4 : (N > 144 ? 10 : 6);
+  // K steps per stage (waits, fences and commits are per stage) and ring slots: what fits one CTA per SM
+  // (160 and 192 columns) or two. Blocked input: one step, as the copies are one thread's.
+  static constexpr int KS = BIN ? 1 : 2, STAGES = (N > 192 ? 4 : (N > 144 ? 10 : 6)) / KS;
+  static constexpr uint32_t STAGE = KS * (2 * A_BYTES + 2 * B_BYTES);
   static constexpr uint32_t SMEM = STAGES * STAGE + 2 * STAGES * 8 + 16 + 1024;  // + barriers, slot, alignment
   static constexpr uint32_t TCOLS = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
 };
@@ -444,10 +445,10 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   // C input channels (K = taps x C), CO output channels (this CTA: [cb, cb + N)); res: add the
   // input row (C == CO). A normalised block is one tile wide: C == CO == N.
   if constexpr (LN) C = CO = N;
-  using S = TcShape<N>;
+  using S = TcShape<N, BIN>;
   constexpr int kStages = S::STAGES;
   const int KC = C / kTcKC;
-  const int STEPS = taps * KC;
+  const int STEPS = taps * KC / S::KS;  // stages (KC is even for every width that is gathered)
   // Grid (column tile, row tile): the CO / N column tiles of the same 128 rows are adjacent
   // in launch order and run side by side, so all but the first read the rows from L2.
   const int cb = blockIdx.x * N;  // first output column of this CTA
@@ -460,6 +461,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   uint64_t* done = full + kStages;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(done + kStages);
   __shared__ int s_abort;
+  __shared__ int8_t s_tap[2][32];  // at most 13 taps (the plus stencil)
   __shared__ float s_sum[2][kTcRows], s_sq[2][kTcRows];  // per-half row sums for the normalisation
   const int tid = threadIdx.x, warp = tid >> 5, row = tid & (kTcRows - 1), part = (tid >> 7) & 1;
   const bool copier = tid < kTcCopy;
@@ -471,6 +473,12 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   const long long R = row0 + (long long)blockIdx.y * kTcRows + row;
   const bool valid = copier && R < rows;
 
+  if (!BIN && tid < taps) {
+    int dx, dy;
+    stencil_tap(stencil, ks, tid, dx, dy);
+    s_tap[0][tid] = (int8_t)dx;
+    s_tap[1][tid] = (int8_t)dy;
+  }
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
       tc::mbar_init(&full[s], BIN ? 1 : 1 + kTcCopy);  // the bulk copies, and the copying threads
@@ -490,7 +498,7 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   int id = 0, ikc = 0;
   const int piece = tid & 3, arow = (tid & (kTcCopy - 1)) >> 2;
   long long acfg[2] = {0, 0};
-  int asite[2] = {-1, -1};
+  int ax[2] = {-1, -1}, ay[2] = {0, 0};  // the rows' sites
   const float* isrc[2] = {in, in};
   uint32_t inb[2] = {0, 0};
   if (!BIN) {
@@ -499,15 +507,24 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
       const long long q = row0 + (long long)blockIdx.y * kTcRows + arow + 64 * u;
       if (q >= rows) continue;
       acfg[u] = q / Ns;
-      asite[u] = (int)(q - acfg[u] * Ns);
+      const int site = (int)(q - acfg[u] * Ns);
+      ay[u] = site / lat.Lx;
+      ax[u] = site - ay[u] * lat.Lx;
     }
   }
+  auto wrap = [](int x, int L, int pbc) {  // no division: the copying warps wait for each new tap
+    if (x >= 0 && x < L) return x;
+    if (!pbc) return -1;
+    while (x < 0) x += L;
+    while (x >= L) x -= L;
+    return x;
+  };
   auto tap_row = [&](int d) {
-    int dx, dy;
-    stencil_tap(stencil, ks, d, dx, dy);
+    const int dx = s_tap[0][d], dy = s_tap[1][d];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const int j = asite[u] >= 0 ? site_off(lat, asite[u], dx, dy) : -1;
+      const int x = wrap(ax[u] + dx, lat.Lx, lat.pbc_x), y = wrap(ay[u] + dy, lat.Ly, lat.pbc_y);
+      const int j = ax[u] >= 0 && x >= 0 && y >= 0 ? y * lat.Lx + x : -1;
       isrc[u] = in + (j >= 0 ? split_off(acfg[u] * Ns + j, C, 0) + piece * 4 : 0);
       inb[u] = j >= 0 ? 16u : 0u;  // zero fill past an open edge or the last row
     }
@@ -516,15 +533,23 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
   const uint32_t a_off = (piece >> 1) * S::A_BYTES + tc_off(arow, (piece & 1) * 4);
   auto issue_next = [&](int b) {
     unsigned char* st = smem + b * S::STAGE;
-    tc::cp_async16_zfill(st + a_off, isrc[0] + ikc * 2 * kTcKC, inb[0]);
-    tc::cp_async16_zfill(st + a_off + tc_off(64, 0), isrc[1] + ikc * 2 * kTcKC, inb[1]);
+#pragma unroll
+    for (int k = 0; k < S::KS; ++k) {
+      tc::cp_async16_zfill(st + k * 2 * S::A_BYTES + a_off, isrc[0] + (ikc + k) * 2 * kTcKC, inb[0]);
+      tc::cp_async16_zfill(st + k * 2 * S::A_BYTES + a_off + tc_off(64, 0), isrc[1] + (ikc + k) * 2 * kTcKC, inb[1]);
+    }
     if (tid == 0) {
       const float* w = bimg + ((size_t)id * KC + ikc) * 2 * CO * kTcKC + (size_t)cb * kTcKC;
-      tc::mbar_arrive_expect_tx(&full[b], 2 * S::B_BYTES);
-      tc::bulk_g2s(st + 2 * S::A_BYTES, w, S::B_BYTES, &full[b]);
-      tc::bulk_g2s(st + 2 * S::A_BYTES + S::B_BYTES, w + CO * kTcKC, S::B_BYTES, &full[b]);
+      unsigned char* sb = st + S::KS * 2 * S::A_BYTES;
+      tc::mbar_arrive_expect_tx(&full[b], S::KS * 2 * S::B_BYTES);
+      if (CO == N) {
+        tc::bulk_g2s(sb, w, S::KS * 2 * S::B_BYTES, &full[b]);
+      } else {
+        for (int k = 0; k < 2 * S::KS; ++k) tc::bulk_g2s(sb + k * S::B_BYTES, w + (size_t)k * CO * kTcKC, S::B_BYTES, &full[b]);
+      }
     }
-    if (++ikc == KC) {
+    ikc += S::KS;
+    if (ikc == KC) {
       ikc = 0;
       if (++id < taps) tap_row(id);
     }
@@ -566,24 +591,32 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
       }
     }
   } else if (tid == kTcCopy) {
+    const uint32_t a0 = tc::smem_u32(smem);
+    const uint64_t da = tc::smem_desc_kmajor(a0, kTcLBO, kTcSBO);  // the address field counts 16 bytes
+    const uint64_t db = tc::smem_desc_kmajor(a0 + S::KS * 2 * S::A_BYTES, kTcLBO, kTcSBO);
+    int b = 0;
+    uint32_t ph = 0;
 #pragma unroll 1
     for (int s = 0; s < STEPS; ++s) {
-      const int b = s % kStages;
-      if (!tc::mbar_wait(&full[b], (uint32_t)(s / kStages) & 1u, kTcWaitPolls)) {
+      if (!tc::mbar_wait(&full[b], ph, kTcWaitPolls)) {
         s_abort = 1;
         break;
       }
       tc::fence_after_sync();
-      tc::fence_proxy_async();
-      const uint32_t a0 = tc::smem_u32(smem + b * S::STAGE);
-      const uint64_t ah = tc::smem_desc_kmajor(a0, kTcLBO, kTcSBO);
-      const uint64_t al = tc::smem_desc_kmajor(a0 + S::A_BYTES, kTcLBO, kTcSBO);
-      const uint64_t bh = tc::smem_desc_kmajor(a0 + 2 * S::A_BYTES, kTcLBO, kTcSBO);
-      const uint64_t bl = tc::smem_desc_kmajor(a0 + 2 * S::A_BYTES + S::B_BYTES, kTcLBO, kTcSBO);
-      tc::mma_tf32(tmem, ah, bh, IDESC, s > 0 ? 1u : 0u);
-      tc::mma_tf32(tmem, al, bh, IDESC, 1u);
-      tc::mma_tf32(tmem, ah, bl, IDESC, 1u);
+      if constexpr (!BIN) tc::fence_proxy_async();
+#pragma unroll
+      for (int k = 0; k < S::KS; ++k) {
+        const uint64_t ah = da + (b * S::STAGE + k * 2 * S::A_BYTES) / 16, al = ah + S::A_BYTES / 16;
+        const uint64_t bh = db + (b * S::STAGE + k * 2 * S::B_BYTES) / 16, bl = bh + S::B_BYTES / 16;
+        tc::mma_tf32(tmem, ah, bh, IDESC, s + k > 0 ? 1u : 0u);
+        tc::mma_tf32(tmem, al, bh, IDESC, 1u);
+        tc::mma_tf32(tmem, ah, bl, IDESC, 1u);
+      }
       tc::mma_commit(&done[b]);
+      if (++b == kStages) {
+        b = 0;
+        ph ^= 1;
+      }
     }
     // every MMA of this thread, before the accumulator is read and the ring's copies are all drained
     const int sl = STEPS - 1;
@@ -706,7 +739,7 @@ template <int N, bool LN, bool BIN = false>
 cudaError_t run_conv_tc(cudaStream_t st, const Lattice& lat, const float* bimg, const float* bias, const float* g,
                         const float* be, int act, float eps, int C, int CO, int res, int ks, int stencil,
                         const float* in, float* out, int omode, long long rows, int* err, const int* vcfg) {
-  using S = TcShape<N>;
+  using S = TcShape<N, BIN>;
   cudaError_t e =
       cudaFuncSetAttribute(k_ace_conv_tc<N, LN, BIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
   if (e != cudaSuccess) return e;
@@ -728,9 +761,9 @@ cudaError_t run_conv_tc(cudaStream_t st, const Lattice& lat, const float* bimg, 
 // (four tiles of 160), 3x3 box or the 5x5 plus.
 bool tc_width(int h) { return h == 48 || h == 144 || h == 192; }
 bool tc_wide_width(int h) { return h == 384 || h == 640; }
-// Site-wise layers on tcgen05 (1x1, no residual): input width a multiple of 8, output width a
+// Site-wise layers on tcgen05 (1x1, no residual): input width a multiple of 16, output width a
 // multiple of 128 (tiles of 128 columns, two CTAs per SM).
-bool tc_sitewise(int cin, int cout) { return cin % kTcKC == 0 && cout % 128 == 0; }
+bool tc_sitewise(int cin, int cout) { return cin % (2 * kTcKC) == 0 && cout % 128 == 0; }
 
 cudaError_t launch_conv_tc(const scale_ctx* c, const Lattice& lat, bool ln, int cin, int cout, int res, int ks,
                            const float* bimg, const float* bias, const float* g, const float* be, int act, float eps,
