@@ -433,9 +433,11 @@ __global__ void k_ace_embed_split(int N, int h, int per_site, const float* __res
 // normalisation, column tiles of N: blockIdx.x selects columns [N x, N x + N)). in: split rows
 // (split_off; BIN: blocked), out: plain FP32 rows (omode 0), split (1) or blocked (2). err: set when
 // a wait ran out. Copying thread t takes the 16-byte piece t % 4 of rows t / 4 and t / 4 + 64 (four lanes a
-// row: 64 contiguous bytes; one lane a row, with hi and lo in separate slabs, asked for 32 lines per load: the
-// blocks of ACE 16x16, 96 walkers, 2.54 ms, now HERE). In the epilogue thread t serves row t % 128, the tile's columns [0, N/2) (warps 0-3) or [N/2, N) (warps
-// 4-7); a warp reads the TMEM lanes of its quarter (warp % 4).
+// row: 64 contiguous bytes). In the epilogue thread t serves row t % 128, the tile's columns [0, N/2) (warps 0-3)
+// or [N/2, N) (warps 4-7); a warp reads the TMEM lanes of its quarter (warp % 4).
+// What bounds it: a gathered block waits for its copies (16x16, 96 walkers: 192 tiles on 152 SMs, 40 SMs with
+// two; the MMAs of a block take 20 of its 123 us, 180 at first), a blocked 512 -> 512 layer runs the MMAs at
+// the tensor pipe's TF32 rate (385 cycles per 8 channels and two CTAs, 435 at the nominal rate).
 template <int N, bool LN, bool BIN>
 __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ace_conv_tc(
     Lattice lat, const float* __restrict__ bimg, const float* __restrict__ bias, const float* __restrict__ gam,
@@ -623,42 +625,25 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
     if (!s_abort && !tc::mbar_wait(&done[sl % kStages], (uint32_t)(sl / kStages) & 1u, kTcWaitPolls)) s_abort = 1;
   }
   __syncwarp();
-  // this thread's half of the tile's residual row (independent of the MMAs: loaded under them);
-  // the 256-column tiles (site-wise layers, no residual) stream their epilogue instead
+  // the 256-column tiles (site-wise layers, no residual) stream their epilogue; the others take residual and
+  // output through the ring's memory, [128][N + 4], so that global memory sees whole rows (one thread a
+  // row, each of its 16-byte accesses was a line of its own and the epilogue a third of an ACE block's time:
+  // 146 us a block of 16x16, 96 walkers, 123 since)
   constexpr bool kStream = N == 256;
+  constexpr int kLd = N + 4, kGroups = N / 4;
+  static_assert(kStream || kTcRows * kLd * 4 <= S::STAGES * S::STAGE, "the tile fits the ring");
   const int c0 = part * H2;
-  float u[kStream ? 1 : H2];
-  if constexpr (kStream) {
-    u[0] = 0.f;
-  } else if (LN || res) {  // the normalised conv blocks are residual
-    const float* xr = in + split_off(valid ? R : 0, C, cb + c0);
-#pragma unroll
-    for (int c = 0; c < H2; c += 4) {
-      const float* x = xr + split_off(0, C, c);
-      const float4 h4 = __ldg(reinterpret_cast<const float4*>(x));
-      const float4 l4 = __ldg(reinterpret_cast<const float4*>(x + kSplitLo));
-      u[c] = h4.x + l4.x;
-      u[c + 1] = h4.y + l4.y;
-      u[c + 2] = h4.z + l4.z;
-      u[c + 3] = h4.w + l4.w;
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < H2; ++c) u[c] = 0.f;
-  }
-  (void)u;
   tc::cp_async_wait_all();
   __syncthreads();
   tc::fence_after_sync();
   const bool aborted = s_abort, run = !aborted && copier;
-  // columns [c, c + 4) of this thread's half of the row
-  auto put = [&](int c, const float(&y)[4]) {
-    const int col = cb + c0 + c;
+  // columns [col, col + 4) of row r of the output
+  auto put = [&](long long r, int col, const float(&y)[4]) {
     if (omode == 0) {
-      *reinterpret_cast<float4*>(out + (size_t)R * CO + col) = make_float4(y[0], y[1], y[2], y[3]);
+      *reinterpret_cast<float4*>(out + (size_t)r * CO + col) = make_float4(y[0], y[1], y[2], y[3]);
       return;
     }
-    float* o = out + (omode == 2 ? ace_blk_off(R, CO, col) : split_off(R, CO, col));
+    float* o = out + (omode == 2 ? ace_blk_off(r, CO, col) : split_off(r, CO, col));
     uint32_t hi[4], lo[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) split_tf32(y[e], hi[e], lo[e]);
@@ -675,8 +660,8 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
 #pragma unroll
         for (int q = 0; q < 8; ++q) z[q] = act_tc(act, z[q] + __ldg(bias + cb + c0 + cc * 8 + q));
         if (valid) {
-          put(cc * 8, reinterpret_cast<const float(&)[4]>(z[0]));
-          put(cc * 8 + 4, reinterpret_cast<const float(&)[4]>(z[4]));
+          put(R, cb + c0 + cc * 8, reinterpret_cast<const float(&)[4]>(z[0]));
+          put(R, cb + c0 + cc * 8 + 4, reinterpret_cast<const float(&)[4]>(z[4]));
         }
       }
     } else if (aborted && tid == 0) {
@@ -687,6 +672,24 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
     if (warp == 0) tc::tmem_dealloc(tmem, S::TCOLS);
     return;
   }
+  float* tile = reinterpret_cast<float*>(smem);
+  const long long R0 = row0 + (long long)blockIdx.y * kTcRows;
+  const bool resid = LN || res;  // the normalised conv blocks are residual
+  if (run && resid) {
+#pragma unroll 6
+    for (int q = tid; q < kTcRows * kGroups; q += kTcCopy) {
+      const int r = q / kGroups, g = q - r * kGroups;
+      if (R0 + r >= rows) continue;
+      const float* x = in + split_off(R0 + r, C, cb + 4 * g);
+      const float4 h4 = __ldg(reinterpret_cast<const float4*>(x));
+      const float4 l4 = __ldg(reinterpret_cast<const float4*>(x + kSplitLo));
+      *reinterpret_cast<float4*>(tile + r * kLd + 4 * g) =
+          make_float4(h4.x + l4.x, h4.y + l4.y, h4.z + l4.z, h4.w + l4.w);
+    }
+  }
+  __syncthreads();
+  float u[kStream ? 1 : H2];  // this thread's half of its row
+  float* urow = tile + row * kLd + c0;
   if (run) {
     const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0;
 #pragma unroll
@@ -694,7 +697,13 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
       float z[8];
       tc::tmem_ld8(trow + cc * 8, z);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) u[cc * 8 + q] += act_tc(act, z[q] + __ldg(bias + cb + c0 + cc * 8 + q));
+      for (int q = 0; q < 8; q += 4) {
+        const float4 x = resid ? *reinterpret_cast<const float4*>(urow + cc * 8 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          u[cc * 8 + q + e] = xs[e] + act_tc(act, z[q + e] + __ldg(bias + cb + c0 + cc * 8 + q + e));
+      }
     }
     if constexpr (LN) {
       float s1 = 0.f;
@@ -725,10 +734,22 @@ __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ac
         if constexpr (LN) y[e] = (u[c + e] - mean) * inv * __ldg(gam + c0 + c + e) + __ldg(bet + c0 + c + e);
         else y[e] = u[c + e];
       }
-      if (valid) put(c, y);
+      *reinterpret_cast<float4*>(urow + c) = make_float4(y[0], y[1], y[2], y[3]);
     }
   } else if (aborted && tid == 0) {
     atomicExch(err, 1);
+  }
+  __syncthreads();
+  if (run) {
+#pragma unroll 2
+    for (int q = tid; q < kTcRows * kGroups; q += kTcCopy) {
+      // along the row, or for blocked rows along the rows of four columns: whole lines either way
+      const int r = omode == 2 ? q % kTcRows : q / kGroups, g = omode == 2 ? q / kTcRows : q - r * kGroups;
+      if (R0 + r >= rows) continue;
+      const float4 v = *reinterpret_cast<const float4*>(tile + r * kLd + 4 * g);
+      const float y[4] = {v.x, v.y, v.z, v.w};
+      put(R0 + r, cb + 4 * g, y);
+    }
   }
   tc::fence_before_sync();
   __syncthreads();
