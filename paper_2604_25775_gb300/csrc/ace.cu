@@ -437,7 +437,7 @@ __global__ void k_ace_embed_split(int N, int h, int per_site, const float* __res
 // or [N/2, N) (warps 4-7); a warp reads the TMEM lanes of its quarter (warp % 4).
 // What bounds it: a gathered block waits for its copies (16x16, 96 walkers: 192 tiles on 152 SMs, 40 SMs with
 // two; the MMAs of a block take 20 of its 123 us, 180 at first), a blocked 512 -> 512 layer runs the MMAs at
-// the tensor pipe's TF32 rate (385 cycles per 8 channels and two CTAs, 435 at the nominal rate).
+// the tensor pipe's TF32 rate (385 cycles per eight channels of a tile, 435 at the nominal rate).
 template <int N, bool LN, bool BIN>
 __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ace_conv_tc(
     Lattice lat, const float* __restrict__ bimg, const float* __restrict__ bias, const float* __restrict__ gam,

@@ -934,7 +934,9 @@ cudaError_t run_gj_split(const GjArgs& a, TOUT* binv) {
 //   n <= 256: many matrices 256 threads, two CTAs per SM, one matrix's panel beside the other's
 //     updates: n = 224, 1500 matrices 8.7 (old 38.3). Up to one per SM 512 threads, whose warps
 //     share the updates: 1.02 alone (1.20 with 256 threads, old 3.83). Up to 32 matrices clusters
-//     of 4 CTAs: 0.69. (Clusters of 4 fill the GPCs' SMs at about 36: 38 matrices 1.37.)
+//     of 4 CTAs: 0.69. (Clusters of 4 fill the GPCs' SMs at about 36: 38 matrices 1.37.) Up to 72
+//     clusters of 2, of which 76 run at once: 0.82 (loads of 40 and 72 walkers 1222 -> 1009 and 1292 ->
+//     1081 us; 76 are two waves).
 //   n <= 512: 512 threads; clusters of 4 also pay in two waves: n = 448 alone 2.37 against 5.36,
 //     38 matrices 4.75 against 5.37.
 //   n <= 1024: two panel rows per thread; n = 896: 152 matrices 43.5 (old 189); alone 39.3, in a
@@ -944,6 +946,7 @@ cudaError_t gj_split(const GjArgs& a, TOUT* binv) {
   if (a.n <= 128) return run_gj_split<TOUT, kInverse, 128, 4, 1, 1>(a, binv);
   if (a.n <= 512) {
     if (a.expect <= (a.n <= 256 ? 32 : 64)) return run_gj_split<TOUT, kInverse, 512, 1, 1, 4>(a, binv);
+    if (a.n <= 256 && a.expect <= 72) return run_gj_split<TOUT, kInverse, 512, 1, 1, 2>(a, binv);
     if (a.n <= 256 && a.expect > kSMs) return run_gj_split<TOUT, kInverse, 256, 2, 1, 1>(a, binv);
     return run_gj_split<TOUT, kInverse, 512, 1, 1, 1>(a, binv);
   }
