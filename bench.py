@@ -558,7 +558,7 @@ def main():
         line["cpu_baseline"] = {"value": n_cpu / dt, "unit": "E_loc/s", "cores": O.num_threads(), "kind": "oracle",
                                 "sample": f"{n_cpu} walkers of the same workload, FP64 full recompute"}
     # per step, as an ncu launch list of the chain step shows: k_eloc, k_commit, k_mark_refresh,
-    # and the refresh of the due samples: k_slots, k_layer, k_mlp_fwd, k_phi, k_gj, k_project
+    # and the refresh of the due samples: k_layer_tile, k_mlp_fwd, k_phi32, k_slots, k_gj_split, k_project32
     line["gpu_launches"] = K * 9
     if rank == 0:
         print(json.dumps(line), flush=True)
