@@ -195,7 +195,8 @@ __global__ void __launch_bounds__(256) k_project(int Ne, int h, const T* __restr
       Ws[kk][col] = (k < Ne) ? proj_w[(size_t)cc * 2 * Ne + s * Ne + k] : T(0);
     }
     __syncthreads();
-    for (int kk = 0; kk < 32; ++kk) {
+    const int kn = c0 + (row & ~3) < Ne ? min(32, Ne - k0) : 0;  // nothing for a warp past the last row
+    for (int kk = 0; kk < kn; ++kk) {
       const T bv = Bs[row][kk];
 #pragma unroll
       for (int u = 0; u < 16; ++u) {
@@ -234,6 +235,8 @@ __global__ void __launch_bounds__(256) k_build_g0(int Ne, int No, const T* __res
   const int nrows = count ? min(*count, B) : B;
   const int j0 = blockIdx.x * 64, o0 = blockIdx.y * 64;
   const int tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
+  // rows j0 + 16 u + tr of this warp (two tr) that exist: the padding of a tile is not worth the FP64 pipe's time
+  const int un = min(4, max(0, (Ne - j0 - (tr & ~1) + 15) >> 4));
   for (int lrow = blockIdx.z; lrow < nrows; lrow += gridDim.z) {
     const int b = list ? list[lrow] : lrow;
     if (b < 0) continue;
@@ -247,8 +250,9 @@ __global__ void __launch_bounds__(256) k_build_g0(int Ne, int No, const T* __res
         Ms[kk][rr] = (o0 + rr < No && k < Ne) ? M0b[(size_t)(o0 + rr) * Ne + k] : T(0);
       }
       __syncthreads();
+      const int kn = min(32, Ne - k0);
 #pragma unroll 4
-      for (int kk = 0; kk < 32; ++kk) {
+      for (int kk = 0; kk < kn; ++kk) {
         T x[4], y[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -256,9 +260,11 @@ __global__ void __launch_bounds__(256) k_build_g0(int Ne, int No, const T* __res
           y[u] = Ms[kk][tc + 16 * u];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 4; ++u) {
+          if (u >= un) break;
 #pragma unroll
           for (int v = 0; v < 4; ++v) acc[u][v] += x[u] * y[v];
+        }
       }
     }
     T* out = G0t + (size_t)b * Ne * No;
