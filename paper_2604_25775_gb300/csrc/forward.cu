@@ -1,6 +1,7 @@
 // forward.cu -- network forward (Sec. II.B), slot bookkeeping,
 // layer-0 conv-of-embedding table and the log|psi| output convention.
 #include <algorithm>
+#include <climits>
 
 #include "mlp_mma.cuh"
 #include "scale_internal.cuh"
@@ -258,17 +259,34 @@ __global__ void k_build_ke(Net<T> net, int Ns, T* __restrict__ KE) {
 }
 
 // log|psi| and sign in the ascending convention: sign = sign_slot * parity of the slot
-// permutation orb_of_slot (inversions counted directly).
+// permutation orb_of_slot (inversions counted directly). Bound by its Ne^2 / 2 comparisons: a thread takes
+// a slot against the later ones, four per broadcast load from shared memory (a division and two loads through
+// L1 per pair before: one sample of 896 electrons 252 us, 2048 of 224 106 us). Up to kLogpsiStaged slots staged.
+constexpr int kLogpsiStaged = 8192;
 __global__ void k_logpsi_out(int Ne, const int32_t* __restrict__ orb_of_slot, const double* __restrict__ la_slot,
                              const int32_t* __restrict__ sg_slot, const int32_t* __restrict__ status,
                              double* __restrict__ logabs, int32_t* __restrict__ sign,
                              const int32_t* __restrict__ list) {
+  extern __shared__ __align__(16) int32_t s_os[];
   const int b = list ? list[blockIdx.x] : blockIdx.x;
   const int32_t* os = orb_of_slot + (size_t)b * Ne;
+  const bool staged = Ne <= kLogpsiStaged;
+  if (staged) {
+    for (int q = threadIdx.x; q < ((Ne + 3) & ~3); q += blockDim.x) s_os[q] = q < Ne ? os[q] : INT_MAX;
+    __syncthreads();
+  }
   int inv = 0;
-  for (int q = threadIdx.x; q < Ne * Ne; q += blockDim.x) {
-    const int a = q / Ne, c = q - a * Ne;
-    inv += (a < c) && (os[a] > os[c]);
+  for (int a = threadIdx.x; a < Ne; a += blockDim.x) {
+    const int v = os[a];
+    if (staged) {
+#pragma unroll 4
+      for (int c = (a & ~31); c < Ne; c += 4) {  // from the warp's first slot on: the lanes read the same words
+        const int4 o = *reinterpret_cast<const int4*>(s_os + c);
+        inv += (c > a && v > o.x) + (c + 1 > a && v > o.y) + (c + 2 > a && v > o.z) + (c + 3 > a && v > o.w);
+      }
+    } else {
+      for (int c = a + 1; c < Ne; ++c) inv += v > os[c];
+    }
   }
   __shared__ int s_inv;
   if (threadIdx.x == 0) s_inv = 0;
@@ -585,14 +603,15 @@ cudaError_t launch_build_ke(scale_ctx* c) {
   return cudaGetLastError();
 }
 
+static size_t logpsi_smem(int Ne) { return Ne <= kLogpsiStaged ? sizeof(int32_t) * ((Ne + 3) & ~3) : 0; }
 cudaError_t launch_logpsi_out(scale_ctx* c, double* logabs, int32_t* sign) {
-  k_logpsi_out<<<c->B, 256, 0, c->stream>>>(c->Ne, c->orb_of_slot, c->logabs, c->sign_slot, c->status,
+  k_logpsi_out<<<c->B, 256, logpsi_smem(c->Ne), c->stream>>>(c->Ne, c->orb_of_slot, c->logabs, c->sign_slot, c->status,
                                              logabs, sign, nullptr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_logpsi_list(scale_ctx* c, const int32_t* list, int n, double* logabs, int32_t* sign) {
-  k_logpsi_out<<<n, 256, 0, c->stream>>>(c->Ne, c->orb_of_slot, c->logabs, c->sign_slot, c->status, logabs, sign,
+  k_logpsi_out<<<n, 256, logpsi_smem(c->Ne), c->stream>>>(c->Ne, c->orb_of_slot, c->logabs, c->sign_slot, c->status, logabs, sign,
                                          list);
   return cudaGetLastError();
 }
