@@ -426,8 +426,11 @@ __device__ __forceinline__ void split_row_tile(const double (&v)[4][2], const in
 
 // One matrix by a cluster of C CTAs of TH threads, R TH >= n, R rows of the panel per thread. The
 // column blocks are dealt out to the CTAs in turn; every CTA takes the panel, (2) and (3) itself,
-// with the same bits, and updates its own columns, so a block costs one cluster barrier and no
-// exchange but through the matrix.
+// with the same bits, and updates its own columns, with no exchange but through the matrix. Two
+// cluster barriers a block: the updates of a block before the next one's panel loads, and the panel loads
+// (before the first block the scan of the rows' exponents too) before any store to the matrix, as the
+// owner of the block's columns stores them swept. The second is split: CTAs arrive with their panel in
+// registers and wait after the pivot steps, which hide it.
 template <typename TOUT, bool kInverse, int TH, int R, int C>
 __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats, int n, int ch, int b,
                              TOUT* __restrict__ binv, double* __restrict__ logabs_out, int32_t* __restrict__ sign_out,
@@ -505,6 +508,7 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
         for (int k = 0; k < kSW; ++k) a[m][k] = (row[m] >= 0 && k < w) ? __ldcg(src + k) : 0.0;
       }
     }
+    if constexpr (C > 1) cg::this_cluster().barrier_arrive();  // the matrix is read as far as this block needs it
     if (tid == 0) s_wild = 0;
     if (tid < kSW * kSW) tri[(tid / kSW) * kSTd + tid % kSW] = tid / kSW == tid % kSW ? 1.0 : 0.0;
     for (int q = TH + tid; q < kSW * kSW; q += TH) tri[(q / kSW) * kSTd + q % kSW] = q / kSW == q % kSW ? 1.0 : 0.0;
@@ -579,6 +583,7 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
         for (int k = jj + 1; k < kSW; ++k) a[m][k] = fma(-f, prow[k], a[m][k]);
       }
     }
+    if constexpr (C > 1) cg::this_cluster().barrier_wait();  // ... by every CTA: stores may follow
     if (singular) break;
     const int c_lo = kInverse ? 0 : K0 + w;
     if (c_lo >= n) break;  // determinant: the last block is done
@@ -867,7 +872,6 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
     const int s = q / n, cf = q - s * n;
     binv[(size_t)b * n * n + q] = (TOUT)__ldcg(A + (size_t)piv[cf] * n + qinv[s]);
   }
-  if constexpr (C > 1) cg::this_cluster().sync();  // the matrix is read before another takes its place
 }
 
 // All B matrices, the listed ones (entries below 0 are skipped), or the first *count entries of a
@@ -882,7 +886,9 @@ __global__ void __launch_bounds__(TH, MINB) k_gj_split(double* __restrict__ mats
   for (int e = blockIdx.x / C; e < total; e += gridDim.x / C) {
     const int b = list ? list[e] : e;
     if (b >= 0) gj_split_one<TOUT, kInverse, TH, R, C>(smem_raw, mats, n, ch, b, binv, logabs_out, sign_out, status);
-    __syncthreads();  // the next matrix takes the same shared memory
+    // the next matrix takes the same shared memory; a cluster goes on to it together
+    if constexpr (C == 1) __syncthreads();
+    else cg::this_cluster().sync();
   }
 }
 
