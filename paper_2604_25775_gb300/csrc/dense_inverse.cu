@@ -321,27 +321,28 @@ cudaError_t run_gj(cudaStream_t st, TW* mats, int n, int B, const int32_t* list,
 //      integer keys.
 //  (2) X = L11^-1 and (inverse) U11^-1 by warp 0, the column slices of the old pivot rows P by
 //      the other warps.
-//  (3) The left factor U = -L21 X of the rows without a pivot, U11^-1 X of the block's pivot rows,
+//  (3) The left factor U = -L21 X of the rows without a pivot, -U11^-1 X of the block's pivot rows,
 //      as split products (its fragment order is that of (4)'s operand, so it stays in registers);
-//      U is also the block's columns of the matrix after the sweep.
+//      X's unit diagonal is left to an FP64 addition. U is also the block's columns of the matrix
+//      after the sweep.
 //  (4) A[i][c] += sum_k U[i][k] P[k][c] outside the block, a pivot row starting from zero.
 //
-// Scales: rows of U by their largest exponent, columns of P per column; between the two, pivot
-// k's column of U is multiplied by the power of two that divides its row of P, the largest
-// exponent of that row of the input matrix, so that rows of very different size do not cost the
-// products of the small ones their low digits. A block whose factors hold an infinity, a NaN
-// or a scale far from 1 (2^+-100 for input rows, 2^+-200 inside the panel, 2^+-300 for the
-// columns: the products' exponents then stay in range) takes (3) and (4) in plain FP64.
+// Elements whose split sum could lose digits that an FP64 chain keeps (split_weak) are taken by
+// such a chain: in (3) from the panel and X in shared memory, in (4) from U in the warp's registers and
+// P in FP64 (the matrix itself without inverse, where no pivot row changes; else a copy in the block
+// of Binv that the inverse is going to overwrite). A tile's weak elements are queued, so that 32 of them
+// share one chain of 16 multiply-adds per lane: a 16 x 16 Hubbard walker has 3% of them, in 6% of the tiles.
 constexpr int kSW = 16;        // pivots per block = k of one mma
 constexpr int kSLd = kSW + 2;  // panel row stride in doubles: 16-byte rows without bank conflicts
 constexpr int kSTd = kSW + 1;  // row stride of the 16 x 16 blocks
 constexpr int kSCols = 224;    // columns whose slices are staged at a time
 constexpr int kSColsTall = 128;  // beside a panel of more than 512 rows
 constexpr int kSplitMaxN = 1024;
+constexpr int kSPkMax = 32;    // rows up to which the block of Binv is too small for P
 constexpr int kSMs = 152;
 
 struct SplitSmem {
-  size_t panel, tri, xs, xf, xe, prow, inv, bf, fexp, rexp, rho, piv, qinv, act, used, total;
+  size_t panel, tri, xs, xf, xe, prow, inv, bf, fexp, pk, piv, qinv, act, used, total;
 };
 __host__ __device__ inline SplitSmem split_smem(int n, int ch) {
   SplitSmem s{};
@@ -360,8 +361,7 @@ __host__ __device__ inline SplitSmem split_smem(int n, int ch) {
   s.inv = take(sizeof(double) * kSW);
   s.bf = take((size_t)(ch / 8) * kSplit * 32 * sizeof(uint2));
   s.fexp = take(sizeof(int) * ch);
-  s.rexp = take(sizeof(int) * n);
-  s.rho = take(sizeof(int) * kSW);
+  s.pk = take(n <= kSPkMax ? sizeof(double) * kSW * n : 0);
   s.piv = take(sizeof(int) * n);
   s.qinv = take(sizeof(int) * n);
   s.act = take(sizeof(int) * n);
@@ -372,53 +372,46 @@ __host__ __device__ inline SplitSmem split_smem(int n, int ch) {
 
 __device__ __forceinline__ uint64_t dbits(double x) { return (uint64_t)__double_as_longlong(x); }
 
-// Exponent field within 2^+-lim of 1, or the value zero (also rejects infinities and NaN).
-__device__ __forceinline__ bool exp_near(int e, bool nonzero, int lim) {
-  return !nonzero || (e >= 1023 - lim && e <= 1023 + lim);
-}
-
 // Slices of the B fragment of one 8-column tile from the lane's values x[q] (row k = 2t + (q & 1)
-// + 8 (q >> 1) of the lane's column g) multiplied by 2^-rho_k; the column's scale to *fe (t == 0).
-// Returns whether the scale is usable.
-__device__ __forceinline__ bool split_column_tile(const uint64_t (&x)[4], const int* rho, uint2* bf, int* fe) {
+// + 8 (q >> 1) of the lane's column g); the column's scale to *fe (t == 0).
+__device__ __forceinline__ void split_column_tile(const uint64_t (&x)[4], uint2* bf, int* fe) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int2 r0 = *reinterpret_cast<const int2*>(rho + 2 * t), r1 = *reinterpret_cast<const int2*>(rho + 2 * t + 8);
-  int e = max(max(exp_scaled(x[0], -r0.x), exp_scaled(x[1], -r0.y)), max(exp_scaled(x[2], -r1.x), exp_scaled(x[3], -r1.y)));
+  int e = max(max(exp_field(x[0]), exp_field(x[1])), max(exp_field(x[2]), exp_field(x[3])));
   int nz = ((x[0] | x[1] | x[2] | x[3]) << 1) != 0;
 #pragma unroll
   for (int off = 1; off < 4; off <<= 1) {
     e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
     nz |= __shfl_xor_sync(0xffffffffu, nz, off);
   }
-  if (t == 0) fe[g] = e;
+  if (t == 0) fe[g] = split_scale(e, nz != 0);
   uint32_t s0[kSplit], s1[kSplit];
-  split_pair(split_fixed(x[0], e + r0.x), split_fixed(x[1], e + r0.y), s0);
-  split_pair(split_fixed(x[2], e + r1.x), split_fixed(x[3], e + r1.y), s1);
+  split_pair(split_fixed(x[0], e), split_fixed(x[1], e), s0);
+  split_pair(split_fixed(x[2], e), split_fixed(x[3], e), s1);
 #pragma unroll
   for (int l = 0; l < kSplit; ++l) bf[l * 32 + lane] = make_uint2(s0[l], s1[l]);
-  return exp_near(e, nz != 0, 300);
 }
 
 // Slices of the A fragment of 16 rows from the lane's values v[q][0..1] (row g + 8 (q & 1), columns
-// 2t, 2t + 1 at q < 2 and 2t + 8, 2t + 9 at q >= 2) times 2^rho of their column; the scales of
-// the lane's two rows come back in ex.
-__device__ __forceinline__ void split_row_tile(const double (&v)[4][2], const int* rho, uint32_t (&a)[kSplit][4],
-                                               int (&ex)[2]) {
-  const int t = threadIdx.x & 3;
-  const int2 r0 = *reinterpret_cast<const int2*>(rho + 2 * t), r1 = *reinterpret_cast<const int2*>(rho + 2 * t + 8);
+// 2t, 2t + 1 at q < 2 and 2t + 8, 2t + 9 at q >= 2); the scales of the lane's two rows come back in ex.
+__device__ __forceinline__ void split_row_tile(const double (&v)[4][2], uint32_t (&a)[kSplit][4], int (&ex)[2]) {
+  int em[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    int e = max(max(exp_scaled(dbits(v[h][0]), r0.x), exp_scaled(dbits(v[h][1]), r0.y)),
-                max(exp_scaled(dbits(v[2 + h][0]), r1.x), exp_scaled(dbits(v[2 + h][1]), r1.y)));
-    e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
-    e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
-    ex[h] = e;
+    const uint64_t x0 = dbits(v[h][0]), x1 = dbits(v[h][1]), x2 = dbits(v[2 + h][0]), x3 = dbits(v[2 + h][1]);
+    int e = max(max(exp_field(x0), exp_field(x1)), max(exp_field(x2), exp_field(x3)));
+    int nz = ((x0 | x1 | x2 | x3) << 1) != 0;
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1) {
+      e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
+      nz |= __shfl_xor_sync(0xffffffffu, nz, off);
+    }
+    em[h] = e;
+    ex[h] = split_scale(e, nz != 0);
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const int2 rk = q < 2 ? r0 : r1;
     uint32_t s[kSplit];
-    split_pair(split_fixed(dbits(v[q][0]), ex[q & 1] - rk.x), split_fixed(dbits(v[q][1]), ex[q & 1] - rk.y), s);
+    split_pair(split_fixed(dbits(v[q][0]), em[q & 1]), split_fixed(dbits(v[q][1]), em[q & 1]), s);
 #pragma unroll
     for (int l = 0; l < kSplit; ++l) a[l][q] = s[l];
   }
@@ -447,8 +440,6 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
   double* inv = reinterpret_cast<double*>(smem_raw + S.inv);      // [16] reciprocal pivots
   uint2* bf = reinterpret_cast<uint2*>(smem_raw + S.bf);          // [ch / 8][kSplit][32] slices of P
   int* fexp = reinterpret_cast<int*>(smem_raw + S.fexp);          // [ch] column scales of P
-  int* rexp = reinterpret_cast<int*>(smem_raw + S.rexp);          // [n] exponent of the largest value of an input row
-  int* rho = reinterpret_cast<int*>(smem_raw + S.rho);            // [16] those of the block's pivot rows
   int* piv = reinterpret_cast<int*>(smem_raw + S.piv);            // [n] pivot row of column k
   int* qinv = reinterpret_cast<int*>(smem_raw + S.qinv);          // [n]
   int* act = reinterpret_cast<int*>(smem_raw + S.act);            // [n] rows in work: all, or those without a pivot
@@ -460,9 +451,15 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
   };
   __shared__ uint4 cand[NW];
   __shared__ int prr[kSW];  // panel rows of the block's pivots
-  __shared__ int s_wild, s_nact, s_sgn;
+  __shared__ unsigned char queue[NW][128];  // a tile's weak elements, 8 row + column
+  __shared__ int s_nact, s_sgn;
 
   double* A = mats + (size_t)b * n * n;
+  // inverse: [16][n] the block's old pivot rows P
+  double* pk = nullptr;
+  if constexpr (kInverse)
+    pk = n <= kSPkMax ? reinterpret_cast<double*>(smem_raw + S.pk)
+                      : reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(binv + (size_t)b * n * n) + 7) & ~(uintptr_t)7);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
   const bool vec = (n & 1) == 0;  // rows of A start on 16 bytes
 
@@ -473,12 +470,6 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
   if (tid == 0) {
     s_nact = n;
     s_sgn = 1;
-  }
-  for (int i = warp; i < n; i += NW) {
-    int e = 0;
-    for (int c = lane; c < n; c += 32) e = max(e, exp_field(dbits(A[(size_t)i * n + c])));
-    e = __reduce_max_sync(0xffffffffu, e);
-    if (lane == 0) rexp[i] = (e == 0 || e == 2047) ? 0 : e - 1023;
   }
   __syncthreads();
 
@@ -509,12 +500,10 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
       }
     }
     if constexpr (C > 1) cg::this_cluster().barrier_arrive();  // the matrix is read as far as this block needs it
-    if (tid == 0) s_wild = 0;
     if (tid < kSW * kSW) tri[(tid / kSW) * kSTd + tid % kSW] = tid / kSW == tid % kSW ? 1.0 : 0.0;
     for (int q = TH + tid; q < kSW * kSW; q += TH) tri[(q / kSW) * kSTd + q % kSW] = q / kSW == q % kSW ? 1.0 : 0.0;
     if (tid < kSW) {
       inv[tid] = 1.0;
-      rho[tid] = 0;
       prr[tid] = -1;
     }
 #pragma unroll
@@ -568,7 +557,6 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
           prr[jj] = rp;
           piv[K0 + jj] = row[m];
           used[row[m]] = blk;
-          rho[jj] = rexp[row[m]];
           pabs[K0 + jj] = fabs(pv);
           if (dbits(pv) >> 63) s_sgn = -s_sgn;
         }
@@ -597,19 +585,10 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
 #pragma unroll
     for (int m = 0; m < R; ++m) {
       if (row[m] < 0 || own[m] >= 0) continue;
-      int e = 0;
-      uint64_t nz = 0;
-#pragma unroll
-      for (int k = 0; k < kSW; ++k) {
-        e = max(e, exp_scaled(dbits(a[m][k]), 0));
-        nz |= dbits(a[m][k]) << 1;
-      }
-      if (!exp_near(e, nz != 0, 200)) atomicOr(&s_wild, 1);
 #pragma unroll
       for (int k = 0; k < kSW; k += 2)
         *reinterpret_cast<double2*>(panel + (tid + TH * m) * kSLd + k) = make_double2(a[m][k], a[m][k + 1]);
     }
-    if (tid < kSW && (rho[tid] > 100 || rho[tid] < -100)) atomicOr(&s_wild, 1);
     // (2)
     if (warp == 0) {
       // lanes 0..15: column `lane` of L11^-1 by forward substitution; lanes 16..31 (inverse): column
@@ -630,14 +609,6 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
 #pragma unroll
         for (int i = s + 1; i < kSW; ++i) x[i] = fma(-l[i], x[s], x[i]);
       }
-      int e = 0;
-      uint64_t nz = 0;
-#pragma unroll
-      for (int i = 0; i < kSW; ++i) {
-        e = max(e, exp_scaled(dbits(x[i]), 0));
-        nz |= dbits(x[i]) << 1;
-      }
-      if ((kInverse || !up) && !exp_near(e, nz != 0, 200)) atomicOr(&s_wild, 1);
       if (!up) {
 #pragma unroll
         for (int i = 0; i < kSW; ++i) xs[i * kSTd + col] = x[i];
@@ -651,8 +622,11 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
       for (int nt = 0; nt < 2; ++nt) {
         uint64_t v[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = dbits(xs[(2 * t + (q & 1) + 8 * (q >> 1)) * kSTd + 8 * nt + g]);
-        split_column_tile(v, rho, xf + nt * kSplit * 32, xe + 8 * nt);
+        for (int q = 0; q < 4; ++q) {
+          const int k = 2 * t + (q & 1) + 8 * (q >> 1), c = 8 * nt + g;
+          v[q] = k == c ? 0ull : dbits(xs[k * kSTd + c]);
+        }
+        split_column_tile(v, xf + nt * kSplit * 32, xe + 8 * nt);
       }
     }
     // this CTA's column blocks from c_lo on: tile nt is half of block jb0 + (nt >> 1) C
@@ -672,143 +646,154 @@ __device__ void gj_split_one(unsigned char* smem_raw, double* __restrict__ mats,
         for (int q = 0; q < 4; ++q) {
           const int k = 2 * t + (q & 1) + 8 * (q >> 1);
           x[q] = (k < w && c < n) ? dbits(A[(size_t)piv[K0 + k] * n + c]) : 0ull;
+          if (kInverse && c < n) pk[(size_t)k * n + c] = __longlong_as_double((long long)x[q]);
         }
-        if (!split_column_tile(x, rho, bf + (size_t)nt * kSplit * 32, fexp + 8 * nt)) atomicOr(&s_wild, 1);
+        split_column_tile(x, bf + (size_t)nt * kSplit * 32, fexp + 8 * nt);
       }
       __syncthreads();
-      if (!s_wild) {
-        // strips of 16 rows in runs of column tiles; as many runs per strip as even out the warps
-        // best (a run's row slices cost about five tiles)
-        const int nstrip = (nact + 15) >> 4;
-        int cs = 1, best = 1 << 30;
-        for (int q = 1; q <= min(ntile, 8); ++q) {
-          const int cost = ((nstrip * q + NW - 1) / NW) * ((ntile + q - 1) / q + 5);
-          if (cost < best) {
-            best = cost;
-            cs = q;
+      // strips of 16 rows in runs of column tiles; as many runs per strip as even out the warps
+      // best (a run's row slices cost about five tiles)
+      const int nstrip = (nact + 15) >> 4;
+      int cs = 1, best = 1 << 30;
+      for (int q = 1; q <= min(ntile, 8); ++q) {
+        const int cost = ((nstrip * q + NW - 1) / NW) * ((ntile + q - 1) / q + 5);
+        if (cost < best) {
+          best = cost;
+          cs = q;
+        }
+      }
+      const int per = (ntile + cs - 1) / cs;
+      for (int task = warp; task < nstrip * cs; task += NW) {
+        const int strip = task % nstrip, run = task / nstrip;
+        const int r0 = strip * 16 + g, r1 = r0 + 8;
+        const int i0 = r0 < nact ? act[r0] : 0, i1 = r1 < nact ? act[r1] : 0;
+        // rows to write; a pivot row of this block starts from zero (inverse) or is done with
+        const bool on0 = r0 < nact && (kInverse || !used[i0]), on1 = r1 < nact && (kInverse || !used[i1]);
+        const bool add0 = on0 && !(kInverse && used[i0] == blk), add1 = on1 && !(kInverse && used[i1] == blk);
+        double* A0 = A + (size_t)i0 * n;
+        double* A1 = A + (size_t)i1 * n;
+        uint32_t as[kSplit][4];
+        int ex[2];
+        float acc[kSplit][4], wt[4];
+        // (3)
+        double u[4][2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          double2 v = make_double2(0.0, 0.0);
+          if ((q & 1) ? on1 : on0)
+            v = *reinterpret_cast<const double2*>(panel + ((q & 1) ? r1 : r0) * kSLd + 2 * t + 8 * (q >> 1));
+          u[q][0] = v.x;
+          u[q][1] = v.y;
+        }
+        split_row_tile(u, as, ex);
+        unsigned weak = 0;  // bit 2 q + e: u[q][e]
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          split_mma(acc, as, xf + nt * kSplit * 32);
+          split_weight(wt, as[0], xf[nt * kSplit * 32 + lane]);
+          const int2 f = *reinterpret_cast<const int2*>(xe + 8 * nt + 2 * t);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            double& l = u[2 * nt + (i >> 1)][i & 1];
+            const int e = ex[i >> 1], fe = (i & 1) ? f.y : f.x;
+            // the diagonal's term counts too: at least 1/16 of the scales
+            if (fe != 0 && split_weak(wt[i], e, fe) && !(e > 0 && fe > 0 && exp_field(dbits(l)) >= e + fe - 1026))
+              weak |= 1u << (4 * nt + i);
+            l = -(l + split_value(acc, i, e, fe));
           }
         }
-        const int per = (ntile + cs - 1) / cs;
-        for (int task = warp; task < nstrip * cs; task += NW) {
-          const int strip = task % nstrip, run = task / nstrip;
-          const int r0 = strip * 16 + g, r1 = r0 + 8;
-          const int i0 = r0 < nact ? act[r0] : 0, i1 = r1 < nact ? act[r1] : 0;
-          // rows to write; a pivot row of this block starts from zero (inverse) or is done with
-          const bool on0 = r0 < nact && (kInverse || !used[i0]), on1 = r1 < nact && (kInverse || !used[i1]);
-          const bool add0 = on0 && !(kInverse && used[i0] == blk), add1 = on1 && !(kInverse && used[i1] == blk);
-          double* A0 = A + (size_t)i0 * n;
-          double* A1 = A + (size_t)i1 * n;
-          uint32_t as[kSplit][4];
-          int ex[2];
-          float acc[kSplit][4];
-          // (3)
-          double u[4][2];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          if (!((weak >> j) & 1u)) continue;
+          const int c = 2 * t + (j & 1) + 8 * (j >> 2);
+          const double* l = panel + (((j >> 1) & 1) ? r1 : r0) * kSLd;
+          double v = -l[c];
+          for (int k = c + 1; k < kSW; ++k) v = fma(-l[k], xs[k * kSTd + c], v);
+          u[j >> 1][j & 1] = v;
+        }
+        if (kInverse && run == 0 && t0 == 0 && (K0 / kSW) % C == cta) {  // the block's columns after the sweep
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            double2 v = make_double2(0.0, 0.0);
-            if ((q & 1) ? on1 : on0)
-              v = *reinterpret_cast<const double2*>(panel + ((q & 1) ? r1 : r0) * kSLd + 2 * t + 8 * (q >> 1));
-            u[q][0] = v.x;
-            u[q][1] = v.y;
+            double* dst = ((q & 1) ? A1 : A0) + K0;
+            const int c = 2 * t + 8 * (q >> 1);
+            if (!((q & 1) ? on1 : on0)) continue;
+            if (c < w) dst[c] = u[q][0];
+            if (c + 1 < w) dst[c + 1] = u[q][1];
           }
-          split_row_tile(u, rho, as, ex);
+        }
+        split_row_tile(u, as, ex);
+        // (4)
+        for (int nt = run * per; nt < min(ntile, (run + 1) * per); ++nt) {
+          const int c0 = tile_col(nt), c = c0 + 2 * t;
+          if (kInverse && (unsigned)(c0 - K0) < (unsigned)kSW) continue;
+          const bool in0 = c < n, in1 = c + 1 < n;
+          double v[4] = {0.0, 0.0, 0.0, 0.0};
+          if (vec) {
+            if (in0 && add0) {
+              const double2 q = *reinterpret_cast<const double2*>(A0 + c);
+              v[0] = q.x;
+              v[1] = q.y;
+            }
+            if (in0 && add1) {
+              const double2 q = *reinterpret_cast<const double2*>(A1 + c);
+              v[2] = q.x;
+              v[3] = q.y;
+            }
+          } else {
+            if (in0 && add0) v[0] = A0[c];
+            if (in1 && add0) v[1] = A0[c + 1];
+            if (in0 && add1) v[2] = A1[c];
+            if (in1 && add1) v[3] = A1[c + 1];
+          }
+          const uint2* bt = bf + (size_t)nt * kSplit * 32;
+          split_mma(acc, as, bt);
+          split_weight(wt, as[0], bt[lane]);
+          const int2 f = *reinterpret_cast<const int2*>(fexp + 8 * nt + 2 * t);
+          v[0] += split_value(acc, 0, ex[0], f.x);
+          v[1] += split_value(acc, 1, ex[0], f.y);
+          v[2] += split_value(acc, 2, ex[1], f.x);
+          v[3] += split_value(acc, 3, ex[1], f.y);
+          const bool k0 = split_weak(wt[0], ex[0], f.x) && on0 && in0, k1 = split_weak(wt[1], ex[0], f.y) && on0 && in1;
+          const bool k2 = split_weak(wt[2], ex[1], f.x) && on1 && in0, k3 = split_weak(wt[3], ex[1], f.y) && on1 && in1;
+          const bool some = __any_sync(0xffffffffu, k0 || k1 || k2 || k3);
+          if (vec && !some) {
+            if (on0 && in0) *reinterpret_cast<double2*>(A0 + c) = make_double2(v[0], v[1]);
+            if (on1 && in0) *reinterpret_cast<double2*>(A1 + c) = make_double2(v[2], v[3]);
+            continue;
+          }
+          if (on0 && in0 && !k0) A0[c] = v[0];
+          if (on0 && in1 && !k1) A0[c + 1] = v[1];
+          if (on1 && in0 && !k2) A1[c] = v[2];
+          if (on1 && in1 && !k3) A1[c + 1] = v[3];
+          if (!some) continue;
+          int cnt = 0;
 #pragma unroll
-          for (int nt = 0; nt < 2; ++nt) {
-            split_mma(acc, as, xf + nt * kSplit * 32);
-            const int2 f = *reinterpret_cast<const int2*>(xe + 8 * nt + 2 * t);
-            u[2 * nt][0] = -split_value(acc, 0, ex[0], f.x);
-            u[2 * nt][1] = -split_value(acc, 1, ex[0], f.y);
-            u[2 * nt + 1][0] = -split_value(acc, 2, ex[1], f.x);
-            u[2 * nt + 1][1] = -split_value(acc, 3, ex[1], f.y);
+          for (int i = 0; i < 4; ++i) {
+            const bool k = i == 0 ? k0 : i == 1 ? k1 : i == 2 ? k2 : k3;
+            const unsigned bal = __ballot_sync(0xffffffffu, k);
+            if (k) queue[warp][cnt + __popc(bal & ((1u << lane) - 1u))] = (unsigned char)(8 * (g + 8 * (i >> 1)) + 2 * t + (i & 1));
+            cnt += __popc(bal);
           }
-          if (kInverse && run == 0 && t0 == 0 && (K0 / kSW) % C == cta) {  // the block's columns after the sweep
+          __syncwarp();
+          for (int q0 = 0; q0 < cnt; q0 += 32) {
+            const bool mine = q0 + lane < cnt;
+            const int code = mine ? queue[warp][q0 + lane] : 0, rr = code >> 3, cc = c0 + (code & 7);
+            const int i = act[strip * 16 + (mine ? rr : 0)];
+            double* dst = A + (size_t)i * n + cc;
+            double s0 = mine && !(kInverse && used[i] == blk) ? *dst : 0.0, s1 = 0.0;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              double* dst = ((q & 1) ? A1 : A0) + K0;
-              const int c = 2 * t + 8 * (q >> 1);
-              if (!((q & 1) ? on1 : on0)) continue;
-              if (c < w) dst[c] = u[q][0];
-              if (c + 1 < w) dst[c + 1] = u[q][1];
+            for (int k = 0; k < kSW; ++k) {
+              const int src = 4 * (rr & 7) + ((k >> 1) & 3);
+              const double ua = __shfl_sync(0xffffffffu, u[2 * (k >> 3)][k & 1], src);
+              const double ub = __shfl_sync(0xffffffffu, u[2 * (k >> 3) + 1][k & 1], src);
+              double p = 0.0;
+              if (mine && k < w) p = kInverse ? pk[(size_t)k * n + cc] : A[(size_t)piv[K0 + k] * n + cc];
+              if (k & 1) s1 = fma(rr < 8 ? ua : ub, p, s1);
+              else s0 = fma(rr < 8 ? ua : ub, p, s0);
             }
+            if (mine) *dst = s0 + s1;
           }
-          split_row_tile(u, rho, as, ex);
-          // (4)
-          for (int nt = run * per; nt < min(ntile, (run + 1) * per); ++nt) {
-            const int c0 = tile_col(nt), c = c0 + 2 * t;
-            if (kInverse && (unsigned)(c0 - K0) < (unsigned)kSW) continue;
-            const bool in0 = c < n, in1 = c + 1 < n;
-            double v[4] = {0.0, 0.0, 0.0, 0.0};
-            if (vec) {
-              if (in0 && add0) {
-                const double2 q = *reinterpret_cast<const double2*>(A0 + c);
-                v[0] = q.x;
-                v[1] = q.y;
-              }
-              if (in0 && add1) {
-                const double2 q = *reinterpret_cast<const double2*>(A1 + c);
-                v[2] = q.x;
-                v[3] = q.y;
-              }
-            } else {
-              if (in0 && add0) v[0] = A0[c];
-              if (in1 && add0) v[1] = A0[c + 1];
-              if (in0 && add1) v[2] = A1[c];
-              if (in1 && add1) v[3] = A1[c + 1];
-            }
-            split_mma(acc, as, bf + (size_t)nt * kSplit * 32);
-            const int2 f = *reinterpret_cast<const int2*>(fexp + 8 * nt + 2 * t);
-            v[0] += split_value(acc, 0, ex[0], f.x);
-            v[1] += split_value(acc, 1, ex[0], f.y);
-            v[2] += split_value(acc, 2, ex[1], f.x);
-            v[3] += split_value(acc, 3, ex[1], f.y);
-            if (vec) {
-              if (on0 && in0) *reinterpret_cast<double2*>(A0 + c) = make_double2(v[0], v[1]);
-              if (on1 && in0) *reinterpret_cast<double2*>(A1 + c) = make_double2(v[2], v[3]);
-            } else {
-              if (on0 && in0) A0[c] = v[0];
-              if (on0 && in1) A0[c + 1] = v[1];
-              if (on1 && in0) A1[c] = v[2];
-              if (on1 && in1) A1[c + 1] = v[3];
-            }
-          }
-        }
-      } else {
-        // (3) and (4) in plain FP64: U takes the place of the panel rows (once per block: bit 1 of
-        // s_wild, which keeps the block's later chunks here), the old pivot rows are staged where
-        // the slices were
-        double* pr = reinterpret_cast<double*>(bf);  // [kSW][ch]
-        __syncthreads();
-        if (!(s_wild & 2)) {
-          for (int r = warp; r < nact; r += NW) {
-            double s = 0.0;
-            if (lane < kSW)
-              for (int k = 0; k < kSW; ++k) s -= panel[r * kSLd + k] * xs[k * kSTd + lane];
-            __syncwarp();
-            if (lane < kSW) {
-              panel[r * kSLd + lane] = s;
-              if (kInverse && lane < w && (K0 / kSW) % C == cta) A[(size_t)act[r] * n + K0 + lane] = s;
-            }
-            __syncwarp();
-          }
-        }
-        const int ncol = 8 * ntile;
-        for (int q = tid; q < w * ncol; q += TH) {
-          const int k = q / ncol, cc = q - k * ncol, c = tile_col(cc >> 3) + (cc & 7);
-          pr[k * ch + cc] = c < n ? A[(size_t)piv[K0 + k] * n + c] : 0.0;
-        }
-        __syncthreads();
-        if (tid == 0) atomicOr(&s_wild, 2);
-        for (int r = warp; r < nact; r += NW) {
-          const int i = act[r];
-          if (!kInverse && used[i]) continue;
-          const bool add = !(kInverse && used[i] == blk);
-          for (int cc = lane; cc < ncol; cc += 32) {
-            const int c = tile_col(cc >> 3) + (cc & 7);
-            if (c >= n || (kInverse && (unsigned)(c - K0) < (unsigned)kSW)) continue;
-            double v = add ? A[(size_t)i * n + c] : 0.0;
-            for (int k = 0; k < w; ++k) v += panel[r * kSLd + k] * pr[k * ch + cc];
-            A[(size_t)i * n + c] = v;
-          }
+          __syncwarp();
         }
       }
       __syncthreads();

@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_phi64(Phi64Args<TH> a) {
     for (int i = 0; i < 4; ++i) {
       const int c = 16 * ks + 2 * t + (i & 1) + 8 * (i >> 1);
       x[i] = (c < h && col < Ne) ? (uint64_t)__double_as_longlong(W[(size_t)c * 2 * Ne + col]) : 0ull;
-      e = max(e, exp_scaled(x[i], 0));
+      e = max(e, exp_field(x[i]));
       nz |= (x[i] << 1) != 0;
     }
 #pragma unroll
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_phi64(Phi64Args<TH> a) {
       e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
       nz |= __shfl_xor_sync(0xffffffffu, nz, off);
     }
-    if (!split_exp_ok(e, nz != 0)) s_plain = 1;
+    if (split_scale(e, nz != 0) == kScaleBad) s_plain = 1;
     if (t == 0) fe[q * 8 + g] = e;
     uint32_t s0[kSplit], s1[kSplit];
     split_pair(split_fixed(x[0], e), split_fixed(x[1], e), s0);
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_phi64(Phi64Args<TH> a) {
           for (int i = 0; i < 4; ++i) {
             const int c = 16 * ks + 2 * t + (i & 1) + 8 * (i >> 1);
             v[i] = (x && c < h) ? (uint64_t)__double_as_longlong((double)x[c]) : 0ull;
-            e = max(e, exp_scaled(v[i], 0));
+            e = max(e, exp_field(v[i]));
             nz |= (v[i] << 1) != 0;
           }
 #pragma unroll
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_phi64(Phi64Args<TH> a) {
             e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
             nz |= __shfl_xor_sync(0xffffffffu, nz, off);
           }
-          if (!split_exp_ok(e, nz != 0)) atomicOr(&s_strip_plain, 1u << st);
+          if (split_scale(e, nz != 0) == kScaleBad) atomicOr(&s_strip_plain, 1u << st);
           if (t == 0) ae[q * 16 + g + 8 * hh] = e;
           uint32_t s0[kSplit], s1[kSplit];
           split_pair(split_fixed(v[0], e), split_fixed(v[1], e), s0);
