@@ -177,9 +177,10 @@ __global__ void __launch_bounds__(kPThreads) k_phi32(Lattice lat, int h, const f
 // two additions and one per 16 channels of every entry instead of h multiply-adds. A CTA keeps the
 // slices of one spin's weights for up to kFTiles / KS column tiles (KS = ceil(h / 16) <= 4) in
 // shared memory and walks over the samples; per sample the slices of up to 16 / KS strips of 16
-// feature rows are built once, then the warps share the (strip, tile) pairs. A strip with an
-// infinity, a NaN or an extreme scale, and every strip when the weights hold one, is taken in plain
-// FP64. (h DFMA an entry: 15.05 ms for 1850 configurations of 224 x 224, h = 32; this 1.35.)
+// feature rows are built once, then the warps share the (strip, tile) pairs. An entry's sum over 16
+// channels that the digits would not carry (split_weak: channels of very different size, large features on
+// small weights and the other way round; an infinity, a NaN or an extreme scale) is taken by FP64
+// multiply-adds. (h DFMA an entry: 15.05 ms for 1850 configurations of 224 x 224, h = 32; this 1.35.)
 constexpr int kFTiles = 28, kFStrips = 16;
 
 template <typename TH>
@@ -232,15 +233,11 @@ __global__ void __launch_bounds__(kPThreads, 2) k_phi64(Phi64Args<TH> a) {
   uint32_t* words = reinterpret_cast<uint32_t*>(psm + S.words);
   int* before = reinterpret_cast<int*>(psm + S.before);
   uint16_t* rows = reinterpret_cast<uint16_t*>(psm + S.rows);
-  __shared__ int s_plain;                             // the weights take the plain path
-  __shared__ unsigned s_strip_plain;                  // bit per strip
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
   const int sp = blockIdx.x / a.chunks, col0 = (blockIdx.x % a.chunks) * a.tiles * 8;
   const int ntile = min(a.tiles, (Ne - col0 + 7) / 8);
   const double* W = a.proj_w + (size_t)sp * Ne;
   const bool vec = (Ne & 1) == 0;
-  if (tid == 0) s_plain = 0;
-  __syncthreads();
   for (int q = warp; q < ntile * KS; q += kPWarps) {
     const int nt = q / KS, ks = q - nt * KS, col = col0 + 8 * nt + g;
     uint64_t x[4];
@@ -257,8 +254,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_phi64(Phi64Args<TH> a) {
       e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
       nz |= __shfl_xor_sync(0xffffffffu, nz, off);
     }
-    if (split_scale(e, nz != 0) == kScaleBad) s_plain = 1;
-    if (t == 0) fe[q * 8 + g] = e;
+    if (t == 0) fe[q * 8 + g] = split_scale(e, nz != 0);
     uint32_t s0[kSplit], s1[kSplit];
     split_pair(split_fixed(x[0], e), split_fixed(x[1], e), s0);
     split_pair(split_fixed(x[2], e), split_fixed(x[3], e), s1);
@@ -284,7 +280,6 @@ __global__ void __launch_bounds__(kPThreads, 2) k_phi64(Phi64Args<TH> a) {
       const int nr = min(16 * per, hi - r0), nstrip = (nr + 15) / 16;
       __syncthreads();  // the previous strips are consumed
       occupied_rows(N, words, before, r0, r0 + nr, rows);
-      if (tid == 0) s_strip_plain = 0u;
       __syncthreads();
       for (int q = warp; q < nstrip * KS; q += kPWarps) {
         const int st = q / KS, ks = q - st * KS;
@@ -307,8 +302,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_phi64(Phi64Args<TH> a) {
             e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
             nz |= __shfl_xor_sync(0xffffffffu, nz, off);
           }
-          if (split_scale(e, nz != 0) == kScaleBad) atomicOr(&s_strip_plain, 1u << st);
-          if (t == 0) ae[q * 16 + g + 8 * hh] = e;
+          if (t == 0) ae[q * 16 + g + 8 * hh] = split_scale(e, nz != 0);
           uint32_t s0[kSplit], s1[kSplit];
           split_pair(split_fixed(v[0], e), split_fixed(v[1], e), s0);
           split_pair(split_fixed(v[2], e), split_fixed(v[3], e), s1);
@@ -332,39 +326,36 @@ __global__ void __launch_bounds__(kPThreads, 2) k_phi64(Phi64Args<TH> a) {
           const int o = i < 2 ? oa : obr, kk = k + (i & 1);
           v[i] = (o >= 0 && kk < Ne) ? a.M0[(size_t)o * Ne + kk] + a.proj_b[sp * Ne + kk] : 0.0;
         }
-        if (!s_plain && !((s_strip_plain >> st) & 1u)) {
-          for (int ks = 0; ks < KS; ++ks) {
-            const uint2* bp = bf + (size_t)(nt * KS + ks) * kSplit * 32 + lane;
-            const uint4* ap = af + (size_t)(st * KS + ks) * kSplit * 32 + lane;
-            uint2 bq[kSplit];
+        for (int ks = 0; ks < KS; ++ks) {
+          const uint2* bp = bf + (size_t)(nt * KS + ks) * kSplit * 32 + lane;
+          const uint4* ap = af + (size_t)(st * KS + ks) * kSplit * 32 + lane;
+          uint2 bq[kSplit];
 #pragma unroll
-            for (int l = 0; l < kSplit; ++l) bq[l] = bp[l * 32];
-            float acc[kSplit][4];
+          for (int l = 0; l < kSplit; ++l) bq[l] = bp[l * 32];
+          float acc[kSplit][4], wt[4];
 #pragma unroll
-            for (int l = 0; l < kSplit; ++l)
+          for (int l = 0; l < kSplit; ++l)
 #pragma unroll
-              for (int i = 0; i < 4; ++i) acc[l][i] = __uint_as_float(kAccBits);
+            for (int i = 0; i < 4; ++i) acc[l][i] = __uint_as_float(kAccBits);
 #pragma unroll
-            for (int sa = 0; sa < kSplit; ++sa) {
-              const uint4 q = ap[sa * 32];
-              const uint32_t aq[4] = {q.x, q.y, q.z, q.w};
+          for (int sa = 0; sa < kSplit; ++sa) {
+            const uint4 q = ap[sa * 32];
+            const uint32_t aq[4] = {q.x, q.y, q.z, q.w};
+            if (sa == 0) split_weight(wt, aq, bq[0]);
 #pragma unroll
-              for (int sb = 0; sa + sb < kSplit; ++sb) mma_f16(acc[sa + sb], aq, bq[sb].x, bq[sb].y);
-            }
-            const int2 f = *reinterpret_cast<const int2*>(fe + (nt * KS + ks) * 8 + 2 * t);
-            const int ea = ae[(st * KS + ks) * 16 + g], eb = ae[(st * KS + ks) * 16 + g + 8];
-            v[0] += split_value(acc, 0, ea, f.x);
-            v[1] += split_value(acc, 1, ea, f.y);
-            v[2] += split_value(acc, 2, eb, f.x);
-            v[3] += split_value(acc, 3, eb, f.y);
+            for (int sb = 0; sa + sb < kSplit; ++sb) mma_f16(acc[sa + sb], aq, bq[sb].x, bq[sb].y);
           }
-        } else {
+          const int2 f = *reinterpret_cast<const int2*>(fe + (nt * KS + ks) * 8 + 2 * t);
+          const int ea = ae[(st * KS + ks) * 16 + g], eb = ae[(st * KS + ks) * 16 + g + 8];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const int o = i < 2 ? oa : obr, kk = k + (i & 1);
-            if (o < 0 || kk >= Ne) continue;
-            const TH* x = Hb + (size_t)(o - sp * N) * h;
-            for (int c = 0; c < h; ++c) v[i] += (double)x[c] * W[(size_t)c * 2 * Ne + kk];
+            const int o = i < 2 ? oa : obr, kk = k + (i & 1), er = i < 2 ? ea : eb, fc = (i & 1) ? f.y : f.x;
+            if (!split_weak(wt[i], er, fc)) {
+              v[i] += split_value(acc, i, er, fc);
+            } else if (o >= 0 && kk < Ne) {
+              const TH* x = Hb + (size_t)(o - sp * N) * h;
+              for (int c = 16 * ks; c < min(h, 16 * ks + 16); ++c) v[i] = fma((double)x[c], W[(size_t)c * 2 * Ne + kk], v[i]);
+            }
           }
         }
 #pragma unroll

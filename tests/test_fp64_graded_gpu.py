@@ -130,3 +130,48 @@ def test_graded_matrices_bit_for_bit_in_every_launch_shape(ne, few, many, kind):
         out.append((*ctx.log_psi(), ctx.ratios(mv[:B].contiguous())))
     for a, b in zip(*out):
         assert torch.equal(torch.nan_to_num(a.double()), torch.nan_to_num(b[:few].double()))
+
+
+@pytest.mark.parametrize("h,spread", [(16, 40), (20, 90), (64, 40), (7, 20)])
+def test_projection_of_channels_of_different_size(h, spread):
+    """Phi = M0 + H W with H's channels times 2^0..2^spread and W's rows times the inverse: sums of terms of one
+    size whose factors differ by `spread` bits. The layer hands the embedding rows on (no kernel, no
+    bias, a residual), so H is the input."""
+    import torch
+    from paper_2604_25775_gb300 import binding as Bd
+    ne, B = 24, 48
+    pb = I.Problem(6, 6, 1, 1, 12, 12, I.MODEL_HUBBARD, 1.0, 0.0, 4.0, 0.0, 1, h, [1], [1], I.ACT_TANH, 1, I.PREC_FP64, 64,
+                   1e-10)
+    rng = np.random.default_rng(h)
+    size = np.ldexp(1.0, rng.integers(0, spread + 1, size=h))
+    params = np.zeros(I.param_count(pb))
+    p = {k: params[o:o + int(np.prod(s))].reshape(s) for k, (o, s) in I.param_offsets(pb).items()}
+    p["embed"][:] = rng.normal(size=(pb.N, 4, h)) * size
+    p["proj_w"][:] = rng.normal(size=(h, 2 * ne)) / size[:, None]
+    M0 = rng.normal(size=(2 * pb.N, ne))
+    occ = I.random_configs(pb, B, 2)
+    ctx = Bd.make_context(pb, params, M0, B)
+    st = torch.empty(B, dtype=torch.int32, device="cuda")
+    ctx.scale_load(torch.from_numpy(occ).cuda(), st)
+    la, sg = (x.cpu().numpy() for x in ctx.log_psi())
+    assert (st.cpu().numpy() == 0).all()
+    err, bound = [], []
+    for b in range(B):
+        res = []
+        for T in (np.longdouble, np.float64):
+            H = p["embed"][np.arange(pb.N), occ[b]].astype(T)
+            rows = []
+            for o in _orbs(occ[b], pb.N):
+                s, i = divmod(o, pb.N)
+                x = M0[o].astype(T)
+                for c in range(h):
+                    x = x + H[i, c] * p["proj_w"][c, s * ne:(s + 1) * ne].astype(T)
+                rows.append(x)
+            res.append(_eliminate(np.stack(rows), 0, T))
+        assert sg[b] == res[0][1]
+        err.append(abs(float(np.longdouble(la[b]) - res[0][0])))
+        bound.append(abs(float(np.longdouble(res[1][0]) - res[0][0])))
+    floor = 2.0 ** -50 * max(1.0, np.abs(la).max())
+    for q, times in ((0.5, 4.0), (0.9, 8.0)):
+        print(f"h {h}: {np.quantile(err, q):.2e} (FP64 {np.quantile(bound, q):.2e}, floor {floor:.2e})")
+        assert np.quantile(err, q) <= times * np.quantile(bound, q) + floor
