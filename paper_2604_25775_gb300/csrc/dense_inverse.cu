@@ -14,7 +14,7 @@
 // so each matrix element is read and written once per block. The matrix stays in global memory
 // (L2-resident while the CTAs in flight fit). Up to 1024 rows (k_gj_split) the update runs on the
 // 16-bit tensor cores as split products; above, where its panel exceeds shared memory, k_gj takes
-// it on the FP64 pipe (8 columns a block, one CTA per matrix).
+// it on the FP64 pipe (8 columns a block, one CTA per matrix; k_gj_cluster eight for the inverses of a list).
 //
 // Pivot choice: largest |value| among unpivoted rows, ties to the lowest row index.
 // Pivoting is implicit (no row swaps); the pivot row of column k is p[k] and the final
@@ -22,6 +22,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "fp64_mma.cuh"
 #include "scale_internal.cuh"
@@ -297,6 +298,246 @@ __global__ void __launch_bounds__(TH) k_gj(TW* __restrict__ mats, int n, const i
     const int s = q / n, cf = q - s * n;
     binv[(size_t)b * n * n + q] = (TOUT)A[(size_t)piv[cf] * n + qinv[s]];
   }
+}
+
+// Inverse mode split over a thread-block cluster of C CTAs per matrix (FP64 working
+// precision). The columns are cut into C contiguous ranges of whole W-column blocks; CTA q
+// owns its range, and only it reads or writes those columns of A. For each block the owner
+// sweeps the W-column panel in its shared memory exactly as k_gj does; after one cluster
+// barrier every CTA copies the swept panel and the block's pivot rows from the owner's
+// shared memory (distributed shared memory) and applies the rank-W update to its own
+// columns. The panel alternates between two buffers, so the owner of the next block can
+// sweep while the others still copy: one cluster barrier per block. A singular panel is told by its
+// block's number, as the others may read the word when the owner is already at the next block. Every
+// element sees the same operations in the same order as in k_gj, so the two kernels give the same bits;
+// the cluster version spreads the O(n^3) FP64 update of one matrix over C SMs, which shortens
+// the refresh of a large matrix (the serial panel steps stay on one SM): 3 matrices of 1100 rows
+// 348 ms by k_gj, 64 here.
+template <typename TOUT, int W, int C>
+__global__ void __launch_bounds__(kThreads) k_gj_cluster(double* __restrict__ mats, int n,
+                                                         const int32_t* __restrict__ list, TOUT* __restrict__ binv,
+                                                         double* __restrict__ logabs_out, int32_t* __restrict__ sign_out,
+                                                         int32_t* __restrict__ status) {
+  extern __shared__ unsigned char smem_raw[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int q = (int)cluster.block_rank();
+  const int mat = blockIdx.x / C;
+  const int b = list ? list[mat] : mat;
+  if (b < 0) return;  // the whole cluster shares mat, so it leaves together
+  double* A = mats + (size_t)b * n * n;
+  const int nblocks = (n + W - 1) / W;
+  const int bpc = (nblocks + C - 1) / C;  // blocks per CTA
+  const int c_lo = min(n, q * bpc * W), c_hi = min(n, (q + 1) * bpc * W);
+  const int ncol = c_hi - c_lo, ldp = bpc * W;
+  double* pabs = reinterpret_cast<double*>(smem_raw);    // [n] |pivot| of the columns this CTA owns
+  double* panels = pabs + n;                             // [2][n][W]
+  double* prow = panels + (size_t)2 * n * W;             // [W][ldp]
+  double* colk = prow + (size_t)W * ldp;                 // [n]
+  double* rowp = colk + n;                               // [W]
+  int* piv = reinterpret_cast<int*>(rowp + W);           // [n]
+  int* qinv = piv + n;                                   // [n]
+  unsigned char* used = reinterpret_cast<unsigned char*>(qinv + n);  // [n]
+  __shared__ unsigned long long red_k[kThreads / 32];
+  __shared__ int red_i[kThreads / 32];
+  __shared__ double s_inv;
+  __shared__ int s_p;
+  __shared__ int s_singular;  // block whose panel is singular (INT_MAX: none)
+  __shared__ int s_sgn;
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < n; i += kThreads) used[i] = 0;
+  if (tid == 0) {
+    s_singular = INT_MAX;
+    s_sgn = 1;
+  }
+  __syncthreads();
+  cluster.sync();  // every CTA of the cluster runs before any reads another's shared memory
+
+  bool singular = false;
+  for (int blk = 0; blk < nblocks; ++blk) {
+    const int K0 = blk * W, w = min(W, n - K0);
+    const int owner = blk / bpc;
+    double* panel = panels + (size_t)(blk & 1) * n * W;
+    if (q == owner) {
+      for (int e = tid; e < n * W; e += kThreads) {
+        const int i = e / W, j = e % W;
+        if (j < w) panel[e] = A[(size_t)i * n + K0 + j];
+      }
+      __syncthreads();
+      for (int jj = 0; jj < w; ++jj) {
+        const int k = K0 + jj;
+        const int bi = pivot_search<double, kThreads>(panel, W, jj, n, used, red_k, red_i);
+        if (tid == 0) {
+          if (bi >= n || !(fabs(panel[bi * W + jj]) > 0.0)) {
+            s_singular = blk;
+          } else {
+            const double pv = panel[bi * W + jj];
+            s_inv = 1.0 / pv;
+            s_p = bi;
+            piv[k] = bi;
+            used[bi] = 1;
+            pabs[k] = fabs(pv);
+            if (pv < 0.0) s_sgn = -s_sgn;
+          }
+        }
+        __syncthreads();
+        if (s_singular == blk) break;
+        const int p = s_p;
+        const double inv = s_inv;
+        for (int j = tid; j < w; j += kThreads) rowp[j] = (j == jj) ? inv : panel[p * W + j] * inv;
+        for (int i = tid; i < n; i += kThreads) colk[i] = panel[i * W + jj];
+        __syncthreads();
+        for (int e = tid; e < n * W; e += kThreads) {
+          const int i = e / W, j = e % W;
+          if (j >= w) continue;
+          if (i == p) {
+            panel[e] = rowp[j];
+          } else {
+            const double f = colk[i];
+            const double base = (j == jj) ? 0.0 : panel[e];
+            panel[e] = base - f * rowp[j];
+          }
+        }
+        __syncthreads();
+      }
+    }
+    cluster.sync();  // the owner's swept panel, pivots and singular flag are visible
+    const int* o_sing = cluster.map_shared_rank(&s_singular, owner);
+    if (*o_sing <= blk) {
+      singular = true;
+      break;
+    }
+    if (q != owner) {
+      const double* o_panel = cluster.map_shared_rank(panel, owner);
+      const int* o_piv = cluster.map_shared_rank(piv, owner);
+      for (int e = tid; e < n * W; e += kThreads)
+        if (e % W < w) panel[e] = o_panel[e];
+      for (int j = tid; j < w; j += kThreads) piv[K0 + j] = o_piv[K0 + j];
+      __syncthreads();
+      for (int j = tid; j < w; j += kThreads) used[piv[K0 + j]] = 1;
+    }
+    // old pivot rows of the block on this CTA's columns (outside the panel)
+    for (int e = tid; e < w * ncol; e += kThreads) {
+      const int j = e / ncol, cc = e - j * ncol;
+      prow[j * ldp + cc] = A[(size_t)piv[K0 + j] * n + c_lo + cc];
+    }
+    __syncthreads();
+    // rank-w update of this CTA's columns outside the panel (the order of k_gj)
+    for (int i = warp; i < n; i += kThreads / 32) {
+      double u[W];
+#pragma unroll
+      for (int j = 0; j < W; ++j) u[j] = (j < w) ? panel[i * W + j] - ((piv[K0 + j] == i) ? 1.0 : 0.0) : 0.0;
+      double* Ai = A + (size_t)i * n;
+      int c = c_lo + lane;
+      for (; c + 32 < c_hi; c += 64) {
+        const int c2 = c + 32;
+        const bool in1 = !(c >= K0 && c < K0 + w);
+        const bool in2 = !(c2 >= K0 && c2 < K0 + w);
+        double a1 = in1 ? Ai[c] : 0.0;
+        double a2 = in2 ? Ai[c2] : 0.0;
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+          if (j < w) {
+            a1 += u[j] * prow[j * ldp + (c - c_lo)];
+            a2 += u[j] * prow[j * ldp + (c2 - c_lo)];
+          }
+        }
+        if (in1) Ai[c] = a1;
+        if (in2) Ai[c2] = a2;
+      }
+      if (c < c_hi && !(c >= K0 && c < K0 + w)) {
+        double a1 = Ai[c];
+#pragma unroll
+        for (int j = 0; j < W; ++j)
+          if (j < w) a1 += u[j] * prow[j * ldp + (c - c_lo)];
+        Ai[c] = a1;
+      }
+    }
+    if (q == owner) {
+      for (int e = tid; e < n * W; e += kThreads) {
+        const int i = e / W, j = e % W;
+        if (j < w) A[(size_t)i * n + K0 + j] = panel[e];
+      }
+    }
+    __syncthreads();
+  }
+  cluster.sync();  // all pivots and flags final: rank 0 gathers the pivots of every block
+  if (q == 0) {
+    // each column's pivot from the CTA that owns its block, summed as in k_gj
+    if (!singular)
+      for (int k = tid; k < n; k += kThreads) pabs[k] = cluster.map_shared_rank(pabs, (k / W) / bpc)[k];
+    __syncthreads();
+    const double logdet = warp == 0 ? sum_log_pivots(pabs, n, singular) : 0.0;
+    if (tid == 0) {
+      double la = logdet;
+      int sg = 1;
+      for (int r = 0; r < C; ++r) sg *= *cluster.map_shared_rank(&s_sgn, r);
+      if (singular) {
+        la = -INFINITY;
+        sg = 0;
+        if (status) status[b] |= SCALE_SAMPLE_SINGULAR;
+      } else {
+        for (int k = 0; k < n; ++k) qinv[k] = 0;
+        int parity = 0;
+        for (int k = 0; k < n; ++k) {
+          if (qinv[k]) continue;
+          int j = k, len = 0;
+          while (!qinv[j]) {
+            qinv[j] = 1;
+            j = piv[j];
+            ++len;
+          }
+          parity += len - 1;
+        }
+        if (parity & 1) sg = -sg;
+      }
+      if (logabs_out) logabs_out[b] = la;
+      if (sign_out) sign_out[b] = sg;
+    }
+  }
+  if (singular) {
+    // zero this CTA's share of the rows of Binv
+    const int r0 = (int)((long long)n * q / C), r1 = (int)((long long)n * (q + 1) / C);
+    for (int e = tid; e < (r1 - r0) * n; e += kThreads) binv[(size_t)b * n * n + (size_t)r0 * n + e] = TOUT(0);
+  } else {
+    // Binv[s][cf] = A^-1[cf][s] = A_final[piv[cf]][col] with s = piv[col], col in this CTA's range
+    for (int e = tid; e < ncol * n; e += kThreads) {
+      const int cc = e / n, cf = e - cc * n, col = c_lo + cc;
+      binv[(size_t)b * n * n + (size_t)piv[col] * n + cf] = (TOUT)A[(size_t)piv[cf] * n + col];
+    }
+  }
+  cluster.sync();  // rank 0 read the others' pivots and signs
+}
+
+template <typename TOUT, int W, int C>
+cudaError_t run_gj_cluster(cudaStream_t st, double* mats, int n, int B, const int32_t* list, TOUT* binv, double* la,
+                           int32_t* sg, int32_t* status) {
+  const int nblocks = (n + W - 1) / W, bpc = (nblocks + C - 1) / C;
+  const size_t smem =
+      sizeof(double) * ((size_t)n + 2 * n * W + (size_t)W * bpc * W + n + W) + sizeof(int) * 2 * n + n + 16;
+  auto kern = k_gj_cluster<TOUT, W, C>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    cudaGetLastError();  // above 1443 rows the panels leave no room
+    return cudaErrorNotSupported;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)B * C);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
+    cudaGetLastError();  // clear; the caller falls back to one CTA per matrix
+    return cudaErrorNotSupported;
+  }
+  return cudaLaunchKernelEx(&cfg, kern, mats, n, list, binv, la, sg, status);
 }
 
 template <typename TW, typename TOUT, bool kInverse, int W, int TH = kThreads>
@@ -961,6 +1202,12 @@ cudaError_t launch_gj(scale_ctx* c, const double* Phi, int n, int B, const int32
     const GjArgs a{c->stream, A, n, B, list, count, expect > 0 ? std::min(expect, B) : B, logabs, sign, status};
     if (!inverse) return gj_split<double, false>(a, nullptr);
     return out_fp64 ? gj_split<double, true>(a, (double*)Binv) : gj_split<float, true>(a, (float*)Binv);
+  }
+  if (inverse && list) {  // a refresh of a few samples is latency-bound
+    const cudaError_t e =
+        out_fp64 ? run_gj_cluster<double, 8, 8>(c->stream, A, n, B, list, (double*)Binv, logabs, sign, status)
+                 : run_gj_cluster<float, 8, 8>(c->stream, A, n, B, list, (float*)Binv, logabs, sign, status);
+    if (e != cudaErrorNotSupported) return e;
   }
   if (inverse)
     return out_fp64 ? run_gj<double, double, true, 8>(c->stream, A, n, B, list, (double*)Binv, logabs, sign, status)
