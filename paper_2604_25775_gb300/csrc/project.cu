@@ -14,11 +14,10 @@ namespace {
 // 2 Ne^2 (2N + 2h) flops a walker, 4 Ne (2N + 2h) bytes written: bound by FP32 FMA. One kernel takes
 // all columns (two read the inverse twice, the projector's with one row a thread). Register tiles of
 // 8 slots x TN columns, 16-byte shared-memory loads along the slots: 5 loads per 48 FMA. Each
-// output is one FMA chain over k ascending. Tiles: 112 x 96 (224 electrons in two, 576 columns in
-// six), or 56 x 160 up to 56 electrons (28 + 28 on 8x8 in one). 1500 walkers of 16x16: 4.82 ms as
-// two kernels, 2.43 here. (On the tensor cores as three TF32 products with rounded additions
-// every 16 terms: 2.33 ms, and the truncation inside the tensor core biased all ratios one way: the
-// error of local energies of well-conditioned walkers grew 1.7-fold.)
+// output is one FMA chain over k ascending, so no result depends on the tile. 1500 walkers of
+// 16x16: 4.82 ms as two kernels, 2.43 here. (On the tensor cores as three TF32 products with rounded
+// additions every 16 terms: 2.33 ms, and the truncation inside the tensor core biased all ratios one way:
+// the error of local energies of well-conditioned walkers grew 1.7-fold.)
 constexpr int kGThreads = 224, kGK = 16;
 
 struct ProjArgs {
@@ -157,11 +156,34 @@ cudaError_t project32(scale_ctx* c, int B, const int32_t* list, const int32_t* c
   const int No = 2 * c->N;
   const ProjArgs a{c->Ne, No, c->h, No + (with_pt ? 2 * c->h : 0), (const float*)c->Binv, (const float*)c->M0b,
                    make_net<float>(c).proj_w, (float*)c->G0t, (float*)c->Pt, list, B, count};
-  if (c->Ne <= 56) return project32_launch<7, 32, 5>(c, a);
+  // A tile's products for rows and columns past the end are not skipped, so the tile is the one of the least
+  // padded area, weighted by the shapes' time per area (112 x 96 and 128 x 84 read the fewest words per FMA).
+  // One-step sweeps, us, 112 x 96 / 56 x 160 / 64 x 140 / 128 x 84, 2048 walkers up to 64 electrons, 1024 up to
+  // 130, 400 above: 8x8 of 56 electrons 299 / 209 / 211 / 300, of 64 318 / 309 / 232 / 320; 16x16 of 112
+  // 557 / 620 / 613 / 616, of 128 1036 / 975 / 711 / 710, of 180 589 / 686 / 538 / 666, of 224
+  // 723 / 856 / 844 / 809, of 256 1132 / 1176 / 973 / 940; 24x24 of 450 3528 / 3934 / 3910 / 3387.
+  struct Tile {
+    int m, n, weight;
+    cudaError_t (*launch)(scale_ctx*, const ProjArgs&);
+  };
+  static constexpr Tile kTiles[] = {{112, 96, 20, project32_launch<14, 16, 6>},
+                                    {56, 160, 22, project32_launch<7, 32, 5>},
+                                    {64, 140, 22, project32_launch<8, 28, 5>},
+                                    {128, 84, 20, project32_launch<16, 14, 6>}};
+  const Tile* best = nullptr;
+  long long least = 0;
+  for (const Tile& t : kTiles) {
+    const long long area = (long long)((c->Ne + t.m - 1) / t.m) * t.m * ((a.ncol + t.n - 1) / t.n) * t.n * t.weight;
+    if (!best || area < least) {
+      best = &t;
+      least = area;
+    }
+  }
   // few walkers: a third of the outputs per thread while the large tiles leave a third of the SMs idle (a
   // one-step sweep of 16x16: 1 walker 92 us against 104, 8 walkers 107 against 111; 12 walkers 128 against 116)
   const long long tiles = (long long)((c->Ne + 111) / 112) * ((a.ncol + 95) / 96) * B;
-  return tiles <= 100 ? project32_launch<7, 32, 2>(c, a) : project32_launch<14, 16, 6>(c, a);
+  if (c->Ne > 56 && tiles <= 100) return project32_launch<7, 32, 2>(c, a);
+  return best->launch(c, a);
 }
 
 // ---- FP64 mode ------------------------------------------------------------------------------
