@@ -108,8 +108,8 @@ __device__ __forceinline__ double sum_log_pivots(const double* pabs, int n, bool
   return part;
 }
 
-// Matrices above 1024 rows. TW: working precision; TOUT: inverse output precision; TH threads per
-// CTA (one matrix).
+// Matrices above 1024 rows, and inverses up to kSmallInverse rows. TW: working precision; TOUT:
+// inverse output precision; TH threads per CTA (one matrix).
 //
 // The FP64 pipe of sm_103a issues one warp-wide DFMA per SM sub-partition about every 64
 // cycles, so the serial part of a pivot step (search, reciprocal, log) is kept off it: the
@@ -1189,6 +1189,11 @@ cudaError_t gj_split(const GjArgs& a, TOUT* binv) {
 
 }  // namespace
 
+// Inverses up to this many rows take k_gj: most of a split block's work is padding and fixed steps (us, k_gj_split / k_gj
+// with 128 threads: n = 8 40 inverses 29 / 18, 8000 354 / 140; n = 14 35 / 34, 431 / 369; n = 17 53 / 45, 784 / 564;
+// n = 24 61 / 58, 898 / 770, but 600 at a time 70 / 84).
+constexpr int kSmallInverse = 20;
+
 // FP64 inverse (out_fp64: Binv in double, else float) or determinant only, for B matrices
 // [B][n][n] stored in Phi (overwritten). count (optional, device): the list is compacted, its
 // first *count entries are taken. expect: how many matrices the caller expects (0: B); it
@@ -1198,6 +1203,9 @@ cudaError_t launch_gj(scale_ctx* c, const double* Phi, int n, int B, const int32
                       int expect) {
   double* A = const_cast<double*>(Phi);
   if (B <= 0) return cudaSuccess;
+  if (inverse && n <= kSmallInverse)
+    return out_fp64 ? run_gj<double, double, true, 8, 128>(c->stream, A, n, B, list, (double*)Binv, logabs, sign, status)
+                    : run_gj<double, float, true, 8, 128>(c->stream, A, n, B, list, (float*)Binv, logabs, sign, status);
   if (n <= kSplitMaxN) {
     const GjArgs a{c->stream, A, n, B, list, count, expect > 0 ? std::min(expect, B) : B, logabs, sign, status};
     if (!inverse) return gj_split<double, false>(a, nullptr);
