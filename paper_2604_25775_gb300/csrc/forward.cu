@@ -92,6 +92,12 @@ __global__ void k_layer0_table(Lattice lat, Net<double> net, const int8_t* __res
   }
 }
 
+// Outputs up to which k_layer takes an FP32 layer: one output per thread then still finds room on the SMs at
+// once, and a tile's 16 outputs are a chain 16 times as long (loads, us, tiles / k_layer: 8x8, h = 32, 64 walkers
+// 110 / 106, 128 walkers 113 / 131; 16x16, h = 32, 16 walkers 108 / 104, 32 walkers 109 / 129). Below 16 tiles a
+// sample most of the tile's block is idle: 4x4, h = 8, 8192 walkers 775 / 756.
+constexpr long long kLayerFew = 160 * 1024;
+
 // The FP32 layer, 4 sites x 4 channels per thread (h % 4 == 0; HC the width as a constant, or 0),
 // in the same order (bias, taps row-major, input channels ascending), so with the same bits.
 // One output per thread issues two loads per multiply-add; the tile eight 16-byte loads per 64.
@@ -523,7 +529,8 @@ cudaError_t forward_t(scale_ctx* c, const int8_t* occ, int B, const int32_t* lis
         k_layer0_table<<<grid, 128, 0, c->stream>>>(c->lat, net, occ, list, out, zo, B, count);
         done = true;
       }
-    } else if (h % 4 == 0) {  // every embedding, kernel and activation row starts on 16 bytes
+    } else if (h % 4 == 0 && ((N + 3) / 4) * (h / 4) >= 16 && (long long)B * N * h > kLayerFew) {
+      // (every embedding, kernel and activation row starts on 16 bytes)
       const dim3 tgrid((((N + 3) / 4) * (h / 4) + 127) / 128, Bgrid);
       if (h == 16) k_layer_tile<16><<<tgrid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);
       else if (h == 32) k_layer_tile<32><<<tgrid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);
