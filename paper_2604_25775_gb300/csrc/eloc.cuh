@@ -153,22 +153,34 @@ size_t eloc_smem(int N) {
 
 template <int H>
 constexpr int kElocWarps = H == 64 ? 16 : 28;  // 64 channels keep 32 activations a lane: registers
-// CTAs per sample for n samples: the number that takes the fewest rounds of moves, ceil(n / slots) / C,
-// with 3% per further CTA for the repeated set-up and enumeration. slots: samples in flight -- one CTA
-// per SM, and clusters of 4 and 8 leave SMs of a GPC over (measured: 38 clusters of 4 and 16 of 8 run
-// as two waves). Local energies do not depend on it. (us, one CTA each / split: 16x16 Hubbard 1
-// walker 665 / 102, 38 walkers 669 / 350, 100 walkers 694 / 542, 333 walkers 1948 / 1760; 64 walkers of
-// 8x8 106 / 61.)
-inline int eloc_split(int n) {
-  constexpr int kSlots[4] = {152, 76, 36, 14};
+// Connected configurations of a sample at the sector's mean densities.
+inline double expected_moves(const scale_ctx* c) {
+  const double fu = (double)c->lat.n_up / c->N, fd = (double)c->lat.n_dn / c->N, bonds = c->nb_nn + c->nb_nnn;
+  if (c->lat.model == SCALE_MODEL_TJ)
+    return 2.0 * bonds * (fu + fd) * (1.0 - fu - fd) + (c->lat.J != 0.0 ? 2.0 * c->nb_nn * fu * fd : 0.0);
+  return 2.0 * bonds * (fu * (1.0 - fu) + fd * (1.0 - fd));
+}
+// CTAs per sample for n samples of `moves` moves: the number of the least time, waves x rounds, in units of
+// one round of moves (a move per warp). Rounds of a sample: 1 up to 0.6 moves per warp (their number varies),
+// 1.1 up to one, then 0.6 + 1.05 per move and warp, the set-up of each CTA included. Waves: samples in flight
+// are one CTA per SM, and clusters of 4 and 8 leave SMs of a GPC over (38 clusters of 4 and 16 of 8 run as
+// two waves); a further wave starts as the last one thins out. FP64: the FP64 pipe is busy with any number
+// of moves, so a CTA's time goes with its share, 3% per further CTA for the repeated set-up. Local energies
+// do not depend on it. (us, C = 1 / 2 / 4 / 8: 16x16 Hubbard 1 walker 677 / 347 / 186 / 107, 40 walkers
+// 720 / 375 / 367 / 310, 100 walkers 725 / 707 / 565 / 719; 8x8 60 walkers 211 / 115 / 129 / 147; 4x4, some 31
+// moves, 14 walkers 38 / 25 / 22 / 22, 40 walkers 39 / 25 / 37 / 52, 100 walkers 40 / 43 / 55 / 112.)
+inline int eloc_split(int n, double moves, int warps, bool fp64) {
   int best = 1;
-  double cost = 1e30;
+  double least = 0.0;
   for (int k = 0; k < 4; ++k) {
     const int C = 1 << k;
-    const double v = (double)((n + kSlots[k] - 1) / kSlots[k]) / C * (1.0 + 0.03 * (C - 1));
-    if (v < cost) {
-      cost = v;
+    const int slots = k == 0 ? 152 : k == 1 ? 76 : k == 2 ? 36 : (fp64 || n <= 14) ? 14 : 16;
+    const int waves = C == 8 && n > 14 ? std::max(2, (n + slots - 1) / slots) : (n + slots - 1) / slots;
+    const double m = moves / (C * warps), rounds = m <= 0.6 ? 1.0 : m <= 1.0 ? 1.1 : 0.6 + 1.05 * m;
+    const double time = fp64 ? waves * (1.0 + 0.03 * (C - 1)) / C : waves == 1 ? rounds : 0.95 * waves * rounds;
+    if (k == 0 || time < least || (!fp64 && time == least)) {
       best = C;
+      least = time;
     }
   }
   return best;
@@ -180,7 +192,7 @@ cudaError_t eloc_launch(scale_ctx* c, const LowrankArgs& a, int n) {
   auto kern = k_eloc<T, H, WARPS, MS>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int C = eloc_split(n);
+  const int C = eloc_split(n, expected_moves(c), WARPS, sizeof(T) == 8);
   if (C > 1) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)n * C);
