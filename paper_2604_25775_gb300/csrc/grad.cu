@@ -746,8 +746,13 @@ cudaError_t grad_t(scale_ctx* c, double* grad, int recompute) {
   int max_taps = 1;
   for (int l = 0; l < L; ++l) max_taps = std::max(max_taps, stencil_taps(net.stencil, net.ksize[l]));
   // one sample's slabs staged in shared memory on small lattices; at 256 sites the 73 KB of slabs
-  // per sample cost more than the L1-served kernels (measured)
-  const bool staged = tiled && N <= kStagedSites && staged_bytes<T>(N, h, max_taps, 2) <= kGradSmemMax &&
+  // per sample cost more than the L1-served kernels (measured). One CTA a sample: in FP64, where the
+  // FP64 pipe of the SMs in use is the limit, a sample of more tiles than a CTA's threads is spread over
+  // several CTAs by the L1-served kernels while fewer than half of the SMs had one (us, staged / L1-served: 66
+  // sites, h = 32, 64 walkers 1519 / 1236, 100 walkers 1517 / 1798; 128 sites, h = 40, 64 walkers 3515 / 2593,
+  // 152 walkers 3541 / 3962; 64 sites, h = 24, 32 walkers 754 / 962).
+  const bool spread = sizeof(T) == 8 && B <= 76 && (N + kConvSites<T> - 1) / kConvSites<T> * (h / 8) > kConvThreads;
+  const bool staged = tiled && !spread && N <= kStagedSites && staged_bytes<T>(N, h, max_taps, 2) <= kGradSmemMax &&
                       conv_bytes<T>(N, h, max_taps) <= kGradSmemMax + 32 * 1024;
   // stored: every layer's input and pre-activation kept from the one forward pass; recompute:
   // only every stride-th layer input, each segment's forward recomputed during the backward
