@@ -531,7 +531,8 @@ cudaError_t forward_t(scale_ctx* c, const int8_t* occ, int B, const int32_t* lis
       }
     } else if (h % 4 == 0 && ((N + 3) / 4) * (h / 4) >= 16 && (long long)B * N * h > kLayerFew) {
       // (every embedding, kernel and activation row starts on 16 bytes)
-      const dim3 tgrid((((N + 3) / 4) * (h / 4) + 127) / 128, Bgrid);
+      dim3 tgrid((((N + 3) / 4) * (h / 4) + 127) / 128);
+      tgrid.y = count ? std::min(B, listed_ctas(tgrid.x)) : B;
       if (h == 16) k_layer_tile<16><<<tgrid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);
       else if (h == 32) k_layer_tile<32><<<tgrid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);
       else k_layer_tile<0><<<tgrid, 128, 0, c->stream>>>(c->lat, net, l, occ, list, in, out, zo, B, count);

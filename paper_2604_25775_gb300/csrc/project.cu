@@ -147,7 +147,8 @@ __global__ void __launch_bounds__(kGThreads, 2) k_project32(ProjArgs a) {
 template <int RG, int CG, int TN>
 cudaError_t project32_launch(scale_ctx* c, const ProjArgs& a) {
   constexpr int M = 8 * RG, N = CG * TN;
-  const dim3 grid((a.Ne + M - 1) / M, (a.ncol + N - 1) / N, a.count ? std::min(a.B, 64) : std::min(a.B, 65535));
+  dim3 grid((a.Ne + M - 1) / M, (a.ncol + N - 1) / N);
+  grid.z = std::min(a.B, a.count ? listed_ctas(grid.x * grid.y) : 65535);
   k_project32<RG, CG, TN><<<grid, kGThreads, 0, c->stream>>>(a);
   return cudaGetLastError();
 }

@@ -20,6 +20,7 @@
 
 #include <cuda_runtime.h>
 #include <math_constants.h>
+#include <algorithm>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -296,6 +297,10 @@ cudaError_t launch_wide_eloc(scale_ctx* c, double* eloc);
 cudaError_t launch_offsets(scale_ctx* c, int B, const int32_t* count, int extra, int64_t* offsets);
 
 // kernels (launch wrappers), each enqueued on ctx->stream
+// Samples in flight of a kernel that walks a compacted list (its count is on the device) with `per` CTAs a sample: 64
+// where a sample fills several SMs, up to 1024 CTAs where it has one or a few (a refresh of 300 walkers of 4x4 with 64
+// of the projector and 256 of the other kernels 141 us, now 102; of 8192 2290 and 978; of 8192 of 8x8 5481 and 4592).
+inline int listed_ctas(unsigned per) { return (int)std::max(64u, 1024u / std::max(1u, per)); }
 // count (optional, device): sample_list is compacted, its first *count entries are used
 cudaError_t launch_forward(scale_ctx* c, const int8_t* occ, int B, const int32_t* sample_list,
                            bool keep_cache, double* phi_out, const int32_t* count = nullptr);

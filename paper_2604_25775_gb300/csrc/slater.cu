@@ -411,7 +411,8 @@ cudaError_t launch_phi(scale_ctx* c, const int8_t* occ, int B, const int32_t* li
   if (proj64) return phi64(c, c->params64 + off_w, c->params64 + off_b, occ, list, (const float*)HL, phi, B, count);
   const int nw = (2 * c->N + 31) / 32;
   const size_t smem = sizeof(float) * kPRows * ((c->h + 3) & ~3) + sizeof(int) * (2 * nw + 1) + 2 * kPRows;
-  const dim3 grid((c->Ne + kPRows - 1) / kPRows, count ? std::min(B, 256) : std::min(B, 65535));
+  dim3 grid((c->Ne + kPRows - 1) / kPRows);
+  grid.y = std::min(B, count ? listed_ctas(grid.x) : 65535);
   k_phi32<<<grid, kPThreads, smem, c->stream>>>(c->lat, c->h, c->params32 + off_w, c->params32 + off_b, c->M0_32, occ, list,
                                                 (const float*)HL, phi, B, count);
   return cudaGetLastError();
