@@ -214,8 +214,9 @@ cudaError_t eloc_launch(scale_ctx* c, const LowrankArgs& a, int n) {
   return cudaGetLastError();
 }
 
-// Launch shape: the most warps per CTA (one CTA per SM) whose move scratch fits shared memory.
-constexpr size_t kElocSmemMax = 227 * 1024;
+// Launch shape: the most warps per CTA (one CTA per SM) whose move scratch fits shared memory beside the
+// kernel's static arrays (WARPS + 2 words).
+constexpr size_t kElocSmemMax = 227 * 1024 - 256;
 template <typename T, int H, typename MS, int W, int... REST>
 cudaError_t eloc_shape(scale_ctx* c, const LowrankArgs& a, int n) {
   if constexpr (sizeof...(REST) == 0) {
