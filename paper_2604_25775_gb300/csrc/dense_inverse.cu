@@ -576,7 +576,7 @@ cudaError_t run_gj(cudaStream_t st, TW* mats, int n, int B, const int32_t* list,
 constexpr int kSW = 16;        // pivots per block = k of one mma
 constexpr int kSLd = kSW + 2;  // panel row stride in doubles: 16-byte rows without bank conflicts
 constexpr int kSTd = kSW + 1;  // row stride of the 16 x 16 blocks
-constexpr int kSCols = 224;    // columns whose slices are staged at a time
+constexpr int kSCols = 256;    // columns whose slices are staged at a time: all of them up to 256 rows
 constexpr int kSColsTall = 128;  // beside a panel of more than 512 rows
 constexpr int kSplitMaxN = 1024;
 constexpr int kSPkMax = 32;    // rows up to which the block of Binv is too small for P
@@ -1132,7 +1132,8 @@ struct GjArgs {
 
 template <typename TOUT, bool kInverse, int TH, int MINB, int R, int C>
 cudaError_t run_gj_split(const GjArgs& a, TOUT* binv) {
-  const int ch = std::min((a.n + 15) & ~15, R == 1 ? kSCols : kSColsTall);
+  // (a determinant's updates leave out the first block)
+  const int ch = std::min(std::max(((a.n + 15) & ~15) - (kInverse ? 0 : kSW), kSW), R == 1 ? kSCols : kSColsTall);
   auto kern = k_gj_split<TOUT, kInverse, TH, MINB, R, C>;
   const size_t smem = split_smem(a.n, ch).total;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
