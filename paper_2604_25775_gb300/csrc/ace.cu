@@ -435,10 +435,10 @@ __global__ void k_ace_embed_split(int N, int h, int per_site, const float* __res
 // a wait ran out. Copying thread t takes the 16-byte piece t % 4 of rows t / 4 and t / 4 + 64 (four lanes a
 // row: 64 contiguous bytes). In the epilogue thread t serves row t % 128, the tile's columns [0, N/2) (warps 0-3)
 // or [N/2, N) (warps 4-7); a warp reads the TMEM lanes of its quarter (warp % 4).
-// What bounds it: the MMAs of a tile are one dependent chain, about 225 cycles each at any N. A block of ACE
-// 16x16 (96 walkers: 192 tiles on 152 SMs, 40 SMs with two) has 486 of them, 55 of its 123 us (180 at first);
-// the rest is the copies' latency, the epilogue and the second tile. A blocked 512 -> 512 layer of two CTAs
-// per SM runs at the tensor pipe's TF32 rate (385 cycles per eight channels of a tile, 435 at the nominal rate).
+// What bounds it: the MMAs of a tile are one dependent chain. A block of ACE 16x16 (96 walkers: 192 tiles on
+// 152 SMs, 40 SMs with two) takes 123 us (180 at first) with the tensor pipe active for 26% of it; the rest is
+// the copies' latency, the epilogue and the second tile. A blocked 512 -> 512 layer, two CTAs per SM, keeps it
+// active for 49%.
 template <int N, bool LN, bool BIN>
 __global__ void __launch_bounds__(kTcThreads, (N > 144 && N < 256 ? 1 : 2)) k_ace_conv_tc(
     Lattice lat, const float* __restrict__ bimg, const float* __restrict__ bias, const float* __restrict__ gam,

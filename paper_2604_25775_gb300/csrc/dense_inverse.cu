@@ -1162,18 +1162,19 @@ cudaError_t run_gj_split(const GjArgs& a, TOUT* binv) {
   return e;
 }
 
-// Launch shapes (inverses of n x n, ms per call on a GB300; "old": every product on the FP64 pipe):
-//   n <= 128: 128 threads, four CTAs per SM. n = 56: 1500 matrices 0.59 (old 2.12).
+// Launch shapes (inverses of Gaussian n x n matrices, ms per call on a GB300; "old": every product on the
+// FP64 pipe):
+//   n <= 128: 128 threads, four CTAs per SM. n = 56: 1500 matrices 0.50 (old 2.12).
 //   n <= 256: many matrices 256 threads, two CTAs per SM, one matrix's panel beside the other's
-//     updates: n = 224, 1500 matrices 8.7 (old 38.3). Up to one per SM 512 threads, whose warps
-//     share the updates: 1.02 alone (1.20 with 256 threads, old 3.83). Up to 32 matrices clusters
-//     of 4 CTAs: 0.69. (Clusters of 4 fill the GPCs' SMs at about 36: 38 matrices 1.37.) Up to 72
-//     clusters of 2, of which 76 run at once: 0.82 (loads of 40 and 72 walkers 1222 -> 1009 and 1292 ->
-//     1081 us; 76 are two waves).
-//   n <= 512: 512 threads; clusters of 4 also pay in two waves: n = 448 alone 2.37 against 5.36,
-//     38 matrices 4.75 against 5.37.
-//   n <= 1024: two panel rows per thread; n = 896: 152 matrices 43.5 (old 189); alone 39.3, in a
-//     cluster of 8 CTAs 8.1 (old cluster of 8 about 30); clusters of 8 run one wave up to 14.
+//     updates: n = 224, 1500 matrices 8.8 (old 38.3; of 16x16 walkers, some of whose products go by FP64
+//     chains, 9.7). Up to one per SM 512 threads, whose warps share the updates: 1.10 alone (1.32 with 256
+//     threads, old 3.83). Up to 32 matrices clusters of 4 CTAs: 0.68. (Clusters of 4 fill the GPCs' SMs at
+//     about 36: 38 matrices 1.36.) Up to 72 clusters of 2, of which 76 run at once: 0.82.
+//   n <= 512: 512 threads; clusters of 4 also pay in two waves: n = 448 alone 2.44 against 6.18,
+//     38 to 64 matrices 4.92 against 6.3.
+//   n <= 1024: two panel rows per thread; n = 896: 152 matrices 50 (old 189); alone 46.9, in a
+//     cluster of 8 CTAs 8.9 (old cluster of 8 about 30); clusters of 8 run one wave up to 14, and 32 to 64
+//     matrices take clusters of 4 (30.5 for 38, 48.7 with one CTA each).
 template <typename TOUT, bool kInverse>
 cudaError_t gj_split(const GjArgs& a, TOUT* binv) {
   if (a.n <= 128) return run_gj_split<TOUT, kInverse, 128, 4, 1, 1>(a, binv);

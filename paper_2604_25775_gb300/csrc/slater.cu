@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kPThreads) k_phi32(Lattice lat, int h, const f
 // feature rows are built once, then the warps share the (strip, tile) pairs. An entry's sum over 16
 // channels that the digits would not carry (split_weak: channels of very different size, large features on
 // small weights and the other way round; an infinity, a NaN or an extreme scale) is taken by FP64
-// multiply-adds. (h DFMA an entry: 15.05 ms for 1850 configurations of 224 x 224, h = 32; this 1.35.)
+// multiply-adds. (h DFMA an entry: 15.05 ms for 1850 configurations of 224 x 224, h = 32; this 1.42.)
 constexpr int kFTiles = 28, kFStrips = 16;
 
 template <typename TH>
